@@ -3,6 +3,7 @@
 // variants is instantiated in a translation unit of its own (sparse_plain.cu, sparse_solve.cu,
 // sparse_cert.cu) so that they compile in parallel.
 #include "sparse_kernel.cuh"
+#include "sparse_step.cuh"
 
 namespace vsa {
 
@@ -25,6 +26,21 @@ size_t sparse_smem_bytes(const Geometry& g, int P, int K_c, bool fused, int thre
 }
 
 int sm_count() { return device_sm_count(); }
+
+// The closed-form family (sparse_step.cuh).  Thread-block size: one block of 512 threads per SM while there are
+// no more units than SMs, two of 256 up to two units per SM, four of 128 beyond (P <= 64: the page selection wants
+// at least P groups of threads).
+int step_threads(const Geometry& g, int P)
+{
+    const long long units = (long long)g.batch * g.n_q_heads;
+    if (units <= sm_count()) return 512;
+    return units > 2 * sm_count() && P <= 64 ? 128 : 256;
+}
+
+size_t step_smem_bytes(const Geometry& g, int P, bool fused)
+{
+    return (size_t)step_layout(step_threads(g, P), g.head_dim, g.max_pages, P, P << g.tile_shift, fused, false).total * 4;
+}
 
 // thread-block size of the per-unit kernel for a launch
 int sparse_block_threads(const Geometry& g, int P, bool solve, bool cert, bool listed, bool two_level = false,
@@ -54,6 +70,7 @@ int sparse_block_threads(const Geometry& g, int P, bool solve, bool cert, bool l
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)
 {
+    if (!solve && !cert && P_super == 0) return step_smem_bytes(g, P, fused) <= (size_t)227 * 1024;
     const int threads = sparse_block_threads(g, P, solve, cert, false, P_super > 0, P_super);
     return sparse_smem_bytes(g, P, K_c, fused, threads, solve, P_super) <= (size_t)227 * 1024;
 }
@@ -68,6 +85,40 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
                           int solver_kind, const int32_t* unit_list, const int32_t* unit_count, int routed_stride,
                           const void* tl_summaries, int P_super, const float* k_scale, const float* v_scale)
 {
+    if ((k_scale || v_scale) && (!k_scale || !v_scale || solve || cert || tl_summaries || g.head_dim != kHeadDim))
+        return cudaErrorInvalidValue;
+    if (g.head_dim != kHeadDim && (solve || cert || tl_summaries)) return cudaErrorInvalidValue;   // (refused by the entry points)
+    if (!solve && !cert && !tl_summaries) {
+        StepParams p;
+        p.geo = g;
+        p.q = (const uint16_t*)q;
+        p.k = (const uint16_t*)k_cache;
+        p.v = (const uint16_t*)v_cache;
+        p.block_table = block_table;
+        p.seq_lens = seq_lens;
+        p.routed_pages = routed_pages;
+        p.page_scores = page_scores;
+        p.P = P;
+        p.K_c = K_c;
+        const int threads = step_threads(g, P);
+        p.lay = step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, page_scores != nullptr, k_scale != nullptr);
+        p.group_shift = 0;
+        while ((1 << p.group_shift) < g.group) ++p.group_shift;
+        p.epsilon = epsilon;
+        p.gap_threshold = gap_threshold;
+        p.out = out;
+        p.diag = diag;
+        p.fallback_list = fallback_list;
+        p.fallback_count = fallback_count;
+        p.solver_iters = 0;
+        p.solve = nullptr;
+        p.k_scale = k_scale;
+        p.v_scale = v_scale;
+        if (k_scale) return launch_step_fp8(p, threads, stream);
+        if (g.head_dim == 64) return launch_step_d64(p, threads, stream);
+        if (g.head_dim == 256) return launch_step_d256(p, threads, stream);
+        return launch_step(p, threads, stream);
+    }
     SparseArgs a;
     a.g = g;
     // no more units than SMs: one larger block per unit (latency shape); otherwise two blocks per SM.
@@ -109,18 +160,10 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
     a.fallback_list = fallback_list;
     a.fallback_count = fallback_count;
     a.stream = stream;
-    if (k_scale || v_scale) {   // fp8 cache
-        if (!k_scale || !v_scale || solve || cert || tl_summaries || g.head_dim != kHeadDim) return cudaErrorInvalidValue;
-        return launch_sparse_plain_fp8(a, threads);
-    }
-    if (g.head_dim != kHeadDim) {
-        if (solve || cert || tl_summaries) return cudaErrorInvalidValue;   // (refused by the entry points)
-        return g.head_dim == 64 ? launch_sparse_plain_d64(a, threads) : launch_sparse_plain_d256(a, threads);
-    }
     if (tl_summaries) return (solve || cert || !page_scores) ? cudaErrorInvalidValue : launch_sparse_two_level(a, threads);
     if (solve) return launch_sparse_solve(a);
     if (cert) return page_scores ? launch_sparse_cert(a, threads) : cudaErrorInvalidValue;
-    return launch_sparse_plain(a, threads);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace vsa

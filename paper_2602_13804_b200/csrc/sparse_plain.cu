@@ -1,12 +1,11 @@
-// Fused sparse pass, closed-form weights: the kernel variants without iterative solve or certificate.
-#include "sparse_kernel.cuh"
+// Fused sparse pass, closed-form weights.
+#include "sparse_step.cuh"
 
 namespace vsa {
 
-cudaError_t launch_sparse_plain(const SparseArgs& a, int threads)
+cudaError_t launch_step(const StepParams& p, int threads, cudaStream_t stream)
 {
-    if (threads == 128) return launch_threads_128<>(a);
-    return threads == 512 ? launch_threads<512, 0, false>(a) : launch_threads<256, 0, false>(a);
+    return launch_step_family<kHeadDim, false>(p, threads, stream);
 }
 
 }  // namespace vsa

@@ -1,13 +1,11 @@
-// Fused sparse pass, closed-form weights, fp8 (e4m3) KV cache.
-#include "sparse_kernel.cuh"
+// Fused sparse pass, closed-form weights, fp8 (e4m3) cache, head dimension 128.
+#include "sparse_step.cuh"
 
 namespace vsa {
 
-cudaError_t launch_sparse_plain_fp8(const SparseArgs& a, int threads)
+cudaError_t launch_step_fp8(const StepParams& p, int threads, cudaStream_t stream)
 {
-    if (threads == 128) return launch_threads_128<kHeadDim, true>(a);
-    return threads == 512 ? launch_threads<512, 0, false, kHeadDim, true>(a)
-                          : launch_threads<256, 0, false, kHeadDim, true>(a);
+    return launch_step_family<kHeadDim, true>(p, threads, stream);
 }
 
 }  // namespace vsa

@@ -1,0 +1,807 @@
+// Fused sparse pass of one (sequence, query head) unit per thread block (paper Sec. 7 steps 2-4, Sec. 8 gap
+// statistic, Cor. 1 leakage bound, Sec. 10.3 fallback flag):
+//   [top-P page selection from the page scores] -> score every valid token of the routed pages -> exact
+//   top-K_c -> weights -> weighted sum of the candidates' value rows -> diagnostics.
+//
+// A unit is a chain of short dependent phases, so what it costs is the number of instructions and block
+// barriers on its longest thread and, since every instruction is executed once or twice per launch, the size
+// of the code (instruction fetch).  Hence: loops that run from memory instead of unrolled register arrays, one
+// template instance for every table width, P and K_c, the rare exact fallbacks out of line, eight barriers.
+//   * Page scores are staged in shared memory (16-byte copies, any table width).  In every warp the r-th largest
+//     of the lanes' maxima, r = ceil(P / warps), has r scores at or above it; the smallest of these over the warps
+//     bounds the P-th best score from below and leaves about 1.6 P scores, which are listed and ranked exactly.
+//   * Routed pages are listed by position, so that the heads of a group walk the pages that they share at about
+//     the same time (L1 and L2 hits).  Ties are decided by (key << 32) | ~position.
+//   * A warp that scored a tile keeps its keys, selects among them and gathers the value rows of the candidates of
+//     its own tiles: no list of the candidates exists across warps.
+//   * Every score is a chain of mixed-precision FMAs on the packed bf16 words (no unpacking).
+// Measured, microseconds per layer before (register-array kernel with seventeen barriers) and after: 15.1 -> 13.1
+// at batch 1, T = 4k with the scan and the empty dense pass; 21.2 -> 17.9 at T = 128k; batch 8, T = 32k 24.6 -> 23.3;
+// 64 sequences of 4k - 128k with 8 heads a group 449 -> 399; batch 32 of short rows at D = 64 44 -> 39.  What bounds it:
+// a tile costs 64 bytes a cycle and SM on the way from L2, then the chain of phases.
+#pragma once
+
+#include <limits.h>
+#include <math.h>
+
+#include <type_traits>
+
+#include "vsa_device.cuh"
+#include "vsa_launch.h"
+#include "vsa_team.cuh"
+
+namespace vsa {
+
+// Shared-memory layout in 4-byte words; every part starts on a 16-byte boundary.
+struct StepLayout {
+    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, work, bt;
+    int tiles_per_group, total;
+    bool stage_bt;   // the block-table row is copied before the wait (blocks that wait for the scan anyway)
+};
+
+// Everything one launch needs.
+struct StepParams {
+    Geometry geo;
+    StepLayout lay;
+    int group_shift;            // log2(query heads per KV head)
+    const uint16_t *q, *k, *v;
+    const int32_t *block_table, *seq_lens;
+    int32_t* routed_pages;
+    const float* page_scores;   // nullptr: routed_pages is an input
+    int P, K_c;
+    float epsilon, gap_threshold;
+    float* out;
+    vsa_diag_t* diag;
+    int32_t *fallback_list, *fallback_count;
+    int solver_iters;
+    vsa_solve_t* solve;
+    const float *k_scale, *v_scale;   // fp8 cache
+};
+
+// one family of instances per translation unit
+cudaError_t launch_step(const StepParams& p, int threads, cudaStream_t stream);        // head dimension 128
+cudaError_t launch_step_d64(const StepParams& p, int threads, cudaStream_t stream);
+cudaError_t launch_step_d256(const StepParams& p, int threads, cudaStream_t stream);
+cudaError_t launch_step_fp8(const StepParams& p, int threads, cudaStream_t stream);    // e4m3 cache
+
+namespace {
+
+constexpr int kStepPages = 512;   // entries of the page list
+constexpr int kStepList = 256;    // entries of the cut bucket's list
+constexpr int kStepBins = 256;    // histogram bins of the token selection
+// control words
+enum : int {
+    kCtlStat = 0,       // 4 words, see publish below
+    kCtlPages = 4,      // listed pages
+    kCtlTokens,         // listed tokens of the cut bucket
+    kCtlOut,            // key of the best rejected token
+    kCtlBad,            // a routed page has no valid pool page
+    kCtlMissing,        // tokens the last page lacks, if it is routed
+    kCtlNp,             // routed pages (when they are an input)
+    kCtlCut,            // (tokens above the cut bucket << 20) | (tokens inside << 8) | bucket
+    kCtlWords = 16
+};
+
+__host__ __device__ constexpr int step_lanes_per_row(int D) { return D / 8; }
+
+inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, bool fused, bool fp8)
+{
+    StepLayout s;
+    const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
+    const int tt = (PT + groups - 1) / groups;
+    s.tiles_per_group = tt;
+    int o = kCtlWords;
+    s.hist = o, o += kStepBins;
+    s.list = o, o += 2 * kStepPages;
+    s.tokens = o, o += 2 * kStepList;
+    s.zeroed = o;
+    s.warp_stat = o, o += 2 * 16;
+    s.misc = o, o += 16;
+    s.win = o, o += (P + 15) & ~15;
+    s.loc = o, o += kStepList;
+    s.tile_off = o, o += 2 * ((PT + 1) & ~1);
+    s.tile_pos = o, o += (PT + 3) & ~3;
+    s.tile_phys = o, o += (PT + 3) & ~3;
+    s.keys = o, o += tt * groups * 16 * (D == 256 ? 2 : 1);   // [round][sub][thread]
+    s.red = o, o += warps * D;
+    s.zred = o, o += (warps + 3) & ~3;
+    s.work = o;
+    // work area: page scores, then the key tiles of the next round, then the lists of value rows (or, in the exact token fallback, the keys in position order)
+    int w = tt * groups * 16 * 4;
+    if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
+    if (tt > 1 && threads * 16 * (fp8 ? 2 : 4) > w) w = threads * 16 * (fp8 ? 2 : 4);
+    o += w;
+    s.bt = o;
+    s.stage_bt = fused && threads >= 256 && max_pages <= 8192;
+    if (s.stage_bt) o += max_pages;
+    s.total = (o + 3) & ~3;
+    return s;
+}
+
+// Exact page selection when the list overflows (many equal scores).  Leaves exactly K entries in list[] and
+// hist[] cleared.  scratch: 16 words + one per warp.
+__device__ __noinline__ void step_pages_exact(const Team& tm, const float* sc, int n, int K, uint32_t* hist,
+                                              uint32_t* scratch, unsigned long long* list, uint32_t* counter)
+{
+    tm.sync();   // every thread has read the counter
+    for (int i = tm.tid; i < kStepPages; i += tm.size) list[i] = 0ull;
+    if (tm.tid == 0) *counter = 0u;
+    tm.sync();
+    auto key = [&](int i) { return float_to_key(sc[i]); };
+    team_exact_topk_slow(tm, key, n, K, hist, scratch, scratch + 16, [&](int i) {
+        list[atomicAdd(counter, 1u)] = ((unsigned long long)key(i) << 32) | (uint32_t)~i;
+    });
+    for (int i = tm.tid; i < kStepBins; i += tm.size) hist[i] = 0u;
+    tm.sync();
+}
+
+// Exact token selection of the R best when the histogram's range is degenerate or its cut bucket crowded: the keys
+// in position order (work[]), then every thread's unselected keys become 0.  Returns the key of the R-th best,
+// which is unselected as well.
+__device__ __noinline__ uint32_t step_tokens_exact(const Team& tm, uint32_t* own_keys, int n_own, const int32_t* tile_pos,
+                                                   int nt, int lanes, int R, uint32_t* hist, uint32_t* scratch, uint32_t* work)
+{
+    const int N = nt * 16;
+    const int tpl = lanes == 8 ? 2 : 1, group = tm.tid / lanes, c = tm.tid % lanes, groups = tm.size / lanes;
+    auto index_of = [&](int o) {   // array index of own key o, or -1 (tiles are in position order)
+        const int slot = (o / tpl) * groups + group;
+        return slot >= nt || (lanes == 32 && (c & 1)) ? -1 : slot * 16 + (lanes == 8 ? 2 * c + o % 2 : lanes == 32 ? c >> 1 : c);
+    };
+    tm.sync();
+    for (int o = 0; o < n_own; ++o) {
+        const int i = index_of(o);
+        if (i >= 0) work[i] = own_keys[o * tm.size + tm.tid];
+    }
+    tm.sync();
+    const TopkResult r = team_exact_topk_slow(tm, [&](int i) { return work[i]; }, N, R, hist, scratch, scratch + 16, [](int) {});
+    for (int o = 0; o < n_own; ++o) {
+        const int i = index_of(o);
+        if (i < 0) continue;
+        const uint32_t k = work[i];
+        if (k < r.kth_key || (k == r.kth_key && i >= r.kth_idx)) own_keys[o * tm.size + tm.tid] = 0u;
+    }
+    tm.sync();
+    return r.kth_key;
+}
+
+// The canonical halving tree over the LPR lanes that hold a row, for the 16 rows of a tile at once.  Lane c ends
+// with rows 2c, 2c + 1 (8 lanes), row c (16) or row c / 2 (32).
+template <int LPR>
+__device__ __forceinline__ void reduce_tile(float (&v)[16], int c)
+{
+    int n = 16;
+#pragma unroll
+    for (int off = LPR / 2; off; off >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool hi = c & off;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (i < n) {
+                    const float send = hi ? v[i] : v[i + n];
+                    const float keep = hi ? v[i + n] : v[i];
+                    v[i] = keep + __shfl_xor_sync(kFullMask, send, off);
+                }
+            }
+        } else {
+            v[0] = v[0] + __shfl_xor_sync(kFullMask, v[0], off);
+        }
+    }
+}
+
+__device__ __noinline__ void step_failed_unit(const Team& tm, const StepParams& p, long long unit, int status, int D,
+                                              bool routed_too)
+{
+    for (int e = tm.tid; e < D; e += tm.size) p.out[unit * D + e] = 0.0f;
+    if (tm.tid == 0) {
+        vsa_diag_t d;
+        d.delta = d.delta12 = d.s_max = d.lse = d.leak_bound = 0.0f;
+        d.n_candidates = 0;
+        d.fallback = 0;
+        d.status = status;
+        p.diag[unit] = d;
+        if (p.solve) p.solve[unit] = vsa_solve_t{0.0f, 0.0f, 0.0f, 0.0f};
+    }
+    if (routed_too)
+        for (int t = tm.tid; t < p.P; t += tm.size) p.routed_pages[unit * p.P + t] = -1;
+}
+
+// Entries of list[0 .. n) that are greater than e, counted by four lanes (part = lane & 3), the total in each of
+// them; list[] is zero up to the next multiple of 32.  All lanes of the warp take part.
+__device__ __forceinline__ int rank_in_list(const unsigned long long* list, int n, unsigned long long e, int part)
+{
+    const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(list) + part;
+    int r0 = 0, r1 = 0;
+#pragma unroll 1
+    for (int j = 0; j < n; j += 32) {
+        ulonglong2 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = l2[j / 2 + 4 * u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            r0 += x[u].x > e;
+            r1 += x[u].y > e;
+        }
+    }
+    r0 += r1;
+    __syncwarp();
+    r0 += __shfl_xor_sync(kFullMask, r0, 1);
+    return r0 + __shfl_xor_sync(kFullMask, r0, 2);
+}
+
+// The same for the position order: entries of win[0 .. n) below l, n padded with INT_MAX to a multiple of 16.
+__device__ __forceinline__ int rank_below(const int32_t* win, int n, int l, int part)
+{
+    const int4* w4 = reinterpret_cast<const int4*>(win) + part;
+    int r0 = 0, r1 = 0;
+#pragma unroll 2
+    for (int j = 0; j < n; j += 16) {
+        const int4 x = w4[j / 4];
+        r0 += (x.x < l) + (x.y < l);
+        r1 += (x.z < l) + (x.w < l);
+    }
+    r0 += r1;
+    __syncwarp();
+    r0 += __shfl_xor_sync(kFullMask, r0, 1);
+    return r0 + __shfl_xor_sync(kFullMask, r0, 2);
+}
+
+// THREADS: 512 (one block per SM) when there are no more units than SMs, 256 (two) up to two units per SM, 128
+//   (four) beyond: a unit is a latency chain, so units in flight count for more than threads per unit.
+// FUSED: the unit's pages are selected here from page_scores; otherwise routed_pages is an input.
+// D: head dimension.  A row is spread over D / 8 lanes, 8 elements (16 bytes; fp8: 8 bytes) each, so a warp works
+//   on 4, 2 or 1 tiles of 16 rows at a time.
+// FP8: k / v hold e4m3 bytes with one scale per (pool page, KV head); strides count bytes.  Scores and weights are
+//   multiplied by the scale afterwards (exact for powers of two).
+template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(const __grid_constant__ StepParams p)
+{
+    constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
+    constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
+    static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
+    extern __shared__ __align__(16) uint32_t smem[];
+    const Geometry& geo = p.geo;
+    const int tid = threadIdx.x;
+    const Team tm{tid, THREADS, 0};   // the whole block
+    const int tsh = geo.tile_shift, P = p.P;
+    const StepLayout& lay = p.lay;
+    uint32_t* ctl = smem;
+    uint32_t* hist = smem + lay.hist;
+    uint32_t* warp_stat = smem + lay.warp_stat;   // page phase: [warp] threshold; token phase: [warp] best two keys
+    unsigned long long* pages = reinterpret_cast<unsigned long long*>(smem + lay.list);
+    unsigned long long* tokens = reinterpret_cast<unsigned long long*>(smem + lay.tokens);
+    int32_t* win = (int32_t*)(smem + lay.win);
+    long long* tile_off = reinterpret_cast<long long*>(smem + lay.tile_off);   // element offset of a tile's first row, -1 = none
+    int32_t* tile_pos = (int32_t*)(smem + lay.tile_pos);                       // its first token's position
+    int32_t* tile_phys = (int32_t*)(smem + lay.tile_phys);                     // its pool page
+    uint32_t* own = smem + lay.keys + tid;                             // this thread's token keys, stride THREADS
+    float* red = (float*)(smem + lay.red);
+    float* zred = (float*)(smem + lay.zred);
+    uint32_t* work = smem + lay.work;
+    int32_t* bt_s = (int32_t*)(smem + lay.bt);
+    const int lane = tid & 31, warp = tid >> 5, c = lane % LPR, grp = tid / LPR;
+    const int h = blockIdx.x, b = blockIdx.y, g = h >> p.group_shift;
+    const long long unit = b * geo.n_q_heads + h;   // (batch * n_q_heads fits 30 bits)
+    const int32_t* bt = p.block_table + (long long)b * geo.max_pages;
+
+    // before the wait on the preceding kernel: the sequence length, the query (the routing kernel that precedes
+    // this one in a step has read both), the block-table row and cleared counters
+    const int T = ld_ca_s32(p.seq_lens + b);
+    const uint4 qraw = ld_nc_16B(p.q + unit * D + c * 8);
+    if (FUSED && lay.stage_bt) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(bt_s);
+        for (int i = tid; i < geo.max_pages; i += THREADS) cp_async_4(dst + 4u * (uint32_t)i, bt + i);
+    }
+    cp_async_commit_group();
+    for (int i = tid; i < lay.zeroed / 4; i += THREADS) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < ((P + 15) & ~15); i += THREADS) win[i] = INT_MAX;
+    const bool length_ok = geo.length_ok(T);
+    const int nb = length_ok ? geo.pages_of(T) : 0;
+    const int r_warp = (P + WARPS - 1) / WARPS;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (!length_ok) {
+        cp_async_wait_all();
+        step_failed_unit(tm, p, unit, VSA_UNIT_BAD_LENGTH, D, FUSED);
+        return;
+    }
+
+    // tiles of a routed page: addresses and positions
+    auto put_page = [&](int slot, int l, int phys) {
+        const bool ok = phys >= 0 && phys < geo.pool_pages;
+        if (!ok) ctl[kCtlBad] = 1u;
+        if (l == nb - 1) ctl[kCtlMissing] = (uint32_t)(nb * geo.page_size - T);
+        for (int hf = 0; hf < (1 << tsh); ++hf) {
+            const int s = (slot << tsh) + hf;
+            tile_off[s] = ok ? (long long)phys * geo.page_stride + (long long)(hf * 16) * geo.token_stride : -1;
+            tile_pos[s] = l * geo.page_size + hf * 16;
+            tile_phys[s] = phys;
+        }
+    };
+
+    int np;
+    if constexpr (FUSED) {
+        // ---- stage the scores of the sequence's pages, four to a chunk; a thread only reads back what it copied.
+        //      Short rows spread over the warps (all of them have to vouch for r_warp scores) ----
+        const float* row = p.page_scores + unit * geo.max_pages;
+        const int mis = (int)((unit * geo.max_pages) & 3), n_chunks = (nb + mis + 3) >> 2;
+        const int chunk0 = n_chunks < THREADS ? lane * WARPS + warp : tid;
+        float* sc = reinterpret_cast<float*>(work);
+        const float4* sc4 = reinterpret_cast<const float4*>(sc);
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sc);
+        for (int i = chunk0; i < n_chunks; i += THREADS) cp_async_16B(dst + 16u * (uint32_t)i, row - mis + 4 * i);
+        cp_async_wait_all();
+        np = min(P, nb);
+        // words of the first and the last chunk that are no scores of this row: NaN fails every comparison
+        if (chunk0 == 0)
+            for (int e = 0; e < mis; ++e) sc[e] = __int_as_float(0x7fffffff);
+        if ((n_chunks - 1) % THREADS == chunk0)
+            for (int e = nb + mis; e < 4 * n_chunks; ++e) sc[e] = __int_as_float(0x7fffffff);
+        // ---- the warp's r-th largest lane maximum ----
+        {
+            float m = -INFINITY;
+#pragma unroll 4
+            for (int i = chunk0; i < n_chunks; i += THREADS) {
+                const float4 v = sc4[i];
+                m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+            }
+            uint32_t v = chunk0 < n_chunks ? float_to_key(m) : 0u, thr = 0u;
+#pragma unroll 1
+            for (int i = 0; i < r_warp; ++i) {
+                thr = __reduce_max_sync(kFullMask, v);
+                const unsigned holders = __ballot_sync(kFullMask, v == thr);
+                if (lane == __ffs(holders) - 1) v = 0u;   // remove one holder of the maximum
+            }
+            if (lane == 0) warp_stat[warp] = thr;   // 0: fewer than r lanes have a score, then every score is listed
+        }
+        __syncthreads();
+        // ---- list every score at or above the smallest of them ----
+        {
+            uint32_t theta_key = 0xffffffffu;
+#pragma unroll
+            for (int w = 0; w < WARPS; w += 4) {
+                const uint4 x = *reinterpret_cast<const uint4*>(warp_stat + w);
+                theta_key = min(theta_key, min(min(x.x, x.y), min(x.z, x.w)));
+            }
+            const float theta = theta_key <= 0x007fffffu ? -INFINITY : key_to_float(theta_key);
+#pragma unroll 1
+            for (int i0 = chunk0; i0 < n_chunks; i0 += 8 * THREADS) {
+                uint32_t hits = 0u;   // four bits per chunk
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int i = i0 + u * THREADS;
+                    if (i < n_chunks) {
+                        const float4 v = sc4[i];
+                        hits |= ((v.x >= theta ? 1u : 0u) | (v.y >= theta ? 2u : 0u) | (v.z >= theta ? 4u : 0u) |
+                                 (v.w >= theta ? 8u : 0u)) << (4 * u);
+                    }
+                }
+                if (hits) {
+                    uint32_t s = atomicAdd(&ctl[kCtlPages], (uint32_t)__popc(hits));
+                    if (s + __popc(hits) <= kStepPages) {
+                        do {
+                            const int bit = __ffs(hits) - 1;
+                            hits &= hits - 1u;
+                            const int i = 4 * (i0 + (bit >> 2) * THREADS) + (bit & 3);
+                            pages[s++] = ((unsigned long long)float_to_key(sc[i]) << 32) | (uint32_t)~(i - mis);
+                        } while (hits);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        int m = (int)ctl[kCtlPages];
+        if (m > kStepPages) {
+            step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, pages, &ctl[kCtlPages]);
+            m = np;
+        }
+        // ---- exact ranks, four lanes per listed page ----
+#pragma unroll 1
+        for (int t0 = 0; t0 < m; t0 += THREADS / 4) {
+            const int t = t0 + (tid >> 2);
+            const unsigned long long e = t < m ? pages[t] : ~0ull;
+            if (t0 + (warp << 3) >= m) break;   // nothing left for this warp
+            const int rank = rank_in_list(pages, m, e, tid & 3);
+            if (t < m && rank < np && (tid & 3) == 0) win[rank] = (int)~(uint32_t)e;
+        }
+        __syncthreads();
+        // ---- routed pages by position ----
+        for (int t = np + tid; t < P; t += THREADS) p.routed_pages[unit * P + t] = -1;
+#pragma unroll 1
+        for (int t0 = 0; t0 < np; t0 += THREADS / 4) {
+            if (t0 + (warp << 3) >= np) break;
+            const int t = t0 + (tid >> 2);
+            const int l = t < np ? win[t] : 0;
+            const int phys = lay.stage_bt ? bt_s[l] : ld_ca_s32(bt + l);
+            const int rank = rank_below(win, np, l, tid & 3);
+            if (t < np && (tid & 3) == 0) {
+                put_page(rank, l, phys);
+                p.routed_pages[unit * P + t] = l;
+            }
+        }
+        __syncthreads();
+    } else {
+        for (int t = tid; t < P; t += THREADS) {
+            const int l = p.routed_pages[unit * P + t];
+            win[t] = l >= 0 && l < nb ? l : INT_MAX;
+        }
+        __syncthreads();
+        for (int t = tid; t < P; t += THREADS) {
+            const int l = win[t];
+            if (l == INT_MAX) continue;
+            const int phys = ld_ca_s32(bt + l);
+            int rank = 0;
+#pragma unroll 4
+            for (int j = 0; j < P; ++j) rank += (int)((win[j] < l) | ((win[j] == l) & (j < t)));
+            put_page(rank, l, phys);
+            atomicAdd(&ctl[kCtlNp], 1u);
+        }
+        __syncthreads();
+        np = (int)ctl[kCtlNp];
+    }
+    if (ctl[kCtlBad]) {
+        step_failed_unit(tm, p, unit, VSA_UNIT_BAD_PAGE, D, false);
+        return;
+    }
+    const int n_valid = np * geo.page_size - (int)ctl[kCtlMissing];   // tokens that get a score
+    const int nt = np << tsh;                                         // their tiles
+    const int rounds = (nt + GROUPS - 1) / GROUPS;
+
+    // ---- token routing: one tile of 16 rows per group of lanes and round ----
+    uint32_t a1 = 0u, a2 = 0u, amin = 0xffffffffu;   // best, second best and smallest key of this thread
+    {
+        // The first tile comes through registers, every later one through shared memory (asynchronous copies that a
+        // lane reads back itself), asked for one round ahead.
+        using Bits = typename std::conditional<FP8, uint2, uint4>::type;
+        constexpr int kElem = FP8 ? 1 : 2;
+        const uint8_t* kbase = reinterpret_cast<const uint8_t*>(p.k) + ((long long)g * geo.head_stride + c * 8) * kElem;
+        const long long stride = (long long)geo.token_stride * kElem;
+        Bits* ring = reinterpret_cast<Bits*>(work) + tid;   // row t at + t * THREADS
+        const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+        auto ahead = [&](int slot) {
+            if (slot < nt) {
+                const uint8_t* src = kbase + tile_off[slot] * kElem;
+#pragma unroll
+                for (int t = 0; t < 16; ++t) {
+                    if constexpr (FP8)
+                        cp_async_8B(ring_s + t * THREADS * 8, src + t * stride);
+                    else
+                        cp_async_16B(ring_s + t * THREADS * 16, src + t * stride);
+                }
+            }
+        };
+#pragma unroll 1
+        for (int r = 0; r < rounds; ++r) {
+            const int slot = r * GROUPS + grp;
+            if (r * GROUPS + warp * GPW >= nt) {   // no tile left for this warp (last round)
+#pragma unroll
+                for (int s = 0; s < TPL; ++s) own[(r * TPL + s) * THREADS] = 0u;
+                break;
+            }
+            const bool active = slot < nt;
+            float kscale = 1.0f;
+            if (FP8 && active) kscale = __ldg(p.k_scale + (long long)tile_phys[slot] * geo.n_kv_heads + g);
+            Bits rows[16];
+            if (r == 0) {
+                const uint8_t* src = kbase + (active ? tile_off[slot] : tile_off[0]) * kElem;
+#pragma unroll
+                for (int t = 0; t < 16; ++t) {
+                    if constexpr (FP8)
+                        rows[t] = ld_nc_8B(src + t * stride);
+                    else
+                        rows[t] = ld_nc_16B(src + t * stride);
+                }
+            } else {
+                cp_async_wait_all();
+#pragma unroll
+                for (int t = 0; t < 16; ++t) rows[t] = ring[t * THREADS];
+            }
+            ahead(slot + GROUPS);
+            float vals[16];
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+                if constexpr (FP8) {
+                    float qf[8], kf[8];
+                    unpack8(qraw, qf);
+                    unpack8_e4m3_mixed(rows[t], kf);
+                    vals[t] = chunk_partial(qf, kf);
+                } else {
+                    vals[t] = chunk_partial_bf16(qraw, rows[t]);
+                }
+            }
+            __syncwarp();
+            reduce_tile<LPR>(vals, c);
+            const int pos = active ? tile_pos[slot] : INT_MAX - 16;
+#pragma unroll
+            for (int s = 0; s < TPL; ++s) {
+                const int tok = LPR == 8 ? 2 * c + s : LPR == 32 ? c >> 1 : c;
+                const bool mine = LPR != 32 || (c & 1) == 0;
+                const float score = FP8 ? __fmul_rn(vals[s], kscale) : vals[s];
+                const uint32_t key = (mine && pos + tok < T) ? float_to_key(score) : 0u;
+                own[(r * TPL + s) * THREADS] = key;
+                a2 = max(a2, min(a1, key));
+                a1 = max(a1, key);
+                amin = min(amin, key != 0u ? key : 0xffffffffu);
+            }
+        }
+    }
+    // Largest and smallest key, and a bracket of the bulk of the scores: the smallest of the warps' largest keys and
+    // the largest of the warps' smallest (the histogram's range; a few outliers do not stretch it).  All four as
+    // maxima, so that lanes 0 .. 3 publish them with one instruction.
+    {
+        const uint32_t wmax = __reduce_max_sync(kFullMask, a1), wmin = __reduce_min_sync(kFullMask, amin);
+        const uint32_t v = lane & 2 ? wmin : wmax;
+        if (lane < 4 && wmax != 0u) atomicMax(&ctl[kCtlStat + lane], lane & 1 ? ~v : v);
+    }
+    __syncthreads();
+    const uint4 stat = *reinterpret_cast<const uint4*>(ctl + kCtlStat);
+    const uint32_t key1 = stat.x;
+    const float s1 = n_valid > 0 ? key_to_float(key1) : -INFINITY;
+    const int ns = min(p.K_c, n_valid);
+    // ---- exact top-(ns + 1): its last element is the best rejected token, the others are the candidates ----
+    const bool has_rejected = n_valid > ns;
+    const int R = ns + 1, n_own = rounds * TPL;
+    int cut = -1, need = 0;   // cut bucket, and how many of its best tokens belong to the top-(ns + 1)
+    float lo = 0.0f, bscale = 0.0f;
+    auto bucket_of = [&](uint32_t key) {
+        return (int)fminf(fmaxf((key_to_float(key) - lo) * bscale, 0.0f), (float)(kStepBins - 1));
+    };
+    if (has_rejected) {
+        float hi = key_to_float(~stat.y);
+        lo = key_to_float(stat.z);
+        if (!(hi > lo)) {
+            hi = s1;
+            lo = key_to_float(~stat.w);
+        }
+        bscale = (float)kStepBins / (hi - lo);
+        bool fast = hi > lo && bscale < INFINITY && hi - lo < INFINITY;
+        if (fast) {
+#pragma unroll 1
+            for (int o = 0; o < n_own; ++o) {
+                const uint32_t key = own[o * THREADS];
+                if (key != 0u) atomicAdd(&hist[bucket_of(key)], 1u);
+            }
+            __syncthreads();
+            // one warp finds the cut: lane j owns bins 8j .. 8j + 7, counts are summed from the top
+            if (warp == 0) {
+                const uint4 na = reinterpret_cast<const uint4*>(hist)[2 * lane], nc = reinterpret_cast<const uint4*>(hist)[2 * lane + 1];
+                const uint32_t n[8] = {na.x, na.y, na.z, na.w, nc.x, nc.y, nc.z, nc.w};
+                uint32_t above[9];   // above[j]: tokens in this lane's bins >= j
+                above[8] = 0u;
+#pragma unroll
+                for (int j = 7; j >= 0; --j) above[j] = above[j + 1] + n[j];
+                uint32_t incl = above[0];
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint32_t o = __shfl_down_sync(kFullMask, incl, off);
+                    if (lane + off < 32) incl += o;
+                }
+                const uint32_t base = incl - above[0];   // tokens in the bins of higher lanes
+                if (base < (uint32_t)R && (uint32_t)R <= incl) {   // exactly one lane
+                    int bin = 0;
+#pragma unroll
+                    for (int j = 1; j < 8; ++j) bin += base + above[j] >= (uint32_t)R;   // the highest bin that reaches R from the top
+                    uint32_t higher = 0u, in_bin = 0u;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (bin == j) higher = above[j + 1], in_bin = n[j];
+                    ctl[kCtlCut] = ((base + higher) << 20) | (in_bin << 8) | (uint32_t)(8 * lane + bin);
+                }
+            }
+            __syncthreads();
+            const uint32_t packed = ctl[kCtlCut];
+            cut = (int)(packed & 255u);
+            need = R - (int)(packed >> 20);
+            fast = ((packed >> 8) & 4095u) <= kStepList;
+        }
+        if (fast) {
+            uint32_t* loc = smem + lay.loc;   // where the listed key lives
+#pragma unroll 2
+            for (int o = 0; o < n_own; ++o) {
+                const uint32_t key = own[o * THREADS];
+                if (key != 0u && bucket_of(key) == cut) {
+                    const int slot = (o / TPL) * GROUPS + grp;
+                    const int pos = tile_pos[slot] + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
+                    const uint32_t i = atomicAdd(&ctl[kCtlTokens], 1u);
+                    tokens[i] = ((unsigned long long)key << 32) | (uint32_t)~pos;
+                    loc[i] = (uint32_t)(o * THREADS + tid);
+                }
+            }
+            __syncthreads();
+            // four lanes rank a listed token; those that do not belong to the candidates lose their key
+            const int m = (int)ctl[kCtlTokens];
+#pragma unroll 1
+            for (int t0 = 0; t0 < m; t0 += THREADS / 4) {
+                if (t0 + (warp << 3) >= m) break;
+                const int t = t0 + (tid >> 2);
+                const unsigned long long e = t < m ? tokens[t] : ~0ull;
+                const int rank = rank_in_list(tokens, m, e, tid & 3);
+                if (t < m && rank >= need - 1 && (tid & 3) == 0) {
+                    smem[lay.keys + loc[t]] = 0u;
+                    if (rank == need - 1) ctl[kCtlOut] = (uint32_t)(e >> 32);
+                }
+            }
+            __syncthreads();
+        } else {
+            cut = -1;
+            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, work);
+            if (tid == 0) ctl[kCtlOut] = k;
+        }
+    }
+
+    // ---- the candidates, compacted for the value gather ----
+    struct __align__(16) Row {
+        long long off;   // element offset of the value row inside its KV head
+        float w;         // weight (fp8: times the scale of the row's page)
+        float pad;
+    };
+    Row* cand = reinterpret_cast<Row*>(work);
+    const float scale = 1.4426950408889634f / p.epsilon;   // log2(e) / epsilon
+    auto is_candidate = [&](uint32_t key) { return key != 0u && (cut < 0 || bucket_of(key) >= cut); };
+    int at = 0;   // first slot of this warp
+    {
+        int mine = 0;
+#pragma unroll 2
+        for (int o = 0; o < n_own; ++o) mine += __popc(__ballot_sync(kFullMask, is_candidate(own[o * THREADS])));
+        if (lane == 0) warp_stat[warp] = (uint32_t)mine;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < WARPS; w += 4) {
+            const uint4 x = *reinterpret_cast<const uint4*>(warp_stat + w);
+            at += (w < warp ? x.x : 0u) + (w + 1 < warp ? x.y : 0u) + (w + 2 < warp ? x.z : 0u) + (w + 3 < warp ? x.w : 0u);
+        }
+    }
+    float z = 0.0f;
+#pragma unroll 2
+    for (int o = 0; o < n_own; ++o) {
+        const uint32_t key = own[o * THREADS];
+        const bool take = is_candidate(key);
+        const unsigned votes = __ballot_sync(kFullMask, take);
+        if (take) {
+            const int slot = (o / TPL) * GROUPS + grp;
+            const int tok = LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c;
+            Row row;
+            row.off = tile_off[slot] + (long long)tok * geo.token_stride;
+            const float w = exp2f((key_to_float(key) - s1) * scale);
+            z += w;
+            row.w = FP8 ? w * __ldg(p.v_scale + (long long)tile_phys[slot] * geo.n_kv_heads + g) : w;
+            row.pad = 0.0f;
+            cand[at + __popc(votes & ((1u << lane) - 1u))] = row;
+        }
+        at += __popc(votes);
+    }
+    __syncthreads();
+
+    // ---- value gather: the candidates dealt out to the groups of lanes, four batches of four rows in flight ----
+    constexpr int UNR = 4;
+    const int n_rows = (ns + GROUPS - 1) / GROUPS;   // of this group of lanes at most; past the end: weight 0
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
+    {
+        constexpr int BATCHES = 4;
+        const uint16_t* vbase = p.v + (long long)g * geo.head_stride + c * 8;
+        const uint8_t* vbase8 = reinterpret_cast<const uint8_t*>(p.v) + (long long)g * geo.head_stride + c * 8;
+        using Bits = typename std::conditional<FP8, uint2, uint4>::type;
+        Bits rows[BATCHES][UNR];
+        float w[BATCHES][UNR];
+        auto fetch = [&](int t, int i) {   // batch t of the registers <- rows i .. i + UNR - 1 of this group
+#pragma unroll
+            for (int u = 0; u < UNR; ++u) {
+                const int j = (i + u) * GROUPS + grp;
+                const Row row = cand[min(j, ns - 1)];
+                w[t][u] = j < ns ? row.w : 0.0f;
+                if constexpr (FP8)
+                    rows[t][u] = ld_nc_8B(vbase8 + row.off);
+                else
+                    rows[t][u] = ld_nc_16B(vbase + row.off);
+            }
+        };
+#pragma unroll
+        for (int t = 0; t < BATCHES; ++t)
+            if (t * UNR < n_rows) fetch(t, t * UNR);
+        // meanwhile: the sum of the weights and the warp's two best keys
+#pragma unroll
+        for (int off = 16; off; off >>= 1) z += __shfl_xor_sync(kFullMask, z, off);
+        const uint32_t best = __reduce_max_sync(kFullMask, a1);
+        const int holder = __ffs(__ballot_sync(kFullMask, a1 == best)) - 1;
+        const uint32_t second = __reduce_max_sync(kFullMask, lane == holder ? a2 : a1);
+        if (lane == 0) {
+            zred[warp] = z;
+            warp_stat[2 * warp] = best;
+            warp_stat[2 * warp + 1] = second;
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int i0 = 0; i0 < n_rows; i0 += BATCHES * UNR)
+#pragma unroll
+            for (int t = 0; t < BATCHES; ++t)
+                if (i0 + t * UNR < n_rows) {
+#pragma unroll
+                    for (int u = 0; u < UNR; ++u) {
+                        float vf[8];
+                        if constexpr (FP8)
+                            unpack8_e4m3_mixed(rows[t][u], vf);
+                        else
+                            unpack8_mixed(rows[t][u], vf);
+#pragma unroll
+                        for (int e = 0; e < 8; e += 2) fma2(acc[e], acc[e + 1], w[t][u], w[t][u], vf[e], vf[e + 1]);
+                    }
+                    if (i0 + (t + BATCHES) * UNR < n_rows) fetch(t, i0 + (t + BATCHES) * UNR);
+                }
+    }
+#pragma unroll
+    for (int off = LPR; off < 32; off <<= 1)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(kFullMask, acc[e], off);
+    if (lane < LPR) {
+        float4* dst = reinterpret_cast<float4*>(red + warp * D + c * 8);
+        dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    }
+    __syncthreads();
+    if (warp >= D / 32 && warp != WARPS - 1) return;
+    float Z = 0.0f;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) Z += zred[w];
+    for (int e = tid; e < D; e += THREADS) {
+        float a = 0.0f;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) a += red[w * D + e];
+        p.out[unit * D + e] = ns > 0 ? a / Z : 0.0f;
+    }
+
+    // ---- diagnostics and fallback flag (the last warp, which has no output row of its own) ----
+    if (warp == WARPS - 1) {
+        // second best key: the best of all but one holder of the best, whose warp offers its own second
+        const uint32_t w1 = lane < WARPS ? warp_stat[2 * lane] : 0u, w2 = lane < WARPS ? warp_stat[2 * lane + 1] : 0u;
+        const int holder = __ffs(__ballot_sync(kFullMask, w1 == key1)) - 1;
+        const uint32_t key2 = __reduce_max_sync(kFullMask, lane == holder ? w2 : w1);
+        if (lane != 0) return;
+        const float s2 = ns > 1 ? key_to_float(key2) : -INFINITY;
+        const float delta = has_rejected ? s1 - key_to_float(ctl[kCtlOut]) : INFINITY;
+        vsa_diag_t d;
+        d.delta = delta;
+        d.delta12 = ns > 0 ? s1 - s2 : INFINITY;
+        d.s_max = s1;
+        d.lse = ns > 0 ? s1 / p.epsilon + logf(Z) : -INFINITY;
+        d.leak_bound = fminf(1.0f, (float)(T - ns) * expf(-delta / p.epsilon));
+        d.n_candidates = ns;
+        d.fallback = (delta < p.gap_threshold && ns < T) ? 1 : 0;
+        d.status = 0;
+        p.diag[unit] = d;
+        if (d.fallback) p.fallback_list[atomicAdd(p.fallback_count, 1)] = (int32_t)unit;
+    }
+}
+
+template <int THREADS, bool FUSED, int D, bool FP8>
+cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
+{
+    static bool attr_done[kMaxDevices] = {};   // per template instance
+    const size_t smem = (size_t)p.lay.total * 4;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8>, attr_done);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8>, dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch),
+                      dim3(THREADS), smem, stream, p);
+}
+
+template <int D, bool FP8>
+cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
+{
+    const bool fused = p.page_scores != nullptr;
+#define VSA_STEP_CASE(T)                                                                    \
+    if (threads == T)                                                                       \
+        return fused ? launch_step_variant<T, true, D, FP8>(p, stream)                      \
+                     : launch_step_variant<T, false, D, FP8>(p, stream);
+    VSA_STEP_CASE(512)
+    VSA_STEP_CASE(256)
+    VSA_STEP_CASE(128)
+#undef VSA_STEP_CASE
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+}  // namespace vsa

@@ -117,6 +117,10 @@ __device__ __forceinline__ void cp_async_16B(uint32_t smem_addr, const void* gpt
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr), "l"(gptr) : "memory");
 }
+__device__ __forceinline__ void cp_async_8B(uint32_t smem_addr, const void* gptr)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr), "l"(gptr) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -151,6 +155,56 @@ __device__ __forceinline__ float chunk_partial(const float (&x)[8], const float 
     fma2(even, odd, x[4], x[5], y[4], y[5]);
     fma2(even, odd, x[6], x[7], y[6], y[7]);
     return even + odd;
+}
+
+// The same chunk straight from the packed bf16 words with mixed-precision FMAs (bf16 x bf16 + fp32, one rounding):
+// no unpacking, which on the integer pipe costs more than the sum itself.  16 chunks per lane take 207 cycles a
+// warp and scheduler against 290 with unpack8 and packed FMAs (both with the loop's 32 other instructions); with
+// four heads sharing an unpacked row 190 against 213, with eight 199 against 190.  The first product starts from
+// +0, so only the sign of a zero can differ.
+__device__ __forceinline__ void fma_bf16_pair(float& even, float& odd, uint32_t x, uint32_t y)
+{
+    asm("{\n\t.reg .b16 xl, xh, yl, yh;\n\tmov.b32 {xl, xh}, %2;\n\tmov.b32 {yl, yh}, %3;\n\t"
+        "fma.rn.f32.bf16 %0, xl, yl, %0;\n\tfma.rn.f32.bf16 %1, xh, yh, %1;\n\t}"
+        : "+f"(even), "+f"(odd)
+        : "r"(x), "r"(y));
+}
+
+__device__ __forceinline__ float chunk_partial_bf16(const uint4& x, const uint4& y)
+{
+    float even = 0.0f, odd = 0.0f;
+    fma_bf16_pair(even, odd, x.x, y.x);
+    fma_bf16_pair(even, odd, x.y, y.y);
+    fma_bf16_pair(even, odd, x.z, y.z);
+    fma_bf16_pair(even, odd, x.w, y.w);
+    return even + odd;
+}
+
+// bf16 -> fp32 with half of the work on the floating-point pipe (x + 0 in mixed precision; -0 becomes +0)
+__device__ __forceinline__ void unpack8_mixed(const uint4& v, float (&f)[8])
+{
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\tadd.rn.f32.bf16 %0, lo, 0f00000000;\n\t}" : "=f"(f[2 * i]) : "r"(w[i]));
+        f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+
+// e4m3 -> fp32, the second step (f16 -> fp32, exact) as a mixed-precision addition instead of a conversion, which
+// runs at a quarter of the rate or less
+__device__ __forceinline__ void unpack8_e4m3_mixed(const uint2& v, float (&f)[8])
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const unsigned short pair = (unsigned short)(((i < 2) ? v.x : v.y) >> (16 * (i & 1)));
+        unsigned int h2;
+        asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"(pair));
+        asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.f16 %0, lo, 0f00000000;\n\t"
+            "add.rn.f32.f16 %1, hi, 0f00000000;\n\t}"
+            : "=f"(f[2 * i]), "=f"(f[2 * i + 1])
+            : "r"(h2));
+    }
 }
 
 // The same tree without any per-lane selection: on entry slot i of lane c holds this lane's partial
