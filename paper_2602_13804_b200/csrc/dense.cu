@@ -153,8 +153,11 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     sm.item_base = (int32_t*)(dense_smem + kRingBytes);
     sm.misc = sm.item_base + n_groups + 1;
     sm.group_mask = (uint8_t*)(sm.misc + 16);
-    pdl_wait();
+    // The list is empty as a rule and the next kernel is what the stream waits for: that one may be scheduled while
+    // this one still waits (0.3 us of a 15.5 us layer at batch 1).  Before its own wait it reads nothing that the
+    // sparse pass, the only kernel it can then overlap, writes.
     pdl_launch_dependents();
+    pdl_wait();
 
     // ---- which heads of which groups are listed? ----
     if (fallback_count) {
