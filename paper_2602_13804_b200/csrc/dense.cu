@@ -25,7 +25,6 @@ namespace vsa {
 
 namespace {
 
-constexpr int kStages = 3;                         // pages in flight per warp
 constexpr int kTileRows = 16;                      // the pass walks tiles of 16 tokens: one per 16-token page, two per 32-token page
 constexpr int kPagesPerItemGoal = 128;             // pages per item and block from which a second round pays
 constexpr int kMaxRounds = 2;
@@ -38,7 +37,10 @@ constexpr int kMaxRoundsRagged = 8;
 // K, 4 KB of V, the four scales) and the tensor cores consume them directly (m16n8k32 e4m3 MMAs).
 template <int D, bool FP8 = false>
 struct DenseCfg {
-    static constexpr int kDenseThreads = D == 256 ? 128 : 256;
+    // fp8: a unit of half the bytes costs the same instructions per token, so the pass is bound by the latency of
+    // each warp's chain: twelve warps with two stages instead of eight with three (254 MB: 100 -> 80 us)
+    static constexpr int kDenseThreads = FP8 ? 384 : D == 256 ? 128 : 256;
+    static constexpr int kStages = FP8 ? 2 : 3;                // units in flight per warp
     static constexpr int kDenseWarps = kDenseThreads / 32;
     static constexpr int kRowBytes = 2 * D;
     static constexpr int kTileBytes = kTileRows * kRowBytes;   // K (or V) rows of one tile and KV head (4 KB at D = 128)
@@ -123,11 +125,11 @@ struct DenseSmem {
     uint8_t* ring;         // [warps][stages][K tile | V tile]; reused for the cross-warp merge
     int32_t* item_base;    // [n_groups + 1] first item of every group (exclusive scan)
     uint8_t* group_mask;   // [n_groups] listed heads of the group
-    int32_t* misc;         // [16]
+    int32_t* misc;         // [32]
 };
 
 template <int G, int D = vsa::kHeadDim, bool FP8 = false>
-__global__ void __launch_bounds__(DenseCfg<D>::kDenseThreads, 1)
+__global__ void __launch_bounds__((DenseCfg<D, FP8>::kDenseThreads), 1)
 dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k_cache,
                    const uint16_t* __restrict__ v_cache, const int32_t* __restrict__ block_table,
                    const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ fallback_list,
@@ -139,7 +141,7 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     using Cfg = DenseCfg<D, FP8>;
     constexpr int kDenseThreads = Cfg::kDenseThreads, kDenseWarps = Cfg::kDenseWarps, kRowBytes = Cfg::kRowBytes,
                   kTileBytes = Cfg::kTileBytes, kStageBytes = Cfg::kStageBytes, kRingBytes = Cfg::kRingBytes,
-                  kPartialFloats = Cfg::kPartialFloats, kMinPagesPerItem = Cfg::kMinPagesPerItem, kHeadDim = D;
+                  kPartialFloats = Cfg::kPartialFloats, kStages = Cfg::kStages, kMinPagesPerItem = Cfg::kMinPagesPerItem, kHeadDim = D;
     constexpr int kUnit = Cfg::kUnitRows;
     constexpr int KS = D / 16;    // 16-element steps of the Q K^T contraction = 16-column steps of P V
     constexpr int NT = D / 8;     // 8-column output tiles
@@ -152,7 +154,7 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     sm.ring = dense_smem;
     sm.item_base = (int32_t*)(dense_smem + kRingBytes);
     sm.misc = sm.item_base + n_groups + 1;
-    sm.group_mask = (uint8_t*)(sm.misc + 16);
+    sm.group_mask = (uint8_t*)(sm.misc + 32);
     // The list is empty as a rule and the next kernel is what the stream waits for: that one may be scheduled while
     // this one still waits (0.3 us of a 15.5 us layer at batch 1).  Before its own wait it reads nothing that the
     // sparse pass, the only kernel it can then overlap, writes.
@@ -175,20 +177,20 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     } else {
         for (int i = tid; i < n_groups; i += kDenseThreads) sm.group_mask[i] = (uint8_t)((1u << G) - 1u);
     }
-    if (tid < 16) sm.misc[tid] = 0;
+    if (tid < 32) sm.misc[tid] = 0;
     __syncthreads();
 
     // ---- pages per item from the amount of flagged work, then the item table ----
-    auto pages_of = [&](int grp) -> int {
-        if (!sm.group_mask[grp]) return 0;
-        const int T = seq_lens[grp / geo.n_kv_heads];
-        if (!geo.length_ok(T)) return 0;
-        return (T + kUnit - 1) / kUnit;
-    };
+    int32_t* group_pages = reinterpret_cast<int32_t*>(sm.ring);   // (the ring is not in use yet; 16 KB at most)
     {
         int pages = 0, groups = 0, longest = 0;
         for (int i = tid; i < n_groups; i += kDenseThreads) {
-            const int p = pages_of(i);
+            int p = 0;
+            if (sm.group_mask[i]) {
+                const int T = seq_lens[i / geo.n_kv_heads];
+                if (geo.length_ok(T)) p = (T + kUnit - 1) / kUnit;
+            }
+            group_pages[i] = p;
             pages += p;
             groups += p > 0;
             longest = max(longest, p);
@@ -236,20 +238,20 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         const int per = (n_groups + kDenseThreads - 1) / kDenseThreads;
         const int lo = tid * per, hi = min(n_groups, lo + per);
         int mine = 0;
-        for (int i = lo; i < hi; ++i) mine += (pages_of(i) + ppi - 1) / ppi;
+        for (int i = lo; i < hi; ++i) mine += (group_pages[i] + ppi - 1) / ppi;
         int incl = mine;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const int o = __shfl_up_sync(kFullMask, incl, off);
             if (lane >= off) incl += o;
         }
-        if (lane == 31) sm.misc[4 + warp] = incl;
+        if (lane == 31) sm.misc[16 + warp] = incl;
         __syncthreads();
         int base = incl - mine;
-        for (int w = 0; w < warp; ++w) base += sm.misc[4 + w];
+        for (int w = 0; w < warp; ++w) base += sm.misc[16 + w];
         for (int i = lo; i < hi; ++i) {
             sm.item_base[i] = base;
-            base += (pages_of(i) + ppi - 1) / ppi;
+            base += (group_pages[i] + ppi - 1) / ppi;
         }
         if (tid == kDenseThreads - 1) sm.item_base[n_groups] = base;
     }
@@ -343,7 +345,25 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         // pages of this warp: first_page + warp, + 8, ...
         const int my_first = first_page + warp;
         const int my_count = my_first < end_page ? (end_page - my_first + kDenseWarps - 1) / kDenseWarps : 0;
+        // fp8: the pool pages of 32 units at a time, one unit per lane (-1: outside the pool, which fails the group's
+        // listed heads); a table load in front of every unit's copies stalls the warp for a trip to L2.  (The bf16 pass
+        // sits at the HBM rate and lost 2 % to it.)
+        int phys0 = 0, phys1 = 0;
+        auto look_up = [&](int k0) {
+            const int pl = my_first + (k0 + lane) * kDenseWarps;
+            auto entry = [&](int tile) {
+                if (k0 + lane >= my_count || tile * kTileRows >= T) return 0;
+                const int ph = bt[tile >> geo.tile_shift];
+                if (ph >= 0 && ph < geo.pool_pages) return ph;
+                sm.misc[13] = 1;   // (cleared at the end of the previous item)
+                return -1;
+            };
+            phys0 = entry(2 * pl);
+            phys1 = entry(2 * pl + 1);
+            __syncwarp();
+        };
         auto issue = [&](int k) {   // k-th unit of this warp into stage k % kStages
+            if (FP8 && (k & 31) == 0) look_up(k);
             const int pl = my_first + k * kDenseWarps;
             const uint32_t dst = ring_addr + (uint32_t)((k % kStages) * kStageBytes);
             if constexpr (FP8) {
@@ -354,10 +374,9 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 for (int hf = 0; hf < 2; ++hf) {
                     const int tile = 2 * pl + hf;
                     const int rows_here = min(kTileRows, T - tile * kTileRows);   // <= 0: the half lies past the sequence
-                    long long phys = rows_here > 0 ? bt[tile >> geo.tile_shift] : -1;
-                    const bool page_ok = phys >= 0 && phys < geo.pool_pages;
-                    if (!page_ok) phys = 0;
-                    const int valid_rows = page_ok ? rows_here : 0;
+                    const int looked_up = __shfl_sync(kFullMask, hf == 0 ? phys0 : phys1, k & 31);
+                    const long long phys = max(looked_up, 0);
+                    const int valid_rows = looked_up >= 0 ? rows_here : 0;
                     const long long off8 = phys * geo.page_stride + (long long)(g / geo.kv_div) * geo.head_stride + ch * 16 +
                                            (long long)((tile & ((1 << geo.tile_shift) - 1)) * kTileRows) * geo.token_stride;
                     const uint8_t* kp = reinterpret_cast<const uint8_t*>(k_cache) + off8;
@@ -378,7 +397,10 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             } else {
             long long phys = bt[pl >> geo.tile_shift];
             const bool page_ok = phys >= 0 && phys < geo.pool_pages;
-            if (!page_ok) phys = 0;
+            if (!page_ok) {
+                phys = 0;
+                sm.misc[13] = 1;   // a page outside the pool: the group's listed heads fail (cleared after the item)
+            }
             const int valid_rows = page_ok ? min(kTileRows, T - pl * kTileRows) : 0;
             const long long head_off = (long long)(g / geo.kv_div) * geo.head_stride + cp_chunk * 8 +
                                        (long long)((pl & ((1 << geo.tile_shift) - 1)) * kTileRows) * geo.token_stride;
@@ -407,16 +429,6 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             if constexpr (FP8) {
             const int pl = my_first + k * kDenseWarps;
             const int valid = min(kUnit, T - pl * kUnit);   // > 0
-            {
-                // a page outside the pool: the group's listed heads fail
-                const long long ph0 = bt[(2 * pl) >> geo.tile_shift];
-                const long long ph1 = valid > kTileRows ? bt[(2 * pl + 1) >> geo.tile_shift] : ph0;
-                if (ph0 < 0 || ph0 >= geo.pool_pages || ph1 < 0 || ph1 >= geo.pool_pages) {
-                    if (lane == 0) sm.misc[13] = 1;   // (cleared at the end of the previous item)
-                    __syncwarp();
-                    continue;
-                }
-            }
             const uint32_t kbase = ring_addr + (uint32_t)((k % kStages) * kStageBytes);
             const uint32_t vbase = kbase + Cfg::kRawBytes;
             const float* scales = reinterpret_cast<const float*>(my_ring + (k % kStages) * kStageBytes + 2 * Cfg::kRawBytes);
@@ -508,14 +520,6 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             } else {
             const int pl = my_first + k * kDenseWarps;
             const int valid = min(kTileRows, T - pl * kTileRows);   // > 0
-            {
-                const long long phys = bt[pl >> geo.tile_shift];   // a page outside the pool: the group's listed heads fail
-                if (phys < 0 || phys >= geo.pool_pages) {
-                    if (lane == 0) sm.misc[13] = 1;   // (cleared at the end of the previous item)
-                    __syncwarp();
-                    continue;
-                }
-            }
             const uint32_t kbase = ring_addr + (uint32_t)((k % kStages) * kStageBytes);
             const uint32_t vbase = kbase + kTileBytes;
 
@@ -682,7 +686,7 @@ size_t dense_smem_bytes(const Geometry& g, bool fp8 = false)
     const size_t ring = fp8 ? DenseCfg<128, true>::kRingBytes
                             : g.head_dim == 64 ? DenseCfg<64>::kRingBytes
                                                : (g.head_dim == 256 ? DenseCfg<256>::kRingBytes : DenseCfg<128>::kRingBytes);
-    return ring + (n_groups + 1) * 4 + 16 * 4 + (n_groups + 15) / 16 * 16;
+    return ring + (n_groups + 1) * 4 + 32 * 4 + (n_groups + 15) / 16 * 16;
 }
 
 }  // namespace
@@ -719,7 +723,7 @@ static cudaError_t launch_dense_gd(const Geometry& g, const uint16_t* q, const u
     const cudaError_t e = allow_large_dynamic_smem(dense_split_kernel<G, D, FP8>, attr_done);
     if (e != cudaSuccess) return e;
     // persistent grid: one block per SM (the ring fills the shared memory)
-    return launch_pdl(dense_split_kernel<G, D, FP8>, dim3((unsigned)num_sms()), dim3(DenseCfg<D>::kDenseThreads), smem,
+    return launch_pdl(dense_split_kernel<G, D, FP8>, dim3((unsigned)num_sms()), dim3(DenseCfg<D, FP8>::kDenseThreads), smem,
                       stream, g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials,
                       counters, out, diag, dense_max_items(g), k_scale, v_scale);
 }
