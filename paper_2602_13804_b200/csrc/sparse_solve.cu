@@ -1,12 +1,17 @@
 // Fused sparse pass with an iterative solve on the candidate set: entropic mirror descent (kind 1) and
-// Frank-Wolfe (kind 2) variants of the kernel, 256 threads.
-#include "sparse_kernel.cuh"
+// Frank-Wolfe (kind 2), 256 threads.
+#include "sparse_step.cuh"
 
 namespace vsa {
 
-cudaError_t launch_sparse_solve(const SparseArgs& a)
+cudaError_t launch_step_solve(const StepParams& p, int kind, cudaStream_t stream)
 {
-    return a.solver_kind == 2 ? launch_threads<256, 2, false>(a) : launch_threads<256, 1, false>(a);
+    const bool fused = p.page_scores != nullptr;
+    if (kind == 2)
+        return fused ? launch_step_variant<256, true, kHeadDim, false, 2>(p, stream)
+                     : launch_step_variant<256, false, kHeadDim, false, 2>(p, stream);
+    return fused ? launch_step_variant<256, true, kHeadDim, false, 1>(p, stream)
+                 : launch_step_variant<256, false, kHeadDim, false, 1>(p, stream);
 }
 
 }  // namespace vsa

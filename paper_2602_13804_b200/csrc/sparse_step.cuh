@@ -26,6 +26,7 @@
 
 #include <type_traits>
 
+#include "step_solve.cuh"
 #include "vsa_device.cuh"
 #include "vsa_launch.h"
 #include "vsa_team.cuh"
@@ -34,7 +35,7 @@ namespace vsa {
 
 // Shared-memory layout in 4-byte words; every part starts on a 16-byte boundary.
 struct StepLayout {
-    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, work, bt;
+    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, cand, solve, work, bt;
     int tiles_per_group, total;
     bool stage_bt;   // the block-table row is copied before the wait (blocks that wait for the scan anyway)
 };
@@ -63,12 +64,15 @@ cudaError_t launch_step(const StepParams& p, int threads, cudaStream_t stream); 
 cudaError_t launch_step_d64(const StepParams& p, int threads, cudaStream_t stream);
 cudaError_t launch_step_d256(const StepParams& p, int threads, cudaStream_t stream);
 cudaError_t launch_step_fp8(const StepParams& p, int threads, cudaStream_t stream);    // e4m3 cache
+cudaError_t launch_step_solve(const StepParams& p, int kind, cudaStream_t stream);     // iterative solves, 256 threads
 
 namespace {
 
 constexpr int kStepPages = 512;   // entries of the page list
 constexpr int kStepList = 256;    // entries of the cut bucket's list
 constexpr int kStepBins = 256;    // histogram bins of the token selection
+// iterative solve: scores and positions of the candidates, weights exchanged inside a warp, the readout
+constexpr int kSolveWords = 3 * VSA_SOLVER_MAX_CANDIDATES + kHeadDim;
 // control words
 enum : int {
     kCtlStat = 0,       // 4 words, see publish below
@@ -84,7 +88,7 @@ enum : int {
 
 __host__ __device__ constexpr int step_lanes_per_row(int D) { return D / 8; }
 
-inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, bool fused, bool fp8)
+inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve)
 {
     StepLayout s;
     const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
@@ -105,11 +109,16 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.keys = o, o += tt * groups * 16 * (D == 256 ? 2 : 1);   // [round][sub][thread]
     s.red = o, o += warps * D;
     s.zred = o, o += (warps + 3) & ~3;
+    s.cand = o, o += 4 * K_c;
+    s.solve = o;
+    if (solve) o += kSolveWords;
     s.work = o;
-    // work area: page scores, then the key tiles of the next round, then the lists of value rows (or, in the exact token fallback, the keys in position order)
-    int w = tt * groups * 16 * 4;
+    // work area: page scores, then the key tiles of the next round, then the candidates' key rows of an iterative solve
+    // or, in the exact token fallback, the keys in position order
+    int w = PT * 16;
     if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
     if (tt > 1 && threads * 16 * (fp8 ? 2 : 4) > w) w = threads * 16 * (fp8 ? 2 : 4);
+    if (solve && ((K_c + 31) & ~31) * 64 > w) w = ((K_c + 31) & ~31) * 64;
     o += w;
     s.bt = o;
     s.stage_bt = fused && threads >= 256 && max_pages <= 8192;
@@ -253,12 +262,14 @@ __device__ __forceinline__ int rank_below(const int32_t* win, int n, int l, int 
 //   on 4, 2 or 1 tiles of 16 rows at a time.
 // FP8: k / v hold e4m3 bytes with one scale per (pool page, KV head); strides count bytes.  Scores and weights are
 //   multiplied by the scale afterwards (exact for powers of two).
-template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false>
+// SOLVE: the weights come from solver_iters entropic (1) or Frank-Wolfe (2) iterations (step_solve.cuh).
+template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(const __grid_constant__ StepParams p)
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
     static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
+    static_assert(SOLVE == 0 || (THREADS == 256 && D == 128 && !FP8), "the solve maps one candidate to each of 256 lanes");
     extern __shared__ __align__(16) uint32_t smem[];
     const Geometry& geo = p.geo;
     const int tid = threadIdx.x;
@@ -635,7 +646,9 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(con
         float w;         // weight (fp8: times the scale of the row's page)
         float pad;
     };
-    Row* cand = reinterpret_cast<Row*>(work);
+    Row* cand = reinterpret_cast<Row*>(smem + lay.cand);
+    float* cand_score = (float*)(smem + lay.solve);                                     // SOLVE only
+    int32_t* cand_pos = (int32_t*)(smem + lay.solve + VSA_SOLVER_MAX_CANDIDATES);
     const float scale = 1.4426950408889634f / p.epsilon;   // log2(e) / epsilon
     auto is_candidate = [&](uint32_t key) { return key != 0u && (cut < 0 || bucket_of(key) >= cut); };
     int at = 0;   // first slot of this warp
@@ -666,11 +679,57 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(con
             z += w;
             row.w = FP8 ? w * __ldg(p.v_scale + (long long)tile_phys[slot] * geo.n_kv_heads + g) : w;
             row.pad = 0.0f;
-            cand[at + __popc(votes & ((1u << lane) - 1u))] = row;
+            const int j = at + __popc(votes & ((1u << lane) - 1u));
+            cand[j] = row;
+            if constexpr (SOLVE != 0) {
+                cand_score[j] = key_to_float(key);
+                cand_pos[j] = tile_pos[slot] + tok;
+            }
         }
         at += __popc(votes);
     }
     __syncthreads();
+
+    float lse_closed = 0.0f;   // log-sum-exp of the closed-form weights (SOLVE only)
+    if constexpr (SOLVE != 0) {
+        // the candidates' key rows once more (L2 hits), then the solve's weights in place of the closed form's
+        if (ns > 0) {
+            uint8_t* tile = reinterpret_cast<uint8_t*>(work);
+            const uint32_t tile_s = (uint32_t)__cvta_generic_to_shared(tile);
+            const uint16_t* kbase = p.k + (long long)g * geo.head_stride + c * 8;
+#pragma unroll 4
+            for (int j = grp; j < ((ns + 31) & ~31); j += GROUPS) {
+                if (j < ns)
+                    cp_async_16B(tile_s + tile_at(j, c), kbase + cand[j].off);
+                else
+                    *reinterpret_cast<uint4*>(tile + tile_at(j, c)) = make_uint4(0u, 0u, 0u, 0u);
+            }
+            cp_async_commit_group();
+            float* spare = (float*)(smem + lay.solve + 2 * VSA_SOLVER_MAX_CANDIDATES);
+            const SolveSmem ss{tile, reinterpret_cast<uint32_t*>(pages), red, spare + VSA_SOLVER_MAX_CANDIDATES, spare};
+            const float s_own = tid < ns ? cand_score[tid] : 0.0f;
+            float z0 = z;
+#pragma unroll
+            for (int off = 16; off; off >>= 1) z0 += __shfl_xor_sync(kFullMask, z0, off);
+            if (lane == 0) zred[warp] = z0;
+            cp_async_wait_all();
+            __syncthreads();
+            if constexpr (SOLVE == 2) {
+                z = solve_frank_wolfe(ss, ns, s_own, tid < ns ? cand_pos[tid] : 0, p.solver_iters, qraw, p.solve + unit);
+                float Z0 = 0.0f;
+#pragma unroll
+                for (int w = 0; w < WARPS; ++w) Z0 += zred[w];
+                lse_closed = s1 / p.epsilon + logf(Z0);
+                __syncthreads();   // zred is rewritten by the value gather
+            } else {
+                z = solve_entropic(ss, ns, s_own, p.solver_iters, p.epsilon, qraw, lse_closed, p.solve + unit);
+            }
+            if (tid < ns) cand[tid].w = z;
+        } else if (tid == 0) {
+            p.solve[unit] = vsa_solve_t{0.0f, 0.0f, 0.0f, 0.0f};
+        }
+        __syncthreads();
+    }
 
     // ---- value gather: the candidates dealt out to the groups of lanes, four batches of four rows in flight ----
     constexpr int UNR = 4;
@@ -764,7 +823,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(con
         d.delta = delta;
         d.delta12 = ns > 0 ? s1 - s2 : INFINITY;
         d.s_max = s1;
-        d.lse = ns > 0 ? s1 / p.epsilon + logf(Z) : -INFINITY;
+        d.lse = ns > 0 ? (SOLVE ? lse_closed : s1 / p.epsilon + logf(Z)) : -INFINITY;
         d.leak_bound = fminf(1.0f, (float)(T - ns) * expf(-delta / p.epsilon));
         d.n_candidates = ns;
         d.fallback = (delta < p.gap_threshold && ns < T) ? 1 : 0;
@@ -774,16 +833,16 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(con
     }
 }
 
-template <int THREADS, bool FUSED, int D, bool FP8>
+template <int THREADS, bool FUSED, int D, bool FP8, int SOLVE = 0>
 cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
 {
     static bool attr_done[kMaxDevices] = {};   // per template instance
     const size_t smem = (size_t)p.lay.total * 4;
     if (smem > 48 * 1024) {
-        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8>, attr_done);
+        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE>, attr_done);
         if (e != cudaSuccess) return e;
     }
-    return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8>, dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch),
+    return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE>, dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch),
                       dim3(THREADS), smem, stream, p);
 }
 

@@ -6,8 +6,8 @@ namespace vsa {
 
 cudaError_t launch_sparse_two_level(const SparseArgs& a, int threads)
 {
-    if (threads == 128) return launch_tok<128, -2, 0, false>(a);
-    return threads == 512 ? launch_tok<512, -2, 0, false>(a) : launch_tok<256, -2, 0, false>(a);
+    if (threads == 128) return launch_tok<128, -2, false>(a);
+    return threads == 512 ? launch_tok<512, -2, false>(a) : launch_tok<256, -2, false>(a);
 }
 
 }  // namespace vsa
