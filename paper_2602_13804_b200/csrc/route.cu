@@ -65,7 +65,9 @@ __device__ __forceinline__ void cp_async_wait()
 // CERT: the radius of every page (radii[page][kv head], see radii_kernel) is copied into logical page
 // order, rad_logical[b][kv head][page], for the certificate that the fused kernel computes.
 // D: head dimension (see sparse_kernel.cuh for how a row of 64 or 256 elements maps to the half-warp's lanes).
-template <int G, bool CERT, int D = kHeadDim>
+// PACKED: the rows stay packed and the dot products are mixed-precision FMAs (a shorter chain); otherwise a row is unpacked
+// once for the heads of the group (fewer FMA-pipe slots).
+template <int G, bool CERT, int D, bool PACKED>
 __global__ void __launch_bounds__(kScanThreads, 2)
 route_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* __restrict__ summaries,
                   const int32_t* __restrict__ block_table, const int32_t* __restrict__ seq_lens,
@@ -149,11 +151,12 @@ route_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
 #pragma unroll
     for (int k = 0; k < kFirstBlocks; ++k)
         if (k < n_blocks) off_tab[k * kBlockPages + lane] = encode(first_entries[k], k * kBlockPages + lane);
-    float qf[G][PIECES][8];
+    float qf[PACKED ? 1 : G][PIECES][8];
+    if constexpr (!PACKED)
 #pragma unroll
-    for (int hh = 0; hh < G; ++hh)
+        for (int hh = 0; hh < G; ++hh)
 #pragma unroll
-        for (int pc = 0; pc < PIECES; ++pc) unpack8(qraw[hh][pc], qf[hh][pc]);
+            for (int pc = 0; pc < PIECES; ++pc) unpack8(qraw[hh][pc], qf[hh][pc]);
     __syncwarp();
 
     const int g_stored = g / geo.kv_div;   // the KV head whose summaries this (possibly virtual) head reads
@@ -215,10 +218,14 @@ route_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
                 const uint4 v = lane_has ? *reinterpret_cast<const uint4*>(src + r * kRowBytes + pc * 256)
                                          : make_uint4(0u, 0u, 0u, 0u);
                 float kf[8];
-                unpack8(v, kf);
+                if constexpr (!PACKED) unpack8(v, kf);
 #pragma unroll
                 for (int hh = 0; hh < G; ++hh) {
-                    const float part = chunk_partial(qf[hh][pc], kf);
+                    float part;
+                    if constexpr (PACKED)
+                        part = chunk_partial_bf16(qraw[hh][pc], v);
+                    else
+                        part = chunk_partial(qf[hh][pc], kf);
                     vals[r * G + hh] = pc == 0 ? part : vals[r * G + hh] + part;
                 }
             }
@@ -462,6 +469,23 @@ int scan_warps_per_block(int warps_per_seq, int batch)
     return best;
 }
 
+template <int G, bool CERT, int D, bool PACKED>
+cudaError_t launch_scan_variant(const dim3& grid, int wpb, int bpw, const Geometry& g, const uint16_t* q,
+                                const uint16_t* summaries, const int32_t* block_table, const int32_t* seq_lens, float* scores,
+                                int32_t* zero_word, int32_t* zero_words, int zero_count, const float* radii,
+                                float* rad_logical, cudaStream_t stream)
+{
+    // The request is padded to 81 KB so that exactly two blocks are resident per SM: with a third one
+    // fewer blocks of the kernel that follows fit beside the scan's to start early, and the step gets
+    // slower although the scan does not (measured: 30.0 against 24.8 us per layer at batch 8, T = 32k).
+    const size_t smem = std::max((size_t)kScanWarps * ScanCfg<G, D>::WARP_BYTES, (size_t)81 * 1024);
+    static bool attr_done[kMaxDevices] = {};   // per template instance
+    const cudaError_t e = allow_large_dynamic_smem(route_scan_kernel<G, CERT, D, PACKED>, attr_done);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(route_scan_kernel<G, CERT, D, PACKED>, grid, dim3(wpb * 32), smem, stream, g, q, summaries,
+                      block_table, seq_lens, scores, bpw, zero_word, zero_words, zero_count, radii, rad_logical);
+}
+
 template <int G, bool CERT, int D = kHeadDim>
 cudaError_t launch_scan_g(const Geometry& g, const uint16_t* q, const uint16_t* summaries, const int32_t* block_table,
                           const int32_t* seq_lens, float* scores, int32_t* zero_word, int32_t* zero_words,
@@ -488,15 +512,13 @@ cudaError_t launch_scan_g(const Geometry& g, const uint16_t* q, const uint16_t* 
     const int warps = slices * g.n_kv_heads;
     const int wpb = scan_warps_per_block(warps, g.batch);
     const dim3 grid((unsigned)((warps + wpb - 1) / wpb), (unsigned)g.batch);
-    // The request is padded to 81 KB so that exactly two blocks are resident per SM: with a third one
-    // fewer blocks of the kernel that follows fit beside the scan's to start early, and the step gets
-    // slower although the scan does not (measured: 30.0 against 24.8 us per layer at batch 8, T = 32k).
-    const size_t smem = std::max((size_t)kScanWarps * ScanCfg<G, D>::WARP_BYTES, (size_t)81 * 1024);
-    static bool attr_done[kMaxDevices] = {};   // per template instance
-    const cudaError_t e = allow_large_dynamic_smem(route_scan_kernel<G, CERT, D>, attr_done);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(route_scan_kernel<G, CERT, D>, grid, dim3(wpb * 32), smem, stream, g, q, summaries,
-                      block_table, seq_lens, scores, bpw, zero_word, zero_words, zero_count, radii, rad_logical);
+    // A grid of one wave is bound by the chain of a warp, longer ones by the FMA pipe: batch 1, T = 4k 0.4 us less with
+    // packed rows, batch 8, T = 32k 0.6 us less (one sequence of 128k tokens 0.1 us more); batch 16, T = 128k, several waves, 1.2 us more.
+    if ((long long)grid.x * grid.y <= 2LL * device_sm_count())
+        return launch_scan_variant<G, CERT, D, true>(grid, wpb, bpw, g, q, summaries, block_table, seq_lens, scores, zero_word,
+                                                     zero_words, zero_count, radii, rad_logical, stream);
+    return launch_scan_variant<G, CERT, D, false>(grid, wpb, bpw, g, q, summaries, block_table, seq_lens, scores, zero_word,
+                                                  zero_words, zero_count, radii, rad_logical, stream);
 }
 
 }  // namespace
