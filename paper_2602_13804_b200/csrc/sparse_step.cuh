@@ -94,11 +94,14 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
     const int tt = (PT + groups - 1) / groups;
     s.tiles_per_group = tt;
+    const int keys = tt * groups * 16 * (D == 256 ? 2 : 1);   // [round][sub][thread]
     int o = kCtlWords;
     s.hist = o, o += kStepBins;
-    s.list = o, o += 2 * kStepPages;
     s.tokens = o, o += 2 * kStepList;
-    s.zeroed = o;
+    s.list = o;
+    s.zeroed = s.list + 2 * kStepPages;
+    s.keys = o;   // the page list is dead when the first token key is written
+    o += keys > 2 * kStepPages ? keys : 2 * kStepPages;
     s.warp_stat = o, o += 2 * 16;
     s.misc = o, o += 16;
     s.win = o, o += (P + 15) & ~15;
@@ -106,16 +109,22 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.tile_off = o, o += 2 * ((PT + 1) & ~1);
     s.tile_pos = o, o += (PT + 3) & ~3;
     s.tile_phys = o, o += (PT + 3) & ~3;
-    s.keys = o, o += tt * groups * 16 * (D == 256 ? 2 : 1);   // [round][sub][thread]
-    s.red = o, o += warps * D;
     s.zred = o, o += (warps + 3) & ~3;
-    s.cand = o, o += 4 * K_c;
-    s.solve = o;
-    if (solve) o += kSolveWords;
+    s.solve = s.cand = s.red = o;
+    if (solve) {
+        s.cand = s.solve + kSolveWords;
+        s.red = s.cand + 4 * K_c;
+        o = s.red + warps * D;
+    }
     s.work = o;
-    // work area: page scores, then the key tiles of the next round, then the candidates' key rows of an iterative solve
-    // or, in the exact token fallback, the keys in position order
+    // work area: page scores, then the key tiles of the next round (or, in the exact token fallback, the keys in position
+    // order), then the candidates and the partial sums, or an iterative solve's key rows
     int w = PT * 16;
+    if (!solve) {
+        s.cand = s.work;
+        s.red = s.work + 4 * K_c;
+        w = 4 * K_c + warps * D > w ? 4 * K_c + warps * D : w;
+    }
     if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
     if (tt > 1 && threads * 16 * (fp8 ? 2 : 4) > w) w = threads * 16 * (fp8 ? 2 : 4);
     if (solve && ((K_c + 31) & ~31) * 64 > w) w = ((K_c + 31) & ~31) * 64;
@@ -129,7 +138,7 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
 
 // Exact page selection when the list overflows (many equal scores).  Leaves exactly K entries in list[] and
 // hist[] cleared.  scratch: 16 words + one per warp.
-__device__ __noinline__ void step_pages_exact(const Team& tm, const float* sc, int n, int K, uint32_t* hist,
+__device__ __noinline__ void step_pages_exact(const BlockTeam& tm, const float* sc, int n, int K, uint32_t* hist,
                                               uint32_t* scratch, unsigned long long* list, uint32_t* counter)
 {
     tm.sync();   // every thread has read the counter
@@ -147,7 +156,7 @@ __device__ __noinline__ void step_pages_exact(const Team& tm, const float* sc, i
 // Exact token selection of the R best when the histogram's range is degenerate or its cut bucket crowded: the keys
 // in position order (work[]), then every thread's unselected keys become 0.  Returns the key of the R-th best,
 // which is unselected as well.
-__device__ __noinline__ uint32_t step_tokens_exact(const Team& tm, uint32_t* own_keys, int n_own, const int32_t* tile_pos,
+__device__ __noinline__ uint32_t step_tokens_exact(const BlockTeam& tm, uint32_t* own_keys, int n_own, const int32_t* tile_pos,
                                                    int nt, int lanes, int R, uint32_t* hist, uint32_t* scratch, uint32_t* work)
 {
     const int N = nt * 16;
@@ -198,7 +207,7 @@ __device__ __forceinline__ void reduce_tile(float (&v)[16], int c)
     }
 }
 
-__device__ __noinline__ void step_failed_unit(const Team& tm, const StepParams& p, long long unit, int status, int D,
+__device__ __noinline__ void step_failed_unit(const BlockTeam& tm, const StepParams& p, long long unit, int status, int D,
                                               bool routed_too)
 {
     for (int e = tm.tid; e < D; e += tm.size) p.out[unit * D + e] = 0.0f;
@@ -256,15 +265,15 @@ __device__ __forceinline__ int rank_below(const int32_t* win, int n, int l, int 
 }
 
 // THREADS: 512 (one block per SM) when there are no more units than SMs, 256 (two) up to two units per SM, 128
-//   (four) beyond: a unit is a latency chain, so units in flight count for more than threads per unit.
+//   (four, or BLOCKS = five) beyond: a unit is a latency chain, so units in flight count for more than threads per unit.
 // FUSED: the unit's pages are selected here from page_scores; otherwise routed_pages is an input.
 // D: head dimension.  A row is spread over D / 8 lanes, 8 elements (16 bytes; fp8: 8 bytes) each, so a warp works
 //   on 4, 2 or 1 tiles of 16 rows at a time.
 // FP8: k / v hold e4m3 bytes with one scale per (pool page, KV head); strides count bytes.  Scores and weights are
 //   multiplied by the scale afterwards (exact for powers of two).
 // SOLVE: the weights come from solver_iters entropic (1) or Frank-Wolfe (2) iterations (step_solve.cuh).
-template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0>
-__global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(const __grid_constant__ StepParams p)
+template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0, int BLOCKS = 512 / THREADS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __grid_constant__ StepParams p)
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
@@ -273,7 +282,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(con
     extern __shared__ __align__(16) uint32_t smem[];
     const Geometry& geo = p.geo;
     const int tid = threadIdx.x;
-    const Team tm{tid, THREADS, 0};   // the whole block
+    const BlockTeam tm{tid, THREADS};
     const int tsh = geo.tile_shift, P = p.P;
     const StepLayout& lay = p.lay;
     uint32_t* ctl = smem;
@@ -833,16 +842,16 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) sparse_step_kernel(con
     }
 }
 
-template <int THREADS, bool FUSED, int D, bool FP8, int SOLVE = 0>
+template <int THREADS, bool FUSED, int D, bool FP8, int SOLVE = 0, int BLOCKS = 512 / THREADS>
 cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
 {
     static bool attr_done[kMaxDevices] = {};   // per template instance
     const size_t smem = (size_t)p.lay.total * 4;
     if (smem > 48 * 1024) {
-        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE>, attr_done);
+        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>, attr_done);
         if (e != cudaSuccess) return e;
     }
-    return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE>, dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch),
+    return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>, dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch),
                       dim3(THREADS), smem, stream, p);
 }
 
@@ -850,6 +859,12 @@ template <int D, bool FP8>
 cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
 {
     const bool fused = p.page_scores != nullptr;
+    // From three waves on five blocks per SM at 96 registers win over four at 128, whose unspilled registers are worth more
+    // while a wave is what counts: 2048 units of 64 pages 228 -> 216 us, 3072 units on an e4m3 cache 135 -> 114, 2048 at
+    // D = 256 155 -> 144; 768 units 52.8 -> 54.4 per layer.  Head dimension 64 loses at any count (4096 units 116 -> 122).
+    if constexpr (D >= 128)
+        if (threads == 128 && fused && (long long)p.geo.batch * p.geo.n_q_heads >= 3LL * 4 * device_sm_count())
+            return launch_step_variant<128, true, D, FP8, 0, 5>(p, stream);
 #define VSA_STEP_CASE(T)                                                                    \
     if (threads == T)                                                                       \
         return fused ? launch_step_variant<T, true, D, FP8>(p, stream)                      \

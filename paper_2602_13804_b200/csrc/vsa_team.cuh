@@ -18,14 +18,21 @@ struct Team {
     }
 };
 
+// The whole block as a team, on the block's own barrier.  (A barrier number in a register makes the compiler reserve all
+// sixteen, and an SM holds 64: four blocks at most.)
+struct BlockTeam {
+    int tid, size;
+    __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+
 // Exact top-K of key(0..n) for any multiplicity of equal keys: MSB-first radix select (8 bits per pass)
 // for the K-th key, then every index with a larger key and the first K - n_greater indices of the equal
 // keys, in index order, are passed to emit().  key(i) is evaluated several times per element (it may
 // re-read memory): this is the path for crowded ties only.  Returns the key and the index of the K-th
 // element.  hist: 256 words, misc: 16 words, wred: one word per warp of the team.  Needs 1 <= K <= number
 // of present keys.  All threads of the team call it; ends with a team barrier.
-template <class KeyFn, class EmitFn>
-__device__ __forceinline__ TopkResult team_exact_topk_slow(const Team& tm, KeyFn key, int n, int K, uint32_t* hist,
+template <class TeamT, class KeyFn, class EmitFn>
+__device__ __forceinline__ TopkResult team_exact_topk_slow(const TeamT& tm, KeyFn key, int n, int K, uint32_t* hist,
                                                            uint32_t* misc, uint32_t* wred, EmitFn emit)
 {
     const int tid = tm.tid, stride = tm.size, lane = tid & 31, warp = tid >> 5, nwarps = stride >> 5;
