@@ -478,7 +478,11 @@ cudaError_t launch_scan_variant(const dim3& grid, int wpb, int bpw, const Geomet
     // The request is padded to 81 KB so that exactly two blocks are resident per SM: with a third one
     // fewer blocks of the kernel that follows fit beside the scan's to start early, and the step gets
     // slower although the scan does not (measured: 30.0 against 24.8 us per layer at batch 8, T = 32k).
-    const size_t smem = std::max((size_t)kScanWarps * ScanCfg<G, D>::WARP_BYTES, (size_t)81 * 1024);
+    // A grid of no more blocks than SMs, of three warps or more each, asks for so much that no SM takes two (beside the
+    // ring of an idle dense block they would pair up: two sequences of 32k tokens 16.1 -> 14.6 us per layer; blocks of
+    // one or two warps do not gain).
+    const bool spread = wpb >= 3 && (long long)grid.x * grid.y <= device_sm_count();
+    const size_t smem = std::max((size_t)kScanWarps * ScanCfg<G, D>::WARP_BYTES, (size_t)(spread ? 120 : 81) * 1024);
     static bool attr_done[kMaxDevices] = {};   // per template instance
     const cudaError_t e = allow_large_dynamic_smem(route_scan_kernel<G, CERT, D, PACKED>, attr_done);
     if (e != cudaSuccess) return e;
