@@ -295,6 +295,25 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
+def step_buffers(shape, P: int, device):
+    """(out, diag, routed pages, fallback list, fallback count) of one step of `shape`: the library writes
+    head_dim floats per (sequence, query head) and checks no sizes."""
+    import torch
+    from paper_2602_13804_b200 import binding as B
+    units = shape.batch * shape.n_q_heads
+    return (torch.empty((shape.batch, shape.n_q_heads, shape.head_dim), dtype=torch.float32, device=device),
+            B.alloc_diag(units, device),
+            torch.empty((shape.batch, shape.n_q_heads, P), dtype=torch.int32, device=device),
+            torch.empty(units, dtype=torch.int32, device=device),
+            torch.zeros(1, dtype=torch.int32, device=device))
+
+
+def e2e_bytes(layers: int, q, out, diag):
+    """(host -> device, device -> host) bytes of one end-to-end step, from the tensors that are copied."""
+    return (layers * q.numel() * q.element_size(),
+            layers * (out.numel() * out.element_size() + diag.numel() * diag.element_size()))
+
+
 class Harness:
     """Layer caches, buffers and the captured step of one workload on one GPU."""
 
@@ -306,7 +325,7 @@ class Harness:
         self.spec, self.dev, self.args = spec, dev, args
         L = spec.layers
         w0 = make_workload(spec, device=dev, rep=0, sub=rank)
-        per_layer = 2 * w0.k_cache.numel() * 2 + w0.pool_pages * spec.n_kv_heads * 256
+        per_layer = 2 * w0.k_cache.numel() * 2 + w0.pool_pages * spec.n_kv_heads * spec.head_dim * 2
         free, _ = torch.cuda.mem_get_info(dev)
         self.distinct = max(1, min(L, int(mem_fraction * free // per_layer) + 1))
         self.layers = [w0] + [make_workload(spec, device=dev, rep=i, sub=rank) for i in range(1, self.distinct)]
@@ -336,11 +355,7 @@ class Harness:
         self.summary_ms_per_layer = ev0.elapsed_time(ev1) / len(self.layers)
 
         P, K_c, units = self.P, self.K_c, self.units
-        self.out = torch.empty((shape.batch, shape.n_q_heads, 128), dtype=torch.float32, device=dev)
-        self.diag = B.alloc_diag(units, dev)
-        self.routed = torch.empty((shape.batch, shape.n_q_heads, P), dtype=torch.int32, device=dev)
-        self.flist = torch.empty(units, dtype=torch.int32, device=dev)
-        self.fcount = torch.zeros(1, dtype=torch.int32, device=dev)
+        self.out, self.diag, self.routed, self.flist, self.fcount = step_buffers(shape, P, dev)
         self.ws = B.alloc_workspace(shape, P, K_c, B.VSA_WS_STEP, dev)
         self.ws_dense = B.alloc_workspace(shape, P, K_c, B.VSA_WS_DENSE, dev)
         self.ws_plain = self.ws
@@ -894,8 +909,7 @@ def run_ours(args):
             e1.record(stream)
             barrier()
             ms_e2e = max_over_ranks(e0.elapsed_time(e1), world, dev) / args.steps
-            h2d = L * units * 128 * 2
-            d2h = L * units * (128 * 4 + B.DIAG_BYTES)
+            h2d, d2h = e2e_bytes(L, q_dev, out_host, diag_host)
             e2e = {"value": us_per_token_per_layer(ms_e2e, world, shape.batch, L), "unit": UNIT, "ms_per_step": ms_e2e,
                    "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                    "api": "vsa_decode_step_host per layer, " +
@@ -1000,7 +1014,7 @@ def run_ours(args):
         "warmup": max(args.warmup, 3), "ms_per_step": ms_per_step, "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": spec.name, "batch": shape.batch, "n_q_heads": shape.n_q_heads,
-                   "n_kv_heads": shape.n_kv_heads, "head_dim": 128, "page_size": spec.page_size,
+                   "n_kv_heads": shape.n_kv_heads, "head_dim": spec.head_dim, "page_size": spec.page_size,
                    "context": int(sl.max()), "P": P, "K_c": K_c, "epsilon": eps, "gap_threshold": tau,
                    "layers_per_step": L, "distinct_layer_caches": distinct,
                    "l2": f"inputs larger than L2: {distinct} distinct layer caches, "

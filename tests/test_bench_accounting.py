@@ -4,6 +4,7 @@ import os
 import sys
 
 import numpy as np
+import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 sys.path.insert(0, ROOT)
@@ -49,3 +50,36 @@ def test_fractions_are_bytes_over_time_over_peak():
     assert abs(k["sparse_decode"]["frac"] - 0.2) < 1e-12 and abs(k["sparse_decode"]["frac_per_head_model"] - 0.8) < 1e-12
     assert abs(k["step"]["achieved_GBps"] - 15_000_000 / 12.5e-6 / 1e9) < 1e-9
     assert abs(k["sparse_decode"]["frac_of_8TBps"] - 1000.0 / 8000.0) < 1e-12
+
+
+@pytest.mark.parametrize("head_dim", [64, 128, 256])
+def test_step_buffers_and_copied_bytes_follow_the_head_dimension(head_dim):
+    from paper_2602_13804_b200 import binding as B
+    shape = B.make_shape(3, 8, 2, 5, 20, head_dim=head_dim)
+    out, diag, routed, flist, fcount = bench.step_buffers(shape, 7, "cpu")
+    assert out.shape == (3, 8, head_dim) and out.element_size() == 4
+    assert diag.numel() * diag.element_size() == 24 * B.DIAG_BYTES
+    assert routed.shape == (3, 8, 7) and flist.shape == (24,) and fcount.shape == (1,)
+    import torch
+    q = torch.empty((3, 8, head_dim), dtype=torch.bfloat16)
+    assert bench.e2e_bytes(2, q, out, diag) == (2 * 24 * head_dim * 2, 2 * 24 * (head_dim * 4 + 32))
+
+
+def test_harness_allocates_what_the_step_writes(monkeypatch):
+    """The harness of a head-dimension-256 workload, built on the CPU with the library call left out."""
+    import torch
+    from dataclasses import replace
+    from paper_2602_13804_b200 import binding as B
+    monkeypatch.setattr(B, "vsa_build_page_summaries", lambda *a, **k: None)
+    monkeypatch.setattr(torch.cuda, "mem_get_info", lambda dev=None: (1 << 34, 1 << 34))
+    monkeypatch.setattr(torch.cuda, "synchronize", lambda *a: None)
+    monkeypatch.setattr(torch.cuda, "Stream", lambda *a, **k: None)
+
+    class Event:
+        def __init__(self, **k): pass
+        def record(self, *a): pass
+        def elapsed_time(self, other): return 0.0
+    monkeypatch.setattr(torch.cuda, "Event", Event)
+    for d in (64, 128, 256):
+        h = bench.Harness(replace(_spec(), head_dim=d, layers=2), torch.device("cpu"))
+        assert h.out.numel() == h.units * d and h.summaries[0].shape[-1] == d and h.layers[0].q.shape[-1] == d
