@@ -145,7 +145,7 @@ __device__ __noinline__ void step_pages_exact(const BlockTeam& tm, const float* 
     for (int i = tm.tid; i < kStepPages; i += tm.size) list[i] = 0ull;
     if (tm.tid == 0) *counter = 0u;
     tm.sync();
-    auto key = [&](int i) { return float_to_key(sc[i]); };
+    auto key = [&](int i) { return max(float_to_key(sc[i]), 1u); };   // 0 (one NaN pattern) would read as no page
     team_exact_topk_slow(tm, key, n, K, hist, scratch, scratch + 16, [&](int i) {
         list[atomicAdd(counter, 1u)] = ((unsigned long long)key(i) << 32) | (uint32_t)~i;
     });
@@ -352,11 +352,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         for (int i = chunk0; i < n_chunks; i += THREADS) cp_async_16B(dst + 16u * (uint32_t)i, row - mis + 4 * i);
         cp_async_wait_all();
         np = min(P, nb);
-        // words of the first and the last chunk that are no scores of this row: NaN fails every comparison
+        // words of the first and the last chunk that are no scores of this row: below or equal to every score
         if (chunk0 == 0)
-            for (int e = 0; e < mis; ++e) sc[e] = __int_as_float(0x7fffffff);
+            for (int e = 0; e < mis; ++e) sc[e] = -INFINITY;
         if ((n_chunks - 1) % THREADS == chunk0)
-            for (int e = nb + mis; e < 4 * n_chunks; ++e) sc[e] = __int_as_float(0x7fffffff);
+            for (int e = nb + mis; e < 4 * n_chunks; ++e) sc[e] = -INFINITY;
         // ---- the warp's r-th largest lane maximum ----
         {
             float m = -INFINITY;
@@ -375,7 +375,9 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             if (lane == 0) warp_stat[warp] = thr;   // 0: fewer than r lanes have a score, then every score is listed
         }
         __syncthreads();
-        // ---- list every score at or above the smallest of them ----
+        // ---- list every score that is not below the smallest of them.  A NaN never is, so whatever the scores are at
+        //      least np pages are listed: every lane that a warp vouched for has one (a lane of NaNs vouches with -inf,
+        //      which lists everything).  Listed by key, a NaN ranks first, as in the exact selections ----
         {
             uint32_t theta_key = 0xffffffffu;
 #pragma unroll
@@ -392,8 +394,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                     const int i = i0 + u * THREADS;
                     if (i < n_chunks) {
                         const float4 v = sc4[i];
-                        hits |= ((v.x >= theta ? 1u : 0u) | (v.y >= theta ? 2u : 0u) | (v.z >= theta ? 4u : 0u) |
-                                 (v.w >= theta ? 8u : 0u)) << (4 * u);
+                        hits |= ((v.x < theta ? 0u : 1u) | (v.y < theta ? 0u : 2u) | (v.z < theta ? 0u : 4u) |
+                                 (v.w < theta ? 0u : 8u)) << (4 * u);
                     }
                 }
                 if (hits) {
@@ -402,8 +404,10 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                         do {
                             const int bit = __ffs(hits) - 1;
                             hits &= hits - 1u;
-                            const int i = 4 * (i0 + (bit >> 2) * THREADS) + (bit & 3);
-                            pages[s++] = ((unsigned long long)float_to_key(sc[i]) << 32) | (uint32_t)~(i - mis);
+                            const int i = 4 * (i0 + (bit >> 2) * THREADS) + (bit & 3), l = i - mis;
+                            // (a word beside the row, listed when everything is, leaves its entry 0: ranked last)
+                            if ((unsigned)l < (unsigned)nb) pages[s] = ((unsigned long long)float_to_key(sc[i]) << 32) | (uint32_t)~l;
+                            ++s;
                         } while (hits);
                     }
                 }
