@@ -80,7 +80,7 @@ enum : int {
     kCtlTokens,         // listed tokens of the cut bucket
     kCtlOut,            // key of the best rejected token
     kCtlBad,            // a routed page has no valid pool page
-    kCtlMissing,        // tokens the last page lacks, if it is routed
+    kCtlMissing,        // tokens the last page lacks, once per time it is routed
     kCtlNp,             // routed pages (when they are an input)
     kCtlCut,            // (tokens above the cut bucket << 20) | (tokens inside << 8) | bucket
     kCtlWords = 16
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     auto put_page = [&](int slot, int l, int phys) {
         const bool ok = phys >= 0 && phys < geo.pool_pages;
         if (!ok) ctl[kCtlBad] = 1u;
-        if (l == nb - 1) ctl[kCtlMissing] = (uint32_t)(nb * geo.page_size - T);
+        if (l == nb - 1) atomicAdd(&ctl[kCtlMissing], (uint32_t)(nb * geo.page_size - T));
         for (int hf = 0; hf < (1 << tsh); ++hf) {
             const int s = (slot << tsh) + hf;
             tile_off[s] = ok ? (long long)phys * geo.page_stride + (long long)(hf * 16) * geo.token_stride : -1;
@@ -625,9 +625,10 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 const uint32_t key = own[o * THREADS];
                 if (key != 0u && bucket_of(key) == cut) {
                     const int slot = (o / TPL) * GROUPS + grp;
-                    const int pos = tile_pos[slot] + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
+                    // (tiles are in position order; a page that the caller lists twice has tiles of its own)
+                    const int order = slot * 16 + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
                     const uint32_t i = atomicAdd(&ctl[kCtlTokens], 1u);
-                    tokens[i] = ((unsigned long long)key << 32) | (uint32_t)~pos;
+                    tokens[i] = ((unsigned long long)key << 32) | (uint32_t)~order;
                     loc[i] = (uint32_t)(o * THREADS + tid);
                 }
             }
