@@ -243,7 +243,8 @@ __device__ __forceinline__ float solve_frank_wolfe(const SolveSmem& sm, int ns, 
             }
             g_own = reduce_scatter16(vals, c) - s_own;
         }
-        arg_best(have ? float_to_key(-g_own) : 0u, 1 + (it & 1), bk, jb);
+        // (a NaN gradient, negated, has key 0: as 1 it is the last choice, but one that names a candidate)
+        arg_best(have ? max(float_to_key(-g_own), 1u) : 0u, 1 + (it & 1), bk, jb);
         gmin = -key_to_float(bk);
         if (it >= iters) break;
         float uj[8], dv[8], rv[8];

@@ -269,7 +269,8 @@ __device__ __forceinline__ float reduce_scatter16(float (&v)[16], int c, unsigne
 // ---- order-preserving keys -----------------------------------------------------------------
 // key(a) > key(b)  <=>  a > b for finite floats and infinities; -0 and +0 map to one key.
 // Key 0 is never produced by a non-NaN float and serves as "no element".  Sums and products that are NaN have the one
-// pattern 0x7fffffff on the GPU, key 0xffffffff: a NaN score is an element, and the first in the order.
+// pattern 0x7fffffff on the GPU, key 0xffffffff: a NaN score is an element, and the first in the order.  (A sign
+// flip turns that pattern into key 0: a key of a negated value that has to name an element is clamped to 1.)
 __device__ __forceinline__ uint32_t float_to_key(float f)
 {
     uint32_t u = __float_as_uint(f);

@@ -106,3 +106,33 @@ def test_step_fp8(batch, hq, hkv, P):
     check_pages(routed_b.numpy(), w, P)
     assert torch.equal(out_b[4:], out[4:]) and torch.equal(routed_b[4:], routed[4:])
     assert torch.equal(diag_b[4 * hq:], diag[4 * hq:])
+
+
+@pytest.mark.parametrize("batch,K_c", [(6, 32), (6, 250), (40, 32)])
+@pytest.mark.parametrize("method", ["entropic", "frank_wolfe"])
+def test_solvers(method, batch, K_c):
+    """Iterative weights: the vertex that Frank-Wolfe picks is a candidate whatever the gradients are."""
+    from paper_2602_13804_b200 import binding as B
+    dev, hq, hkv, P = "cuda:0", 8, 2, 32
+    w = clean_workload(batch, hq, hkv, P, K_c)
+
+    def run(w):
+        wd = w.to(dev)
+        shape = B.shape_of(wd.q, wd.k_cache, wd.block_table)
+        units = batch * hq
+        summ = torch.zeros((shape.num_pool_pages, hkv, 128), dtype=torch.bfloat16, device=dev)
+        B.vsa_build_page_summaries(shape, wd.k_cache, wd.block_table, wd.seq_lens, None, summ)
+        out = torch.empty((batch, hq, 128), dtype=torch.float32, device=dev)
+        diag, sol, flist = B.alloc_diag(units, dev), B.alloc_solve(units, dev), torch.empty(units, dtype=torch.int32, device=dev)
+        routed, fcount = torch.empty((batch, hq, P), dtype=torch.int32, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+        getattr(B, "vsa_decode_step_" + method)(shape, wd.q, summ, wd.k_cache, wd.v_cache, wd.block_table, wd.seq_lens, P, K_c,
+                                                w.epsilon, -INF, 4, out, diag, sol, routed, flist, fcount,
+                                                B.alloc_workspace(shape, P, K_c, B.VSA_WS_STEP, dev))
+        torch.cuda.synchronize()
+        return out.cpu(), diag.cpu(), sol.cpu(), routed.cpu()
+
+    out, diag, sol, routed = run(w)
+    out_b, diag_b, sol_b, routed_b = run(poison(w))
+    check_pages(routed_b.numpy(), w, P)
+    assert torch.equal(out_b[4:], out[4:]) and torch.equal(routed_b[4:], routed[4:])
+    assert torch.equal(diag_b[4 * hq:], diag[4 * hq:]) and torch.equal(sol_b[4 * hq:], sol[4 * hq:])
