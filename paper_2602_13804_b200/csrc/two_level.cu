@@ -12,7 +12,7 @@
 //
 //   super_summaries_kernel  cache maintenance: representative (and its logical page) per super-page
 //   (the page-routing scan, run on the representatives with a geometry whose pages are super-pages)
-//   inner_scan_kernel       per unit: top-P_super super-pages, -inf over the unit's score row, exact scores
+//   inner_scan_kernel       per unit: top-P_super super-pages, "not scored" over the unit's score row, exact scores
 //                           of the pages inside the kept super-pages
 #include <math.h>
 
@@ -68,7 +68,7 @@ super_summaries_kernel(Geometry geo, const uint16_t* __restrict__ summaries, con
 }
 
 // One block (256 or 512 threads) per (sequence, query head): exact top-P_super of the unit's representative scores (score
-// descending, super-page ascending); the unit's score row [0, n_b) is set to -inf; then every page of the
+// descending, super-page ascending); the unit's score row [0, n_b) is set to not_scored(); then every page of the
 // kept super-pages gets its exact score (one super-page = 16 summary rows = one 16-value reduction per
 // half-warp, lane c ending with the score of page 16 s + c).  page_budget[unit] = pages scored.
 __global__ void __launch_bounds__(512)
@@ -100,7 +100,7 @@ inner_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
     int* scored = (int*)ps.ts.misc;   // pages that get a score (selection scratch, free after its last barrier)
     if (tid == 0) *scored = 0;
     float* row = scores + unit * geo.max_pages;
-    for (int i = tid; i < nb; i += blockDim.x) row[i] = -INFINITY;
+    for (int i = tid; i < nb; i += blockDim.x) row[i] = not_scored();
     __syncthreads();
     float qf[8];
     unpack8(qraw, qf);
@@ -133,7 +133,7 @@ inner_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
         if (c == 0) atomicAdd(scored, n_ok);
     }
     __syncthreads();
-    // no more than the scored pages may be routed (every other entry of the row holds -inf)
+    // no more than the scored pages may be routed (a score may be -inf itself: large finite inputs overflow)
     if (tid == 0) page_budget[unit] = *scored;
 }
 

@@ -278,6 +278,9 @@ __device__ __forceinline__ uint32_t float_to_key(float f)
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// the float of key 0: a score row's mark for "not scored" (no score has it, see above)
+__device__ __forceinline__ float not_scored() { return __uint_as_float(0xffffffffu); }
+
 __device__ __forceinline__ float key_to_float(uint32_t k)
 {
     const uint32_t u = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;

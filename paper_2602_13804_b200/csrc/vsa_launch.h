@@ -131,7 +131,7 @@ cudaError_t launch_route_scan(const Geometry& g, const void* q, const void* summ
                               int zero_count, cudaStream_t stream, const float* radii = nullptr,
                               float* rad_logical = nullptr);
 // page_budget (device, per unit, or nullptr): at most that many pages of a unit are routed (two-level
-// routing: the pages that were scored; the rest of the unit's score row is -inf)
+// routing: the pages that were scored; the rest of the unit's score row is marked)
 cudaError_t launch_route_select(const Geometry& g, const void* ws, const int32_t* seq_lens, int P,
                                 int32_t* routed_pages, float* routed_scores, cudaStream_t stream,
                                 const int32_t* page_budget = nullptr);
@@ -143,7 +143,7 @@ cudaError_t launch_build_super_summaries(const Geometry& g, const void* summarie
                                          const int32_t* seq_lens, const int32_t* first_super, void* super_summaries,
                                          int32_t* super_rep, cudaStream_t stream);
 // selects the P_super best super-pages of every unit from super_scores (the representative scan's output)
-// and writes the exact scores of the pages inside them (everything else -inf) and the number of scored
+// and writes the exact scores of the pages inside them (everything else marked as not scored) and the number of scored
 // pages per unit; super_routed_out (nullable) receives the kept super-pages
 cudaError_t launch_inner_scan(const Geometry& g, const void* q, const void* summaries, const int32_t* block_table,
                               const int32_t* seq_lens, const float* super_scores, int P_super,

@@ -66,15 +66,12 @@ __device__ __forceinline__ void order_winners(int K, const PageSelectSmem& s)
 
 // Exact top-min(P, n) of sc[0..n) under (score descending, page ascending), keys staged in shared
 // memory (any n up to the carve size).  Returns K; winners in s.win_* / s.asc_idx.
-// sparse_row: scores of -inf mark pages that were never scored (two-level routing); they are treated as
-// absent, and the caller guarantees P <= the number of scored pages.
-__device__ __forceinline__ int select_top_pages(const float* __restrict__ sc, int n, int P, const PageSelectSmem& s,
-                                                bool sparse_row = false)
+// Entries of not_scored() (two-level routing) are absent; the caller guarantees P <= the number of the others.
+__device__ __forceinline__ int select_top_pages(const float* __restrict__ sc, int n, int P, const PageSelectSmem& s)
 {
     const int K = min(P, n);
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const float v = __ldcg(sc + i);
-        s.keys[i] = (sparse_row && v == -INFINITY) ? 0u : float_to_key(v);
+        s.keys[i] = float_to_key(__ldcg(sc + i));
         s.take[i] = 0;
     }
     if (threadIdx.x == 0) s.ts.misc[8] = 0u;
@@ -213,14 +210,13 @@ __device__ __forceinline__ int select_top_pages_keys(const uint32_t (&key)[KPT],
 // The register variant fed from the scores in global memory.
 template <int KPT>
 __device__ __forceinline__ int select_top_pages_reg(const float* __restrict__ sc, int n, int P,
-                                                    const PageSelectSmem& s, bool sparse_row = false)
+                                                    const PageSelectSmem& s)
 {
     uint32_t key[KPT];
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
         const int i = threadIdx.x + j * blockDim.x;
-        const float v = i < n ? __ldcg(sc + i) : 0.0f;
-        key[j] = (i < n && !(sparse_row && v == -INFINITY)) ? float_to_key(v) : 0u;
+        key[j] = i < n ? float_to_key(__ldcg(sc + i)) : 0u;
     }
     return select_top_pages_keys<KPT>(key, n, P, s);
 }

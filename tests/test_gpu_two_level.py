@@ -122,3 +122,22 @@ def test_gqa8_and_a_long_sequence_recall():
     w = make_workload(spec, seed=914)
     recall = _compare(w, _run(w, 32, 32, 256), 32, 32, 256)
     assert recall >= 0.9, recall
+
+
+def test_scores_that_overflow_to_minus_infinity_are_still_scores():
+    """Finite inputs whose sums overflow: pages with a score of -inf were scored, so they are routed in page order
+    after the finite ones, and never a page outside the kept super-pages."""
+    spec = WorkloadSpec(name="tl", config=9, batch=2, n_q_heads=4, n_kv_heads=2, P=40, K_c=32, seq_lens=(3000, 1700),
+                        needles=0)
+    w = make_workload(spec, seed=916)
+    w.q[:, :2] = 3e38
+    w.k_cache[:, 0] = -w.k_cache[:, 0].abs() - 1.0          # KV head 0, query heads 0 and 1: every score is -inf
+    g = _run(w, 3, 40, 32)
+    geo = geometry(w)
+    q, K, V, bt, sl = host_arrays(w)
+    summ = oracle.build_summaries(geo, K, bt, sl)
+    sup, _ = oracle.build_super_summaries(geo, summ, bt, sl)
+    tl = oracle.route_two_level(geo, q, summ, sup, bt, sl, 3, 40)
+    assert np.isneginf(tl.scores[:, :2]).all() and (tl.pages[:, :2] >= 0).all()
+    assert np.array_equal(g["routed"], tl.pages) and np.array_equal(g["rscores"], tl.scores)
+    assert np.array_equal(g["routed2"], tl.pages)
