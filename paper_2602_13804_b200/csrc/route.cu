@@ -20,10 +20,10 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kScanWarps = kScanThreads / 32;
 constexpr int kBlockPages = 32;      // pages per block-table block (one coalesced 128-byte load per warp)
-// Blocks of 32 pages one warp takes at most.  More per warp would amortise its start-up further, but
-// the launch then has fewer, longer warps and a ragged batch (whose short sequences leave most of a
-// grid sized for the longest one idle) ends on a long tail: 4 measured best from batch 16, T = 128k
-// (87.7 against 93.6 us per layer with 16) to a 64-sequence log-uniform batch (455 against 482 us).
+// Blocks of 32 pages one warp takes at most.  Fewer pay a warp's start-up more often, more leave fewer, longer warps
+// and a longer tail.  Microseconds per layer with 2 / 4 / 8 / 16: batch 16, T = 128k 85.4 / 83.4 / 85.3 / 86.8; 64
+// sequences of 32k 145 / 141 / 144 / 152; 32 sequences of 16k - 64k 84.4 / 82.9 / 80.9 / 96.1; 64 sequences of
+// 4k - 128k at head dimension 64 143 / 132 / 130 / 136.
 constexpr int kMaxBlocksPerWarp = 4;
 
 template <int G, int D = kHeadDim>
@@ -248,13 +248,17 @@ route_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
     }
 }
 
-// ---- the scan over a list of pages, for batches whose sequences cannot all be as long as the table is wide ----
+// ---- the scan over a list of pages, for large batches that are probably ragged ----
 // The grid of the kernel above is sized for the longest sequence; in a ragged batch most of its blocks find no page,
 // and the others run in waves that each pay the start-up of a block.  Here the pages of all sequences, in units of 8,
 // form one list that one wave of warps shares evenly: warp w takes KV head w % n_kv and the (w / n_kv)-th range of the
 // list, part by part as it crosses sequences.  The start is a longer chain (lengths, their sums, then the table), so
-// regular batches keep the kernel above (batch 8, T = 32k: 2.4 us less).  64 sequences of 4k - 128k tokens: 399 -> 371 us
-// per layer.  DEPTH rounds of a warp's rows are in flight in registers.
+// small batches keep the kernel above (batch 8, T = 32k: 2.4 us less).  DEPTH rounds of a warp's rows are in flight in
+// registers.
+// Equal shares end together only if the blocks start together, two on every SM.  The kernel is therefore launched in
+// stream order, not as a programmatic dependent: scheduled early, its blocks pile up on the SMs that an idle dense block
+// of the step before does not hold, and the rest runs as a second wave (64 sequences of 4k - 128k, four heads a group:
+// 198 us per layer early, 149 in order, 162 with the kernel above).
 constexpr int kUnitPages = 8;
 constexpr int kHalfPages = 128;   // pages of one half of a warp's offset table
 
@@ -284,7 +288,6 @@ route_list_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
         const int T = ld_ca_s32(seq_lens + b);
         return geo.length_ok(T) ? geo.pages_of(T) : 0;
     };
-    // before the wait, as above: lengths and table entries
     if (warp == 0) {
         int base = 0;
         for (int b0 = 0; b0 < geo.batch; b0 += 32) {
@@ -326,7 +329,6 @@ route_list_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
     };
     if (lo < hi) look_up(first_page);
 
-    pdl_wait();
     pdl_launch_dependents();
     if (zero_word && blockIdx.x == 0 && threadIdx.x == 0) *zero_word = 0;
     if (zero_words)
@@ -495,9 +497,14 @@ cudaError_t launch_scan_g(const Geometry& g, const uint16_t* q, const uint16_t* 
                           const int32_t* seq_lens, float* scores, int32_t* zero_word, int32_t* zero_words,
                           int zero_count, const float* radii, float* rad_logical, cudaStream_t stream)
 {
-    if constexpr (!CERT && D == kHeadDim) {
-        // At least half of the grid would be blocks without a page (the pool cannot hold `batch` sequences of the table's
-        // width) and it is more than two waves of blocks: share the pages that exist.
+    if constexpr (!CERT && D == kHeadDim && G != 2) {
+        // The pool has fewer than half of the pages that `batch` sequences of the table's width would have of their own -
+        // the sequences are of uneven length, or share prefixes - and the grid is more than two waves of blocks: share
+        // the pages that exist.  Lengths are not known here; where they are even after all the list costs nothing (64
+        // sequences of 16k that share three quarters 100 us per layer against 102, 64 of 32k without 141 against 142).
+        // Uneven ones, list against grid: 64 sequences of 4k - 128k with four heads a group 149 / 162, with eight
+        // 253 / 288; 32 of 2k - 128k 75.5 / 84.8, with one head a group 129 / 149; 48 of 2k - 32k 86.7 / 86.9.  With two
+        // heads a group the list loses (64 of 8k - 96k 251 / 226, 64 of 4k - 64k 180 / 172).
         const long long warps = (long long)g.batch * g.n_kv_heads * ((g.max_pages + kBlockPages - 1) / kBlockPages);
         const long long wave = 2LL * kScanWarps * device_sm_count();
         if (!g.super_pages && (long long)g.batch * g.max_pages >= 2 * g.pool_pages && warps > 2 * wave && g.n_kv_heads <= wave) {
@@ -506,9 +513,9 @@ cudaError_t launch_scan_g(const Geometry& g, const uint16_t* q, const uint16_t* 
             static bool attr_done[kMaxDevices] = {};
             const cudaError_t e = allow_large_dynamic_smem(route_list_kernel<G>, attr_done);
             if (e != cudaSuccess) return e;
-            return launch_pdl(route_list_kernel<G>, dim3((unsigned)((ranges * g.n_kv_heads + kScanWarps - 1) / kScanWarps)),
-                              dim3(kScanThreads), smem, stream, g, q, summaries, block_table, seq_lens, scores, ranges,
-                              zero_word, zero_words, zero_count);
+            return launch_in_order(route_list_kernel<G>, dim3((unsigned)((ranges * g.n_kv_heads + kScanWarps - 1) / kScanWarps)),
+                                   dim3(kScanThreads), smem, stream, g, q, summaries, block_table, seq_lens, scores, ranges,
+                                   zero_word, zero_words, zero_count);
         }
     }
     const int bpw = scan_blocks_per_warp(g);
