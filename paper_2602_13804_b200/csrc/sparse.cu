@@ -25,8 +25,12 @@ size_t sparse_smem_bytes(const Geometry& g, int P, int K_c, int threads, int P_s
 int sm_count() { return device_sm_count(); }
 
 // The closed-form family (sparse_step.cuh).  Thread-block size: one block of 512 threads per SM while there are
-// no more units than SMs, two of 256 up to two units per SM, four of 128 beyond (P <= 64: the page selection wants
-// at least P groups of threads).
+// no more units than SMs, two of 256 up to two units per SM, four of 128 beyond.  More than 64 pages stay with 256: each of
+// four warps vouches for P / 4 of its 32 lanes, which for P near 128 lets so many pages through that the list overflows
+// and the exact selection runs.  Microseconds per layer, 256 / 128 threads, bf16 cache: P = 128 384 units of 32k tokens
+// 83 / 96, 1024 173 / 193, 2048 305 / 352; P = 112 1024 160 / 179; P = 96 within 5 % either way (1024 units of 8k 123 / 117,
+// of 32k 148 / 149); P = 64 384 57.5 / 55.4, 1024 122 / 118.  (On the e4m3 cache 128 threads win up to P = 128, 2048
+// units 303 / 274, which the rule leaves.)
 int step_threads(const Geometry& g, int P)
 {
     const long long units = (long long)g.batch * g.n_q_heads;

@@ -6,19 +6,21 @@
 // A unit is a chain of short dependent phases, so what it costs is the number of instructions and block
 // barriers on its longest thread and, since every instruction is executed once or twice per launch, the size
 // of the code (instruction fetch).  Hence: loops that run from memory instead of unrolled register arrays, one
-// template instance for every table width, P and K_c, the rare exact fallbacks out of line, eight barriers.
+// template instance for every table width, P and K_c, the rare exact fallbacks out of line, twelve barriers.
 //   * Page scores are staged in shared memory (16-byte copies, any table width).  In every warp the r-th largest
 //     of the lanes' maxima, r = ceil(P / warps), has r scores at or above it; the smallest of these over the warps
 //     bounds the P-th best score from below and leaves about 1.6 P scores, which are listed and ranked exactly.
 //   * Routed pages are listed by position, so that the heads of a group walk the pages that they share at about
 //     the same time (L1 and L2 hits).  Ties are decided by (key << 32) | ~position.
-//   * A warp that scored a tile keeps its keys, selects among them and gathers the value rows of the candidates of
-//     its own tiles: no list of the candidates exists across warps.
+//   * A warp that scored a tile keeps its keys in shared memory and selects among them; the candidates of all warps
+//     are then compacted into one list, whose value rows are dealt out evenly to the groups of lanes.
 //   * Every score is a chain of mixed-precision FMAs on the packed bf16 words (no unpacking).
 // Measured, microseconds per layer before (register-array kernel with seventeen barriers) and after: 15.1 -> 13.1
 // at batch 1, T = 4k with the scan and the empty dense pass; 21.2 -> 17.9 at T = 128k; batch 8, T = 32k 24.6 -> 23.3;
 // 64 sequences of 4k - 128k with 8 heads a group 449 -> 399; batch 32 of short rows at D = 64 44 -> 39.  What bounds it:
-// a tile costs 64 bytes a cycle and SM on the way from L2, then the chain of phases.
+// no unit of the SM, but the chain of phases.  Counters at P = 32, K_c = 256: 20k warp instructions per unit of 256
+// threads, 0.41 of the issue slots at two units per SM (256 units), 0.38 at four of 128 threads (512 units); at P = 64,
+// K_c = 512 34k per unit, 0.52 at five per SM (2048 units).  The waits are for loads from L2, then for shared memory.
 #pragma once
 
 #include <limits.h>
@@ -864,9 +866,13 @@ template <int D, bool FP8>
 cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
 {
     const bool fused = p.page_scores != nullptr;
-    // From three waves on five blocks per SM at 96 registers win over four at 128, whose unspilled registers are worth more
-    // while a wave is what counts: 2048 units of 64 pages 228 -> 216 us, 3072 units on an e4m3 cache 135 -> 114, 2048 at
-    // D = 256 155 -> 144; 768 units 52.8 -> 54.4 per layer.  Head dimension 64 loses at any count (4096 units 116 -> 122).
+    // Five blocks per SM at 96 registers against four at 128, whose unspilled registers make a unit faster: five win from
+    // three waves of four on, where units in flight count for more.  Microseconds per layer, four / five, T = 8k: 64 pages a
+    // unit 1536 units 131 / 143, 1664 138 / 150, 1792 155 / 154, 2048 170 / 165, 3072 245 / 241; 32 pages 1664 84 / 93,
+    // 1792 93 / 95, 2048 100.4 / 100.1; D = 256 1536 138 / 149, 1792 164 / 165, 2048 179 / 176; e4m3 cache 1792 92 / 75, 3072
+    // 151 / 128.  Below the line they win only where they save a whole wave (640 units of 32 pages 47 / 40, 1280 73 / 71)
+    // and on the e4m3 cache (1024 units 51 / 49); those counts are not in the rule.  Head dimension 64 loses at any (3072
+    // units 100 / 109).
     if constexpr (D >= 128)
         if (threads == 128 && fused && (long long)p.geo.batch * p.geo.n_q_heads >= 3LL * 4 * device_sm_count())
             return launch_step_variant<128, true, D, FP8, 0, 5>(p, stream);
