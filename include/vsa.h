@@ -28,7 +28,8 @@
  *   - Data-dependent anomalies (a block-table entry outside the pool, a sequence longer
  *     than its block-table row, a non-positive length) never trap: the unit's
  *     diag.status becomes non-zero and its output row is zero-filled.
- *   - Inputs are assumed finite (no NaN/Inf in q, K, V).
+ *   - Inputs are assumed finite (no NaN/Inf in q, K, V).  Others give unspecified results in the units
+ *     that read them; no unit reads or writes outside the buffers for them, and the others stay correct.
  *   - v1 shapes: head_dim = 128 (every entry point) or 64 / 256 (page summaries, routing, the closed-form
  *     sparse pass, the dense pass and the steps built from them; the iterative solves, the certificate,
  *     two-level and group-shared routing, vsa_build_page_radii and vsa_append_kv return
