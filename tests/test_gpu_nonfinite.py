@@ -136,3 +136,54 @@ def test_solvers(method, batch, K_c):
     check_pages(routed_b.numpy(), w, P)
     assert torch.equal(out_b[4:], out[4:]) and torch.equal(routed_b[4:], routed[4:])
     assert torch.equal(diag_b[4 * hq:], diag[4 * hq:]) and torch.equal(sol_b[4 * hq:], sol[4 * hq:])
+
+
+@pytest.mark.parametrize("variant", ["certified", "expand", "two_level", "group_shared"])
+@pytest.mark.parametrize("batch", [6, 40])
+def test_routing_variants(variant, batch):
+    from paper_2602_13804_b200 import binding as B
+    dev, hq, hkv, P, K_c = "cuda:0", 8, 2, 32, 100
+    w = clean_workload(batch, hq, hkv, P, K_c)
+
+    def run(w):
+        wd = w.to(dev)
+        shape = B.shape_of(wd.q, wd.k_cache, wd.block_table)
+        units = batch * hq
+        summ = torch.zeros((shape.num_pool_pages, hkv, 128), dtype=torch.bfloat16, device=dev)
+        B.vsa_build_page_summaries(shape, wd.k_cache, wd.block_table, wd.seq_lens, None, summ)
+        out = torch.empty((batch, hq, 128), dtype=torch.float32, device=dev)
+        diag, flist = B.alloc_diag(units, dev), torch.empty(units, dtype=torch.int32, device=dev)
+        fcount, cert = torch.zeros(1, dtype=torch.int32, device=dev), B.alloc_cert(units, dev)
+        radii = torch.zeros((shape.num_pool_pages, hkv), dtype=torch.float32, device=dev)
+        B.vsa_build_page_radii(shape, wd.k_cache, summ, wd.block_table, wd.seq_lens, None, radii)
+        routed = torch.empty((batch, hkv if variant == "group_shared" else hq, 64 if variant == "expand" else P),
+                             dtype=torch.int32, device=dev)
+        cache = (wd.k_cache, wd.v_cache, wd.block_table, wd.seq_lens)
+        after = (K_c, w.epsilon, -INF, out, diag)
+        if variant == "two_level":
+            sup = torch.zeros((batch, B.n_super_pages(shape), hkv, 128), dtype=torch.bfloat16, device=dev)
+            B.vsa_build_super_summaries(shape, summ, wd.block_table, wd.seq_lens, None, sup)
+            B.vsa_decode_step_two_level(shape, wd.q, summ, sup, *cache, 4, P, *after, routed, flist, fcount,
+                                        B.alloc_workspace(shape, 4, K_c, B.VSA_WS_STEP_TWO_LEVEL, dev))
+        elif variant == "group_shared":
+            B.vsa_decode_step_group_shared(shape, wd.q, summ, *cache, P, *after, routed, flist, fcount,
+                                           B.alloc_workspace(shape, P, K_c, B.VSA_WS_STEP, dev))
+        elif variant == "expand":
+            B.vsa_decode_step_certified_expand(shape, wd.q, summ, radii, *cache, P, 64, *after, cert, routed, flist, fcount,
+                                               B.alloc_workspace(shape, 64, K_c, B.VSA_WS_STEP_EXPAND, dev))
+        else:
+            B.vsa_decode_step_certified(shape, wd.q, summ, radii, *cache, P, *after, cert, routed, flist, fcount,
+                                        B.alloc_workspace(shape, P, K_c, B.VSA_WS_STEP_CERTIFIED, dev))
+        torch.cuda.synchronize()
+        return out.cpu(), diag.cpu(), routed.cpu().numpy()
+
+    out, diag, routed = run(w)
+    out_b, diag_b, routed_b = run(poison(w))
+    for b in range(batch):
+        nb = -(-int(w.seq_lens[b]) // w.spec.page_size)
+        assert ((routed_b[b] >= -1) & (routed_b[b] < nb)).all()
+        for row in routed_b[b]:
+            row = row[row >= 0]
+            assert len(set(row.tolist())) == len(row) > 0
+    assert torch.equal(out_b[4:], out[4:]) and np.array_equal(routed_b[4:], routed[4:])
+    assert torch.equal(diag_b[4 * hq:], diag[4 * hq:])
