@@ -1,5 +1,6 @@
 """The page scan over a list of pages (ragged batches in a pool that could not hold that many long sequences): parts that
-cross sequences, single pages, ranges past the last page, groups of 1 to 16 heads, 32-token pages."""
+cross sequences, single pages, ranges past the last page, groups of 1 to 16 heads, 32-token pages.  (Two heads a group
+take the grid scan on the same kind of batch.)"""
 import pytest
 
 from gpu_runner import compare, run_gpu
