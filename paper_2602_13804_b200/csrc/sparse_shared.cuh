@@ -37,41 +37,6 @@ constexpr int kSlotsPerWarp = 2;
 constexpr int kSharedSlots = kSharedWarps * kSlotsPerWarp;
 constexpr int kPageKeysCached = 16;                   // summed page scores per thread kept in registers
 constexpr int kTeamScratchWords = 256 + 16 + 72 + kTopkList;
-constexpr uint32_t kWaitLimit = 1u << 22;             // polls of a tile's barrier before the group is failed
-
-// ---- bulk copies global -> shared with completion on an mbarrier -------------------------------------
-__device__ __forceinline__ void mbar_init(uint32_t addr, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t addr, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(addr), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(mbar)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t addr, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok)
-                 : "r"(addr), "r"(parity)
-                 : "memory");
-    return ok != 0u;
-}
-// bounded wait: false when the copy has not landed after kWaitLimit polls
-__device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity)
-{
-    for (uint32_t it = 0; it < kWaitLimit; ++it)
-        if (mbar_try_wait(addr, parity)) return true;
-    return false;
-}
-__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---- shared-memory layout, in 4-byte words from the start of dynamic shared memory ---------------------
 struct SharedLayout {

@@ -5,8 +5,9 @@
 //
 // A unit is a chain of short dependent phases, so what it costs is the number of instructions and block
 // barriers on its longest thread and, since every instruction is executed once or twice per launch, the size
-// of the code (instruction fetch).  Hence: loops that run from memory instead of unrolled register arrays, one
-// template instance for every table width, P and K_c, the rare exact fallbacks out of line, twelve barriers.
+// of the code (instruction fetch: an SM caches about 2000 instructions, straight code that is not there takes three or more
+// cycles each).  Hence: loops that run from memory instead of unrolled register arrays, one template instance for every
+// table width, P and K_c, the rare exact fallbacks out of line, twelve barriers.
 //   * Page scores are staged in shared memory (16-byte copies, any table width).  In every warp the r-th largest
 //     of the lanes' maxima, r = ceil(P / warps), has r scores at or above it; the smallest of these over the warps
 //     bounds the P-th best score from below and leaves about 1.6 P scores, which are listed and ranked exactly.
@@ -17,7 +18,10 @@
 //   * Every score is a chain of mixed-precision FMAs on the packed bf16 words (no unpacking).
 // Measured, microseconds per layer before (register-array kernel with seventeen barriers) and after: 15.1 -> 13.1
 // at batch 1, T = 4k with the scan and the empty dense pass; 21.2 -> 17.9 at T = 128k; batch 8, T = 32k 24.6 -> 23.3;
-// 64 sequences of 4k - 128k with 8 heads a group 449 -> 399; batch 32 of short rows at D = 64 44 -> 39.  What bounds it:
+// 64 sequences of 4k - 128k with 8 heads a group 449 -> 399; batch 32 of short rows at D = 64 44 -> 39.  Then, with bulk
+// copies of the key tiles and the value rows streamed through shared memory (128 threads), 355 -> 312 for the 64 sequences and
+// 83.0 -> 81.5 at batch 16, T = 128k; with scores in registers where a thread has one chunk, 14.5 -> 14.2 at batch 1, T = 4k.
+// What bounds it:
 // no unit of the SM, but the chain of phases.  Counters at P = 32, K_c = 256: 20k warp instructions per unit of 256
 // threads, 0.41 of the issue slots at two units per SM (256 units), 0.38 at four of 128 threads (512 units); at P = 64,
 // K_c = 512 34k per unit, 0.52 at five per SM (2048 units).  The waits are for loads from L2, then for shared memory.
@@ -37,8 +41,8 @@ namespace vsa {
 
 // Shared-memory layout in 4-byte words; every part starts on a 16-byte boundary.
 struct StepLayout {
-    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, cand, solve, work, bt;
-    int tiles_per_group, total;
+    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, bar, cand, solve, work, vring, bt;
+    int total;
     bool stage_bt;   // the block-table row is copied before the wait (blocks that wait for the scan anyway)
 };
 
@@ -84,18 +88,22 @@ enum : int {
     kCtlBad,            // a routed page has no valid pool page
     kCtlMissing,        // tokens the last page lacks, once per time it is routed
     kCtlNp,             // routed pages (when they are an input)
+    kCtlLate,           // a tile's copy did not arrive
     kCtlCut,            // (tokens above the cut bucket << 20) | (tokens inside << 8) | bucket
     kCtlWords = 16
 };
 
 __host__ __device__ constexpr int step_lanes_per_row(int D) { return D / 8; }
+// Value rows in flight per group of lanes, in stages of four in shared memory (0: in registers, see the value gather).
+__host__ __device__ constexpr int step_value_stages(int threads) { return threads == 128 ? 2 : threads == 256 ? 3 : 0; }
 
 inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve)
 {
     StepLayout s;
     const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
-    const int tt = (PT + groups - 1) / groups;
-    s.tiles_per_group = tt;
+    const int tt = (PT + groups - 1) / groups;   // tiles of a group of lanes
+    const int cands = (K_c + 4 * groups - 1) / (4 * groups) * (4 * groups);   // (the value gather takes four rows per group at a time)
+    const int lane_words = fp8 ? 2 : 4;          // a lane's piece of a row
     const int keys = tt * groups * 16 * (D == 256 ? 2 : 1);   // [round][sub][thread]
     int o = kCtlWords;
     s.hist = o, o += kStepBins;
@@ -112,27 +120,32 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.tile_pos = o, o += (PT + 3) & ~3;
     s.tile_phys = o, o += (PT + 3) & ~3;
     s.zred = o, o += (warps + 3) & ~3;
+    s.bar = o, o += 2 * groups;
     s.solve = s.cand = s.red = o;
     if (solve) {
         s.cand = s.solve + kSolveWords;
-        s.red = s.cand + 4 * K_c;
+        s.red = s.cand + 4 * cands;
         o = s.red + warps * D;
     }
     s.work = o;
     // work area: page scores, then the key tiles of the next round (or, in the exact token fallback, the keys in position
-    // order), then the candidates and the partial sums, or an iterative solve's key rows
+    // order), then the candidates, the partial readouts and the value rows in flight, or an iterative solve's key rows
     int w = PT * 16;
+    s.vring = s.work;
     if (!solve) {
         s.cand = s.work;
-        s.red = s.work + 4 * K_c;
-        w = 4 * K_c + warps * D > w ? 4 * K_c + warps * D : w;
+        s.red = s.work + 4 * cands;
+        s.vring = s.red + warps * D;
     }
+    const int vring_end = s.vring + 4 * step_value_stages(threads) * threads * lane_words - s.work;
+    w = vring_end > w ? vring_end : w;
     if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
-    if (tt > 1 && threads * 16 * (fp8 ? 2 : 4) > w) w = threads * 16 * (fp8 ? 2 : 4);
+    if (tt > 1 && threads * 16 * lane_words > w) w = threads * 16 * lane_words;
     if (solve && ((K_c + 31) & ~31) * 64 > w) w = ((K_c + 31) & ~31) * 64;
     o += w;
     s.bt = o;
-    s.stage_bt = fused && threads >= 256 && max_pages <= 8192;
+    // (not where it would cost the second block of an SM)
+    s.stage_bt = fused && threads >= 256 && max_pages <= 8192 && (threads == 512 || o + max_pages <= 113 * 256);
     if (s.stage_bt) o += max_pages;
     s.total = (o + 3) & ~3;
     return s;
@@ -209,6 +222,30 @@ __device__ __forceinline__ void reduce_tile(float (&v)[16], int c)
     }
 }
 
+// The same where slot i of lane c holds its partial of row i ^ tile_xor(c): at every level the slot that a lane sends and
+// the slot that it adds into are then fixed, which saves the selects.
+template <int LPR>
+__device__ __forceinline__ int tile_xor(int c)
+{
+    return LPR == 8 ? 2 * c : LPR == 32 ? c >> 1 : c;
+}
+template <int LPR>
+__device__ __forceinline__ void reduce_tile_xor(float (&v)[16])
+{
+    int n = 16;
+#pragma unroll
+    for (int off = LPR / 2; off; off >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < n) v[i] += __shfl_xor_sync(kFullMask, v[i + n], off);
+        } else {
+            v[0] += __shfl_xor_sync(kFullMask, v[0], off);
+        }
+    }
+}
+
 __device__ __noinline__ void step_failed_unit(const BlockTeam& tm, const StepParams& p, long long unit, int status, int D,
                                               bool routed_too)
 {
@@ -278,6 +315,7 @@ template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE
 __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __grid_constant__ StepParams p)
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
+    constexpr bool BULK = THREADS == 128;   // key tiles by bulk copies
     constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
     static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
     static_assert(SOLVE == 0 || (THREADS == 256 && D == 128 && !FP8), "the solve maps one candidate to each of 256 lanes");
@@ -319,6 +357,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     for (int i = tid; i < ((P + 15) & ~15); i += THREADS) win[i] = INT_MAX;
     const bool length_ok = geo.length_ok(T);
     const int nb = length_ok ? geo.pages_of(T) : 0;
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(smem + lay.bar) + 8u * (uint32_t)grp;   // BULK: of this group of lanes
+    if constexpr (BULK) {
+        if (c == 0) mbar_init(bar, 1u);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     const int r_warp = (P + WARPS - 1) / WARPS;
     pdl_wait();
     pdl_launch_dependents();
@@ -347,26 +390,44 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         //      Short rows spread over the warps (all of them have to vouch for r_warp scores) ----
         const float* row = p.page_scores + unit * geo.max_pages;
         const int mis = (int)((unit * geo.max_pages) & 3), n_chunks = (nb + mis + 3) >> 2;
-        const int chunk0 = n_chunks < THREADS ? lane * WARPS + warp : tid;
+        const bool single = n_chunks <= THREADS;   // a chunk per thread at most: it stays in registers
+        const int chunk0 = single ? lane * WARPS + warp : tid, l0 = 4 * chunk0 - mis;
         float* sc = reinterpret_cast<float*>(work);
-        const float4* sc4 = reinterpret_cast<const float4*>(sc);
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sc);
-        for (int i = chunk0; i < n_chunks; i += THREADS) cp_async_16B(dst + 16u * (uint32_t)i, row - mis + 4 * i);
-        cp_async_wait_all();
+        float4* sc4 = reinterpret_cast<float4*>(sc);
         np = min(P, nb);
+        auto in_row = [&](int l) { return (unsigned)l < (unsigned)nb; };
+        float4 own_chunk = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         // words of the first and the last chunk that are no scores of this row: below or equal to every score
-        if (chunk0 == 0)
-            for (int e = 0; e < mis; ++e) sc[e] = -INFINITY;
-        if ((n_chunks - 1) % THREADS == chunk0)
-            for (int e = nb + mis; e < 4 * n_chunks; ++e) sc[e] = -INFINITY;
+        if (single) {
+            if (chunk0 < n_chunks) {
+                const float4 v = ld_cg_f32x4(row + l0);
+                if (in_row(l0)) own_chunk.x = v.x;
+                if (in_row(l0 + 1)) own_chunk.y = v.y;
+                if (in_row(l0 + 2)) own_chunk.z = v.z;
+                if (in_row(l0 + 3)) own_chunk.w = v.w;
+            }
+        } else {
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sc);
+            for (int i = chunk0; i < n_chunks; i += THREADS) cp_async_16B(dst + 16u * (uint32_t)i, row - mis + 4 * i);
+        }
+        cp_async_wait_all();
+        if (!single) {
+            if (chunk0 == 0)
+                for (int e = 0; e < mis; ++e) sc[e] = -INFINITY;
+            if ((n_chunks - 1) % THREADS == chunk0)
+                for (int e = nb + mis; e < 4 * n_chunks; ++e) sc[e] = -INFINITY;
+        }
         // ---- the warp's r-th largest lane maximum ----
         {
-            float m = -INFINITY;
+            float m = fmaxf(fmaxf(own_chunk.x, own_chunk.y), fmaxf(own_chunk.z, own_chunk.w));
+            if (!single) {
 #pragma unroll 4
-            for (int i = chunk0; i < n_chunks; i += THREADS) {
-                const float4 v = sc4[i];
-                m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                for (int i = chunk0; i < n_chunks; i += THREADS) {
+                    const float4 v = sc4[i];
+                    m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                }
             }
+            __syncwarp();
             uint32_t v = chunk0 < n_chunks ? float_to_key(m) : 0u, thr = 0u;
 #pragma unroll 1
             for (int i = 0; i < r_warp; ++i) {
@@ -388,36 +449,59 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 theta_key = min(theta_key, min(min(x.x, x.y), min(x.z, x.w)));
             }
             const float theta = theta_key <= 0x007fffffu ? -INFINITY : key_to_float(theta_key);
-#pragma unroll 1
-            for (int i0 = chunk0; i0 < n_chunks; i0 += 8 * THREADS) {
-                uint32_t hits = 0u;   // four bits per chunk
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u * THREADS;
-                    if (i < n_chunks) {
-                        const float4 v = sc4[i];
-                        hits |= ((v.x < theta ? 0u : 1u) | (v.y < theta ? 0u : 2u) | (v.z < theta ? 0u : 4u) |
-                                 (v.w < theta ? 0u : 8u)) << (4 * u);
+            auto entry = [&](float score, int l) { return ((unsigned long long)float_to_key(score) << 32) | (uint32_t)~l; };
+            if (single) {
+                const float4 v = own_chunk;
+                const bool h0 = in_row(l0) && !(v.x < theta), h1 = in_row(l0 + 1) && !(v.y < theta),
+                           h2 = in_row(l0 + 2) && !(v.z < theta), h3 = in_row(l0 + 3) && !(v.w < theta);
+                const unsigned b0 = __ballot_sync(kFullMask, h0), b1 = __ballot_sync(kFullMask, h1),
+                               b2 = __ballot_sync(kFullMask, h2), b3 = __ballot_sync(kFullMask, h3);
+                const int n0 = __popc(b0), n1 = n0 + __popc(b1), n2 = n1 + __popc(b2), n3 = n2 + __popc(b3);
+                if (n3) {
+                    int s = 0;
+                    if (lane == 0) s = (int)atomicAdd(&ctl[kCtlPages], (uint32_t)n3);
+                    __syncwarp();
+                    s = __shfl_sync(kFullMask, s, 0);
+                    if (s + n3 <= kStepPages) {   // otherwise the list overflows and the exact selection runs
+                        const unsigned below = (1u << lane) - 1u;
+                        if (h0) pages[s + __popc(b0 & below)] = entry(v.x, l0);
+                        if (h1) pages[s + n0 + __popc(b1 & below)] = entry(v.y, l0 + 1);
+                        if (h2) pages[s + n1 + __popc(b2 & below)] = entry(v.z, l0 + 2);
+                        if (h3) pages[s + n2 + __popc(b3 & below)] = entry(v.w, l0 + 3);
                     }
                 }
-                if (hits) {
-                    uint32_t s = atomicAdd(&ctl[kCtlPages], (uint32_t)__popc(hits));
-                    if (s + __popc(hits) <= kStepPages) {
-                        do {
-                            const int bit = __ffs(hits) - 1;
-                            hits &= hits - 1u;
-                            const int i = 4 * (i0 + (bit >> 2) * THREADS) + (bit & 3), l = i - mis;
-                            // (a word beside the row, listed when everything is, leaves its entry 0: ranked last)
-                            if ((unsigned)l < (unsigned)nb) pages[s] = ((unsigned long long)float_to_key(sc[i]) << 32) | (uint32_t)~l;
-                            ++s;
-                        } while (hits);
+            } else {
+#pragma unroll 1
+                for (int i1 = 0; i1 < n_chunks; i1 += 8 * THREADS) {
+                    const int i0 = i1 + chunk0;
+                    uint32_t hits = 0u;   // four bits per chunk
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int i = i0 + u * THREADS;
+                        if (i < n_chunks) {
+                            const float4 v = sc4[i];
+                            hits |= ((v.x < theta ? 0u : 1u) | (v.y < theta ? 0u : 2u) | (v.z < theta ? 0u : 4u) |
+                                     (v.w < theta ? 0u : 8u)) << (4 * u);
+                        }
                     }
+                    uint32_t s = hits ? atomicAdd(&ctl[kCtlPages], (uint32_t)__popc(hits)) : 0u;
+                    if (s + __popc(hits) > kStepPages) hits = 0u;
+                    while (hits) {
+                        const int bit = __ffs(hits) - 1;
+                        hits &= hits - 1u;
+                        const int i = 4 * (i0 + (bit >> 2) * THREADS) + (bit & 3), l = i - mis;
+                        // (a word beside the row, listed when everything is, leaves its entry 0: ranked last)
+                        if (in_row(l)) pages[s] = entry(sc[i], l);
+                        ++s;
+                    }
+                    __syncwarp();
                 }
             }
         }
         __syncthreads();
         int m = (int)ctl[kCtlPages];
         if (m > kStepPages) {
+            if (single && chunk0 < n_chunks) sc4[chunk0] = own_chunk;
             step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, pages, &ctl[kCtlPages]);
             m = np;
         }
@@ -476,17 +560,32 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     // ---- token routing: one tile of 16 rows per group of lanes and round ----
     uint32_t a1 = 0u, a2 = 0u, amin = 0xffffffffu;   // best, second best and smallest key of this thread
     {
-        // The first tile comes through registers, every later one through shared memory (asynchronous copies that a
-        // lane reads back itself), asked for one round ahead.
+        // The first tile comes through registers, every later one through shared memory, asked for one round ahead: by
+        // asynchronous copies that a lane reads back itself or (BULK) by one bulk copy of 16 contiguous rows, which a lane reads
+        // in the order t ^ tile_xor(c) (from global memory that order would take a sector per lane).  BULK saves 16 copies with
+        // their addresses and 30 selects of the 360 instructions of a round: 19.2k -> 16.4k cycles of a unit with 64 tiles in a
+        // full chip, 8.2k -> 5.8k with 32 at D = 64.  Larger blocks have one or two rounds, which its set-up costs (batch 8,
+        // T = 32k 22.6 -> 22.9 us per layer).  Streams of four rows with eight in flight were slower (28k cycles).
         using Bits = typename std::conditional<FP8, uint2, uint4>::type;
-        constexpr int kElem = FP8 ? 1 : 2;
+        constexpr int kElem = FP8 ? 1 : 2, ROW = D * kElem, TILE = 16 * ROW;
         const uint8_t* kbase = reinterpret_cast<const uint8_t*>(p.k) + ((long long)g * geo.head_stride + c * 8) * kElem;
         const long long stride = (long long)geo.token_stride * kElem;
-        Bits* ring = reinterpret_cast<Bits*>(work) + tid;   // row t at + t * THREADS
-        const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+        const uint8_t* ring = reinterpret_cast<const uint8_t*>(work);
+        // BULK: the group's tile, row t ^ tile_xor(c) at mine ^ t * ROW; otherwise row t at mine + t * THREADS
+        const uint32_t mine = BULK ? (uint32_t)(grp * TILE + tile_xor<LPR>(c) * ROW + c * 8 * kElem) : (uint32_t)(tid * sizeof(Bits));
+        const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring) + (BULK ? (uint32_t)(grp * TILE) : mine);
         auto ahead = [&](int slot) {
-            if (slot < nt) {
-                const uint8_t* src = kbase + tile_off[slot] * kElem;
+            if (slot >= nt) return;
+            const uint8_t* src = kbase + tile_off[slot] * kElem;
+            if constexpr (BULK) {
+                if (c == 0) {
+                    mbar_expect_tx(bar, TILE);
+                    if (geo.token_stride == D)
+                        bulk_load(ring_s, src, TILE, bar);
+                    else
+                        for (int t = 0; t < 16; ++t) bulk_load(ring_s + t * ROW, src + t * stride, ROW, bar);
+                }
+            } else {
 #pragma unroll
                 for (int t = 0; t < 16; ++t) {
                     if constexpr (FP8)
@@ -496,6 +595,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 }
             }
         };
+        if (BULK && rounds > 1) fence_async_proxy();   // the page scores lay where the copies go
 #pragma unroll 1
         for (int r = 0; r < rounds; ++r) {
             const int slot = r * GROUPS + grp;
@@ -517,10 +617,15 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                     else
                         rows[t] = ld_nc_16B(src + t * stride);
                 }
+            } else if constexpr (BULK) {
+                if (active && !mbar_wait(bar, (uint32_t)(r - 1) & 1u)) ctl[kCtlLate] = 1u;
+#pragma unroll
+                for (int t = 0; t < 16; ++t) rows[t] = *reinterpret_cast<const Bits*>(ring + (mine ^ (uint32_t)(t * ROW)));
+                __syncwarp();   // read by all lanes: the next tile may land
             } else {
                 cp_async_wait_all();
 #pragma unroll
-                for (int t = 0; t < 16; ++t) rows[t] = ring[t * THREADS];
+                for (int t = 0; t < 16; ++t) rows[t] = reinterpret_cast<const Bits*>(ring + mine)[t * THREADS];
             }
             ahead(slot + GROUPS);
             float vals[16];
@@ -536,7 +641,10 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 }
             }
             __syncwarp();
-            reduce_tile<LPR>(vals, c);
+            if (BULK && r != 0)
+                reduce_tile_xor<LPR>(vals);
+            else
+                reduce_tile<LPR>(vals, c);
             const int pos = active ? tile_pos[slot] : INT_MAX - 16;
 #pragma unroll
             for (int s = 0; s < TPL; ++s) {
@@ -561,6 +669,10 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     }
     __syncthreads();
     const uint4 stat = *reinterpret_cast<const uint4*>(ctl + kCtlStat);
+    if (BULK && ctl[kCtlLate]) {
+        step_failed_unit(tm, p, unit, VSA_UNIT_COPY_TIMEOUT, D, false);
+        return;
+    }
     const uint32_t key1 = stat.x;
     const float s1 = n_valid > 0 ? key_to_float(key1) : -INFINITY;
     const int ns = min(p.K_c, n_valid);
@@ -579,7 +691,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             hi = s1;
             lo = key_to_float(~stat.w);
         }
-        bscale = (float)kStepBins / (hi - lo);
+        bscale = __fdividef((float)kStepBins, hi - lo);   // (0 for a huge range: one bucket, the exact selection)
         bool fast = hi > lo && bscale < INFINITY && hi - lo < INFINITY;
         if (fast) {
 #pragma unroll 1
@@ -704,6 +816,13 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         }
         at += __popc(votes);
     }
+    constexpr int UNR = 4;   // rows of a group of lanes that the value gather takes at a time
+    const int n_rows = (ns + UNR * GROUPS - 1) / (UNR * GROUPS) * UNR;   // past the candidates: the last one, weight 0
+    static_assert(UNR * GROUPS <= THREADS, "fewer than a row each");
+    if (ns < n_rows * GROUPS) {   // (the same for the block; K_c is a multiple as a rule)
+        __syncthreads();
+        if (ns + tid < n_rows * GROUPS) cand[ns + tid] = Row{cand[ns - 1].off, 0.0f, 0.0f};
+    }
     __syncthreads();
 
     float lse_closed = 0.0f;   // log-sum-exp of the closed-form weights (SOLVE only)
@@ -747,63 +866,102 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         __syncthreads();
     }
 
-    // ---- value gather: the candidates dealt out to the groups of lanes, four batches of four rows in flight ----
-    constexpr int UNR = 4;
-    const int n_rows = (ns + GROUPS - 1) / GROUPS;   // of this group of lanes at most; past the end: weight 0
+    // ---- value gather: the candidates dealt out to the groups of lanes, four rows at a time.  A block of 128 or 256 threads
+    //      streams them through stages in shared memory: the loop is a quarter of the code of sixteen rows in registers (the SM
+    //      caches some 2000 instructions, a kernel with units in all phases needs its code again and again: 20.7k -> 14k
+    //      cycles of a unit with K_c = 512 in a full chip, 4.0k -> 3.4k at K_c = 256 and two units per SM).  With 512 threads
+    //      every instruction runs once, and rows in registers are faster (batch 1, T = 4k 14.4 against 14.7 us per layer) ----
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
     {
-        constexpr int BATCHES = 4;
-        const uint16_t* vbase = p.v + (long long)g * geo.head_stride + c * 8;
-        const uint8_t* vbase8 = reinterpret_cast<const uint8_t*>(p.v) + (long long)g * geo.head_stride + c * 8;
         using Bits = typename std::conditional<FP8, uint2, uint4>::type;
-        Bits rows[BATCHES][UNR];
-        float w[BATCHES][UNR];
-        auto fetch = [&](int t, int i) {   // batch t of the registers <- rows i .. i + UNR - 1 of this group
+        constexpr int kElem = FP8 ? 1 : 2, STAGES = step_value_stages(THREADS);
+        const uint8_t* vbase = reinterpret_cast<const uint8_t*>(p.v) + ((long long)g * geo.head_stride + c * 8) * kElem;
+        const Row* mine = cand + grp;
+        auto add = [&](const Bits& row, float w) {
+            float vf[8];
+            if constexpr (FP8)
+                unpack8_e4m3_mixed(row, vf);
+            else
+                unpack8_mixed(row, vf);
 #pragma unroll
-            for (int u = 0; u < UNR; ++u) {
-                const int j = (i + u) * GROUPS + grp;
-                const Row row = cand[min(j, ns - 1)];
-                w[t][u] = j < ns ? row.w : 0.0f;
-                if constexpr (FP8)
-                    rows[t][u] = ld_nc_8B(vbase8 + row.off);
-                else
-                    rows[t][u] = ld_nc_16B(vbase + row.off);
-            }
+            for (int e = 0; e < 8; e += 2) fma2(acc[e], acc[e + 1], w, w, vf[e], vf[e + 1]);
         };
-#pragma unroll
-        for (int t = 0; t < BATCHES; ++t)
-            if (t * UNR < n_rows) fetch(t, t * UNR);
         // meanwhile: the sum of the weights and the warp's two best keys
+        auto statistics = [&] {
+            __syncwarp();
 #pragma unroll
-        for (int off = 16; off; off >>= 1) z += __shfl_xor_sync(kFullMask, z, off);
-        const uint32_t best = __reduce_max_sync(kFullMask, a1);
-        const int holder = __ffs(__ballot_sync(kFullMask, a1 == best)) - 1;
-        const uint32_t second = __reduce_max_sync(kFullMask, lane == holder ? a2 : a1);
-        if (lane == 0) {
-            zred[warp] = z;
-            warp_stat[2 * warp] = best;
-            warp_stat[2 * warp + 1] = second;
-        }
-        __syncwarp();
-#pragma unroll 1
-        for (int i0 = 0; i0 < n_rows; i0 += BATCHES * UNR)
+            for (int off = 16; off; off >>= 1) z += __shfl_xor_sync(kFullMask, z, off);
+            const uint32_t best = __reduce_max_sync(kFullMask, a1);
+            const int holder = __ffs(__ballot_sync(kFullMask, a1 == best)) - 1;
+            const uint32_t second = __reduce_max_sync(kFullMask, lane == holder ? a2 : a1);
+            if (lane == 0) {
+                zred[warp] = z;
+                warp_stat[2 * warp] = best;
+                warp_stat[2 * warp + 1] = second;
+            }
+            __syncwarp();
+        };
+        if constexpr (STAGES == 0) {
+            constexpr int BATCHES = 4;
+            Bits rows[BATCHES][UNR];
+            float w[BATCHES][UNR];
+            auto fetch = [&](int t, int i) {   // batch t of the registers <- rows i .. i + UNR - 1 of this group
+#pragma unroll
+                for (int u = 0; u < UNR; ++u) {
+                    const Row row = mine[(i + u) * GROUPS];
+                    w[t][u] = row.w;
+                    if constexpr (FP8)
+                        rows[t][u] = ld_nc_8B(vbase + row.off * kElem);
+                    else
+                        rows[t][u] = ld_nc_16B(vbase + row.off * kElem);
+                }
+            };
 #pragma unroll
             for (int t = 0; t < BATCHES; ++t)
-                if (i0 + t * UNR < n_rows) {
+                if (t * UNR < n_rows) fetch(t, t * UNR);
+            statistics();
+#pragma unroll 1
+            for (int i0 = 0; i0 < n_rows; i0 += BATCHES * UNR)
 #pragma unroll
-                    for (int u = 0; u < UNR; ++u) {
-                        float vf[8];
-                        if constexpr (FP8)
-                            unpack8_e4m3_mixed(rows[t][u], vf);
-                        else
-                            unpack8_mixed(rows[t][u], vf);
+                for (int t = 0; t < BATCHES; ++t)
+                    if (i0 + t * UNR < n_rows) {
 #pragma unroll
-                        for (int e = 0; e < 8; e += 2) fma2(acc[e], acc[e + 1], w[t][u], w[t][u], vf[e], vf[e + 1]);
+                        for (int u = 0; u < UNR; ++u) add(rows[t][u], w[t][u]);
+                        if (i0 + (t + BATCHES) * UNR < n_rows) fetch(t, i0 + (t + BATCHES) * UNR);
                     }
-                    if (i0 + (t + BATCHES) * UNR < n_rows) fetch(t, i0 + (t + BATCHES) * UNR);
+        } else {
+            const Bits* ring = reinterpret_cast<const Bits*>(smem + lay.vring) + tid;   // row t of a stage at + t * THREADS
+            const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+            auto fetch = [&](int i, int stage) {   // stage <- rows i .. i + UNR - 1 of this group
+#pragma unroll
+                for (int u = 0; u < UNR; ++u) {
+                    const uint8_t* src = vbase + mine[(i + u) * GROUPS].off * kElem;
+                    const uint32_t dst = ring_s + (uint32_t)((stage * UNR + u) * THREADS * sizeof(Bits));
+                    if constexpr (FP8)
+                        cp_async_8B(dst, src);
+                    else
+                        cp_async_16B(dst, src);
                 }
+            };
+#pragma unroll 1
+            for (int s = 0; s < STAGES; ++s) {
+                if (UNR * s < n_rows) fetch(UNR * s, s);
+                cp_async_commit_group();
+            }
+            statistics();
+            int stage = 0;
+#pragma unroll 1
+            for (int i = 0; i < n_rows; i += UNR) {
+                cp_async_wait_group<STAGES - 1>();
+#pragma unroll
+                for (int u = 0; u < UNR; ++u) add(ring[(stage * UNR + u) * THREADS], mine[(i + u) * GROUPS].w);
+                if (i + UNR * STAGES < n_rows) fetch(i + UNR * STAGES, stage);
+                cp_async_commit_group();
+                stage = stage + 1 == STAGES ? 0 : stage + 1;
+            }
+        }
     }
 #pragma unroll
     for (int off = LPR; off < 32; off <<= 1)
