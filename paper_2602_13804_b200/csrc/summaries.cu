@@ -259,31 +259,59 @@ __global__ void __launch_bounds__(256) append_kernel(Geometry geo, const uint16_
                                                      uint16_t* __restrict__ summaries, float* __restrict__ radii)
 {
     // Launched with programmatic serialisation like the kernels of the step, so that neither side of it pays a full
-    // launch gap (0.8 us of a 16 us layer at batch 1).  Everything, the lengths included, is read after the wait.
-    pdl_wait();
-    pdl_launch_dependents();
+    // launch gap (0.8 us of a 16 us layer at batch 1).  What bounds it is a chain of loads: length, table entry, rows.  So the
+    // length and the entry are read once ahead of the wait, when they may still be about to change, and only to know where
+    // the page probably is: its rows are asked for in L2, and after the wait everything is read (again) at once.  Where the
+    // length or the entry did change, the chain is walked as it is.
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int c = (int)(idx & 15);
     const long long pair = idx >> 4;
     if (pair >= (long long)geo.batch * geo.n_kv_heads) return;
     const int b = (int)(pair / geo.n_kv_heads), g = (int)(pair % geo.n_kv_heads);
-    const int T = seq_lens[b];
-    if (T <= 0 || T > geo.max_pages * PS) return;
-    const int l = (T - 1) / PS, n = (T - 1) % PS + 1;   // page of the new token, rows it holds now
-    const long long p = block_table[(long long)b * geo.max_pages + l];
-    if (p < 0 || p >= geo.pool_pages) return;
     const unsigned hmask = 0xffffu << (threadIdx.x & 16);
+    const int32_t* bt = block_table + (long long)b * geo.max_pages;
+    auto length_ok = [&](int T) { return T > 0 && T <= geo.max_pages * PS; };
+    auto page_ok = [&](long long p) { return p >= 0 && p < geo.pool_pages; };
+    const int T0 = ld_cg_s32(seq_lens + b), l0 = length_ok(T0) ? (T0 - 1) / PS : 0;
+    const long long p0 = ld_cg_s32(bt + l0);
+    const bool expected = length_ok(T0) && page_ok(p0);
+    const long long head_off = (long long)g * geo.head_stride + c * 8;
+    if (expected) {
+        const uint16_t* page = k_cache + p0 * geo.page_stride + (long long)g * geo.head_stride;
+        for (int t = c; t < (T0 - 1) % PS; t += 16) {
+            prefetch_L2(page + (long long)t * geo.token_stride);
+            prefetch_L2(page + (long long)t * geo.token_stride + kHeadDim / 2);
+        }
+    }
 
-    const long long row0 = p * geo.page_stride + (long long)g * geo.head_stride + c * 8;
-    const uint4 kn = *reinterpret_cast<const uint4*>(k_new + pair * kHeadDim + c * 8);
-    const uint4 vn = *reinterpret_cast<const uint4*>(v_new + pair * kHeadDim + c * 8);
-    *reinterpret_cast<uint4*>(k_cache + row0 + (long long)(n - 1) * geo.token_stride) = kn;
-    *reinterpret_cast<uint4*>(v_cache + row0 + (long long)(n - 1) * geo.token_stride) = vn;
+    pdl_wait();
+    pdl_launch_dependents();
+    int T = ld_cg_s32(seq_lens + b);
+    long long p = ld_cg_s32(bt + l0);
+    const uint4 kn = ld_cg_16B(k_new + pair * kHeadDim + c * 8);
+    const uint4 vn = ld_cg_16B(v_new + pair * kHeadDim + c * 8);
     uint4 rows[PS];
+    auto fetch = [&](long long page, int n) {   // the rows before the new one
+#pragma unroll
+        for (int t = 0; t < PS; ++t)
+            rows[t] = t < n - 1 ? ld_cg_16B(k_cache + page * geo.page_stride + head_off + (long long)t * geo.token_stride)
+                                : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (expected) fetch(p0, (T0 - 1) % PS + 1);
+    if (!expected || T != T0 || p != p0) {
+        if (!length_ok(T)) return;
+        p = ld_cg_s32(bt + (T - 1) / PS);
+        if (!page_ok(p)) return;
+        fetch(p, (T - 1) % PS + 1);
+    }
+    __syncwarp(hmask);
+
+    const int n = (T - 1) % PS + 1;   // rows that the page holds now
+    *reinterpret_cast<uint4*>(k_cache + p * geo.page_stride + head_off + (long long)(n - 1) * geo.token_stride) = kn;
+    *reinterpret_cast<uint4*>(v_cache + p * geo.page_stride + head_off + (long long)(n - 1) * geo.token_stride) = vn;
 #pragma unroll
     for (int t = 0; t < PS; ++t)
-        rows[t] = t < n - 1 ? *reinterpret_cast<const uint4*>(k_cache + row0 + (long long)t * geo.token_stride)
-                            : (t == n - 1 ? kn : make_uint4(0u, 0u, 0u, 0u));
+        if (t == n - 1) rows[t] = kn;
     const uint4 mu_bits = mean_of_rows<PS>(rows, n);
     *reinterpret_cast<uint4*>(summaries + (p * geo.n_kv_heads + g) * kHeadDim + c * 8) = mu_bits;
     if (radii) {

@@ -108,6 +108,23 @@ __device__ __forceinline__ float4 ld_cg_f32x4(const float* p)
     return v;
 }
 
+__device__ __forceinline__ int ld_cg_s32(const int32_t* p)
+{
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// 16 bytes from L2 (never from a line that this SM's L1 kept from before a wait)
+__device__ __forceinline__ uint4 ld_cg_16B(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void prefetch_L2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 __device__ __forceinline__ int ld_ca_s32(const int32_t* p)
 {
     int v;
