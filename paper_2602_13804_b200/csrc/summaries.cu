@@ -7,10 +7,11 @@ namespace vsa {
 
 // Chunks of 256 threads' work that one block of the summary kernels takes: the grid is sized for the longest
 // sequence, and with one chunk per block the blocks past the shorter ones cost 10 us of 120 (8 prompts of 8k - 32k
-// tokens, two layers); four such waves of blocks (three per SM) stay, so small prompts still spread over the chip.
+// tokens, two layers); six waves of blocks (four per SM) stay, so small prompts still spread over the chip and the last
+// wave is a small part (three waves: 153.6 against 149.4 us over 32 prompts of 2k - 16k tokens in 32-token pages).
 static int summary_chunks(long long threads, int batch)
 {
-    const long long c = threads * batch / (256LL * 12 * device_sm_count());
+    const long long c = threads * batch / (256LL * 24 * device_sm_count());
     return (int)(c < 1 ? 1 : c > 8 ? 8 : c);
 }
 
@@ -107,11 +108,11 @@ __device__ __forceinline__ float radius_of_rows(const uint4 (&rows)[PS], int n, 
 
 // One thread per (logical page, kv head, slice of 8 elements): the D / 8 threads of a (page, head) read one
 // contiguous key row per load.  fp32 sum in ascending token order, IEEE division by the number of valid rows,
-// round-to-nearest-even to bf16.  Bound by HBM: eight rows of a page in flight per thread and three blocks per SM
-// keep 96 KB in flight while other blocks add (16 rows, two blocks per SM, unpacked sums and 64-bit index
-// divisions: 4.3 TB/s over 8 prompts of 8k - 32k tokens; now 5.6).  Grid: x = chunks of pages, y = sequence.
+// round-to-nearest-even to bf16.  Bound by HBM: eight rows of a page in flight per thread and four blocks per SM
+// keep 128 KB in flight while other blocks add (8 prompts of 8k - 32k tokens, two layers: 112.9 us with three blocks, 103.3
+// with four, 109.4 with five, whose registers spill; e4m3 64.6 / 57.8 / 66.0).  Grid: x = chunks of pages, y = sequence.
 template <int PS, int D>
-__global__ void __launch_bounds__(256, 3) summaries_kernel(Geometry geo, const uint16_t* __restrict__ k_cache,
+__global__ void __launch_bounds__(256, 4) summaries_kernel(Geometry geo, const uint16_t* __restrict__ k_cache,
                                                            const int32_t* __restrict__ block_table,
                                                            const int32_t* __restrict__ seq_lens,
                                                            const int32_t* __restrict__ first_page,
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(256, 3) summaries_kernel(Geometry geo, const u
 // holds the same values.
 // One thread per (logical page, kv head, 8-byte slice); head dimension 128.
 template <int PS>
-__global__ void __launch_bounds__(256, 3) summaries_fp8_kernel(Geometry geo, const uint8_t* __restrict__ k_cache,
+__global__ void __launch_bounds__(256, 4) summaries_fp8_kernel(Geometry geo, const uint8_t* __restrict__ k_cache,
                                                                const float* __restrict__ k_scale,
                                                                const int32_t* __restrict__ block_table,
                                                                const int32_t* __restrict__ seq_lens,
