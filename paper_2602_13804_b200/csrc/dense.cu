@@ -16,7 +16,7 @@
 // the block that finishes the last item of a (sequence, KV head) combines its partials.
 #include <math.h>
 
-#include <cuda_fp8.h>
+#include <cuda.h>
 
 #include "vsa_device.cuh"
 #include "vsa_launch.h"
@@ -29,16 +29,21 @@ constexpr int kTileRows = 16;                      // the pass walks tiles of 16
 constexpr int kPagesPerItemGoal = 128;             // pages per item and block from which a second round pays
 constexpr int kMaxRounds = 2;
 constexpr int kMaxRoundsRagged = 8;
+constexpr float kPScale = 16384.0f;                // FP8: the probabilities' place in the f16 range
 
 // Sizes that depend on the head dimension D (64, 128 or 256).  The ring of a block holds three stages of a
 // K tile and a V tile per warp: 192 KB with eight warps at D = 128; D = 256 runs four warps per block so
 // that the same ring fits.
 // FP8 (D = 128): the unit of work is 32 tokens (two tiles); a stage holds their e4m3 rows as they are (4 KB of
-// K, 4 KB of V, the four scales) and the tensor cores consume them directly (m16n8k32 e4m3 MMAs).
+// K, 4 KB of V), brought by four TMA tile loads in the 128-byte swizzle that ldmatrix wants; fragments are converted to f16
+// (exact) for m16n8k16 MMAs with the tokens, then the columns, as rows and the heads as columns.
 template <int D, bool FP8 = false>
 struct DenseCfg {
-    // fp8: a unit of half the bytes costs the same instructions per token, so the pass is bound by the latency of
-    // each warp's chain: twelve warps with two stages instead of eight with three (254 MB: 100 -> 80 us)
+    // fp8: a unit of half the bytes costs the same instructions per token, so the pass is bound by the latency of each
+    // warp's chain: twelve warps with two stages.  Microseconds per layer, 16 sequences of 16k - 32k that all fall back
+    // (754 MB), with 8 / 10 / 12 warps: 228 / 221 / 207.  Before, with m16n8k32 e4m3 MMAs of two terms per
+    // operand (860 instructions per 32 tokens against 560 now) and 16-byte copies in place of TMA tiles, 290; a quarter of the
+    // sequences (246 MB, the kernel alone 62 us, DRAM at half its rate, 0.40 of the issue slots) 116 -> 92.
     static constexpr int kDenseThreads = FP8 ? 384 : D == 256 ? 128 : 256;
     static constexpr int kStages = FP8 ? 2 : 3;                // units in flight per warp
     static constexpr int kDenseWarps = kDenseThreads / 32;
@@ -46,9 +51,10 @@ struct DenseCfg {
     static constexpr int kTileBytes = kTileRows * kRowBytes;   // K (or V) rows of one tile and KV head (4 KB at D = 128)
     static constexpr int kUnitRows = FP8 ? 32 : kTileRows;     // tokens per unit of work of a warp
     static constexpr int kRawBytes = 32 * D;                   // FP8: K (or V) rows of a unit as e4m3 bytes
-    static constexpr int kStageBytes = FP8 ? 2 * kRawBytes + 16 : 2 * kTileBytes;   // K + V (+ scales)
+    static constexpr int kStageBytes = FP8 ? 2 * kRawBytes : 2 * kTileBytes;   // K + V
     static constexpr int kWarpBytes = kStages * kStageBytes;
     static constexpr int kRingBytes = kDenseWarps * kWarpBytes;
+    static constexpr int kBarBytes = FP8 ? kDenseWarps * kStages * 8 : 0;   // one mbarrier per stage
     static constexpr int kPartialFloats = 2 + D;               // per (item, head): max (log2 domain), sum, acc[D]
     static constexpr int kMinPagesPerItem = 2 * kDenseWarps;   // at least two pages per warp: one would expose the DRAM latency
 };
@@ -85,16 +91,34 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a2
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(zero), "r"(a2), "r"(zero), "r"(b0), "r"(b1));
 }
-// D (16x8, fp32) += A (16x32, e4m3, row) * B (32x8, e4m3, col).  The (at most eight) heads occupy rows 0..7 of
-// A with the high e4m3 term of each operand value and rows 8..15 with the low term (a1, a3), so that one MMA
-// forms both partial products: d[0], d[1] (row g) and d[2], d[3] (row g + 8) are added by the caller.
-__device__ __forceinline__ void mma_e4m3(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                         uint32_t b1)
+// D (16x8, fp32) += A (16x16, f16, row) * B (16x8, f16, col)
+__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1)
 {
-    asm volatile("mma.sync.aligned.m16n8k32.row.col.f32.e4m3.e4m3.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                  "{%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// an 8 x 8 matrix of 16-bit elements, two of a row per lane, transposed across the warp
+__device__ __forceinline__ uint32_t transpose_8x8(uint32_t x)
+{
+    uint32_t r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
+}
+// four e4m3 bytes as f16 (exact), bytes 0, 1 and bytes 2, 3
+__device__ __forceinline__ void e4m3x4_to_f16(uint32_t bytes, uint32_t& lo, uint32_t& hi)
+{
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tcvt.rn.f16x2.e4m3x2 %0, l;\n\tcvt.rn.f16x2.e4m3x2 %1, h;\n\t}"
+        : "=r"(lo), "=r"(hi)
+        : "r"(bytes));
+}
+__device__ __forceinline__ uint32_t pack_f16x2(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
 }
 // 16 x 16 bytes, transposed: lane (g = lane / 4, t = lane % 4) receives rows 4t .. 4t+3 of column g (first
 // register) and of column g + 8 (second); .x2 loads a second matrix (addresses from lanes 16 .. 31) into r2, r3
@@ -104,22 +128,28 @@ __device__ __forceinline__ void ldmatrix_x2_trans_b8(uint32_t (&r)[4], uint32_t 
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
-// x = hi + lo with hi, lo e4m3 (x of up to eight significant bits inside the e4m3 range splits exactly)
-__device__ __forceinline__ void split_e4m3x2(float x0, float x1, uint32_t& hi, uint32_t& lo)
-{
-    const __nv_fp8x2_storage_t h = __nv_cvt_float2_to_fp8x2(make_float2(x0, x1), __NV_SATFINITE, __NV_E4M3);
-    const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2(h, __NV_E4M3);
-    const float2 hf = __half22float2(*reinterpret_cast<const __half2*>(&hr));
-    const __nv_fp8x2_storage_t l = __nv_cvt_float2_to_fp8x2(make_float2(x0 - hf.x, x1 - hf.y), __NV_SATFINITE, __NV_E4M3);
-    hi = h;
-    lo = l;
-}
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+
+// one tile of 16 rows of 128 bytes: rows row .. row + 15 of KV head `head` of pool page `page`
+__device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, int row, int head, int page, uint32_t mbar)
+{
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+                 ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(head), "r"(page), "r"(mbar)
+                 : "memory");
+}
+
+// e4m3 cache: the K and V pools as tensors [page][head][token][128 bytes], box = one tile
+template <bool FP8>
+struct DenseMaps {};
+template <>
+struct DenseMaps<true> {
+    CUtensorMap k, v;
+};
 
 struct DenseSmem {
     uint8_t* ring;         // [warps][stages][K tile | V tile]; reused for the cross-warp merge
@@ -135,7 +165,8 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                    const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ fallback_list,
                    const int32_t* __restrict__ fallback_count, float epsilon, float* __restrict__ partials,
                    int32_t* __restrict__ counters, float* __restrict__ out, vsa_diag_t* __restrict__ diag,
-                   int max_items, const float* __restrict__ k_scale, const float* __restrict__ v_scale)
+                   int max_items, const float* __restrict__ k_scale, const float* __restrict__ v_scale,
+                   const __grid_constant__ DenseMaps<FP8> maps)
 {
     static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
     using Cfg = DenseCfg<D, FP8>;
@@ -147,12 +178,13 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     constexpr int NT = D / 8;     // 8-column output tiles
     constexpr int CPR = D / 8;    // 16-byte chunks per row
     constexpr int RPI = 32 / (CPR < 32 ? CPR : 32);   // rows one copy instruction of a warp covers
-    extern __shared__ __align__(128) uint8_t dense_smem[];
+    extern __shared__ __align__(1024) uint8_t dense_smem[];   // (the TMA swizzle is one of address bits)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_groups = geo.batch * geo.n_kv_heads;
     DenseSmem sm;
     sm.ring = dense_smem;
-    sm.item_base = (int32_t*)(dense_smem + kRingBytes);
+    const uint32_t bars = (uint32_t)__cvta_generic_to_shared(dense_smem + kRingBytes);   // FP8: [warp][stage]
+    sm.item_base = (int32_t*)(dense_smem + kRingBytes + Cfg::kBarBytes);
     sm.misc = sm.item_base + n_groups + 1;
     sm.group_mask = (uint8_t*)(sm.misc + 32);
     // The list is empty as a rule and the next kernel is what the stream waits for: that one may be scheduled while
@@ -178,6 +210,10 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         for (int i = tid; i < n_groups; i += kDenseThreads) sm.group_mask[i] = (uint8_t)((1u << G) - 1u);
     }
     if (tid < 32) sm.misc[tid] = 0;
+    if constexpr (FP8) {
+        if (tid < kDenseWarps * kStages) mbar_init(bars + 8u * (uint32_t)tid, 1u);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     __syncthreads();
 
     // ---- pages per item from the amount of flagged work, then the item table ----
@@ -255,6 +291,7 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         }
         if (tid == kDenseThreads - 1) sm.item_base[n_groups] = base;
     }
+    if constexpr (FP8) fence_async_proxy();   // group_pages lay where the copies go
     __syncthreads();
     const int n_items = sm.item_base[n_groups];
 
@@ -265,6 +302,7 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     const uint32_t ring_addr = (uint32_t)__cvta_generic_to_shared(my_ring);
     // copy mapping: lane covers 16-byte chunk lane % CPR of rows lane / CPR + RPI i, i = 0 .. 16 / RPI - 1
     const int cp_chunk = lane % CPR, cp_row0 = lane / CPR;
+    int used = 0;   // FP8: units that this warp has asked for in earlier items
 
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         // group of this item: last g with item_base[g] <= item
@@ -290,40 +328,33 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         uint32_t qa0[KS], qa2[KS];
         float q_unscale = 1.0f;
         if constexpr (FP8) {
-            // q as e4m3 operands: scaled by a power of two into the top of the e4m3 range, split into hi + lo
-            // (qa0 / qa2 hold, per 32-column step, {hi, lo} of columns 4 quad .. + 3 and of 16 + the same)
+            // q as f16 operands, scaled by a power of two into the top of the f16 range: exact down to 2^-28 of the head's
+            // largest element.  Step ks holds columns 16 ks + 4 quad, + 1 (qa0) and + 2, + 3 (qa2) of head lane / 4: the
+            // order in which a lane receives the bytes of a key row.
             const uint16_t* qrow = q + ((long long)b * geo.n_q_heads + g * G + (head < G ? head : 0)) * kHeadDim;
-            float qv[4][8];
+            float qv[KS][4];
             float amax = 0.0f;
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
+            for (int ks = 0; ks < KS; ++ks) {
+                const uint2 raw = *reinterpret_cast<const uint2*>(qrow + ks * 16 + quad * 4);
+                qv[ks][0] = __uint_as_float(raw.x << 16);
+                qv[ks][1] = __uint_as_float(raw.x & 0xffff0000u);
+                qv[ks][2] = __uint_as_float(raw.y << 16);
+                qv[ks][3] = __uint_as_float(raw.y & 0xffff0000u);
 #pragma unroll
-                for (int part = 0; part < 2; ++part) {
-                    const uint2 raw = *reinterpret_cast<const uint2*>(qrow + ks * 32 + part * 16 + quad * 4);
-                    qv[ks][part * 4 + 0] = __uint_as_float(raw.x << 16);
-                    qv[ks][part * 4 + 1] = __uint_as_float(raw.x & 0xffff0000u);
-                    qv[ks][part * 4 + 2] = __uint_as_float(raw.y << 16);
-                    qv[ks][part * 4 + 3] = __uint_as_float(raw.y & 0xffff0000u);
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) amax = fmaxf(amax, fabsf(qv[ks][i]));
+                for (int i = 0; i < 4; ++i) amax = fmaxf(amax, fabsf(qv[ks][i]));
             }
             amax = fmaxf(amax, __shfl_xor_sync(kFullMask, amax, 1));
             amax = fmaxf(amax, __shfl_xor_sync(kFullMask, amax, 2));
-            const int sq = amax > 0.0f ? 7 - ilogbf(amax) : 0;   // largest |q| of the head lands in [128, 256)
+            const int sq = amax > 0.0f ? 13 - ilogbf(amax) : 0;   // largest |q| of the head lands in [2^13, 2^14)
             q_unscale = ldexpf(1.0f, -sq);
+            const float up0 = ldexpf(1.0f, sq >> 1), up1 = ldexpf(1.0f, sq - (sq >> 1));   // 2^sq may be no float
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                uint32_t h01, l01, h23, l23, h45, l45, h67, l67;
-                split_e4m3x2(ldexpf(qv[ks][0], sq), ldexpf(qv[ks][1], sq), h01, l01);
-                split_e4m3x2(ldexpf(qv[ks][2], sq), ldexpf(qv[ks][3], sq), h23, l23);
-                split_e4m3x2(ldexpf(qv[ks][4], sq), ldexpf(qv[ks][5], sq), h45, l45);
-                split_e4m3x2(ldexpf(qv[ks][6], sq), ldexpf(qv[ks][7], sq), h67, l67);
-                const bool on = head < G;
-                qa0[2 * ks] = on ? (h01 | (h23 << 16)) : 0u;       // hi: columns 4 quad .. + 3
-                qa0[2 * ks + 1] = on ? (h45 | (h67 << 16)) : 0u;   // hi: columns 16 + 4 quad .. + 3
-                qa2[2 * ks] = on ? (l01 | (l23 << 16)) : 0u;       // lo, likewise
-                qa2[2 * ks + 1] = on ? (l45 | (l67 << 16)) : 0u;
+            for (int ks = 0; ks < KS; ++ks) {
+                const uint32_t v0 = pack_f16x2(qv[ks][0] * up0 * up1, qv[ks][1] * up0 * up1);
+                const uint32_t v2 = pack_f16x2(qv[ks][2] * up0 * up1, qv[ks][3] * up0 * up1);
+                qa0[ks] = head < G ? v0 : 0u;
+                qa2[ks] = head < G ? v2 : 0u;
             }
         } else {
             const uint16_t* qrow = q + ((long long)b * geo.n_q_heads + g * G + (head < G ? head : 0)) * kHeadDim;
@@ -335,66 +366,68 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 qa2[ks] = head < G ? v2 : 0u;
             }
         }
+        float vref = 0.0f;                       // FP8: the largest value scale so far; o is in units of vref / kPScale
         float m_run = -INFINITY, l_run = 0.0f;   // per lane: head `head`, partial over this lane's columns
-        float o[NT][4];
+        // FP8: the lane's score columns are heads 2 quad, 2 quad + 1; o[n]: columns 16 n + head and + 8 of both
+        const float q_unscale0 = FP8 ? __shfl_sync(kFullMask, q_unscale, 8 * quad) * scale : 0.0f;
+        const float q_unscale1 = FP8 ? __shfl_sync(kFullMask, q_unscale, 8 * quad + 4) * scale : 0.0f;
+        float m_run1 = -INFINITY, l_run1 = 0.0f;   // FP8: of head 2 quad + 1 (m_run, l_run: of head 2 quad)
+        constexpr int OT = FP8 ? D / 16 : NT;
+        float o[OT][4];
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
+        for (int n = 0; n < OT; ++n)
 #pragma unroll
             for (int i = 0; i < 4; ++i) o[n][i] = 0.0f;
 
         // pages of this warp: first_page + warp, + 8, ...
         const int my_first = first_page + warp;
         const int my_count = my_first < end_page ? (end_page - my_first + kDenseWarps - 1) / kDenseWarps : 0;
-        // fp8: the pool pages of 32 units at a time, one unit per lane (-1: outside the pool, which fails the group's
-        // listed heads); a table load in front of every unit's copies stalls the warp for a trip to L2.  (The bf16 pass
-        // sits at the HBM rate and lost 2 % to it.)
+        // fp8: the pool pages and the scales of 32 units at a time, one unit per lane (a page outside the pool fails the
+        // group's listed heads); a table load in front of every unit's copies stalls the warp for a trip to L2.  (The bf16
+        // pass sits at the HBM rate and lost 2 % to it.)  Tiles past the sequence and pages outside the pool are copied from
+        // page 0, with scales of 0, and masked.
         int phys0 = 0, phys1 = 0;
+        float kscale0 = 0.0f, kscale1 = 0.0f, vscale0 = 0.0f, vscale1 = 0.0f;
         auto look_up = [&](int k0) {
             const int pl = my_first + (k0 + lane) * kDenseWarps;
-            auto entry = [&](int tile) {
+            auto entry = [&](int tile, float& ks, float& vs) {
+                ks = vs = 0.0f;
                 if (k0 + lane >= my_count || tile * kTileRows >= T) return 0;
                 const int ph = bt[tile >> geo.tile_shift];
-                if (ph >= 0 && ph < geo.pool_pages) return ph;
-                sm.misc[13] = 1;   // (cleared at the end of the previous item)
-                return -1;
+                if (ph < 0 || ph >= geo.pool_pages) {
+                    atomicMax(&sm.misc[13], 1);   // (cleared at the end of the previous item)
+                    return 0;
+                }
+                const long long at = (long long)ph * geo.kv_heads_stored + g / geo.kv_div;
+                ks = k_scale[at];
+                vs = v_scale[at];
+                return ph;
             };
-            phys0 = entry(2 * pl);
-            phys1 = entry(2 * pl + 1);
+            phys0 = entry(2 * pl, kscale0, vscale0);
+            phys1 = entry(2 * pl + 1, kscale1, vscale1);
             __syncwarp();
         };
         auto issue = [&](int k) {   // k-th unit of this warp into stage k % kStages
             if (FP8 && (k & 31) == 0) look_up(k);
             const int pl = my_first + k * kDenseWarps;
-            const uint32_t dst = ring_addr + (uint32_t)((k % kStages) * kStageBytes);
             if constexpr (FP8) {
-                // 32 rows of 128 bytes per cache: lane covers 16-byte chunk lane % 8 of rows lane / 8 + 4 i; the two
-                // halves of the unit are tiles 2 pl and 2 pl + 1 (one page, or two pages with their own scales)
-                const int ch = lane & 7, r0 = lane >> 3;
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    const int tile = 2 * pl + hf;
-                    const int rows_here = min(kTileRows, T - tile * kTileRows);   // <= 0: the half lies past the sequence
-                    const int looked_up = __shfl_sync(kFullMask, hf == 0 ? phys0 : phys1, k & 31);
-                    const long long phys = max(looked_up, 0);
-                    const int valid_rows = looked_up >= 0 ? rows_here : 0;
-                    const long long off8 = phys * geo.page_stride + (long long)(g / geo.kv_div) * geo.head_stride + ch * 16 +
-                                           (long long)((tile & ((1 << geo.tile_shift) - 1)) * kTileRows) * geo.token_stride;
-                    const uint8_t* kp = reinterpret_cast<const uint8_t*>(k_cache) + off8;
-                    const uint8_t* vp = reinterpret_cast<const uint8_t*>(v_cache) + off8;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int r = r0 + 4 * i, row = hf * 16 + r;
-                        const uint32_t off = (uint32_t)(row * 128 + ((ch ^ (row & 7)) << 4));
-                        const bool ok = r < valid_rows;
-                        cp_async_16_zfill(dst + off, kp + (long long)r * geo.token_stride, ok);
-                        cp_async_16_zfill(dst + Cfg::kRawBytes + off, vp + (long long)r * geo.token_stride, ok);
-                    }
-                    if (lane < 2) {   // the half's two scales ride the same stage: [k0, k1, v0, v1]
-                        const float* sp = (lane == 0 ? k_scale : v_scale) + phys * geo.kv_heads_stored + g / geo.kv_div;
-                        cp_async_4(dst + 2 * Cfg::kRawBytes + 8 * lane + 4 * hf, sp);
-                    }
+                // four tiles of 2 KB, asked for by one lane (16 copies of 16 bytes per lane, with their addresses, took 116 us
+                // per layer where the tiles took 108, all else the same)
+                const int page0 = __shfl_sync(kFullMask, phys0, k & 31), page1 = __shfl_sync(kFullMask, phys1, k & 31);
+                if (lane == 0) {
+                    const int stage = (used + k) % kStages, in_page = (1 << geo.tile_shift) - 1, head_at = g / geo.kv_div;
+                    const int row0 = ((2 * pl) & in_page) * kTileRows, row1 = ((2 * pl + 1) & in_page) * kTileRows;
+                    const uint32_t dst = ring_addr + (uint32_t)(stage * kStageBytes);
+                    const uint32_t bar = bars + 8u * (uint32_t)(warp * kStages + stage);
+                    mbar_expect_tx(bar, kStageBytes);
+                    tma_tile(dst, &maps.k, row0, head_at, page0, bar);
+                    tma_tile(dst + Cfg::kRawBytes / 2, &maps.k, row1, head_at, page1, bar);
+                    tma_tile(dst + Cfg::kRawBytes, &maps.v, row0, head_at, page0, bar);
+                    tma_tile(dst + Cfg::kRawBytes * 3 / 2, &maps.v, row1, head_at, page1, bar);
                 }
+                __syncwarp();
             } else {
+            const uint32_t dst = ring_addr + (uint32_t)((k % kStages) * kStageBytes);
             long long phys = bt[pl >> geo.tile_shift];
             const bool page_ok = phys >= 0 && phys < geo.pool_pages;
             if (!page_ok) {
@@ -419,102 +452,129 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
 #pragma unroll
         for (int s = 0; s < kStages - 1; ++s) {
             if (s < my_count) issue(s);
-            cp_async_commit();
+            if constexpr (!FP8) cp_async_commit();
         }
         for (int k = 0; k < my_count; ++k) {
+            float ks0 = 0.0f, ks1 = 0.0f, vs0 = 0.0f, vs1 = 0.0f;
+            if constexpr (FP8) {   // (before the next look-up)
+                static_assert(kStages == 2, "a look-up is one unit ahead at most");
+                ks0 = __shfl_sync(kFullMask, kscale0, k & 31), ks1 = __shfl_sync(kFullMask, kscale1, k & 31);
+                vs0 = __shfl_sync(kFullMask, vscale0, k & 31), vs1 = __shfl_sync(kFullMask, vscale1, k & 31);
+            }
             if (k + kStages - 1 < my_count) issue(k + kStages - 1);
-            cp_async_commit();
-            cp_async_wait<kStages - 1>();
+            if constexpr (FP8) {
+                const int seq = used + k;
+                const uint32_t bar = bars + 8u * (uint32_t)(warp * kStages + seq % kStages);
+                // (waited for once more before the stage can be written again or the block can end)
+                if (!mbar_wait(bar, (uint32_t)(seq / kStages) & 1u)) {
+                    atomicMax(&sm.misc[13], 2);
+                    mbar_wait(bar, (uint32_t)(seq / kStages) & 1u);
+                }
+            } else {
+                cp_async_commit();
+                cp_async_wait<kStages - 1>();
+            }
             __syncwarp();
             if constexpr (FP8) {
             const int pl = my_first + k * kDenseWarps;
             const int valid = min(kUnit, T - pl * kUnit);   // > 0
-            const uint32_t kbase = ring_addr + (uint32_t)((k % kStages) * kStageBytes);
+            const int stage = (used + k) % kStages;
+            const uint32_t kbase = ring_addr + (uint32_t)(stage * kStageBytes);
             const uint32_t vbase = kbase + Cfg::kRawBytes;
-            const float* scales = reinterpret_cast<const float*>(my_ring + (k % kStages) * kStageBytes + 2 * Cfg::kRawBytes);
-            const float ks0 = scales[0], ks1 = scales[1], vs0 = scales[2], vs1 = scales[3];
+            if (valid < kUnit) {   // value rows past the sequence have weight 0, but may hold NaN
+                uint4* row = reinterpret_cast<uint4*>(my_ring + stage * kStageBytes + Cfg::kRawBytes + lane * 128);
+                if (lane >= valid)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) row[i] = make_uint4(0u, 0u, 0u, 0u);
+                __syncwarp();
+            }
 
-            // S = Q K^T for the 32 tokens of the unit (four 8-token column tiles), q = hi + lo
-            float sc4[4][4];
+            // S^T = K Q^T for the 32 tokens of the unit (two 16-token row tiles): tokens are the rows of the MMA, which the
+            // few heads of a group would leave half empty
+            float st[2][4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < 2; ++j)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sc4[j][i] = 0.0f;
+                for (int i = 0; i < 4; ++i) st[j][i] = 0.0f;
             {
                 // ldmatrix.x4 on byte rows: matrix mi = lane / 8 is (tokens 8 (mi / 2) .. + 7) x (16-byte chunk 2 ks + mi % 2);
-                // a lane receives 4 consecutive columns of one token: the B fragment of an m16n8k32 MMA
+                // a lane receives 4 consecutive columns of one token: two slots of either half of a step, see qa0
                 const int mi = lane >> 3, rr = lane & 7;
 #pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    const int tok = hf * 16 + (mi >> 1) * 8 + rr;
+                for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const int ch = 2 * ks + (mi & 1);
-                        uint32_t r[4];
+                    for (int hf = 0; hf < 2; ++hf) {
+                        const int tok = hf * 16 + (mi >> 1) * 8 + rr, ch = 2 * ks + (mi & 1);
+                        uint32_t r[4], a[4];
                         ldmatrix_x4(r, kbase + (uint32_t)(tok * 128 + ((ch ^ (tok & 7)) << 4)));
-                        mma_e4m3(sc4[2 * hf], qa0[2 * ks], qa2[2 * ks], qa0[2 * ks + 1], qa2[2 * ks + 1], r[0], r[1]);
-                        mma_e4m3(sc4[2 * hf + 1], qa0[2 * ks], qa2[2 * ks], qa0[2 * ks + 1], qa2[2 * ks + 1], r[2], r[3]);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            e4m3x4_to_f16(r[i], a[0], a[2]);
+                            e4m3x4_to_f16(r[2 + i], a[1], a[3]);
+                            mma_f16(st[hf], a[0], a[1], a[2], a[3], qa0[2 * ks + i], qa2[2 * ks + i]);
+                        }
                     }
-                }
             }
-            // this lane: head `head`, tokens 8 j + 2 quad, + 1 of column tile j = 0 .. 3
-            float t[8];
+            // this lane: heads 2 quad (ta) and 2 quad + 1 (tb), tokens head + 8 j (head = lane / 4)
+            float ta[4], tb[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {   // the page's key scale folded in
+                ta[j] = st[j >> 1][2 * (j & 1)] * (q_unscale0 * (j < 2 ? ks0 : ks1));
+                tb[j] = st[j >> 1][2 * (j & 1) + 1] * (q_unscale1 * (j < 2 ? ks0 : ks1));
+            }
+            if (valid < kUnit)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (head + 8 * j >= valid) ta[j] = tb[j] = -INFINITY;
+            float ma = fmaxf(fmaxf(ta[0], ta[1]), fmaxf(ta[2], ta[3])), mb = fmaxf(fmaxf(tb[0], tb[1]), fmaxf(tb[2], tb[3]));
+            const float vmax = fmaxf(vs0, vs1);
+            // a new maximum (of the scores or of the value scales), rarer with every unit: reduce it and rescale the sums
+            if (__any_sync(kFullMask, ma > m_run || mb > m_run1) || vmax > vref) {
+#pragma unroll
+                for (int off = 4; off < 32; off <<= 1) {
+                    ma = fmaxf(ma, __shfl_xor_sync(kFullMask, ma, off));
+                    mb = fmaxf(mb, __shfl_xor_sync(kFullMask, mb, off));
+                }
+                ma = fmaxf(ma, m_run), mb = fmaxf(mb, m_run1);   // finite: token 0 of a unit is always valid
+                const float fa = exp2f(m_run - ma), fb = exp2f(m_run1 - mb);   // 0 on the first unit
+                l_run *= fa, l_run1 *= fb;
+                const float fv = vmax > vref ? vref / vmax : 1.0f;
+                vref = fmaxf(vref, vmax);
+#pragma unroll
+                for (int n = 0; n < OT; ++n) {
+                    o[n][0] *= fa * fv, o[n][1] *= fb * fv;
+                    o[n][2] *= fa * fv, o[n][3] *= fb * fv;
+                }
+                m_run = ma, m_run1 = mb;
+            }
+            // P as f16 operands: p * (value scale of its page / vref) * kPScale, normal numbers down to p = 2^-28; packed by
+            // token, then transposed into the B fragment (tokens are the contraction's index)
+            auto weight = [&](float vs) { return vs == vref ? kPScale : vref > 0.0f ? kPScale * (vs / vref) : 0.0f; };
+            const float w0 = weight(vs0), w1 = weight(vs1);
+            uint32_t pb[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float ts = scale * q_unscale * (j < 2 ? ks0 : ks1);   // the page's key scale folded in
-                t[2 * j] = (8 * j + 2 * quad < valid) ? (sc4[j][0] + sc4[j][2]) * ts : -INFINITY;   // hi + lo rows
-                t[2 * j + 1] = (8 * j + 2 * quad + 1 < valid) ? (sc4[j][1] + sc4[j][3]) * ts : -INFINITY;
+                const float pa = exp2f(ta[j] - m_run), pc = exp2f(tb[j] - m_run1);
+                l_run += pa, l_run1 += pc;
+                pb[j] = transpose_8x8(pack_f16x2(pa * (j < 2 ? w0 : w1), pc * (j < 2 ? w0 : w1)));
             }
-            float pm = fmaxf(fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])), fmaxf(fmaxf(t[4], t[5]), fmaxf(t[6], t[7])));
-            pm = fmaxf(pm, __shfl_xor_sync(kFullMask, pm, 1));
-            pm = fmaxf(pm, __shfl_xor_sync(kFullMask, pm, 2));
-            const float m_new = fmaxf(m_run, pm);       // finite: token 0 of a unit is always valid
-            const float corr = exp2f(m_run - m_new);    // 0 on the first unit
-            float p[8], psum = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                p[i] = exp2f(t[i] - m_new);
-                psum += p[i];
-            }
-            l_run = fmaf(l_run, corr, psum);
-            if (__any_sync(kFullMask, m_new > m_run)) {
-#pragma unroll
-                for (int n = 0; n < NT; ++n) {
-                    o[n][0] *= corr;
-                    o[n][1] *= corr;
-                }
-            }
-            m_run = m_new;
-            // P as e4m3 operands: p * (value scale of its page / the larger of the two scales) * 2^8 = hi + lo.
-            // The 8 tokens of this lane take the lane's 8 slots of the contraction index: slots 4 quad .. + 3 are
-            // tokens 2 quad, 2 quad + 1, 8 + 2 quad, 9 + 2 quad, slots 16 + 4 quad .. + 3 the same + 16; the V rows
-            // are fetched in the matching order below.
-            const float vref = fmaxf(vs0, vs1);
-            const float w0 = vref > 0.0f ? 256.0f * (vs0 / vref) : 0.0f, w1 = vref > 0.0f ? 256.0f * (vs1 / vref) : 0.0f;
-            uint32_t h01, l01, h23, l23, h45, l45, h67, l67;
-            split_e4m3x2(p[0] * w0, p[1] * w0, h01, l01);
-            split_e4m3x2(p[2] * w0, p[3] * w0, h23, l23);
-            split_e4m3x2(p[4] * w1, p[5] * w1, h45, l45);
-            split_e4m3x2(p[6] * w1, p[7] * w1, h67, l67);
-            const uint32_t ph0 = h01 | (h23 << 16), ph2 = h45 | (h67 << 16), pl0 = l01 | (l23 << 16), pl2 = l45 | (l67 << 16);
-            const float oscale = vref * (1.0f / 256.0f);
 
-            // O += P V, 16 columns at a time: one transposing byte load per 32 tokens x 16 columns
+            // O^T += V^T P^T, 16 columns at a time: one transposing byte load per 32 tokens x 16 columns.  A lane's four rows
+            // of a column are tokens 2 quad, 2 quad + 1, 8 + 2 quad, 9 + 2 quad of the half: two slots of either half of a step.
             {
                 const int rrow = lane & 15, qd = rrow >> 2, ii = rrow & 3;
                 const int tokp = (lane >> 4) * 16 + ((ii < 2) ? 0 : 8) + 2 * qd + (ii & 1);
                 const uint32_t vrow = vbase + (uint32_t)(tokp * 128);
 #pragma unroll
                 for (int dp = 0; dp < 8; ++dp) {
-                    uint32_t r[4];
+                    uint32_t r[4], a[4];
                     ldmatrix_x2_trans_b8(r, vrow + (uint32_t)((dp ^ (tokp & 7)) << 4));
-                    float ta[4] = {0.f, 0.f, 0.f, 0.f}, tb[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma_e4m3(ta, ph0, pl0, ph2, pl2, r[0], r[2]);
-                    mma_e4m3(tb, ph0, pl0, ph2, pl2, r[1], r[3]);
-                    o[2 * dp][0] = fmaf(ta[0] + ta[2], oscale, o[2 * dp][0]);
-                    o[2 * dp][1] = fmaf(ta[1] + ta[3], oscale, o[2 * dp][1]);
-                    o[2 * dp + 1][0] = fmaf(tb[0] + tb[2], oscale, o[2 * dp + 1][0]);
-                    o[2 * dp + 1][1] = fmaf(tb[1] + tb[3], oscale, o[2 * dp + 1][1]);
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf) {
+                        e4m3x4_to_f16(r[2 * hf], a[0], a[2]);
+                        e4m3x4_to_f16(r[2 * hf + 1], a[1], a[3]);
+                        mma_f16(o[dp], a[0], a[1], a[2], a[3], pb[2 * hf], pb[2 * hf + 1]);
+                    }
                 }
             }
             } else {
@@ -577,23 +637,51 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             }
             __syncwarp();   // the stage is overwritten by a later issue
         }
-        cp_async_wait<0>();
+        if constexpr (FP8)
+            used += my_count;   // (every one of them has been waited for)
+        else
+            cp_async_wait<0>();
 
-        // ---- merge: quad lanes share a head (sum l), then the warps, into one partial per head ----
-        l_run += __shfl_xor_sync(kFullMask, l_run, 1);
-        l_run += __shfl_xor_sync(kFullMask, l_run, 2);
-        __syncthreads();   // every warp is done with its ring: reuse it for the merge
-        float* mg = reinterpret_cast<float*>(sm.ring);   // [warps][G][2 + 128]
-        if (head < G) {
-            float* rec = mg + (warp * G + head) * kPartialFloats;
-            if (quad == 0) {
-                rec[0] = m_run;
-                rec[1] = l_run;
-            }
+        // ---- merge: the lanes that share a head (sum l), then the warps, into one partial per head ----
+        float* mg = reinterpret_cast<float*>(sm.ring);   // [warps][G][2 + 128], in the place of the ring
+        if constexpr (FP8) {
 #pragma unroll
-            for (int n = 0; n < NT; ++n) {
-                rec[2 + n * 8 + quad * 2] = o[n][0];
-                rec[2 + n * 8 + quad * 2 + 1] = o[n][1];
+            for (int off = 4; off < 32; off <<= 1) {
+                l_run += __shfl_xor_sync(kFullMask, l_run, off);
+                l_run1 += __shfl_xor_sync(kFullMask, l_run1, off);
+            }
+            __syncthreads();   // every warp is done with its ring
+            const float o_unit = vref * (1.0f / kPScale);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int hh = 2 * quad + i;
+                if (hh >= G) continue;
+                float* rec = mg + (warp * G + hh) * kPartialFloats;
+                if (head == 0) {
+                    rec[0] = i ? m_run1 : m_run;
+                    rec[1] = i ? l_run1 : l_run;
+                }
+#pragma unroll
+                for (int n = 0; n < OT; ++n) {
+                    rec[2 + n * 16 + head] = o[n][i] * o_unit;
+                    rec[2 + n * 16 + 8 + head] = o[n][2 + i] * o_unit;
+                }
+            }
+        } else {
+            l_run += __shfl_xor_sync(kFullMask, l_run, 1);
+            l_run += __shfl_xor_sync(kFullMask, l_run, 2);
+            __syncthreads();   // every warp is done with its ring
+            if (head < G) {
+                float* rec = mg + (warp * G + head) * kPartialFloats;
+                if (quad == 0) {
+                    rec[0] = m_run;
+                    rec[1] = l_run;
+                }
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    rec[2 + n * 8 + quad * 2] = o[n][0];
+                    rec[2 + n * 8 + quad * 2 + 1] = o[n][1];
+                }
             }
         }
         __syncthreads();
@@ -615,7 +703,8 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             dst[2 + e] = a;
             if (e == 0) {
                 dst[0] = M;
-                dst[1] = sm.misc[13] ? -1.0f : L;   // sums are never negative: -1 marks a page outside the pool
+                // sums are never negative: -1 marks a page outside the pool, -2 a copy that did not land
+                dst[1] = sm.misc[13] ? -(float)sm.misc[13] : L;
             }
         }
 
@@ -642,18 +731,17 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 const int hh = idx / kHeadDim, e = idx % kHeadDim;
                 if (!((mask >> hh) & 1u)) continue;
                 float M = -INFINITY;
-                bool bad_page = false;
+                float failed = 0.0f;   // -1: a page outside the pool, -2: a copy that did not land
                 for (int it = 0; it < items_of_group; ++it) {
                     M = fmaxf(M, ms_s[it * G + hh]);
-                    bad_page |= ls_s[it * G + hh] < 0.0f;
+                    failed = fminf(failed, ls_s[it * G + hh]);
                 }
                 const long long unit = (long long)b * geo.n_q_heads + g * G + hh;
-                if (bad_page) {
-                    // a block-table entry of the sequence is outside the pool: no dense result exists
+                if (failed < 0.0f) {   // no dense result exists
                     out[unit * kHeadDim + e] = 0.0f;
                     if (e == 0 && diag) {
                         diag[unit].lse = 0.0f;
-                        diag[unit].status = VSA_UNIT_BAD_PAGE;
+                        diag[unit].status = failed < -1.0f ? VSA_UNIT_COPY_TIMEOUT : VSA_UNIT_BAD_PAGE;
                     }
                     continue;
                 }
@@ -671,6 +759,7 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             }
         }
         if (tid == 0) sm.misc[13] = 0;
+        if constexpr (FP8) fence_async_proxy();
         __syncthreads();   // the ring (merge buffer) and misc are reused by the next item
     }
 }
@@ -683,13 +772,37 @@ int dense_max_items(const Geometry& g) { return g.batch * g.n_kv_heads + 2048; }
 size_t dense_smem_bytes(const Geometry& g, bool fp8 = false)
 {
     const size_t n_groups = (size_t)g.batch * g.n_kv_heads;
-    const size_t ring = fp8 ? DenseCfg<128, true>::kRingBytes
+    const size_t ring = fp8 ? DenseCfg<128, true>::kRingBytes + DenseCfg<128, true>::kBarBytes
                             : g.head_dim == 64 ? DenseCfg<64>::kRingBytes
                                                : (g.head_dim == 256 ? DenseCfg<256>::kRingBytes : DenseCfg<128>::kRingBytes);
     return ring + (n_groups + 1) * 4 + 32 * 4 + (n_groups + 15) / 16 * 16;
 }
 
 }  // namespace
+
+// A pool of e4m3 rows as a 4-d tensor, box = one tile of 16 rows, swizzled as ldmatrix reads it.  The entry points have
+// checked what the encoding asks for: base and strides are multiples of 16 bytes.  (The stride of an extent of one page or
+// head is never used; it may be any number.)
+static bool encode_pool(CUtensorMap* map, const void* pool, const Geometry& g)
+{
+    using Encode = decltype(&cuTensorMapEncodeTiled);
+    static const Encode encode = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<Encode>(f);
+    }();
+    if (!encode) return false;
+    const cuuint64_t dims[4] = {128, (cuuint64_t)g.page_size, (cuuint64_t)g.kv_heads_stored, (cuuint64_t)g.pool_pages};
+    const cuuint64_t strides[3] = {(cuuint64_t)g.token_stride, (cuuint64_t)(g.kv_heads_stored > 1 ? g.head_stride : 128),
+                                   (cuuint64_t)(g.pool_pages > 1 ? g.page_stride : 128)};
+    const cuuint32_t box[4] = {128, kTileRows, 1, 1}, element_strides[4] = {1, 1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(pool), dims, strides, box, element_strides,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 static size_t dense_counter_bytes(const Geometry& g_in)
 {
@@ -722,10 +835,13 @@ static cudaError_t launch_dense_gd(const Geometry& g, const uint16_t* q, const u
     static bool attr_done[kMaxDevices] = {};   // per template instance
     const cudaError_t e = allow_large_dynamic_smem(dense_split_kernel<G, D, FP8>, attr_done);
     if (e != cudaSuccess) return e;
+    DenseMaps<FP8> maps;
+    if constexpr (FP8)
+        if (!encode_pool(&maps.k, k, g) || !encode_pool(&maps.v, v, g)) return cudaErrorInvalidValue;
     // persistent grid: one block per SM (the ring fills the shared memory)
     return launch_pdl(dense_split_kernel<G, D, FP8>, dim3((unsigned)num_sms()), dim3(DenseCfg<D, FP8>::kDenseThreads), smem,
                       stream, g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials,
-                      counters, out, diag, dense_max_items(g), k_scale, v_scale);
+                      counters, out, diag, dense_max_items(g), k_scale, v_scale, maps);
 }
 
 template <int G>
