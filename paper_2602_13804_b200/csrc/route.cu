@@ -3,7 +3,7 @@
 //
 //   route_scan_kernel    streams the summary rows (the only part of the step whose traffic grows
 //                        with the context length) and writes all page scores to scratch.
-//   route_list_kernel    the same for ragged batches: the pages that exist, shared evenly.
+//   route_list_kernel    the same where the grid is several waves: the pages that exist, shared evenly.
 //   route_select_kernel  one block per (sequence, query head): exact top-P selection.
 #include <math.h>
 
@@ -25,6 +25,9 @@ constexpr int kBlockPages = 32;      // pages per block-table block (one coalesc
 // sequences of 32k 145 / 141 / 144 / 152; 32 sequences of 16k - 64k 84.4 / 82.9 / 80.9 / 96.1; 64 sequences of
 // 4k - 128k at head dimension 64 143 / 132 / 130 / 136.
 constexpr int kMaxBlocksPerWarp = 4;
+// Table width from which, and sequences up to which, the list scan takes batches of even lengths.
+constexpr int kListPages = 2048;
+constexpr int kListBatch = 256;
 
 template <int G, int D = kHeadDim>
 struct ScanCfg {
@@ -248,9 +251,9 @@ route_scan_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* 
     }
 }
 
-// ---- the scan over a list of pages, for large batches that are probably ragged ----
+// ---- the scan over a list of pages, for several waves of blocks ----
 // The grid of the kernel above is sized for the longest sequence; in a ragged batch most of its blocks find no page,
-// and the others run in waves that each pay the start-up of a block.  Here the pages of all sequences, in units of 8,
+// and in any the others run in waves that each pay the start-up of a block.  Here the pages of all sequences, in units of 8,
 // form one list that one wave of warps shares evenly: warp w takes KV head w % n_kv and the (w / n_kv)-th range of the
 // list, part by part as it crosses sequences.  The start is a longer chain (lengths, their sums, then the table), so
 // small batches keep the kernel above (batch 8, T = 32k: 2.4 us less).  DEPTH rounds of a warp's rows are in flight in
@@ -498,16 +501,30 @@ cudaError_t launch_scan_g(const Geometry& g, const uint16_t* q, const uint16_t* 
                           int zero_count, const float* radii, float* rad_logical, cudaStream_t stream)
 {
     if constexpr (!CERT && D == kHeadDim && G != 2) {
-        // The pool has fewer than half of the pages that `batch` sequences of the table's width would have of their own -
-        // the sequences are of uneven length, or share prefixes - and the grid is more than two waves of blocks: share
-        // the pages that exist.  Lengths are not known here; where they are even after all the list costs nothing (64
-        // sequences of 16k that share three quarters 100 us per layer against 102, 64 of 32k without 141 against 142).
-        // Uneven ones, list against grid: 64 sequences of 4k - 128k with four heads a group 149 / 162, with eight
-        // 253 / 288; 32 of 2k - 128k 75.5 / 84.8, with one head a group 129 / 149; 48 of 2k - 32k 86.7 / 86.9.  With two
-        // heads a group the list loses (64 of 8k - 96k 251 / 226, 64 of 4k - 64k 180 / 172).
+        // Share the pages that exist, instead of a grid sized for the longest sequence.  A wave of the grid ends with its
+        // slowest warp and each warp pays its start-up; the list pays a longer start and an ordinary launch once, about
+        // 3 us.  It wins from so many waves of 32-page blocks on, where the table holds long sequences; microseconds per
+        // layer, grid / list, by waves:
+        //   four heads a group: 2.2 33 / 36, 3.5 27.7 / 28.8 (4 of 128k) and 39.2 / 39.1 (16 of 32k), 4.3 44.9 / 42.3 (10 of
+        //   64k), 5.2 39.7 / 37.1 (6 of 128k) and 62.2 / 61.5 (24 of 32k), 6.9 46.8 / 43.1 (8 of 128k) and 70.9 / 69.4 (32
+        //   of 32k), 13.8 79.2 / 75.9 (16 of 128k);
+        //   eight, whose round computes twice as long on a row: 1.7 42.1 / 40.0, 2.2 58.3 / 57.2, 3.5 40.6 / 37.8, 13.8 149 / 144;
+        //   one: 1.7 19.6 / 20.1, 2.6 22.9 / 23.1, 3.5 25.7 / 26.1, 4.3 33.3 / 29.0, 6.9 37.8 / 35.0, 13.8 68.6 / 58.8;
+        //   two: the list loses (6.9 78.2 / 82.2, 104 / 111).
+        // Short sequences gain nothing: with four heads 64 of 16k 94.8 / 94.8, 48 of 16k 80.1 / 80.9, 64 of 12k 88.5 / 89.4;
+        // with eight 64 of 8k 150 / 150; with one 16 of 8k 40.4 / 41.1.
+        // Where the pool has fewer than half of the pages that `batch` sequences of the table's width would have of their own -
+        // the sequences are of uneven length, or share prefixes - two waves are enough (lengths are not known here): 64
+        // sequences of 4k - 128k with four heads a group 162 / 149, with eight 288 / 253; 32 of 2k - 128k 84.8 / 75.5, with
+        // one head a group 149 / 129; 48 of 2k - 32k 86.9 / 86.7.
+        // (The sums over the lengths are formed by every block, hence a bound on their number.)
         const long long warps = (long long)g.batch * g.n_kv_heads * ((g.max_pages + kBlockPages - 1) / kBlockPages);
         const long long wave = 2LL * kScanWarps * device_sm_count();
-        if (!g.super_pages && (long long)g.batch * g.max_pages >= 2 * g.pool_pages && warps > 2 * wave && g.n_kv_heads <= wave) {
+        const bool uneven = (long long)g.batch * g.max_pages >= 2 * g.pool_pages;
+        constexpr int kHalfWaves = G == 8 ? 3 : 8;
+        const bool enough = (uneven && warps > 2 * wave) ||
+                            (g.max_pages >= kListPages && g.batch <= kListBatch && 2 * warps >= kHalfWaves * wave);
+        if (!g.super_pages && enough && g.n_kv_heads <= wave) {
             const int ranges = (int)(wave / g.n_kv_heads);
             const size_t smem = std::max(kScanWarps * (size_t)ListCfg<G>::WARP_BYTES + ((size_t)g.batch + 1) * 4, (size_t)81 * 1024);
             static bool attr_done[kMaxDevices] = {};

@@ -28,3 +28,15 @@ def test_list_scan(hq, hkv, page, long, short):
     assert w.block_table.shape[0] * w.block_table.shape[1] >= 2 * w.pool_pages
     assert batch * heads * blocks > 2 * 2368
     compare(w, run_gpu(w), dense_sample=4)
+
+@pytest.mark.parametrize("hq,hkv,batch,blocks", [(16, 2, 28, 65), (8, 8, 19, 65)])
+def test_list_scan_of_a_full_pool(hq, hkv, batch, blocks):
+    # (sequences of one table width in a pool that holds them, from so many waves of warps on)
+    assert 2 * batch * hkv * blocks >= (3 if hq > hkv else 8) * 2368
+    pages = 32 * blocks - 5      # 2048 at least
+    lens = [(1, 17, 300, 1025)[i % 4] for i in range(batch)]
+    lens[0] = lens[-1] = pages * 16 - 3
+    w = make_workload(WorkloadSpec(name="list", config=9, batch=batch, n_q_heads=hq, n_kv_heads=hkv, P=8, K_c=40,
+                                   seq_lens=tuple(lens), needles=3, pool_pages=batch * pages // 2 + 1), seed=8500 + hq + hkv)
+    assert w.block_table.shape[0] * w.block_table.shape[1] < 2 * w.pool_pages
+    compare(w, run_gpu(w), dense_sample=4)
