@@ -1024,16 +1024,20 @@ template <int D, bool FP8>
 cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
 {
     const bool fused = p.page_scores != nullptr;
-    // Five blocks per SM at 96 registers against four at 128, whose unspilled registers make a unit faster: five win from
-    // three waves of four on, where units in flight count for more.  Microseconds per layer, four / five, T = 8k: 64 pages a
-    // unit 1536 units 131 / 143, 1664 138 / 150, 1792 155 / 154, 2048 170 / 165, 3072 245 / 241; 32 pages 1664 84 / 93,
-    // 1792 93 / 95, 2048 100.4 / 100.1; D = 256 1536 138 / 149, 1792 164 / 165, 2048 179 / 176; e4m3 cache 1792 92 / 75, 3072
-    // 151 / 128.  Below the line they win only where they save a whole wave (640 units of 32 pages 47 / 40, 1280 73 / 71)
-    // and on the e4m3 cache (1024 units 51 / 49); those counts are not in the rule.  Head dimension 64 loses at any (3072
-    // units 100 / 109).
-    if constexpr (D >= 128)
-        if (threads == 128 && fused && (long long)p.geo.batch * p.geo.n_q_heads >= 3LL * 4 * device_sm_count())
-            return launch_step_variant<128, true, D, FP8, 0, 5>(p, stream);
+    // Five blocks per SM at 96 registers against four at 128, whose unspilled registers make a unit 5 - 10 % faster: five
+    // where they save a wave of blocks, and from three waves of four on, where units in flight count for more.  Microseconds
+    // per layer, four / five, T = 8k.  A wave saved: 32 pages a unit, 640 units 41.6 / 31.9, 704 43.5 / 32.5, 1280 65.4 / 56.0,
+    // 1472 68.1 / 63.6; 64 pages 640 66.0 / 48.0, 1472 107 / 100; e4m3 cache 640 39.6 / 29.0, 1472 68.6 / 56.6; D = 64 640
+    // 36.0 / 29.2, 1472 63.6 / 60.4; D = 256 640 66.4 / 50.7, 1472 109 / 102.  None saved: 512 26.6 / 29.1, 768 45.1 / 44.5,
+    // 1024 47.7 / 50.6, 1152 49.2 / 52.8.  From three waves on: 32 pages 1792 84.0 / 75.9,
+    // 2240 90.1 / 90.1, 3200 131 / 120; 64 pages 2048 140 / 124; e4m3 cache 2048 89.2 / 78.7; D = 64 2240 75.8 / 75.7, 3200
+    // 114 / 106; D = 256 2240 146 / 147, 3200 214 / 199.  Not where five do not fit the shared memory of an SM (D = 256, 64
+    // pages a unit: four 1 % faster).
+    const long long units = (long long)p.geo.batch * p.geo.n_q_heads, four = 4LL * device_sm_count(), five = 5LL * device_sm_count();
+    const bool fits = (size_t)p.lay.total * 4 + 1024 <= (size_t)228 * 1024 / 5;   // (1 KB of each block is the system's)
+    if (threads == 128 && fused && fits &&
+        ((units + five - 1) / five < (units + four - 1) / four || units >= 3 * four))
+        return launch_step_variant<128, true, D, FP8, 0, 5>(p, stream);
 #define VSA_STEP_CASE(T)                                                                    \
     if (threads == T)                                                                       \
         return fused ? launch_step_variant<T, true, D, FP8>(p, stream)                      \
