@@ -158,6 +158,98 @@ struct DenseSmem {
     int32_t* misc;         // [32]
 };
 
+// The partials of a (sequence, KV head) combined by the block that finished its last item.  Out of line: the kernel's
+// registers and code are those of its main loop.
+template <int G, int D, bool FP8>
+__device__ __noinline__ void combine_items(float* ring, float* misc, const float* gp, int items_of_group, uint32_t mask,
+                                           long long first_unit, float* out, vsa_diag_t* diag)
+{
+    using Cfg = DenseCfg<D, FP8>;
+    constexpr int kDenseThreads = Cfg::kDenseThreads, kDenseWarps = Cfg::kDenseWarps, kPartialFloats = Cfg::kPartialFloats, kHeadDim = D;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // Every item's (max, sum) of every head in shared memory, then the listed heads and their items dealt out to the
+    // warps: the loads are independent, and one head keeps every warp busy.  A thread per column that walked all
+    // items paid a memory round trip for every eight of them: with this and the 32-bit divisions above one
+    // sequence of 128k that falls back 131 -> 118 us per layer, one unit of four in 4 of 2k - 8k 36.8 -> 34.5, the
+    // same at D = 256 63.9 -> 56.4.
+    float* ms_s = ring;                                 // [items][G]
+    float* ls_s = ms_s + (size_t)items_of_group * G;    // [items][G]
+    float* sums = ms_s + ((size_t)2 * items_of_group * G + 3) / 4 * 4;   // [warps][G][2 + D]
+    for (int i = tid; i < items_of_group * G; i += kDenseThreads) {
+        const float* rec = gp + (long long)i * kPartialFloats;
+        ms_s[i] = __ldcg(rec);
+        ls_s[i] = __ldcg(rec + 1);
+    }
+    __syncthreads();
+    const int heads = __popc(mask), per_head = heads < kDenseWarps ? kDenseWarps / heads : 1;   // warps for each head
+    const int slice = warp % per_head;
+#pragma unroll 1
+    for (int n = warp / per_head; n < heads; n += kDenseWarps / per_head) {
+        uint32_t from_nth = mask;
+        for (int i = 0; i < n; ++i) from_nth &= from_nth - 1u;
+        const int hh = __ffs(from_nth) - 1;   // the n-th listed head
+        float M = -INFINITY, failed = 0.0f;   // failed: -1 a page outside the pool, -2 a copy that did not land
+        for (int it = lane; it < items_of_group; it += 32) {
+            M = fmaxf(M, ms_s[it * G + hh]);
+            failed = fminf(failed, ls_s[it * G + hh]);
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) {
+            M = fmaxf(M, __shfl_xor_sync(kFullMask, M, off));
+            failed = fminf(failed, __shfl_xor_sync(kFullMask, failed, off));
+        }
+        constexpr int PAIRS = D / 64;   // columns 64 j + 2 lane, + 1
+        float2 acc[PAIRS];
+        float L = 0.0f;
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) acc[j] = make_float2(0.0f, 0.0f);
+#pragma unroll 4
+        for (int it = slice; it < items_of_group; it += per_head) {
+            const float ms = ms_s[it * G + hh];
+            const float f = ms == -INFINITY ? 0.0f : exp2f(ms - M);
+            const float2* rec = reinterpret_cast<const float2*>(gp + ((long long)it * G + hh) * kPartialFloats + 2) + lane;
+#pragma unroll
+            for (int j = 0; j < PAIRS; ++j) {
+                const float2 x = __ldcg(rec + 32 * j);
+                acc[j].x = fmaf(x.x, f, acc[j].x);
+                acc[j].y = fmaf(x.y, f, acc[j].y);
+            }
+            L = fmaf(ls_s[it * G + hh], f, L);
+        }
+        float* mine = sums + (slice * G + hh) * kPartialFloats;
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) reinterpret_cast<float2*>(mine + 2)[lane + 32 * j] = acc[j];
+        if (lane == 0) mine[0] = L;
+        if (lane == 0 && slice == 0) {
+            misc[hh] = M;
+            misc[16 + hh] = failed;
+        }
+    }
+    __syncthreads();
+    for (int idx = tid; idx < G * kHeadDim; idx += kDenseThreads) {
+        const int hh = idx / kHeadDim, e = idx % kHeadDim;
+        if (!((mask >> hh) & 1u)) continue;
+        const long long unit = first_unit + hh;
+        const float M = misc[hh], failed = misc[16 + hh];
+        float acc = 0.0f, L = 0.0f;
+        for (int w = 0; w < per_head; ++w) {
+            const float* rec = sums + (w * G + hh) * kPartialFloats;
+            acc += rec[2 + e];
+            L += rec[0];
+        }
+        if (failed < 0.0f) {   // no dense result exists
+            out[unit * kHeadDim + e] = 0.0f;
+            if (e == 0 && diag) {
+                diag[unit].lse = 0.0f;
+                diag[unit].status = failed < -1.0f ? VSA_UNIT_COPY_TIMEOUT : VSA_UNIT_BAD_PAGE;
+            }
+            continue;
+        }
+        out[unit * kHeadDim + e] = L > 0.0f ? acc / L : 0.0f;
+        if (e == 0 && diag) diag[unit].lse = (M + log2f(L)) * 0.6931471805599453f;
+    }
+}
+
 template <int G, int D = vsa::kHeadDim, bool FP8 = false>
 __global__ void __launch_bounds__((DenseCfg<D, FP8>::kDenseThreads), 1)
 dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k_cache,
@@ -252,19 +344,20 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         // microseconds of fixed overhead: query fragments, pipeline fill, merge, ticket), two when items
         // stay long.  Every group may add one ragged item, so sizing for (target - groups) full items
         // keeps the count within the target and no block starts a round the others do not have.
-        long long rounds = total_pages / ((long long)gridDim.x * kPagesPerItemGoal);
+        // (32-bit divisions, which are a shorter chain; the counts are below 2^31)
+        const unsigned blocks = gridDim.x, total = (unsigned)total_pages, listed = (unsigned)flagged_groups;
+        unsigned rounds = total / (blocks * kPagesPerItemGoal);
         rounds = rounds < 1 ? 1 : (rounds > kMaxRounds ? kMaxRounds : rounds);   // 1 or 2
         // many flagged groups of uneven length (the longest more than twice the mean): about four items
         // per group, so that short and long groups mix over the blocks
         if ((long long)longest_group * flagged_groups > 2LL * total_pages) {
-            const long long by_groups = (4LL * flagged_groups + gridDim.x - 1) / gridDim.x;
+            const unsigned by_groups = (4 * listed + blocks - 1) / blocks;
             if (rounds < by_groups) rounds = by_groups < kMaxRoundsRagged ? by_groups : kMaxRoundsRagged;
         }
-        const long long target = (long long)gridDim.x * rounds;
-        long long want = target > 2LL * flagged_groups ? (total_pages + (target - flagged_groups) - 1) / (target - flagged_groups)
-                                                       : (total_pages + target - 1) / target;
-        const long long room = max_items - flagged_groups;
-        const long long need = (total_pages + room - 1) / room;
+        const unsigned target = blocks * rounds, parts = target > 2 * listed ? target - listed : target;
+        unsigned want = (total + parts - 1) / parts;
+        const unsigned room = (unsigned)max_items - listed;
+        const unsigned need = (total + room - 1) / room;
         if (want < need) want = need;
         ppi = (int)((want + kDenseWarps - 1) / kDenseWarps) * kDenseWarps;
         if (ppi < kMinPagesPerItem) ppi = kMinPagesPerItem;
@@ -324,53 +417,8 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         const int end_page = min(nb, first_page + even);
         const int32_t* bt = block_table + (long long)b * geo.max_pages;
 
-        // Q fragments of the group: bf16 pairs straight from memory, rows >= G are zero
-        uint32_t qa0[KS], qa2[KS];
-        float q_unscale = 1.0f;
-        if constexpr (FP8) {
-            // q as f16 operands, scaled by a power of two into the top of the f16 range: exact down to 2^-28 of the head's
-            // largest element.  Step ks holds columns 16 ks + 4 quad, + 1 (qa0) and + 2, + 3 (qa2) of head lane / 4: the
-            // order in which a lane receives the bytes of a key row.
-            const uint16_t* qrow = q + ((long long)b * geo.n_q_heads + g * G + (head < G ? head : 0)) * kHeadDim;
-            float qv[KS][4];
-            float amax = 0.0f;
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint2 raw = *reinterpret_cast<const uint2*>(qrow + ks * 16 + quad * 4);
-                qv[ks][0] = __uint_as_float(raw.x << 16);
-                qv[ks][1] = __uint_as_float(raw.x & 0xffff0000u);
-                qv[ks][2] = __uint_as_float(raw.y << 16);
-                qv[ks][3] = __uint_as_float(raw.y & 0xffff0000u);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) amax = fmaxf(amax, fabsf(qv[ks][i]));
-            }
-            amax = fmaxf(amax, __shfl_xor_sync(kFullMask, amax, 1));
-            amax = fmaxf(amax, __shfl_xor_sync(kFullMask, amax, 2));
-            const int sq = amax > 0.0f ? 13 - ilogbf(amax) : 0;   // largest |q| of the head lands in [2^13, 2^14)
-            q_unscale = ldexpf(1.0f, -sq);
-            const float up0 = ldexpf(1.0f, sq >> 1), up1 = ldexpf(1.0f, sq - (sq >> 1));   // 2^sq may be no float
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint32_t v0 = pack_f16x2(qv[ks][0] * up0 * up1, qv[ks][1] * up0 * up1);
-                const uint32_t v2 = pack_f16x2(qv[ks][2] * up0 * up1, qv[ks][3] * up0 * up1);
-                qa0[ks] = head < G ? v0 : 0u;
-                qa2[ks] = head < G ? v2 : 0u;
-            }
-        } else {
-            const uint16_t* qrow = q + ((long long)b * geo.n_q_heads + g * G + (head < G ? head : 0)) * kHeadDim;
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint32_t v0 = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + quad * 2);
-                const uint32_t v2 = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + quad * 2);
-                qa0[ks] = head < G ? v0 : 0u;
-                qa2[ks] = head < G ? v2 : 0u;
-            }
-        }
         float vref = 0.0f;                       // FP8: the largest value scale so far; o is in units of vref / kPScale
         float m_run = -INFINITY, l_run = 0.0f;   // per lane: head `head`, partial over this lane's columns
-        // FP8: the lane's score columns are heads 2 quad, 2 quad + 1; o[n]: columns 16 n + head and + 8 of both
-        const float q_unscale0 = FP8 ? __shfl_sync(kFullMask, q_unscale, 8 * quad) * scale : 0.0f;
-        const float q_unscale1 = FP8 ? __shfl_sync(kFullMask, q_unscale, 8 * quad + 4) * scale : 0.0f;
         float m_run1 = -INFINITY, l_run1 = 0.0f;   // FP8: of head 2 quad + 1 (m_run, l_run: of head 2 quad)
         constexpr int OT = FP8 ? D / 16 : NT;
         float o[OT][4];
@@ -454,6 +502,52 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
             if (s < my_count) issue(s);
             if constexpr (!FP8) cp_async_commit();
         }
+
+        // Q fragments of the group, while the first tiles are on their way: bf16 pairs straight from memory, rows >= G are zero
+        uint32_t qa0[KS], qa2[KS];
+        float q_unscale = 1.0f;
+        if constexpr (FP8) {
+            // q as f16 operands, scaled by a power of two into the top of the f16 range: exact down to 2^-28 of the head's
+            // largest element.  Step ks holds columns 16 ks + 4 quad, + 1 (qa0) and + 2, + 3 (qa2) of head lane / 4: the
+            // order in which a lane receives the bytes of a key row.
+            const uint16_t* qrow = q + ((long long)b * geo.n_q_heads + g * G + (head < G ? head : 0)) * kHeadDim;
+            float qv[KS][4];
+            float amax = 0.0f;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                const uint2 raw = *reinterpret_cast<const uint2*>(qrow + ks * 16 + quad * 4);
+                qv[ks][0] = __uint_as_float(raw.x << 16);
+                qv[ks][1] = __uint_as_float(raw.x & 0xffff0000u);
+                qv[ks][2] = __uint_as_float(raw.y << 16);
+                qv[ks][3] = __uint_as_float(raw.y & 0xffff0000u);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) amax = fmaxf(amax, fabsf(qv[ks][i]));
+            }
+            amax = fmaxf(amax, __shfl_xor_sync(kFullMask, amax, 1));
+            amax = fmaxf(amax, __shfl_xor_sync(kFullMask, amax, 2));
+            const int sq = amax > 0.0f ? 13 - ilogbf(amax) : 0;   // largest |q| of the head lands in [2^13, 2^14)
+            q_unscale = ldexpf(1.0f, -sq);
+            const float up0 = ldexpf(1.0f, sq >> 1), up1 = ldexpf(1.0f, sq - (sq >> 1));   // 2^sq may be no float
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                const uint32_t v0 = pack_f16x2(qv[ks][0] * up0 * up1, qv[ks][1] * up0 * up1);
+                const uint32_t v2 = pack_f16x2(qv[ks][2] * up0 * up1, qv[ks][3] * up0 * up1);
+                qa0[ks] = head < G ? v0 : 0u;
+                qa2[ks] = head < G ? v2 : 0u;
+            }
+        } else {
+            const uint16_t* qrow = q + ((long long)b * geo.n_q_heads + g * G + (head < G ? head : 0)) * kHeadDim;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+                const uint32_t v0 = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + quad * 2);
+                const uint32_t v2 = *reinterpret_cast<const uint32_t*>(qrow + ks * 16 + 8 + quad * 2);
+                qa0[ks] = head < G ? v0 : 0u;
+                qa2[ks] = head < G ? v2 : 0u;
+            }
+        }
+        // FP8: the lane's score columns are heads 2 quad, 2 quad + 1; o[n]: columns 16 n + head and + 8 of both
+        const float q_unscale0 = FP8 ? __shfl_sync(kFullMask, q_unscale, 8 * quad) * scale : 0.0f;
+        const float q_unscale1 = FP8 ? __shfl_sync(kFullMask, q_unscale, 8 * quad + 4) * scale : 0.0f;
         for (int k = 0; k < my_count; ++k) {
             float ks0 = 0.0f, ks1 = 0.0f, vs0 = 0.0f, vs1 = 0.0f;
             if constexpr (FP8) {   // (before the next look-up)
@@ -709,54 +803,18 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         }
 
         // ---- the block that finishes the last item of this (sequence, KV head) combines them ----
-        __threadfence();
         __syncthreads();
-        if (tid == 0) sm.misc[12] = atomicAdd(&counters[grp], 1) == items_of_group - 1;
+        if (tid == 0) {
+            __threadfence();   // (cumulative over the barrier)
+            const bool last = atomicAdd(&counters[grp], 1) == items_of_group - 1;
+            if (last) __threadfence();
+            sm.misc[12] = last;
+        }
         __syncthreads();
         if (sm.misc[12]) {
-            __threadfence();
-            const float* gp = partials + (long long)sm.item_base[grp] * G * kPartialFloats;
-            // Stage every item's (max, sum) of every head in shared memory first: the weighted sums below
-            // then consist of independent loads only (a running maximum would make each load wait for the
-            // previous item's, which costs a memory round trip per item).
-            float* ms_s = reinterpret_cast<float*>(sm.ring);          // [items][G]
-            float* ls_s = ms_s + (size_t)items_of_group * G;           // [items][G]
-            for (int i = tid; i < items_of_group * G; i += kDenseThreads) {
-                const float* rec = gp + (long long)i * kPartialFloats;
-                ms_s[i] = __ldcg(rec);
-                ls_s[i] = __ldcg(rec + 1);
-            }
-            __syncthreads();
-            for (int idx = tid; idx < G * kHeadDim; idx += kDenseThreads) {
-                const int hh = idx / kHeadDim, e = idx % kHeadDim;
-                if (!((mask >> hh) & 1u)) continue;
-                float M = -INFINITY;
-                float failed = 0.0f;   // -1: a page outside the pool, -2: a copy that did not land
-                for (int it = 0; it < items_of_group; ++it) {
-                    M = fmaxf(M, ms_s[it * G + hh]);
-                    failed = fminf(failed, ls_s[it * G + hh]);
-                }
-                const long long unit = (long long)b * geo.n_q_heads + g * G + hh;
-                if (failed < 0.0f) {   // no dense result exists
-                    out[unit * kHeadDim + e] = 0.0f;
-                    if (e == 0 && diag) {
-                        diag[unit].lse = 0.0f;
-                        diag[unit].status = failed < -1.0f ? VSA_UNIT_COPY_TIMEOUT : VSA_UNIT_BAD_PAGE;
-                    }
-                    continue;
-                }
-                // one pass in item order
-                float acc = 0.0f, L = 0.0f;
-#pragma unroll 8
-                for (int it = 0; it < items_of_group; ++it) {
-                    const float ms = ms_s[it * G + hh];
-                    const float f = ms == -INFINITY ? 0.0f : exp2f(ms - M);
-                    acc = fmaf(__ldcg(gp + ((long long)it * G + hh) * kPartialFloats + 2 + e), f, acc);
-                    L = fmaf(ls_s[it * G + hh], f, L);
-                }
-                out[unit * kHeadDim + e] = L > 0.0f ? acc / L : 0.0f;
-                if (e == 0 && diag) diag[unit].lse = (M + log2f(L)) * 0.6931471805599453f;
-            }
+            combine_items<G, D, FP8>(reinterpret_cast<float*>(sm.ring), reinterpret_cast<float*>(sm.misc),
+                                     partials + (long long)sm.item_base[grp] * G * kPartialFloats, items_of_group, mask,
+                                     (long long)b * geo.n_q_heads + g * G, out, diag);
         }
         if (tid == 0) sm.misc[13] = 0;
         if constexpr (FP8) fence_async_proxy();
