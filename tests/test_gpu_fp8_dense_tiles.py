@@ -31,3 +31,20 @@ def test_rows_outside_the_sequences(page, hq, hkv, lens, alt):
     k8[at], v8[at] = 0x7f, 0xff
     wq, g = run_fp8(w, gap_threshold=math.inf, alt_strides=alt, quantised=(wq, k8, v8, ke, ve))
     compare(wq, g, gap_threshold=math.inf)
+
+
+@pytest.mark.parametrize("page,token,head_pad,page_pad", [(16, 144, 32, 48), (32, 128, 16, 0), (16, 272, 0, 4096)])
+def test_padded_strides(page, token, head_pad, page_pad):
+    lens, hkv = (700, 33, 16), 2
+    w = make_workload(spec(batch=len(lens), n_q_heads=8, n_kv_heads=hkv, seq_lens=lens, page_size=page, P=2, K_c=8), seed=8400 + page + token)
+    wq, k8, v8, ke, ve = quantize_kv_fp8(w)
+    head = page * token + head_pad
+    strides = (hkv * head + page_pad, head, token, 1)
+
+    def padded(x):
+        out = torch.full((x.shape[0] * strides[0],), 0x7f, dtype=torch.uint8, device="cuda:0").as_strided(x.shape, strides)
+        out.copy_(x)
+        return out
+
+    wq, g = run_fp8(w, gap_threshold=math.inf, quantised=(wq, padded(k8), padded(v8), ke, ve))
+    compare(wq, g, gap_threshold=math.inf)
