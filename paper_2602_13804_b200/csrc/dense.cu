@@ -417,7 +417,6 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         const int end_page = min(nb, first_page + even);
         const int32_t* bt = block_table + (long long)b * geo.max_pages;
 
-        float vref = 0.0f;                       // FP8: the largest value scale so far; o is in units of vref / kPScale
         float m_run = -INFINITY, l_run = 0.0f;   // per lane: head `head`, partial over this lane's columns
         float m_run1 = -INFINITY, l_run1 = 0.0f;   // FP8: of head 2 quad + 1 (m_run, l_run: of head 2 quad)
         constexpr int OT = FP8 ? D / 16 : NT;
@@ -621,9 +620,8 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 for (int j = 0; j < 4; ++j)
                     if (head + 8 * j >= valid) ta[j] = tb[j] = -INFINITY;
             float ma = fmaxf(fmaxf(ta[0], ta[1]), fmaxf(ta[2], ta[3])), mb = fmaxf(fmaxf(tb[0], tb[1]), fmaxf(tb[2], tb[3]));
-            const float vmax = fmaxf(vs0, vs1);
-            // a new maximum (of the scores or of the value scales), rarer with every unit: reduce it and rescale the sums
-            if (__any_sync(kFullMask, ma > m_run || mb > m_run1) || vmax > vref) {
+            // a new maximum, rarer with every unit: reduce it and rescale the sums
+            if (__any_sync(kFullMask, ma > m_run || mb > m_run1)) {
 #pragma unroll
                 for (int off = 4; off < 32; off <<= 1) {
                     ma = fmaxf(ma, __shfl_xor_sync(kFullMask, ma, off));
@@ -632,25 +630,21 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 ma = fmaxf(ma, m_run), mb = fmaxf(mb, m_run1);   // finite: token 0 of a unit is always valid
                 const float fa = exp2f(m_run - ma), fb = exp2f(m_run1 - mb);   // 0 on the first unit
                 l_run *= fa, l_run1 *= fb;
-                const float fv = vmax > vref ? vref / vmax : 1.0f;
-                vref = fmaxf(vref, vmax);
 #pragma unroll
                 for (int n = 0; n < OT; ++n) {
-                    o[n][0] *= fa * fv, o[n][1] *= fb * fv;
-                    o[n][2] *= fa * fv, o[n][3] *= fb * fv;
+                    o[n][0] *= fa, o[n][1] *= fb;
+                    o[n][2] *= fa, o[n][3] *= fb;
                 }
                 m_run = ma, m_run1 = mb;
             }
-            // P as f16 operands: p * (value scale of its page / vref) * kPScale, normal numbers down to p = 2^-28; packed by
-            // token, then transposed into the B fragment (tokens are the contraction's index)
-            auto weight = [&](float vs) { return vs == vref ? kPScale : vref > 0.0f ? kPScale * (vs / vref) : 0.0f; };
-            const float w0 = weight(vs0), w1 = weight(vs1);
+            // P as f16 operands: p * kPScale, normal numbers down to p = 2^-28; packed by token, then transposed into the B
+            // fragment (tokens are the contraction's index)
             uint32_t pb[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float pa = exp2f(ta[j] - m_run), pc = exp2f(tb[j] - m_run1);
                 l_run += pa, l_run1 += pc;
-                pb[j] = transpose_8x8(pack_f16x2(pa * (j < 2 ? w0 : w1), pc * (j < 2 ? w0 : w1)));
+                pb[j] = transpose_8x8(pack_f16x2(pa * kPScale, pc * kPScale));
             }
 
             // O^T += V^T P^T, 16 columns at a time: one transposing byte load per 32 tokens x 16 columns.  A lane's four rows
@@ -659,15 +653,20 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 const int rrow = lane & 15, qd = rrow >> 2, ii = rrow & 3;
                 const int tokp = (lane >> 4) * 16 + ((ii < 2) ? 0 : 8) + 2 * qd + (ii & 1);
                 const uint32_t vrow = vbase + (uint32_t)(tokp * 128);
+                const float out0 = vs0 * (1.0f / kPScale), out1 = vs1 * (1.0f / kPScale);
 #pragma unroll
                 for (int dp = 0; dp < 8; ++dp) {
                     uint32_t r[4], a[4];
                     ldmatrix_x2_trans_b8(r, vrow + (uint32_t)((dp ^ (tokp & 7)) << 4));
 #pragma unroll
                     for (int hf = 0; hf < 2; ++hf) {
+                        float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                         e4m3x4_to_f16(r[2 * hf], a[0], a[2]);
                         e4m3x4_to_f16(r[2 * hf + 1], a[1], a[3]);
-                        mma_f16(o[dp], a[0], a[1], a[2], a[3], pb[2 * hf], pb[2 * hf + 1]);
+                        mma_f16(t, a[0], a[1], a[2], a[3], pb[2 * hf], pb[2 * hf + 1]);
+#pragma unroll
+                        for (int i = 0; i < 4; i += 2)
+                            fma2(o[dp][i], o[dp][i + 1], t[i], t[i + 1], hf ? out1 : out0, hf ? out1 : out0);
                     }
                 }
             }
@@ -745,7 +744,6 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 l_run1 += __shfl_xor_sync(kFullMask, l_run1, off);
             }
             __syncthreads();   // every warp is done with its ring
-            const float o_unit = vref * (1.0f / kPScale);
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const int hh = 2 * quad + i;
@@ -757,8 +755,8 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
                 }
 #pragma unroll
                 for (int n = 0; n < OT; ++n) {
-                    rec[2 + n * 16 + head] = o[n][i] * o_unit;
-                    rec[2 + n * 16 + 8 + head] = o[n][2 + i] * o_unit;
+                    rec[2 + n * 16 + head] = o[n][i];
+                    rec[2 + n * 16 + 8 + head] = o[n][2 + i];
                 }
             }
         } else {
