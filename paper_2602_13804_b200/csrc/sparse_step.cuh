@@ -94,8 +94,12 @@ enum : int {
 };
 
 __host__ __device__ constexpr int step_lanes_per_row(int D) { return D / 8; }
-// Value rows in flight per group of lanes, in stages of four in shared memory (0: in registers, see the value gather).
-__host__ __device__ constexpr int step_value_stages(int threads) { return threads == 128 ? 2 : threads == 256 ? 3 : 0; }
+// Value rows in flight per group of lanes, in stages of four in shared memory (0: in registers, see the value gather).  An
+// iterative solve asks for all of its rows at once (16 per group at most), in the place of its key tile.
+__host__ __device__ constexpr int step_value_stages(int threads, bool solve)
+{
+    return solve ? 4 : threads == 128 ? 2 : threads == 256 ? 3 : 0;
+}
 
 inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve)
 {
@@ -137,7 +141,8 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
         s.red = s.work + 4 * cands;
         s.vring = s.red + warps * D;
     }
-    const int vring_end = s.vring + 4 * step_value_stages(threads) * threads * lane_words - s.work;
+    const int stages = solve ? cands / (4 * groups) : step_value_stages(threads, false);   // (of a solve: those that K_c needs)
+    const int vring_end = s.vring + 4 * stages * threads * lane_words - s.work;
     w = vring_end > w ? vring_end : w;
     if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
     if (tt > 1 && threads * 16 * lane_words > w) w = threads * 16 * lane_words;
@@ -870,13 +875,18 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     //      streams them through stages in shared memory: the loop is a quarter of the code of sixteen rows in registers (the SM
     //      caches some 2000 instructions, a kernel with units in all phases needs its code again and again: 20.7k -> 14k
     //      cycles of a unit with K_c = 512 in a full chip, 4.0k -> 3.4k at K_c = 256 and two units per SM).  With 512 threads
-    //      every instruction runs once, and rows in registers are faster (batch 1, T = 4k 14.4 against 14.7 us per layer) ----
+    //      every instruction runs once, and rows in registers are faster (batch 1, T = 4k 14.4 against 14.7 us per layer).  After
+    //      an iterative solve nothing else overlaps the loads: all rows at once (three stages and four, mean over six orders of
+    //      loading the kernels, whose place in memory moves one and the same code by 1.5 %: batch 8, T = 32k, four Frank-Wolfe
+    //      iterations 32.4 -> 32.0 us per layer, two entropic ones 33.0 -> 32.8, four 37.3 -> 37.2; batch 24 89.0 -> 88.2; batch 1,
+    //      T = 8k 22.6 -> 22.8) ----
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0f;
     {
         using Bits = typename std::conditional<FP8, uint2, uint4>::type;
-        constexpr int kElem = FP8 ? 1 : 2, STAGES = step_value_stages(THREADS);
+        constexpr int kElem = FP8 ? 1 : 2, STAGES = step_value_stages(THREADS, SOLVE != 0);
+        static_assert(SOLVE == 0 || STAGES * UNR * GROUPS == VSA_SOLVER_MAX_CANDIDATES, "a solve's rows are asked for once");
         const uint8_t* vbase = reinterpret_cast<const uint8_t*>(p.v) + ((long long)g * geo.head_stride + c * 8) * kElem;
         const Row* mine = cand + grp;
         auto add = [&](const Bits& row, float w) {

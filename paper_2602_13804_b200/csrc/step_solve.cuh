@@ -6,7 +6,7 @@
 // A pass of the descent is y = sum_i a_i k_i followed by g_i = <k_i, y> - s_i, two products of the 64 KB of keys with a
 // vector, fp32 on the floating-point pipe; half of the unpacking runs there too, as mixed-precision additions.  Bound by
 // the instructions of the passes and by shared-memory bandwidth (two blocks read 256 KB a pass).  Four iterations at
-// batch 8, T = 32k: 41.0 -> 38.1 us per layer.  The same products on the tensor cores (the vector as three bf16 columns,
+// batch 8, T = 32k: 41.0 -> 37.2 us per layer.  The same products on the tensor cores (the vector as three bf16 columns,
 // which is exact) took 41.6: a warp-level MMA costs about twelve cycles and an ldmatrix the bandwidth of these loads.
 // Frank-Wolfe picks vertices, integers that the CPU oracle mirrors bit for bit, so it keeps the canonical fp32 order.
 #pragma once
