@@ -5,7 +5,8 @@
 
 A "step" is one decode token for every sequence of the batch through all layers of the
 workload: per layer vsa_decode_step (page routing -> fused sparse pass -> dense fallback) on
-that layer's own KV cache.  Prints ONE JSON line (rank 0).  Workloads:
+that layer's own KV cache.  Prints ONE JSON line of at most LINE_LIMIT characters on stdout (rank 0), and the full
+record - per-kernel times, byte counts, sweep points - as one JSON line on stderr.  Workloads:
     cfg1            batch 8, T = 32768, 32 layers, P = 32, K_c = 256  (default; the metric's config)
     cfg0 | cfg3 | cfg4
     cfg2:B:T        a point of the context sweep, e.g. cfg2:1:131072
@@ -13,7 +14,7 @@ With --gpus N > 1 and no torchrun environment the script starts its N ranks itse
 (python -m torch.distributed.run ... bench.py, one process per GPU, no data-path collective).
 Extra flags: --layers L (override), --dense-baseline (time the split-K dense kernel on the same
 caches instead of the sparse path), --no-graph (plain stream launches for `value`), --no-sweep
-(skip the context sweep / fallback / scan points that the default run adds to its line),
+(skip the context sweep / fallback / scan points that the default run adds to its record),
 --grid (the (P, K_c) ablation grid of the paper's Table 3 as one JSON line),
 --leak-curve (leakage against the gap statistic, CPU oracle only, one JSON line).
 """
@@ -37,6 +38,7 @@ METRIC = "decode_attn_us_per_token_per_layer"
 UNIT = "us/token/layer"
 FALLBACK_HBM_GBS = 6650.0
 NOMINAL_HBM_GBS = 8000.0      # the denominator the metric names ("vs 8 TB/s")
+LINE_LIMIT = 1500             # characters of the stdout line: logs keep the end of an output, a longer line loses its start
 SUSTAIN_S = 0.6               # length of the event-timed region the clock samples come from
 
 
@@ -151,6 +153,27 @@ class ClockSampler:
         return {"sm_mhz": sm[len(sm) // 2], "sm_max_mhz": float(rows[0][1]),
                 "power_w_max": max(float(r[2]) for r in rows), "reasons": reasons, "samples": len(rows),
                 "samples_inside_timed_region": len(inside)}
+
+
+# what of the record the stdout line holds: top-level keys, and of nested objects the keys listed (None: all)
+LINE_KEYS = {
+    "metric": None, "value": None, "unit": None, "n_gpus": None, "steps": None, "warmup": None, "ms_per_step": None,
+    "higher_is_better": None, "scaling": None, "vs_baseline": None, "dtype": None, "data": None, "gpu_launches": None,
+    "config": ("workload", "batch", "n_q_heads", "n_kv_heads", "head_dim", "page_size", "context", "P", "K_c", "layers_per_step",
+               "l2", "path"),
+    "clocks": ("sm_mhz", "sm_max_mhz", "reasons"),
+    "e2e": ("value", "unit", "ms_per_step", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel"),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
+}
+
+
+def short_line(record: dict) -> str:
+    line = {}
+    for key, inner in LINE_KEYS.items():
+        v = record.get(key)
+        line[key] = {k: v[k] for k in inner if k in v} if inner and isinstance(v, dict) else v
+    return json.dumps(line)
 
 
 def max_over_ranks(ms: float, world: int, device) -> float:
@@ -1044,7 +1067,8 @@ def run_ours(args):
         "gpu_launches": args.steps * L * kernels_per_layer, "clocks": clocks, "e2e": e2e, "roofline": roofline,
         "cpu_baseline": cpu_baseline, "sweep": sweep_obj,
     }
-    print(json.dumps(line), flush=True)
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(short_line(line), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()

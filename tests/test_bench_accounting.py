@@ -83,3 +83,38 @@ def test_harness_allocates_what_the_step_writes(monkeypatch):
     for d in (64, 128, 256):
         h = bench.Harness(replace(_spec(), head_dim=d, layers=2), torch.device("cpu"))
         assert h.out.numel() == h.units * d and h.summaries[0].shape[-1] == d and h.layers[0].q.shape[-1] == d
+
+
+def test_the_line_on_stdout_keeps_what_is_asked_for_and_stays_short():
+    """A record of the default run, with the longest texts that its fields take, as one line of at most LINE_LIMIT characters."""
+    import json
+    x = 12345.678901234567
+    path = ("route -> sparse with routing certificate -> retries of the refused units with up to 1024 pages -> dense fallback")
+    record = {
+        "metric": bench.METRIC, "value": x, "unit": bench.UNIT, "n_gpus": 8, "steps": 1000, "warmup": 100, "ms_per_step": x,
+        "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
+        "config": {"workload": "cfg2_b16_t131072_P1024_Kc1024_per_qhead_round_robin", "batch": 64, "n_q_heads": 64, "n_kv_heads": 32,
+                   "head_dim": 256, "page_size": 16, "context": 131072, "P": 1024, "K_c": 1024, "epsilon": x, "gap_threshold": x,
+                   "layers_per_step": 32, "distinct_layer_caches": 32,
+                   "l2": "inputs larger than L2: 32 distinct layer caches, 123456 MB touched per pass over them",
+                   "launch": "cuda graph replay of the whole step", "path": path},
+        "sustained": {"steps": 1, "note": "n" * 200}, "kernels": {"route_scan": "k" * 1000}, "gpu_launches": 123456,
+        "clocks": {"sm_mhz": 1965.0, "sm_max_mhz": 1965.0, "power_w_max": x, "reasons": ["sw_power_cap"], "samples": 5},
+        "e2e": {"value": x, "unit": bench.UNIT, "ms_per_step": x, "h2d_bytes_per_step": 1 << 30, "d2h_bytes_per_step": 1 << 30,
+                "api": "a" * 200},
+        "roofline": {"bound": "hbm", "achieved": x, "peak": x, "unit": "GB/s", "frac": x / 1e5, "traffic": x * 1e6,
+                     "kernel": "dense_fallback", "us_is": "u" * 400},
+        "cpu_baseline": {"value": x, "unit": bench.UNIT, "cores": 128, "kind": "oracle",
+                         "sample": "one layer of 32, all 64 sequences, 200 repetitions of one oracle decode step (summaries "
+                                   "prebuilt)", "extra_samples": "e" * 300},
+        "sweep": {"points": ["s" * 17000]},
+    }
+    text = bench.short_line(record)
+    line = json.loads(text)
+    assert len(text) <= bench.LINE_LIMIT and "\n" not in text
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                "dtype", "data", "gpu_launches"):
+        assert line[key] == record[key]
+    assert line["e2e"]["value"] == x and line["clocks"]["reasons"] == ["sw_power_cap"] and line["cpu_baseline"]["cores"] == 128
+    assert line["config"]["l2"] == record["config"]["l2"] and line["roofline"]["frac"] == record["roofline"]["frac"]
+    assert bench.short_line({**record, "e2e": None, "cpu_baseline": None})       # variants without an end-to-end form
