@@ -479,8 +479,9 @@ int vsa_route_pages_static(const vsa_shape_t* shape, const void* q, const void* 
  * Token scores are the fixed-order dot of q with the decoded bytes, multiplied by the page's key scale;
  * the readout multiplies each candidate's weight by its page's value scale.  With POWER-OF-TWO scales every
  * one of those multiplications is exact, and all results equal - discrete ones bit for bit - those of
- * the bf16 entry points on a bf16 cache that holds the same values; with other scales the score carries
- * one more rounding.  head_dim 128; page_size 16 or 32; closed-form weights only.  Otherwise the four entry
+ * the bf16 entry points on a bf16 cache that holds the same values (the dense pass's outputs up to the
+ * rounding of its probabilities, to f16 here and to bf16 there; no page's share depends on another page's
+ * scale); with other scales the score carries one more rounding.  head_dim 128; page_size 16 or 32; closed-form weights only.  Otherwise the four entry
  * points take the arguments, workspaces and error rules of the entry points they are named after.
  */
 int vsa_build_page_summaries_fp8(const vsa_shape_t* shape, const void* k_cache, const float* k_scale,

@@ -43,7 +43,7 @@ struct DenseCfg {
     // warp's chain: twelve warps with two stages.  Microseconds per layer, 16 sequences of 16k - 32k that all fall back
     // (754 MB), with 8 / 10 / 12 warps: 228 / 221 / 207.  Before, with m16n8k32 e4m3 MMAs of two terms per
     // operand (860 instructions per 32 tokens against 560 now) and 16-byte copies in place of TMA tiles, 290; a quarter of the
-    // sequences (246 MB, the kernel alone 62 us, DRAM at half its rate, 0.40 of the issue slots) 116 -> 92.
+    // sequences (246 MB, the kernel alone 62 us, DRAM at half its rate, 0.40 of the issue slots) 116 -> 90.
     static constexpr int kDenseThreads = FP8 ? 384 : D == 256 ? 128 : 256;
     static constexpr int kStages = FP8 ? 2 : 3;                // units in flight per warp
     static constexpr int kDenseWarps = kDenseThreads / 32;
@@ -169,7 +169,7 @@ __device__ __noinline__ void combine_items(float* ring, float* misc, const float
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // Every item's (max, sum) of every head in shared memory, then the listed heads and their items dealt out to the
     // warps: the loads are independent, and one head keeps every warp busy.  A thread per column that walked all
-    // items paid a memory round trip for every eight of them: with this and the 32-bit divisions above one
+    // items paid a memory round trip for every eight of them: with this and the 32-bit divisions of the item sizes one
     // sequence of 128k that falls back 131 -> 118 us per layer, one unit of four in 4 of 2k - 8k 36.8 -> 34.5, the
     // same at D = 256 63.9 -> 56.4.
     float* ms_s = ring;                                 // [items][G]

@@ -20,7 +20,8 @@
 // at batch 1, T = 4k with the scan and the empty dense pass; 21.2 -> 17.9 at T = 128k; batch 8, T = 32k 24.6 -> 23.3;
 // 64 sequences of 4k - 128k with 8 heads a group 449 -> 399; batch 32 of short rows at D = 64 44 -> 39.  Then, with bulk
 // copies of the key tiles and the value rows streamed through shared memory (128 threads), 355 -> 312 for the 64 sequences and
-// 83.0 -> 81.5 at batch 16, T = 128k; with scores in registers where a thread has one chunk, 14.5 -> 14.2 at batch 1, T = 4k.
+// 83.0 -> 81.5 at batch 16, T = 128k; with scores in registers where a thread has one chunk (and the append's reads side by
+// side), 14.4 -> 14.2 at batch 1, T = 4k, the append included.
 // What bounds it:
 // no unit of the SM, but the chain of phases.  Counters at P = 32, K_c = 256: 20k warp instructions per unit of 256
 // threads, 0.41 of the issue slots at two units per SM (256 units), 0.38 at four of 128 threads (512 units); at P = 64,
@@ -1034,7 +1035,7 @@ template <int D, bool FP8>
 cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
 {
     const bool fused = p.page_scores != nullptr;
-    // Five blocks per SM at 96 registers against four at 128, whose unspilled registers make a unit 5 - 10 % faster: five
+    // Five blocks per SM at 96 registers against four at 128, which make a unit 5 - 10 % faster: five
     // where they save a wave of blocks, and from three waves of four on, where units in flight count for more.  Microseconds
     // per layer, four / five, T = 8k.  A wave saved: 32 pages a unit, 640 units 41.6 / 31.9, 704 43.5 / 32.5, 1280 65.4 / 56.0,
     // 1472 68.1 / 63.6; 64 pages 640 66.0 / 48.0, 1472 107 / 100; e4m3 cache 640 39.6 / 29.0, 1472 68.6 / 56.6; D = 64 640

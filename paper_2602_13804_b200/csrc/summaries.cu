@@ -110,7 +110,8 @@ __device__ __forceinline__ float radius_of_rows(const uint4 (&rows)[PS], int n, 
 // contiguous key row per load.  fp32 sum in ascending token order, IEEE division by the number of valid rows,
 // round-to-nearest-even to bf16.  Bound by HBM: eight rows of a page in flight per thread and four blocks per SM
 // keep 128 KB in flight while other blocks add (8 prompts of 8k - 32k tokens, two layers: 112.9 us with three blocks, 103.3
-// with four, 109.4 with five, whose registers spill; e4m3 64.6 / 57.8 / 66.0).  Grid: x = chunks of pages, y = sequence.
+// with four, 109.4 with five; e4m3 64.6 / 57.8 / 66.0).  At four the 64 registers leave 28 bytes of spills (e4m3, 32-token
+// pages, 8), which cost less than the fourth block brings; three have none, five more.  Grid: x = chunks of pages, y = sequence.
 template <int PS, int D>
 __global__ void __launch_bounds__(256, 4) summaries_kernel(Geometry geo, const uint16_t* __restrict__ k_cache,
                                                            const int32_t* __restrict__ block_table,
