@@ -539,6 +539,18 @@ static int decode_step_impl(const vsa_shape_t* shape, const void* q, const void*
             ev[i] = (cudaEvent_t)events[i];
         }
     void* ws_dense = (char*)ws + step_route_part(g);
+    if (!events && !cert && vsa::step_scans(g, P, K_c, fp8, solve != nullptr)) {
+        // two launches: the sparse pass scores the pages itself, and the dense pass makes the list from its flags
+        // (in the place of the page scores)
+        int32_t* flags = (int32_t*)ws;
+        cudaError_t e = vsa::launch_sparse(g, q, k_cache, v_cache, block_table, seq_lens, routed_pages, nullptr, P, K_c, epsilon,
+                                           gap_threshold, out, diag, fallback_list, fallback_count, st, solver_iters, solve, nullptr,
+                                           nullptr, solver_kind, nullptr, nullptr, 0, nullptr, 0, k_scale, v_scale, summaries, flags,
+                                           vsa::dense_tickets(ws_dense));
+        if (e != cudaSuccess) return VSA_ERR_CUDA;
+        return cuda_rc(vsa::launch_dense(g, q, k_cache, v_cache, block_table, seq_lens, fallback_list, fallback_count, epsilon, out,
+                                         diag, ws_dense, st, /*tickets_cleared=*/true, k_scale, v_scale, flags));
+    }
     if (ev[0] && cudaEventRecord(ev[0], st) != cudaSuccess) return VSA_ERR_CUDA;
     // the scan kernel clears fallback_count and the dense pass's tickets: the step enqueues no memset
     cudaError_t e = vsa::launch_route_scan(g, q, summaries, block_table, seq_lens, ws, fallback_count,

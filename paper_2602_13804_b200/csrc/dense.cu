@@ -254,8 +254,8 @@ template <int G, int D = vsa::kHeadDim, bool FP8 = false>
 __global__ void __launch_bounds__((DenseCfg<D, FP8>::kDenseThreads), 1)
 dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k_cache,
                    const uint16_t* __restrict__ v_cache, const int32_t* __restrict__ block_table,
-                   const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ fallback_list,
-                   const int32_t* __restrict__ fallback_count, float epsilon, float* __restrict__ partials,
+                   const int32_t* __restrict__ seq_lens, int32_t* __restrict__ fallback_list,
+                   int32_t* __restrict__ fallback_count, const int32_t* __restrict__ flags, float epsilon, float* __restrict__ partials,
                    int32_t* __restrict__ counters, float* __restrict__ out, vsa_diag_t* __restrict__ diag,
                    int max_items, const float* __restrict__ k_scale, const float* __restrict__ v_scale,
                    const __grid_constant__ DenseMaps<FP8> maps)
@@ -286,7 +286,29 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     pdl_wait();
 
     // ---- which heads of which groups are listed? ----
-    if (fallback_count) {
+    if (flags) {
+        // one flag per unit (a step whose sparse pass ran the scan itself: nothing ahead of it could clear a counter); the
+        // list is made here
+        const int units = geo.batch * geo.n_q_heads;
+        int mine = 0;
+        for (int i = tid; i < units; i += kDenseThreads) mine |= __ldcg(flags + i);
+        if (!__syncthreads_or(mine)) {
+            if (blockIdx.x == 0 && tid == 0) *fallback_count = 0;
+            return;
+        }
+        for (int i = tid; i < n_groups; i += kDenseThreads) sm.group_mask[i] = 0;
+        if (tid == 0) sm.misc[31] = 0;
+        __syncthreads();
+        for (int i = tid; i < units; i += kDenseThreads) {
+            if (__ldcg(flags + i) == 0) continue;
+            const int grp = i / G;   // (heads of a group are neighbours)
+            atomicOr(reinterpret_cast<unsigned int*>(sm.group_mask) + (grp >> 2), (1u << (i % G)) << (8 * (grp & 3)));
+            if (blockIdx.x == 0) fallback_list[atomicAdd(&sm.misc[31], 1)] = i;
+        }
+        __syncthreads();
+        if (blockIdx.x == 0 && tid == 0) *fallback_count = sm.misc[31];
+        __syncthreads();
+    } else if (fallback_count) {
         const int count = *fallback_count;
         if (count <= 0) return;
         for (int i = tid; i < n_groups; i += kDenseThreads) sm.group_mask[i] = 0;
@@ -882,8 +904,8 @@ size_t dense_workspace_bytes(const Geometry& g_in)
 
 template <int G, int D, bool FP8 = false>
 static cudaError_t launch_dense_gd(const Geometry& g, const uint16_t* q, const uint16_t* k, const uint16_t* v,
-                                   const int32_t* block_table, const int32_t* seq_lens, const int32_t* fallback_list,
-                                   const int32_t* fallback_count, float epsilon, float* partials, int32_t* counters,
+                                   const int32_t* block_table, const int32_t* seq_lens, int32_t* fallback_list,
+                                   int32_t* fallback_count, const int32_t* flags, float epsilon, float* partials, int32_t* counters,
                                    float* out, vsa_diag_t* diag, cudaStream_t stream, const float* k_scale = nullptr,
                                    const float* v_scale = nullptr)
 {
@@ -896,37 +918,38 @@ static cudaError_t launch_dense_gd(const Geometry& g, const uint16_t* q, const u
         if (!encode_pool(&maps.k, k, g) || !encode_pool(&maps.v, v, g)) return cudaErrorInvalidValue;
     // persistent grid: one block per SM (the ring fills the shared memory)
     return launch_pdl(dense_split_kernel<G, D, FP8>, dim3((unsigned)num_sms()), dim3(DenseCfg<D, FP8>::kDenseThreads), smem,
-                      stream, g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials,
+                      stream, g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon, partials,
                       counters, out, diag, dense_max_items(g), k_scale, v_scale, maps);
 }
 
 template <int G>
 static cudaError_t launch_dense_g(const Geometry& g, const uint16_t* q, const uint16_t* k, const uint16_t* v,
-                                  const int32_t* block_table, const int32_t* seq_lens, const int32_t* fallback_list,
-                                  const int32_t* fallback_count, float epsilon, float* partials, int32_t* counters,
+                                  const int32_t* block_table, const int32_t* seq_lens, int32_t* fallback_list,
+                                  int32_t* fallback_count, const int32_t* flags, float epsilon, float* partials, int32_t* counters,
                                   float* out, vsa_diag_t* diag, cudaStream_t stream, const float* k_scale,
                                   const float* v_scale)
 {
     if (k_scale)
-        return launch_dense_gd<G, 128, true>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon,
+        return launch_dense_gd<G, 128, true>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon,
                                              partials, counters, out, diag, stream, k_scale, v_scale);
     if (g.head_dim == 64)
-        return launch_dense_gd<G, 64>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon,
+        return launch_dense_gd<G, 64>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon,
                                       partials, counters, out, diag, stream);
     if (g.head_dim == 256)
-        return launch_dense_gd<G, 256>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon,
+        return launch_dense_gd<G, 256>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon,
                                        partials, counters, out, diag, stream);
-    return launch_dense_gd<G, 128>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials,
+    return launch_dense_gd<G, 128>(g, q, k, v, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon, partials,
                                    counters, out, diag, stream);
 }
 
 cudaError_t launch_dense(const Geometry& g_in, const void* q, const void* k_cache, const void* v_cache,
-                         const int32_t* block_table, const int32_t* seq_lens, const int32_t* fallback_list,
-                         const int32_t* fallback_count, float epsilon, float* out, vsa_diag_t* diag, void* ws,
-                         cudaStream_t stream, bool tickets_cleared, const float* k_scale, const float* v_scale)
+                         const int32_t* block_table, const int32_t* seq_lens, const int32_t* fallback_list_in,
+                         const int32_t* fallback_count_in, float epsilon, float* out, vsa_diag_t* diag, void* ws,
+                         cudaStream_t stream, bool tickets_cleared, const float* k_scale, const float* v_scale, const int32_t* flags)
 {
     if ((k_scale || v_scale) && (!k_scale || !v_scale || g_in.head_dim != kHeadDim)) return cudaErrorInvalidValue;
     const Geometry g = with_virtual_kv_heads(g_in);
+    int32_t *fallback_list = const_cast<int32_t*>(fallback_list_in), *fallback_count = const_cast<int32_t*>(fallback_count_in);   // (written with flags only)
     int32_t* counters = (int32_t*)ws;
     float* partials = (float*)((char*)ws + dense_counter_bytes(g));
     if (!tickets_cleared) {
@@ -935,10 +958,10 @@ cudaError_t launch_dense(const Geometry& g_in, const void* q, const void* k_cach
     }
     const uint16_t *qq = (const uint16_t*)q, *kk = (const uint16_t*)k_cache, *vv = (const uint16_t*)v_cache;
     switch (g.group) {
-        case 1: return launch_dense_g<1>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
-        case 2: return launch_dense_g<2>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
-        case 4: return launch_dense_g<4>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
-        case 8: return launch_dense_g<8>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
+        case 1: return launch_dense_g<1>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
+        case 2: return launch_dense_g<2>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
+        case 4: return launch_dense_g<4>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
+        case 8: return launch_dense_g<8>(g, qq, kk, vv, block_table, seq_lens, fallback_list, fallback_count, flags, epsilon, partials, counters, out, diag, stream, k_scale, v_scale);
         default: return cudaErrorInvalidValue;
     }
 }

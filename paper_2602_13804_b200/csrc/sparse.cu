@@ -44,6 +44,31 @@ size_t step_smem_bytes(const Geometry& g, int P, int K_c, bool fused, bool solve
                                false, solve).total * 4;
 }
 
+// Query heads of a cluster: those of a KV head, eight at most (the portable cluster size).
+int scan_heads(const Geometry& g) { return g.group < 8 ? g.group : 8; }
+
+// Blocks of a cluster when the sparse pass scans the pages itself, 0 when a scan ahead of it is faster.  The kernel boundary
+// and the scores' way through memory are 1.5 us of a step, but the scan then runs on the SMs of the units only, two or more
+// (tile of 16 pages, head) items to a group of lanes cost what that saves, and with 256 threads two units share an SM.
+// Up to `half`: one item for every other group of lanes.  Blocks that only help with the scan double this where that many
+// SMs are free anyway.  Microseconds per layer, scan ahead / here, by items of the largest context per block: one sequence,
+// 8 KV heads of 4 heads, 4k 12.6 / 11.1 (16), 8k 12.6 / 12.2 (32), with helpers 11.8 (16), 16k 12.6 / 12.8 (32, with helpers); two
+// of 4k 12.8 / 11.7, four 13.1 / 12.1; eight of 4k (256 threads) 16.1 / 16.1.  One head a group 4k 12.9 / 11.6 (16), 16k 14.1 /
+// 14.7 (32); two heads 4k 12.8 / 11.4.  Eight heads, whose scan ahead is slower: 4k 14.9 / 12.9 (16), 16k 14.2 / 13.7 (64).
+// A cluster needs its SMs in one GPC: of 148 one block each, 132 are within reach of clusters of four and 120 of eight.  128 units
+// of one head a group, which share no rows: 15.4 / 15.7.
+int scan_cluster(const Geometry& g, bool solve)
+{
+    const int heads = scan_heads(g), groups = (solve ? 256 : 512) / step_lanes_per_row(g.head_dim);
+    const long long clusters = (long long)g.batch * g.n_q_heads / heads, tiles = (g.max_pages + 15) / 16;
+    const int sms = sm_count(), half = groups / 2;
+    auto items = [&](int c) { return (tiles + c - 1) / c * heads; };
+    int c = heads;
+    while (items(c) > half && 2 * c <= 8 && 2 * c * clusters * 16 <= 7 * sms) c *= 2;
+    if (items(c) > (heads == 8 ? 4 * half : half)) return 0;
+    return clusters * c * 16 <= (c == 8 ? 13 : c == 1 ? 7 : 14) * sms ? c : 0;
+}
+
 // thread-block size of the routing variants for a launch
 int sparse_block_threads(const Geometry& g, int P, bool listed, bool two_level, int P_super)
 {
@@ -56,6 +81,15 @@ int sparse_block_threads(const Geometry& g, int P, bool listed, bool two_level, 
 }
 
 }  // namespace
+
+bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve)
+{
+    const int cluster = scan_cluster(g, solve);
+    if (!cluster) return false;
+    const int threads = solve ? 256 : step_threads(g, P);
+    return (size_t)step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, true, fp8, solve, cluster, scan_heads(g)).total * 4 <=
+           (size_t)227 * 1024;
+}
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)
 {
@@ -71,7 +105,8 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
                           vsa_diag_t* diag, int32_t* fallback_list, int32_t* fallback_count, cudaStream_t stream,
                           int solver_iters, vsa_solve_t* solve, const float* rad_logical, vsa_cert_t* cert,
                           int solver_kind, const int32_t* unit_list, const int32_t* unit_count, int routed_stride,
-                          const void* tl_summaries, int P_super, const float* k_scale, const float* v_scale)
+                          const void* tl_summaries, int P_super, const float* k_scale, const float* v_scale,
+                          const void* scan_summaries, int32_t* flags, int32_t* tickets)
 {
     if ((k_scale || v_scale) && (!k_scale || !v_scale || solve || cert || tl_summaries || g.head_dim != kHeadDim))
         return cudaErrorInvalidValue;
@@ -88,9 +123,17 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         p.page_scores = page_scores;
         p.P = P;
         p.K_c = K_c;
-        const int threads = solve ? 256 : step_threads(g, P);
-        p.lay = step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, page_scores != nullptr, k_scale != nullptr,
-                            solve != nullptr);
+        const int threads = solve ? 256 : step_threads(g, P), cluster = scan_summaries ? scan_cluster(g, solve != nullptr) : 0;
+        p.lay = step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, page_scores || scan_summaries,
+                            k_scale != nullptr, solve != nullptr, cluster, scan_heads(g));
+        p.summaries = (const uint16_t*)scan_summaries;
+        p.cluster_shift = 0;
+        while ((1 << p.cluster_shift) < cluster) ++p.cluster_shift;
+        p.heads_shift = 0;
+        while ((1 << p.heads_shift) < scan_heads(g)) ++p.heads_shift;
+        p.flags = flags;
+        p.tickets = tickets;
+        p.n_tickets = tickets ? dense_ticket_count(g) : 0;
         p.group_shift = 0;
         while ((1 << p.group_shift) < g.group) ++p.group_shift;
         p.epsilon = epsilon;

@@ -42,7 +42,7 @@ namespace vsa {
 
 // Shared-memory layout in 4-byte words; every part starts on a 16-byte boundary.
 struct StepLayout {
-    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, bar, cand, solve, work, vring, bt;
+    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, bar, cand, solve, work, vring, bt, scan_q, scan_ring;
     int total;
     bool stage_bt;   // the block-table row is copied before the wait (blocks that wait for the scan anyway)
 };
@@ -55,7 +55,13 @@ struct StepParams {
     const uint16_t *q, *k, *v;
     const int32_t *block_table, *seq_lens;
     int32_t* routed_pages;
-    const float* page_scores;   // nullptr: routed_pages is an input
+    const float* page_scores;   // nullptr: routed_pages is an input, or (summaries) the scores are computed here
+    const uint16_t* summaries;  // not nullptr: the page scan runs here, by a cluster of the blocks of a KV head's query heads
+    int cluster_shift;          // log2(blocks of a cluster): those of the heads, the first of them, and others that only scan
+    int heads_shift;            // log2(heads of a cluster)
+    int32_t* flags;             // with summaries: fallback flag of every unit, from which the dense pass makes the list
+    int32_t* tickets;           // with summaries: the dense pass's tickets, cleared here
+    int n_tickets;
     int P, K_c;
     float epsilon, gap_threshold;
     float* out;
@@ -102,7 +108,8 @@ __host__ __device__ constexpr int step_value_stages(int threads, bool solve)
     return solve ? 4 : threads == 128 ? 2 : threads == 256 ? 3 : 0;
 }
 
-inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve)
+inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
+                              int cluster = 0, int heads = 0)
 {
     StepLayout s;
     const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
@@ -146,13 +153,21 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     const int vring_end = s.vring + 4 * stages * threads * lane_words - s.work;
     w = vring_end > w ? vring_end : w;
     if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
+    // page scan: the queries of the cluster's heads and the summary rows of the next round, beside the scores
+    s.scan_q = s.work + ((max_pages + 11) & ~3);
+    s.scan_ring = s.scan_q + heads * (D / 2);
+    if (cluster) {
+        const bool ahead = (max_pages + 15) / 16 > cluster * groups;   // more than one round
+        const int scan_end = s.scan_ring + (ahead ? threads * 16 * 4 : 0) - s.work;
+        w = scan_end > w ? scan_end : w;
+    }
     if (tt > 1 && threads * 16 * lane_words > w) w = threads * 16 * lane_words;
     if (solve && ((K_c + 31) & ~31) * 64 > w) w = ((K_c + 31) & ~31) * 64;
     o += w;
     s.bt = o;
     // (not where it would cost the second block of an SM)
-    s.stage_bt = fused && threads >= 256 && max_pages <= 8192 && (threads == 512 || o + max_pages <= 113 * 256);
-    if (s.stage_bt) o += max_pages;
+    s.stage_bt = fused && (cluster || (threads >= 256 && max_pages <= 8192 && (threads == 512 || o + max_pages <= 113 * 256)));
+    if (s.stage_bt) o += (max_pages + 15) & ~15;
     s.total = (o + 3) & ~3;
     return s;
 }
@@ -252,6 +267,116 @@ __device__ __forceinline__ void reduce_tile_xor(float (&v)[16])
     }
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// the place of a shared-memory address of this block in block `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+// The page scan of one (sequence, KV head) by the cluster of the blocks of its query heads and their helpers: tiles of 16 summary rows are
+// dealt out to the blocks and, there, to the groups of lanes; a tile is scored for all heads of the cluster in the way of
+// token routing, and every head's scores go to the shared memory of its own block.  Where there are fewer tiles than
+// groups of lanes, the heads are dealt out as well.  The first tile of a group of lanes comes through registers, every
+// later one through shared memory, asked for one round ahead.  Ends with the scores of this block's head complete in sc.
+// Bound by one load from memory (0.6 us), the chain of a tile's sums (0.6) and the barrier of the cluster (0.4), where a kernel
+// ahead takes 3.1 with its boundary and 0.5 to read its scores: one sequence of 4k 12.6 -> 11.2 us per layer, as one call 12.0 -> 10.5.
+template <int THREADS, int D>
+__device__ __forceinline__ void step_scan_pages(const StepParams& p, const int32_t* bt_s, const uint8_t* qs, const uint8_t* ring,
+                                                const float* sc, int nb, int g)
+{
+    constexpr int LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR, ROW = 2 * D, TPL = LPR == 8 ? 2 : 1;
+    const Geometry& geo = p.geo;
+    const int tid = threadIdx.x, warp = tid >> 5, c = tid % LPR, grp = tid / LPR;
+    const int cs = p.cluster_shift, C = 1 << cs, rank = (int)blockIdx.x & (C - 1), hs = p.heads_shift;
+    const int n_tiles = (nb + 15) >> 4, mine = (n_tiles - rank + C - 1) >> cs;   // tiles rank, rank + C, ...
+    int ss = 0;   // log2 of the parts that the heads are dealt out in
+    while (ss < hs && (mine << (ss + 1)) <= GROUPS) ++ss;
+    const int n_items = mine << ss, per = (1 << hs) >> ss;
+    const uint8_t* base = reinterpret_cast<const uint8_t*>(p.summaries) + (long long)g * ROW + c * 16;
+    const unsigned page_bytes = (unsigned)(geo.n_kv_heads * ROW);
+    const uint32_t sc_s = (uint32_t)__cvta_generic_to_shared(sc);
+    const uint8_t* own_ring = ring + grp * 16 * ROW;
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(own_ring) + c * 16, at = (uint32_t)(tile_xor<LPR>(c) * ROW + c * 16);
+    auto tile_of = [&](int item) { return rank + ((item >> ss) << cs); };
+    auto page_ok = [&](int e) { return e >= 0 && e < geo.pool_pages; };
+    // rows without a valid page read row 0 of the pool instead (their score becomes -inf)
+    auto row_of = [&](int e) { return base + (unsigned long long)(unsigned)(page_ok(e) ? e : 0) * page_bytes; };
+    auto entries = [&](int item, int (&e)[16]) {   // (entries past the sequence are whatever the table holds)
+        const int4* t4 = reinterpret_cast<const int4*>(bt_s + 16 * tile_of(item));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int4 x = t4[i];
+            e[4 * i] = x.x, e[4 * i + 1] = x.y, e[4 * i + 2] = x.z, e[4 * i + 3] = x.w;
+        }
+    };
+    const bool any = warp * GPW < n_items;
+    uint4 rows[16];
+    auto ahead = [&](int item) {
+        if (item >= n_items) return;
+        int e[16];
+        entries(item, e);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) cp_async_16B(ring_s + (uint32_t)(t * ROW), row_of(e[t]));
+    };
+    if (any) {
+        int e[16];
+        entries(grp < n_items ? grp : 0, e);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) rows[t] = ld_cg_16B(row_of(e[t]));
+        cp_async_commit_group();   // (the queries)
+        ahead(grp + GROUPS);
+    } else {
+        cp_async_commit_group();
+    }
+    cp_async_commit_group();
+    cp_async_wait_group<1>();
+    __syncthreads();
+    cluster_wait();   // the other blocks of the cluster run
+#pragma unroll 1
+    for (int i0 = 0; i0 + warp * GPW < n_items; i0 += GROUPS) {
+        const int item = i0 + grp;
+        if (i0 != 0) {
+            cp_async_wait_all();
+            __syncwarp();   // the other lanes' pieces of the tile
+#pragma unroll
+            for (int t = 0; t < 16; ++t) rows[t] = *reinterpret_cast<const uint4*>(own_ring + (at ^ (uint32_t)(t * ROW)));
+            __syncwarp();
+            ahead(item + GROUPS);
+        }
+        const int first = tile_of(item) * 16, head0 = (item & ((1 << ss) - 1)) * per;
+#pragma unroll 1
+        for (int hh = head0; hh < head0 + per; ++hh) {
+            const uint4 qv = *reinterpret_cast<const uint4*>(qs + hh * ROW + c * 16);
+            float vals[16];
+#pragma unroll
+            for (int t = 0; t < 16; ++t) vals[t] = chunk_partial_bf16(qv, rows[t]);
+            __syncwarp();
+            if (i0 != 0)
+                reduce_tile_xor<LPR>(vals);
+            else
+                reduce_tile<LPR>(vals, c);
+            const uint32_t dst = cluster_address(sc_s, hh);
+#pragma unroll
+            for (int s = 0; s < TPL; ++s) {
+                const int l = first + (LPR == 8 ? 2 * c + s : LPR == 32 ? c >> 1 : c);
+                if (item < n_items && l < nb && (LPR != 32 || (c & 1) == 0))
+                    cluster_store(dst + 4u * (uint32_t)l, page_ok(bt_s[l]) ? vals[s] : -INFINITY);
+            }
+        }
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+}
+
 __device__ __noinline__ void step_failed_unit(const BlockTeam& tm, const StepParams& p, long long unit, int status, int D,
                                               bool routed_too)
 {
@@ -264,6 +389,7 @@ __device__ __noinline__ void step_failed_unit(const BlockTeam& tm, const StepPar
         d.status = status;
         p.diag[unit] = d;
         if (p.solve) p.solve[unit] = vsa_solve_t{0.0f, 0.0f, 0.0f, 0.0f};
+        if (p.flags) p.flags[unit] = 0;
     }
     if (routed_too)
         for (int t = tm.tid; t < p.P; t += tm.size) p.routed_pages[unit * p.P + t] = -1;
@@ -311,13 +437,14 @@ __device__ __forceinline__ int rank_below(const int32_t* win, int n, int l, int 
 
 // THREADS: 512 (one block per SM) when there are no more units than SMs, 256 (two) up to two units per SM, 128
 //   (four, or BLOCKS = five) beyond: a unit is a latency chain, so units in flight count for more than threads per unit.
-// FUSED: the unit's pages are selected here from page_scores; otherwise routed_pages is an input.
+// FUSED: the unit's pages are selected here from page_scores (1) or from scores computed here (2: the blocks of a cluster are
+//   the query heads of a KV head, eight at most); otherwise (0) routed_pages is an input.
 // D: head dimension.  A row is spread over D / 8 lanes, 8 elements (16 bytes; fp8: 8 bytes) each, so a warp works
 //   on 4, 2 or 1 tiles of 16 rows at a time.
 // FP8: k / v hold e4m3 bytes with one scale per (pool page, KV head); strides count bytes.  Scores and weights are
 //   multiplied by the scale afterwards (exact for powers of two).
 // SOLVE: the weights come from solver_iters entropic (1) or Frank-Wolfe (2) iterations (step_solve.cuh).
-template <int THREADS, bool FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0, int BLOCKS = 512 / THREADS>
+template <int THREADS, int FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0, int BLOCKS = 512 / THREADS>
 __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __grid_constant__ StepParams p)
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
@@ -346,14 +473,20 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     uint32_t* work = smem + lay.work;
     int32_t* bt_s = (int32_t*)(smem + lay.bt);
     const int lane = tid & 31, warp = tid >> 5, c = lane % LPR, grp = tid / LPR;
-    const int h = blockIdx.x, b = blockIdx.y, g = h >> p.group_shift;
+    int h = blockIdx.x, helper = 0;
+    if constexpr (FUSED == 2) {   // (a helper: the first head of its cluster)
+        helper = (h & ((1 << p.cluster_shift) - 1)) >> p.heads_shift;
+        h = ((h >> p.cluster_shift) << p.heads_shift) + (helper ? 0 : h & ((1 << p.heads_shift) - 1));
+    }
+    const int b = blockIdx.y, g = h >> p.group_shift;
     const long long unit = b * geo.n_q_heads + h;   // (batch * n_q_heads fits 30 bits)
     const int32_t* bt = p.block_table + (long long)b * geo.max_pages;
 
-    // before the wait on the preceding kernel: the sequence length, the query (the routing kernel that precedes
-    // this one in a step has read both), the block-table row and cleared counters
+    // before the wait on the preceding kernel: the sequence length, the query (unless the scan runs here: the routing kernel
+    // that precedes this one in a step has read both), the block-table row and cleared counters
     const int T = ld_ca_s32(p.seq_lens + b);
-    const uint4 qraw = ld_nc_16B(p.q + unit * D + c * 8);
+    uint4 qraw;
+    if constexpr (FUSED != 2) qraw = ld_nc_16B(p.q + unit * D + c * 8);
     if (FUSED && lay.stage_bt) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(bt_s);
         for (int i = tid; i < geo.max_pages; i += THREADS) cp_async_4(dst + 4u * (uint32_t)i, bt + i);
@@ -369,9 +502,17 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int r_warp = (P + WARPS - 1) / WARPS;
+    if constexpr (FUSED == 2) {
+        cluster_arrive();
+        cp_async_wait_all();
+        __syncthreads();
+    }
     pdl_wait();
     pdl_launch_dependents();
+    if (FUSED == 2 && tid == 0 && unit < p.n_tickets) p.tickets[unit] = 0;
     if (!length_ok) {
+        if constexpr (FUSED == 2) cluster_wait();
+        if (helper) return;
         cp_async_wait_all();
         step_failed_unit(tm, p, unit, VSA_UNIT_BAD_LENGTH, D, FUSED);
         return;
@@ -394,25 +535,35 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     if constexpr (FUSED) {
         // ---- stage the scores of the sequence's pages, four to a chunk; a thread only reads back what it copied.
         //      Short rows spread over the warps (all of them have to vouch for r_warp scores) ----
-        const float* row = p.page_scores + unit * geo.max_pages;
-        const int mis = (int)((unit * geo.max_pages) & 3), n_chunks = (nb + mis + 3) >> 2;
+        const float* row = FUSED == 1 ? p.page_scores + unit * geo.max_pages : nullptr;
+        const int mis = FUSED == 1 ? (int)((unit * geo.max_pages) & 3) : 0, n_chunks = (nb + mis + 3) >> 2;
         const bool single = n_chunks <= THREADS;   // a chunk per thread at most: it stays in registers
         const int chunk0 = single ? lane * WARPS + warp : tid, l0 = 4 * chunk0 - mis;
         float* sc = reinterpret_cast<float*>(work);
         float4* sc4 = reinterpret_cast<float4*>(sc);
         np = min(P, nb);
         auto in_row = [&](int l) { return (unsigned)l < (unsigned)nb; };
+        if constexpr (FUSED == 2) {
+            const int heads = 1 << p.heads_shift, first = h & ~(heads - 1);
+            const uint8_t* qs = reinterpret_cast<const uint8_t*>(smem + lay.scan_q);
+            const uint32_t qs_s = (uint32_t)__cvta_generic_to_shared(qs);
+            for (int i = tid; i < heads * (D / 8); i += THREADS)
+                cp_async_16B(qs_s + 16u * (uint32_t)i, p.q + ((long long)b * geo.n_q_heads + first) * D + i * 8);
+            step_scan_pages<THREADS, D>(p, bt_s, qs, reinterpret_cast<const uint8_t*>(smem + lay.scan_ring), sc, nb, g);
+            if (helper) return;
+            qraw = *reinterpret_cast<const uint4*>(qs + (h - first) * 2 * D + c * 16);
+        }
         float4 own_chunk = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         // words of the first and the last chunk that are no scores of this row: below or equal to every score
         if (single) {
             if (chunk0 < n_chunks) {
-                const float4 v = ld_cg_f32x4(row + l0);
+                const float4 v = FUSED == 1 ? ld_cg_f32x4(row + l0) : sc4[chunk0];
                 if (in_row(l0)) own_chunk.x = v.x;
                 if (in_row(l0 + 1)) own_chunk.y = v.y;
                 if (in_row(l0 + 2)) own_chunk.z = v.z;
                 if (in_row(l0 + 3)) own_chunk.w = v.w;
             }
-        } else {
+        } else if constexpr (FUSED == 1) {
             const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sc);
             for (int i = chunk0; i < n_chunks; i += THREADS) cp_async_16B(dst + 16u * (uint32_t)i, row - mis + 4 * i);
         }
@@ -621,7 +772,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                     if constexpr (FP8)
                         rows[t] = ld_nc_8B(src + t * stride);
                     else
-                        rows[t] = ld_nc_16B(src + t * stride);
+                        rows[t] = FUSED == 2 ? ld_cg_16B(src + t * stride) : ld_nc_16B(src + t * stride);
                 }
             } else if constexpr (BULK) {
                 if (active && !mbar_wait(bar, (uint32_t)(r - 1) & 1u)) ctl[kCtlLate] = 1u;
@@ -1014,27 +1165,39 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         d.fallback = (delta < p.gap_threshold && ns < T) ? 1 : 0;
         d.status = 0;
         p.diag[unit] = d;
-        if (d.fallback) p.fallback_list[atomicAdd(p.fallback_count, 1)] = (int32_t)unit;
+        if (FUSED == 2)
+            p.flags[unit] = d.fallback;
+        else if (d.fallback)
+            p.fallback_list[atomicAdd(p.fallback_count, 1)] = (int32_t)unit;
     }
 }
 
-template <int THREADS, bool FUSED, int D, bool FP8, int SOLVE = 0, int BLOCKS = 512 / THREADS>
+template <int THREADS, int FUSED, int D, bool FP8, int SOLVE = 0, int BLOCKS = 512 / THREADS>
 cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
 {
     static bool attr_done[kMaxDevices] = {};   // per template instance
-    const size_t smem = (size_t)p.lay.total * 4;
+    size_t smem = (size_t)p.lay.total * 4;
+    // a scanning block has an SM of its own (two units of a solve on one SM, which a cluster's blocks otherwise share: one
+    // sequence of 4k, four entropic iterations 27.2 against 20.7 us per layer)
+    if (FUSED == 2 && smem < 120 * 1024) smem = 120 * 1024;
     if (smem > 48 * 1024) {
         const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>, attr_done);
         if (e != cudaSuccess) return e;
     }
-    return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>, dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch),
-                      dim3(THREADS), smem, stream, p);
+    if constexpr (FUSED == 2)
+        return launch_pdl_cluster(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>,
+                                  dim3((unsigned)(p.geo.n_q_heads >> p.heads_shift << p.cluster_shift), (unsigned)p.geo.batch),
+                                  dim3(THREADS), 1u << p.cluster_shift, smem, stream, p);
+    else
+        return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>,
+                          dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch), dim3(THREADS), smem, stream, p);
 }
 
 template <int D, bool FP8>
 cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
 {
     const bool fused = p.page_scores != nullptr;
+    if (p.summaries) return threads == 512 ? launch_step_variant<512, 2, D, FP8>(p, stream) : cudaErrorInvalidValue;
     // Five blocks per SM at 96 registers against four at 128, which make a unit 5 - 10 % faster: five
     // where they save a wave of blocks, and from three waves of four on, where units in flight count for more.  Microseconds
     // per layer, four / five, T = 8k.  A wave saved: 32 pages a unit, 640 units 41.6 / 31.9, 704 43.5 / 32.5, 1280 65.4 / 56.0,
@@ -1048,11 +1211,11 @@ cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t st
     const bool fits = (size_t)p.lay.total * 4 + 1024 <= (size_t)228 * 1024 / 5;   // (1 KB of each block is the system's)
     if (threads == 128 && fused && fits &&
         ((units + five - 1) / five < (units + four - 1) / four || units >= 3 * four))
-        return launch_step_variant<128, true, D, FP8, 0, 5>(p, stream);
+        return launch_step_variant<128, 1, D, FP8, 0, 5>(p, stream);
 #define VSA_STEP_CASE(T)                                                                    \
     if (threads == T)                                                                       \
-        return fused ? launch_step_variant<T, true, D, FP8>(p, stream)                      \
-                     : launch_step_variant<T, false, D, FP8>(p, stream);
+        return fused ? launch_step_variant<T, 1, D, FP8>(p, stream)                      \
+                     : launch_step_variant<T, 0, D, FP8>(p, stream);
     VSA_STEP_CASE(512)
     VSA_STEP_CASE(256)
     VSA_STEP_CASE(128)

@@ -28,6 +28,27 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The same with thread-block clusters of `cluster` blocks along x.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, unsigned cluster, size_t smem,
+                                      cudaStream_t stream, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // Ordinary kernel launch: starts when everything before it in the stream has finished.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_in_order(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
@@ -178,7 +199,11 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
                           vsa_cert_t* cert = nullptr, int solver_kind = 1, const int32_t* unit_list = nullptr,
                           const int32_t* unit_count = nullptr, int routed_stride = 0,
                           const void* tl_summaries = nullptr, int P_super = 0, const float* k_scale = nullptr,
-                          const float* v_scale = nullptr);
+                          const float* v_scale = nullptr, const void* scan_summaries = nullptr, int32_t* flags = nullptr,
+                          int32_t* tickets = nullptr);
+// scan_summaries != nullptr (step_scans() of the shape, page_scores nullptr): the kernel scores the pages itself, writes
+// every unit's fallback flag instead of the list and clears the dense pass's tickets.
+bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve);
 // k_scale / v_scale != nullptr: k_cache / v_cache hold e4m3 bytes, value = byte * scale[pool page][KV head]
 // (closed-form family, head dimension 128).
 // tl_summaries != nullptr: the two-level front end - page_scores then holds the scores of the super-pages'
@@ -218,7 +243,8 @@ cudaError_t launch_dense(const Geometry& g, const void* q, const void* k_cache, 
                          const int32_t* block_table, const int32_t* seq_lens, const int32_t* fallback_list,
                          const int32_t* fallback_count, float epsilon, float* out, vsa_diag_t* diag, void* ws,
                          cudaStream_t stream, bool tickets_cleared = false, const float* k_scale = nullptr,
-                         const float* v_scale = nullptr);
+                         const float* v_scale = nullptr, const int32_t* flags = nullptr);
+// flags != nullptr: the units with a flag other than 0 are the list; fallback_list and fallback_count are written
 // the per-(sequence, KV head) tickets at the start of the dense workspace, and how many there are
 int32_t* dense_tickets(void* ws_dense);
 int dense_ticket_count(const Geometry& g);
