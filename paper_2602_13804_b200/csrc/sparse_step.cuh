@@ -173,16 +173,17 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
 }
 
 // Exact page selection when the list overflows (many equal scores).  Leaves exactly K entries in list[] and
-// hist[] cleared.  scratch: 16 words + one per warp.
+// hist[] cleared.  scratch: 16 words; wred: one word per warp (not the words behind scratch, where the winners' list is padded for
+// the ranks that follow).
 __device__ __noinline__ void step_pages_exact(const BlockTeam& tm, const float* sc, int n, int K, uint32_t* hist,
-                                              uint32_t* scratch, unsigned long long* list, uint32_t* counter)
+                                              uint32_t* scratch, uint32_t* wred, unsigned long long* list, uint32_t* counter)
 {
     tm.sync();   // every thread has read the counter
     for (int i = tm.tid; i < kStepPages; i += tm.size) list[i] = 0ull;
     if (tm.tid == 0) *counter = 0u;
     tm.sync();
     auto key = [&](int i) { return max(float_to_key(sc[i]), 1u); };   // 0 (one NaN pattern) would read as no page
-    team_exact_topk_slow(tm, key, n, K, hist, scratch, scratch + 16, [&](int i) {
+    team_exact_topk_slow(tm, key, n, K, hist, scratch, wred, [&](int i) {
         list[atomicAdd(counter, 1u)] = ((unsigned long long)key(i) << 32) | (uint32_t)~i;
     });
     for (int i = tm.tid; i < kStepBins; i += tm.size) hist[i] = 0u;
@@ -659,7 +660,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         int m = (int)ctl[kCtlPages];
         if (m > kStepPages) {
             if (single && chunk0 < n_chunks) sc4[chunk0] = own_chunk;
-            step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, pages, &ctl[kCtlPages]);
+            step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, warp_stat, pages, &ctl[kCtlPages]);
             m = np;
         }
         // ---- exact ranks, four lanes per listed page ----

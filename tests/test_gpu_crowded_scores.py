@@ -13,6 +13,8 @@ pytestmark = pytest.mark.gpu
     (2, 4, 2, 128, 1030),    # the same with several tiles per group of lanes
     (40, 4, 2, 70, 513),     # 160 units: 256 threads
     (80, 4, 4, 64, 600),     # 320 units: 128 threads
+    (2, 4, 2, 5, 40),        # fewer pages than the block has warps
+    (80, 4, 4, 3, 30),
 ])
 @pytest.mark.parametrize("distinct", [1, 3])
 def test_equal_scores(batch, hq, hkv, P, K_c, distinct):
