@@ -552,17 +552,24 @@ static int decode_step_impl(const vsa_shape_t* shape, const void* q, const void*
                                          diag, ws_dense, st, /*tickets_cleared=*/true, k_scale, v_scale, flags));
     }
     if (ev[0] && cudaEventRecord(ev[0], st) != cudaSuccess) return VSA_ERR_CUDA;
-    // the scan kernel clears fallback_count and the dense pass's tickets: the step enqueues no memset
-    cudaError_t e = vsa::launch_route_scan(g, q, summaries, block_table, seq_lens, ws, fallback_count,
-                                           vsa::dense_tickets(ws_dense), vsa::dense_ticket_count(g), st,
-                                           cert ? radii : nullptr, rad_logical);
+    // The scan kernel clears fallback_count and the dense pass's tickets: the step enqueues no memset.  The bounds of scores by
+    // MMAs lie in the place of the dense pass's partial results.
+    uint32_t* bounds = nullptr;
+    if (!cert && !solve && vsa::step_takes_bounds(g, P) && vsa::route_mma_wins(g) && vsa::route_bound_bytes(g) <= vsa::dense_partials_bytes(g))
+        bounds = (uint32_t*)vsa::dense_partials(g, ws_dense);
+    cudaError_t e = bounds ? vsa::launch_route_mma(g, q, summaries, block_table, seq_lens, (float*)ws, bounds, fallback_count,
+                                                   vsa::dense_tickets(ws_dense), vsa::dense_ticket_count(g), st)
+                           : vsa::launch_route_scan(g, q, summaries, block_table, seq_lens, ws, fallback_count,
+                                                    vsa::dense_tickets(ws_dense), vsa::dense_ticket_count(g), st,
+                                                    cert ? radii : nullptr, rad_logical);
     if (e != cudaSuccess) return VSA_ERR_CUDA;
     if (ev[1] && cudaEventRecord(ev[1], st) != cudaSuccess) return VSA_ERR_CUDA;
     // the top-P selection runs inside the fused kernel, on the scores the scan left in ws
     if (ev[2] && cudaEventRecord(ev[2], st) != cudaSuccess) return VSA_ERR_CUDA;
     e = vsa::launch_sparse(g, q, k_cache, v_cache, block_table, seq_lens, routed_pages, (const float*)ws, P, K_c,
                            epsilon, gap_threshold, out, diag, fallback_list, fallback_count, st, solver_iters, solve,
-                           rad_logical, cert, solver_kind, nullptr, nullptr, 0, nullptr, 0, k_scale, v_scale);
+                           rad_logical, cert, solver_kind, nullptr, nullptr, 0, nullptr, 0, k_scale, v_scale,
+                           bounds ? summaries : nullptr, nullptr, nullptr, bounds);
     if (e != cudaSuccess) return VSA_ERR_CUDA;
     if (ev[3] && cudaEventRecord(ev[3], st) != cudaSuccess) return VSA_ERR_CUDA;
     e = vsa::launch_dense(g, q, k_cache, v_cache, block_table, seq_lens, fallback_list, fallback_count, epsilon,

@@ -902,6 +902,10 @@ size_t dense_workspace_bytes(const Geometry& g_in)
     return dense_counter_bytes(g) + (size_t)dense_max_items(g) * g.group * (2 + g.head_dim) * sizeof(float);
 }
 
+void* dense_partials(const Geometry& g, void* ws_dense) { return (char*)ws_dense + dense_counter_bytes(g); }
+
+size_t dense_partials_bytes(const Geometry& g) { return dense_workspace_bytes(g) - dense_counter_bytes(g); }
+
 template <int G, int D, bool FP8 = false>
 static cudaError_t launch_dense_gd(const Geometry& g, const uint16_t* q, const uint16_t* k, const uint16_t* v,
                                    const int32_t* block_table, const int32_t* seq_lens, int32_t* fallback_list,
@@ -951,7 +955,7 @@ cudaError_t launch_dense(const Geometry& g_in, const void* q, const void* k_cach
     const Geometry g = with_virtual_kv_heads(g_in);
     int32_t *fallback_list = const_cast<int32_t*>(fallback_list_in), *fallback_count = const_cast<int32_t*>(fallback_count_in);   // (written with flags only)
     int32_t* counters = (int32_t*)ws;
-    float* partials = (float*)((char*)ws + dense_counter_bytes(g));
+    float* partials = (float*)dense_partials(g, ws);
     if (!tickets_cleared) {
         cudaError_t e = cudaMemsetAsync(counters, 0, dense_counter_bytes(g), stream);
         if (e != cudaSuccess) return e;

@@ -47,26 +47,45 @@ size_t step_smem_bytes(const Geometry& g, int P, int K_c, bool fused, bool solve
 // Query heads of a cluster: those of a KV head, eight at most (the portable cluster size).
 int scan_heads(const Geometry& g) { return g.group < 8 ? g.group : 8; }
 
-// Blocks of a cluster when the sparse pass scans the pages itself, 0 when a scan ahead of it is faster.  The kernel boundary
-// and the scores' way through memory are 1.5 us of a step, but the scan then runs on the SMs of the units only, two or more
-// (tile of 16 pages, head) items to a group of lanes cost what that saves, and with 256 threads two units share an SM.
-// Up to `half`: one item for every other group of lanes.  Blocks that only help with the scan double this where that many
-// SMs are free anyway.  Microseconds per layer, scan ahead / here, by items of the largest context per block: one sequence,
-// 8 KV heads of 4 heads, 4k 12.6 / 11.1 (16), 8k 12.6 / 12.2 (32), with helpers 11.8 (16), 16k 12.6 / 12.8 (32, with helpers); two
-// of 4k 12.8 / 11.7, four 13.1 / 12.1; eight of 4k (256 threads) 16.1 / 16.1.  One head a group 4k 12.9 / 11.6 (16), 16k 14.1 /
-// 14.7 (32); two heads 4k 12.8 / 11.4.  Eight heads, whose scan ahead is slower: 4k 14.9 / 12.9 (16), 16k 14.2 / 13.7 (64).
+// The clusters of a sparse pass that scans the pages itself, or none where a scan ahead of it is faster.  The kernel boundary
+// and the scores' way through memory are 1.5 us of a step, but the scan then runs on the SMs of the units only.
+//
+// Few pages, fixed-order scores: two or more (tile of 16 pages, head) items to a group of lanes cost what that saves, and with 256
+// threads two units share an SM.  Up to `half`: one item for every other group of lanes.  Blocks that only help with the scan
+// double this where that many SMs are free anyway.  Microseconds per layer, scan ahead / here, by items of the largest context per
+// block: one sequence, 8 KV heads of 4 heads, 4k 12.6 / 11.1 (16), 8k 12.6 / 12.2 (32), with helpers 11.8 (16), 16k 12.6 / 12.8 (32, with
+// helpers); two of 4k 12.8 / 11.7, four 13.1 / 12.1; eight of 4k (256 threads) 16.1 / 16.1.  One head a group 4k 12.9 / 11.6 (16), 16k
+// 14.1 / 14.7 (32); two heads 4k 12.8 / 11.4.  Eight heads, whose scan ahead is slower: 4k 14.9 / 12.9 (16), 16k 14.2 / 13.7 (64).
+//
+// Many pages, scores by MMAs (0.6 us slower than the fixed order where every warp has a tile at most: 4k 11.2 / 11.8): four tiles to a
+// warp at least, on most of the SMs; two blocks of 256 threads share one.  Ahead / here: 8 of 32k (4 tiles) 22.3 / 21.2, 8 of
+// 64k 29.2 / 27.7, 4 of 64k 20.5 / 19.4, 4 of 128k (8) 27.1 / 26.8, D = 64 8 of 32k 22.0 / 18.7, D = 256 34.1 / 33.0, four entropic
+// iterations 4 of 32k 33.1 / 28.0, 8 of 32k 36.9 / 36.6; with two tiles 8 of 16k 19.1 / 19.3, 4 of 32k 17.4 / 17.4, on 32 SMs one of 128k
+// 17.9 / 22.5, and with helpers on 64 19.4.  Eight heads, whose scan ahead is slower: any number, 4 of 20k (2 KV heads) 14.6 / 13.8, 16
+// heads of one KV head 2 of 64k 15.4 / 14.8, but no more than one on few SMs, one of 32k 14.9 / 14.6.
+//
 // A cluster needs its SMs in one GPC: of 148 one block each, 132 are within reach of clusters of four and 120 of eight.  128 units
 // of one head a group, which share no rows: 15.4 / 15.7.
-int scan_cluster(const Geometry& g, bool solve)
+struct ScanCluster {
+    int blocks;   // 0: a scan ahead
+    int per_sm;   // blocks that share an SM
+    bool mma;     // scores by MMAs
+};
+
+ScanCluster scan_cluster(const Geometry& g, int threads)
 {
-    const int heads = scan_heads(g), groups = (solve ? 256 : 512) / step_lanes_per_row(g.head_dim);
+    const int heads = scan_heads(g), groups = threads / step_lanes_per_row(g.head_dim), half = groups / 2, sms = sm_count();
     const long long clusters = (long long)g.batch * g.n_q_heads / heads, tiles = (g.max_pages + 15) / 16;
-    const int sms = sm_count(), half = groups / 2;
+    if (threads < 256) return {0, 0, false};
+    auto fits = [&](int c, int per_sm) { return clusters * c * 16 <= (long long)per_sm * (c == 8 ? 13 : c == 1 ? 7 : 14) * sms; };
     auto items = [&](int c) { return (tiles + c - 1) / c * heads; };
     int c = heads;
     while (items(c) > half && 2 * c <= 8 && 2 * c * clusters * 16 <= 7 * sms) c *= 2;
-    if (items(c) > (heads == 8 ? 4 * half : half)) return 0;
-    return clusters * c * 16 <= (c == 8 ? 13 : c == 1 ? 7 : 14) * sms ? c : 0;
+    if (items(c) <= (heads == 8 ? 4 * half : half) && fits(c, 1)) return {c, 1, false};
+    const long long blocks = clusters * heads, warps = (long long)heads * (threads / 32);
+    if (3 * blocks >= 2 * sms ? heads < 8 && tiles < 4 * warps : heads < 8 || tiles > warps) return {0, 0, false};
+    if (fits(heads, 1)) return {heads, 1, true};
+    return threads == 256 && fits(heads, 2) ? ScanCluster{heads, 2, true} : ScanCluster{0, 0, false};
 }
 
 // thread-block size of the routing variants for a launch
@@ -84,12 +103,14 @@ int sparse_block_threads(const Geometry& g, int P, bool listed, bool two_level, 
 
 bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve)
 {
-    const int cluster = scan_cluster(g, solve);
-    if (!cluster) return false;
     const int threads = solve ? 256 : step_threads(g, P);
-    return (size_t)step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, true, fp8, solve, cluster, scan_heads(g)).total * 4 <=
-           (size_t)227 * 1024;
+    const ScanCluster c = scan_cluster(g, threads);
+    if (!c.blocks || threads < 256) return false;
+    return (size_t)step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, true, fp8, solve, c.blocks, scan_heads(g), c.mma).total * 4 <=
+           (size_t)(c.per_sm == 2 ? 113 : 227) * 1024;
 }
+
+bool step_takes_bounds(const Geometry& g, int P) { return step_threads(g, P) == 128; }
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)
 {
@@ -106,7 +127,7 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
                           int solver_iters, vsa_solve_t* solve, const float* rad_logical, vsa_cert_t* cert,
                           int solver_kind, const int32_t* unit_list, const int32_t* unit_count, int routed_stride,
                           const void* tl_summaries, int P_super, const float* k_scale, const float* v_scale,
-                          const void* scan_summaries, int32_t* flags, int32_t* tickets)
+                          const void* scan_summaries, int32_t* flags, int32_t* tickets, const uint32_t* bounds)
 {
     if ((k_scale || v_scale) && (!k_scale || !v_scale || solve || cert || tl_summaries || g.head_dim != kHeadDim))
         return cudaErrorInvalidValue;
@@ -123,10 +144,15 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         p.page_scores = page_scores;
         p.P = P;
         p.K_c = K_c;
-        const int threads = solve ? 256 : step_threads(g, P), cluster = scan_summaries ? scan_cluster(g, solve != nullptr) : 0;
+        const int threads = solve ? 256 : step_threads(g, P);
+        const ScanCluster scan = page_scores || !scan_summaries ? ScanCluster{0, 0, false} : scan_cluster(g, threads);
+        const int cluster = scan.blocks;
         p.lay = step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, page_scores || scan_summaries,
-                            k_scale != nullptr, solve != nullptr, cluster, scan_heads(g));
+                            k_scale != nullptr, solve != nullptr, cluster, scan_heads(g), scan.mma);
         p.summaries = (const uint16_t*)scan_summaries;
+        p.bounds = bounds;
+        p.scan_per_sm = scan.per_sm;
+        p.scan_mma = scan.mma;
         p.cluster_shift = 0;
         while ((1 << p.cluster_shift) < cluster) ++p.cluster_shift;
         p.heads_shift = 0;

@@ -33,6 +33,7 @@
 
 #include <type_traits>
 
+#include "page_mma.cuh"
 #include "step_solve.cuh"
 #include "vsa_device.cuh"
 #include "vsa_launch.h"
@@ -42,7 +43,7 @@ namespace vsa {
 
 // Shared-memory layout in 4-byte words; every part starts on a 16-byte boundary.
 struct StepLayout {
-    int hist, warp_stat, misc, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, bar, cand, solve, work, vring, bt, scan_q, scan_ring;
+    int hist, warp_stat, misc, win_key, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, bar, cand, solve, work, vring, bt, scan_q, scan_ring;
     int total;
     bool stage_bt;   // the block-table row is copied before the wait (blocks that wait for the scan anyway)
 };
@@ -56,9 +57,12 @@ struct StepParams {
     const int32_t *block_table, *seq_lens;
     int32_t* routed_pages;
     const float* page_scores;   // nullptr: routed_pages is an input, or (summaries) the scores are computed here
-    const uint16_t* summaries;  // not nullptr: the page scan runs here, by a cluster of the blocks of a KV head's query heads
+    const uint16_t* summaries;  // without page_scores: the page scan runs here, by a cluster of the blocks of a KV head's query heads
+    const uint32_t* bounds;     // not nullptr: page_scores are within page_score_slack() / 2 of the fixed-order ones, see route_mma.cu
     int cluster_shift;          // log2(blocks of a cluster): those of the heads, the first of them, and others that only scan
     int heads_shift;            // log2(heads of a cluster)
+    int scan_per_sm;            // blocks of such a launch that share an SM
+    bool scan_mma;              // scores by MMAs (page_mma.cuh)
     int32_t* flags;             // with summaries: fallback flag of every unit, from which the dense pass makes the list
     int32_t* tickets;           // with summaries: the dense pass's tickets, cleared here
     int n_tickets;
@@ -83,6 +87,7 @@ namespace {
 
 constexpr int kStepPages = 512;   // entries of the page list
 constexpr int kStepList = 256;    // entries of the cut bucket's list
+constexpr int kMaxRouted = 128;   // routed pages of a unit at most
 constexpr int kStepBins = 256;    // histogram bins of the token selection
 // iterative solve: scores and positions of the candidates, weights exchanged inside a warp, the readout
 constexpr int kSolveWords = 3 * VSA_SOLVER_MAX_CANDIDATES + kHeadDim;
@@ -96,8 +101,12 @@ enum : int {
     kCtlMissing,        // tokens the last page lacks, once per time it is routed
     kCtlNp,             // routed pages (when they are an input)
     kCtlLate,           // a tile's copy did not arrive
+    kCtlNext,           // key of the best page that is not routed
     kCtlCut,            // (tokens above the cut bucket << 20) | (tokens inside << 8) | bucket
-    kCtlWords = 16
+    kCtlNear = 16,      // 4 words: bit t, the scores of the pages of rank t and t + 1 are too close to tell (P is 128 at most)
+    kCtlClose = 20,     // pages that have such a neighbour
+    kCtlBound,          // bits of the largest sum |q_i k_i| of the pages (scan by the cluster)
+    kCtlWords = 24
 };
 
 __host__ __device__ constexpr int step_lanes_per_row(int D) { return D / 8; }
@@ -108,8 +117,11 @@ __host__ __device__ constexpr int step_value_stages(int threads, bool solve)
     return solve ? 4 : threads == 128 ? 2 : threads == 256 ? 3 : 0;
 }
 
+// Tiles of 16 summary rows in flight per warp of a scanning block: 8 KB.
+__host__ __device__ constexpr int step_scan_stages(int D) { return D == 64 ? 4 : D == 128 ? 2 : 1; }
+
 inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
-                              int cluster = 0, int heads = 0)
+                              int cluster = 0, int heads = 0, bool mma = false)
 {
     StepLayout s;
     const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
@@ -127,6 +139,7 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.warp_stat = o, o += 2 * 16;
     s.misc = o, o += 16;
     s.win = o, o += (P + 15) & ~15;
+    s.win_key = o, o += (P + 3) & ~3;
     s.loc = o, o += kStepList;
     s.tile_off = o, o += 2 * ((PT + 1) & ~1);
     s.tile_pos = o, o += (PT + 3) & ~3;
@@ -158,7 +171,7 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.scan_ring = s.scan_q + heads * (D / 2);
     if (cluster) {
         const bool ahead = (max_pages + 15) / 16 > cluster * groups;   // more than one round
-        const int scan_end = s.scan_ring + (ahead ? threads * 16 * 4 : 0) - s.work;
+        const int scan_end = s.scan_ring + (mma ? threads * step_scan_stages(D) * (D / 32) * 8 : ahead ? threads * 16 * 4 : 0) - s.work;
         w = scan_end > w ? scan_end : w;
     }
     if (tt > 1 && threads * 16 * lane_words > w) w = threads * 16 * lane_words;
@@ -190,11 +203,82 @@ __device__ __noinline__ void step_pages_exact(const BlockTeam& tm, const float* 
     tm.sync();
 }
 
+// Fixed-order scores of pages, one per group of LPR lanes: the canonical chain and halving tree (complete in every lane).
+template <int LPR>
+__device__ __forceinline__ float page_score(const uint4& q, const uint4& row)
+{
+    float v = chunk_partial_bf16(q, row);
+#pragma unroll
+    for (int off = LPR / 2; off; off >>= 1) v += __shfl_xor_sync(kFullMask, v, off);
+    return v + 0.0f;   // (the sums over more lanes end in +0 for -0)
+}
+
+// All fixed-order scores of the unit's pages into sc[].
+template <int THREADS, int D>
+__device__ __noinline__ void step_rescore_row(const StepParams& p, const int32_t* bt, uint4 qraw, float* sc, int nb, int g)
+{
+    constexpr int LPR = step_lanes_per_row(D), GROUPS = THREADS / LPR, U = 4;
+    const int c = (threadIdx.x & 31) % LPR, grp = threadIdx.x / LPR;
+    const uint8_t* base = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
+    const unsigned page_bytes = (unsigned)(p.geo.n_kv_heads * 2 * D);
+    __syncthreads();   // every thread has read its own part
+#pragma unroll 1
+    for (int l0 = 0; l0 < nb; l0 += U * GROUPS) {
+        int e[U];
+        uint4 row[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int l = l0 + u * GROUPS + grp;
+            e[u] = l < nb ? ld_ca_s32(bt + l) : -1;
+            if (e[u] >= p.geo.pool_pages) e[u] = -1;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) row[u] = ld_nc_16B(base + (unsigned long long)(unsigned)max(e[u], 0) * page_bytes);
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float s = page_score<LPR>(qraw, row[u]);
+            const int l = l0 + u * GROUPS + grp;
+            if (c == 0 && l < nb) sc[l] = e[u] >= 0 ? s : -INFINITY;
+        }
+    }
+    __syncthreads();
+}
+
+// The P-th and the next of the listed pages' scores are too close to tell: the pages from `lowest` on get their fixed-order
+// scores, which then decide.  Pages below it are not among the P best, whatever the rounding (the P-th best score moves by no more than
+// the scores do).
+template <int THREADS, int D>
+__device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_t* bt, uint4 qraw, unsigned long long* list, int m,
+                                               float lowest, int g)
+{
+    constexpr int LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
+    const int c = (threadIdx.x & 31) % LPR, grp = threadIdx.x / LPR, warp = threadIdx.x >> 5;
+    const uint8_t* base = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
+    const unsigned page_bytes = (unsigned)(p.geo.n_kv_heads * 2 * D);
+#pragma unroll 1
+    for (int t0 = 0; t0 + warp * GPW < m; t0 += GROUPS) {
+        const int t = t0 + grp;
+        const unsigned long long e = t < m ? list[t] : 0ull;
+        // (0: a word beside the row; -inf, a page outside the pool, is exact)
+        const float s = e != 0ull ? key_to_float((uint32_t)(e >> 32)) : -INFINITY;
+        const bool near = s != -INFINITY && !(s < lowest);
+        const int phys = near ? ld_ca_s32(bt + (int)~(uint32_t)e) : 0;
+        const uint4 row = ld_nc_16B(base + (unsigned long long)(unsigned)phys * page_bytes);
+        __syncwarp();
+        const float exact = page_score<LPR>(qraw, row);
+        if (c == 0 && s != -INFINITY)   // (key 1: below the rest, -inf included)
+            list[t] = ((unsigned long long)(near ? float_to_key(exact) : 1u) << 32) | (uint32_t)e;
+    }
+    __syncthreads();
+}
+
 // Exact token selection of the R best when the histogram's range is degenerate or its cut bucket crowded: the keys
 // in position order (work[]), then every thread's unselected keys become 0.  Returns the key of the R-th best,
 // which is unselected as well.
 __device__ __noinline__ uint32_t step_tokens_exact(const BlockTeam& tm, uint32_t* own_keys, int n_own, const int32_t* tile_pos,
-                                                   int nt, int lanes, int R, uint32_t* hist, uint32_t* scratch, uint32_t* work)
+                                                   int nt, int lanes, int R, uint32_t* hist, uint32_t* scratch, uint32_t* wred,
+                                                   uint32_t* work)
 {
     const int N = nt * 16;
     const int tpl = lanes == 8 ? 2 : 1, group = tm.tid / lanes, c = tm.tid % lanes, groups = tm.size / lanes;
@@ -208,7 +292,7 @@ __device__ __noinline__ uint32_t step_tokens_exact(const BlockTeam& tm, uint32_t
         if (i >= 0) work[i] = own_keys[o * tm.size + tm.tid];
     }
     tm.sync();
-    const TopkResult r = team_exact_topk_slow(tm, [&](int i) { return work[i]; }, N, R, hist, scratch, scratch + 16, [](int) {});
+    const TopkResult r = team_exact_topk_slow(tm, [&](int i) { return work[i]; }, N, R, hist, scratch, wred, [](int) {});
     for (int o = 0; o < n_own; ++o) {
         const int i = index_of(o);
         if (i < 0) continue;
@@ -280,6 +364,11 @@ __device__ __forceinline__ uint32_t cluster_address(uint32_t addr, int rank)
 __device__ __forceinline__ void cluster_store(uint32_t addr, float v)
 {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+__device__ __forceinline__ void cluster_max(uint32_t addr, uint32_t v)
+{
+    asm volatile("red.shared::cluster.max.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 // The page scan of one (sequence, KV head) by the cluster of the blocks of its query heads and their helpers: tiles of 16 summary rows are
@@ -378,6 +467,86 @@ __device__ __forceinline__ void step_scan_pages(const StepParams& p, const int32
     cluster_wait();
 }
 
+// The page scan of one (sequence, KV head) by the cluster of the blocks of its query heads and their helpers: tiles of 16 summary
+// rows are dealt out to the warps of all blocks, scored for all heads of the cluster by MMAs (page_mma.cuh: near ties
+// are settled later), and every head's scores go to the shared memory of its own block, the bound of their rounding to all.
+// Rows come through shared memory, every lane copying what it reads itself: loads into registers need lines of the L1, of
+// which blocks with this much shared memory leave 28 KB.  Ends with the scores of this block's head complete in sc.
+template <int THREADS, int D>
+__device__ __forceinline__ void step_scan_pages_mma(const StepParams& p, const int32_t* bt_s, const uint8_t* qs, uint8_t* ring_base,
+                                                const float* sc, uint32_t* bound, int nb, int g)
+{
+    constexpr int ROW = 2 * D, KC = D / 32, STAGES = step_scan_stages(D), WARPS = THREADS / 32;
+    const Geometry& geo = p.geo;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = lane >> 2, j = lane & 3;
+    cp_async_commit_group();   // (the queries)
+    const int cs = p.cluster_shift, C = 1 << cs, rank = (int)blockIdx.x & (C - 1), heads = 1 << p.heads_shift;
+    // warps of the cluster take tiles in turn, block by block, so that few tiles are spread over all SMs
+    const int n_tiles = (nb + 15) >> 4, first_tile = (warp << cs) + rank, step = WARPS << cs;
+    const uint8_t* base = reinterpret_cast<const uint8_t*>(p.summaries) + (long long)g * ROW + j * 16;
+    const unsigned page_bytes = (unsigned)(geo.n_kv_heads * ROW);
+    uint4* own = reinterpret_cast<uint4*>(ring_base) + warp * (STAGES * 2 * KC * 32) + lane;   // piece i of stage s: own[(s * 2 KC + i) * 32]
+    const uint32_t own_s = (uint32_t)__cvta_generic_to_shared(own);
+    auto page_ok = [&](int e) { return e >= 0 && e < geo.pool_pages; };
+    auto issue = [&](int tile, int stage) {   // rows without a valid page read row 0 of the pool instead (their score becomes -inf)
+        if (tile >= n_tiles) return;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int e = bt_s[tile * 16 + h * 8 + r];   // (entries past the sequence are whatever the table holds)
+            const uint8_t* row = base + (unsigned long long)(unsigned)(page_ok(e) ? e : 0) * page_bytes;
+#pragma unroll
+            for (int i = 0; i < KC; ++i) cp_async_16B(own_s + (uint32_t)((stage * 2 * KC + h * KC + i) * 512), row + 64 * i);
+        }
+    };
+#pragma unroll
+    for (int s = 0; s < STAGES; ++s) {
+        issue(first_tile + s * step, s);
+        cp_async_commit_group();
+    }
+    cp_async_wait_group<STAGES>();   // the queries, asked for before
+    __syncthreads();
+    uint4 q[KC];
+#pragma unroll
+    for (int i = 0; i < KC; ++i) q[i] = r < heads ? *reinterpret_cast<const uint4*>(qs + r * ROW + (j + 4 * i) * 16) : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t sc_s = (uint32_t)__cvta_generic_to_shared(sc);
+    const bool has0 = 2 * j < heads, has1 = 2 * j + 1 < heads;
+    const uint32_t dst0 = has0 ? cluster_address(sc_s, 2 * j) : 0u, dst1 = has1 ? cluster_address(sc_s, 2 * j + 1) : 0u;
+    uint32_t most = 0u;
+    cluster_wait();   // the other blocks of the cluster run
+    int stage = 0;
+#pragma unroll 1
+    for (int tile = first_tile; tile < n_tiles; tile += step) {
+        cp_async_wait_group<STAGES - 1>();
+        PageTile<D> t;
+#pragma unroll
+        for (int i = 0; i < KC; ++i) {
+            t.row[0][i] = own[(stage * 2 * KC + i) * 32];
+            t.row[1][i] = own[(stage * 2 * KC + KC + i) * 32];
+        }
+        float s[4], a[4];
+        t.dot(q, s, a);
+        __syncwarp();
+        issue(tile + STAGES * step, stage);
+        cp_async_commit_group();
+        stage = stage + 1 == STAGES ? 0 : stage + 1;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int l = tile * 16 + h * 8 + r;
+            if (l >= nb) continue;
+            const bool ok = page_ok(bt_s[l]);
+            if (ok) most = max(most, max(__float_as_uint(a[2 * h]), __float_as_uint(a[2 * h + 1])));
+            if (has0) cluster_store(dst0 + 4u * (uint32_t)l, ok ? s[2 * h] : -INFINITY);
+            if (has1) cluster_store(dst1 + 4u * (uint32_t)l, ok ? s[2 * h + 1] : -INFINITY);
+        }
+    }
+    __syncwarp();
+    most = __reduce_max_sync(kFullMask, most);
+    if (lane < heads && most != 0u) cluster_max(cluster_address((uint32_t)__cvta_generic_to_shared(bound), lane), most);
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+}
+
 __device__ __noinline__ void step_failed_unit(const BlockTeam& tm, const StepParams& p, long long unit, int status, int D,
                                               bool routed_too)
 {
@@ -450,6 +619,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     constexpr bool BULK = THREADS == 128;   // key tiles by bulk copies
+    constexpr bool CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED >= 3;
     constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
     static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
     static_assert(SOLVE == 0 || (THREADS == 256 && D == 128 && !FP8), "the solve maps one candidate to each of 256 lanes");
@@ -465,6 +635,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     unsigned long long* pages = reinterpret_cast<unsigned long long*>(smem + lay.list);
     unsigned long long* tokens = reinterpret_cast<unsigned long long*>(smem + lay.tokens);
     int32_t* win = (int32_t*)(smem + lay.win);
+    uint32_t* win_key = smem + lay.win_key;   // key of the page with that rank
     long long* tile_off = reinterpret_cast<long long*>(smem + lay.tile_off);   // element offset of a tile's first row, -1 = none
     int32_t* tile_pos = (int32_t*)(smem + lay.tile_pos);                       // its first token's position
     int32_t* tile_phys = (int32_t*)(smem + lay.tile_phys);                     // its pool page
@@ -475,7 +646,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     int32_t* bt_s = (int32_t*)(smem + lay.bt);
     const int lane = tid & 31, warp = tid >> 5, c = lane % LPR, grp = tid / LPR;
     int h = blockIdx.x, helper = 0;
-    if constexpr (FUSED == 2) {   // (a helper: the first head of its cluster)
+    if constexpr (CLUSTER) {   // (a helper: the first head of its cluster)
         helper = (h & ((1 << p.cluster_shift) - 1)) >> p.heads_shift;
         h = ((h >> p.cluster_shift) << p.heads_shift) + (helper ? 0 : h & ((1 << p.heads_shift) - 1));
     }
@@ -487,7 +658,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     // that precedes this one in a step has read both), the block-table row and cleared counters
     const int T = ld_ca_s32(p.seq_lens + b);
     uint4 qraw;
-    if constexpr (FUSED != 2) qraw = ld_nc_16B(p.q + unit * D + c * 8);
+    if constexpr (!CLUSTER) qraw = ld_nc_16B(p.q + unit * D + c * 8);
     if (FUSED && lay.stage_bt) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(bt_s);
         for (int i = tid; i < geo.max_pages; i += THREADS) cp_async_4(dst + 4u * (uint32_t)i, bt + i);
@@ -503,16 +674,16 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int r_warp = (P + WARPS - 1) / WARPS;
-    if constexpr (FUSED == 2) {
+    if constexpr (CLUSTER) {
         cluster_arrive();
         cp_async_wait_all();
         __syncthreads();
     }
     pdl_wait();
     pdl_launch_dependents();
-    if (FUSED == 2 && tid == 0 && unit < p.n_tickets) p.tickets[unit] = 0;
+    if (CLUSTER && tid == 0 && unit < p.n_tickets) p.tickets[unit] = 0;
     if (!length_ok) {
-        if constexpr (FUSED == 2) cluster_wait();
+        if constexpr (CLUSTER) cluster_wait();
         if (helper) return;
         cp_async_wait_all();
         step_failed_unit(tm, p, unit, VSA_UNIT_BAD_LENGTH, D, FUSED);
@@ -533,38 +704,50 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     };
 
     int np;
+    float slack = 0.0f;   // page scores further apart than this are in the order of the fixed-order ones (0: they are those)
     if constexpr (FUSED) {
         // ---- stage the scores of the sequence's pages, four to a chunk; a thread only reads back what it copied.
         //      Short rows spread over the warps (all of them have to vouch for r_warp scores) ----
-        const float* row = FUSED == 1 ? p.page_scores + unit * geo.max_pages : nullptr;
-        const int mis = FUSED == 1 ? (int)((unit * geo.max_pages) & 3) : 0, n_chunks = (nb + mis + 3) >> 2;
+        const float* row = !CLUSTER ? p.page_scores + unit * geo.max_pages : nullptr;
+        const int mis = !CLUSTER ? (int)((unit * geo.max_pages) & 3) : 0, n_chunks = (nb + mis + 3) >> 2;
         const bool single = n_chunks <= THREADS;   // a chunk per thread at most: it stays in registers
         const int chunk0 = single ? lane * WARPS + warp : tid, l0 = 4 * chunk0 - mis;
         float* sc = reinterpret_cast<float*>(work);
         float4* sc4 = reinterpret_cast<float4*>(sc);
         np = min(P, nb);
         auto in_row = [&](int l) { return (unsigned)l < (unsigned)nb; };
-        if constexpr (FUSED == 2) {
+        if constexpr (CLUSTER) {
             const int heads = 1 << p.heads_shift, first = h & ~(heads - 1);
             const uint8_t* qs = reinterpret_cast<const uint8_t*>(smem + lay.scan_q);
             const uint32_t qs_s = (uint32_t)__cvta_generic_to_shared(qs);
             for (int i = tid; i < heads * (D / 8); i += THREADS)
                 cp_async_16B(qs_s + 16u * (uint32_t)i, p.q + ((long long)b * geo.n_q_heads + first) * D + i * 8);
-            step_scan_pages<THREADS, D>(p, bt_s, qs, reinterpret_cast<const uint8_t*>(smem + lay.scan_ring), sc, nb, g);
+            uint8_t* ring = reinterpret_cast<uint8_t*>(smem + lay.scan_ring);
+            if constexpr (MMA)
+                step_scan_pages_mma<THREADS, D>(p, bt_s, qs, ring, sc, &ctl[kCtlBound], nb, g);
+            else
+                step_scan_pages<THREADS, D>(p, bt_s, qs, ring, sc, nb, g);
             if (helper) return;
             qraw = *reinterpret_cast<const uint4*>(qs + (h - first) * 2 * D + c * 16);
+        }
+        // the bound of the scores' rounding, over the blocks of pages that the sequence has
+        uint32_t bound = FUSED == 4 ? ctl[kCtlBound] : 0u;
+        if constexpr (FUSED == 3) {
+            const int hs = min(p.group_shift, 3), blocks = bound_blocks(nb);
+            const int32_t* from = reinterpret_cast<const int32_t*>(p.bounds) + (long long)(unit >> hs) * bound_blocks(geo.max_pages);
+            for (int i = tid; i < blocks; i += THREADS) bound = max(bound, (uint32_t)ld_cg_s32(from + i));
         }
         float4 own_chunk = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
         // words of the first and the last chunk that are no scores of this row: below or equal to every score
         if (single) {
             if (chunk0 < n_chunks) {
-                const float4 v = FUSED == 1 ? ld_cg_f32x4(row + l0) : sc4[chunk0];
+                const float4 v = !CLUSTER ? ld_cg_f32x4(row + l0) : sc4[chunk0];
                 if (in_row(l0)) own_chunk.x = v.x;
                 if (in_row(l0 + 1)) own_chunk.y = v.y;
                 if (in_row(l0 + 2)) own_chunk.z = v.z;
                 if (in_row(l0 + 3)) own_chunk.w = v.w;
             }
-        } else if constexpr (FUSED == 1) {
+        } else if constexpr (!CLUSTER) {
             const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sc);
             for (int i = chunk0; i < n_chunks; i += THREADS) cp_async_16B(dst + 16u * (uint32_t)i, row - mis + 4 * i);
         }
@@ -594,8 +777,20 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 if (lane == __ffs(holders) - 1) v = 0u;   // remove one holder of the maximum
             }
             if (lane == 0) warp_stat[warp] = thr;   // 0: fewer than r lanes have a score, then every score is listed
+            if constexpr (FUSED == 3) {
+                bound = __reduce_max_sync(kFullMask, bound);
+                if (lane == 0) smem[lay.misc + warp] = bound;
+            }
         }
         __syncthreads();
+        if constexpr (FUSED == 3) {
+#pragma unroll
+            for (int w = 0; w < WARPS; w += 4) {
+                const uint4 x = *reinterpret_cast<const uint4*>(smem + lay.misc + w);
+                bound = max(bound, max(max(x.x, x.y), max(x.z, x.w)));
+            }
+        }
+        if constexpr (MMA) slack = page_score_slack(__uint_as_float(bound));
         // ---- list every score that is not below the smallest of them.  A NaN never is, so whatever the scores are at
         //      least np pages are listed: every lane that a warp vouched for has one (a lane of NaNs vouches with -inf,
         //      which lists everything).  Listed by key, a NaN ranks first, as in the exact selections ----
@@ -606,7 +801,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 const uint4 x = *reinterpret_cast<const uint4*>(warp_stat + w);
                 theta_key = min(theta_key, min(min(x.x, x.y), min(x.z, x.w)));
             }
-            const float theta = theta_key <= 0x007fffffu ? -INFINITY : key_to_float(theta_key);
+            const float theta = theta_key <= 0x007fffffu ? -INFINITY : key_to_float(theta_key) - (MMA ? slack : 0.0f);
             auto entry = [&](float score, int l) { return ((unsigned long long)float_to_key(score) << 32) | (uint32_t)~l; };
             if (single) {
                 const float4 v = own_chunk;
@@ -658,21 +853,43 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         }
         __syncthreads();
         int m = (int)ctl[kCtlPages];
-        if (m > kStepPages) {
+        // (a bound that is no ordinary number, or so large that a sum may overflow: the fixed-order scores of all pages)
+        const bool unbounded = MMA && bound >= 0x7e800000u;
+        if (m > kStepPages || unbounded) {
             if (single && chunk0 < n_chunks) sc4[chunk0] = own_chunk;
+            if constexpr (MMA) {
+                step_rescore_row<THREADS, D>(p, bt, qraw, sc + mis, nb, g);
+                slack = 0.0f;
+            }
             step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, warp_stat, pages, &ctl[kCtlPages]);
             m = np;
         }
         // ---- exact ranks, four lanes per listed page ----
 #pragma unroll 1
-        for (int t0 = 0; t0 < m; t0 += THREADS / 4) {
-            const int t = t0 + (tid >> 2);
-            const unsigned long long e = t < m ? pages[t] : ~0ull;
-            if (t0 + (warp << 3) >= m) break;   // nothing left for this warp
-            const int rank = rank_in_list(pages, m, e, tid & 3);
-            if (t < m && rank < np && (tid & 3) == 0) win[rank] = (int)~(uint32_t)e;
+        while (true) {
+#pragma unroll 1
+            for (int t0 = 0; t0 < m; t0 += THREADS / 4) {
+                const int t = t0 + (tid >> 2);
+                const unsigned long long e = t < m ? pages[t] : ~0ull;
+                if (t0 + (warp << 3) >= m) break;   // nothing left for this warp
+                const int rank = rank_in_list(pages, m, e, tid & 3);
+                if (t < m && rank < np + (MMA ? 1 : 0) && (tid & 3) == 0) {
+                    if (rank < np) {
+                        win[rank] = (int)~(uint32_t)e;
+                        if constexpr (MMA) win_key[rank] = (uint32_t)(e >> 32);
+                    } else if constexpr (MMA) {
+                        ctl[kCtlNext] = (uint32_t)(e >> 32);
+                    }
+                }
+            }
+            __syncthreads();
+            if (!MMA || slack == 0.0f || m <= np) break;
+            const uint32_t next = ctl[kCtlNext];   // (0: no page, but a word beside the row)
+            const float kth = key_to_float(win_key[np - 1]);
+            if (next == 0u || kth - key_to_float(next) > slack) break;
+            step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, g);
+            slack = 0.0f;   // the scores are the fixed-order ones
         }
-        __syncthreads();
         // ---- routed pages by position ----
         for (int t = np + tid; t < P; t += THREADS) p.routed_pages[unit * P + t] = -1;
 #pragma unroll 1
@@ -681,10 +898,24 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             const int t = t0 + (tid >> 2);
             const int l = t < np ? win[t] : 0;
             const int phys = lay.stage_bt ? bt_s[l] : ld_ca_s32(bt + l);
+            // too close to tell from the neighbours in the order by score?  (-inf, a page outside the pool, is exact)
+            bool near = false, close = false;
+            if (MMA && slack != 0.0f && t < np) {
+                const float s = key_to_float(win_key[t]), next = t + 1 < np ? key_to_float(win_key[t + 1]) : -INFINITY,
+                            last = t > 0 ? key_to_float(win_key[t - 1]) : INFINITY;
+                near = next != -INFINITY && !(s - next > slack);
+                close = near || (s != -INFINITY && !(last - s > slack));
+            }
             const int rank = rank_below(win, np, l, tid & 3);
             if (t < np && (tid & 3) == 0) {
                 put_page(rank, l, phys);
                 p.routed_pages[unit * P + t] = l;
+                if (MMA && close) {
+                    if (near) atomicOr(&ctl[kCtlNear + (t >> 5)], 1u << (t & 31));
+                    const uint32_t i = atomicAdd(&ctl[kCtlClose], 1u);
+                    smem[lay.loc + i] = (uint32_t)t;
+                    smem[lay.loc + kMaxRouted + i] = (uint32_t)phys;
+                }
             }
         }
         __syncthreads();
@@ -707,13 +938,45 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         __syncthreads();
         np = (int)ctl[kCtlNp];
     }
+    // The list of routed pages is ordered by score (nothing else depends on that order): pages whose scores are too close to tell
+    // get their fixed-order scores, each by a group of lanes, ...
+    const int n_close = MMA ? (int)ctl[kCtlClose] : 0;
+    auto close_row = [&](int i) {
+        const uint8_t* from = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
+        return ld_nc_16B(from + (unsigned long long)smem[lay.loc + kMaxRouted + min(i, n_close - 1)] * (unsigned)(geo.n_kv_heads * 2 * D));
+    };
+    auto settle_score = [&](int i, const uint4& row) {   // (by all lanes of a warp)
+        const float s = page_score<LPR>(qraw, row);
+        if (c == 0 && i < n_close) win_key[smem[lay.loc + i]] = float_to_key(s);
+    };
+    // ... and, later, their places among the neighbours that are close to one another
+    auto settle_places = [&](int first, int step) {
+        auto near = [&](int x) { return x >= 0 && ((ctl[kCtlNear + (x >> 5)] >> (x & 31)) & 1u); };
+#pragma unroll 1
+        for (int t = first; t < np; t += step) {
+            if (!near(t) && !near(t - 1)) continue;
+            const uint32_t key = win_key[t];
+            const int l = win[t];
+            auto before = [&](int x) { return win_key[x] > key || (win_key[x] == key && win[x] < l); };
+            int at = t;
+            for (int x = t - 1; near(x); --x) at -= !before(x);
+            for (int x = t + 1; near(x - 1); ++x) at += before(x);
+            p.routed_pages[unit * P + at] = l;
+        }
+    };
     if (ctl[kCtlBad]) {
+        for (int i0 = 0; i0 + warp * GPW < n_close; i0 += GROUPS) settle_score(i0 + grp, close_row(i0 + grp));
+        __syncthreads();
+        if (n_close) settle_places(tid, THREADS);
         step_failed_unit(tm, p, unit, VSA_UNIT_BAD_PAGE, D, false);
         return;
     }
     const int n_valid = np * geo.page_size - (int)ctl[kCtlMissing];   // tokens that get a score
     const int nt = np << tsh;                                         // their tiles
     const int rounds = (nt + GROUPS - 1) / GROUPS;
+
+    uint4 first_close;   // asked for ahead of the keys
+    if (warp * GPW < n_close) first_close = close_row(grp);
 
     // ---- token routing: one tile of 16 rows per group of lanes and round ----
     uint32_t a1 = 0u, a2 = 0u, amin = 0xffffffffu;   // best, second best and smallest key of this thread
@@ -773,7 +1036,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                     if constexpr (FP8)
                         rows[t] = ld_nc_8B(src + t * stride);
                     else
-                        rows[t] = FUSED == 2 ? ld_cg_16B(src + t * stride) : ld_nc_16B(src + t * stride);
+                        rows[t] = CLUSTER ? ld_cg_16B(src + t * stride) : ld_nc_16B(src + t * stride);
                 }
             } else if constexpr (BULK) {
                 if (active && !mbar_wait(bar, (uint32_t)(r - 1) & 1u)) ctl[kCtlLate] = 1u;
@@ -817,6 +1080,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             }
         }
     }
+    if (warp * GPW < n_close) {
+        settle_score(grp, first_close);
+#pragma unroll 1
+        for (int i0 = GROUPS; i0 + warp * GPW < n_close; i0 += GROUPS) settle_score(i0 + grp, close_row(i0 + grp));
+    }
     // Largest and smallest key, and a bracket of the bulk of the scores: the smallest of the warps' largest keys and
     // the largest of the warps' smallest (the histogram's range; a few outliers do not stretch it).  All four as
     // maxima, so that lanes 0 .. 3 publish them with one instruction.
@@ -828,6 +1096,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     __syncthreads();
     const uint4 stat = *reinterpret_cast<const uint4*>(ctl + kCtlStat);
     if (BULK && ctl[kCtlLate]) {
+        if (n_close) settle_places(tid, THREADS);
         step_failed_unit(tm, p, unit, VSA_UNIT_COPY_TIMEOUT, D, false);
         return;
     }
@@ -921,7 +1190,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             __syncthreads();
         } else {
             cut = -1;
-            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, work);
+            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, warp_stat, work);
             if (tid == 0) ctl[kCtlOut] = k;
         }
     }
@@ -1136,6 +1405,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
     }
     __syncthreads();
+    constexpr int SETTLER = D / 32 < WARPS - 1 ? D / 32 : 0;   // a warp that has nothing else to do, if there is one
+    if (MMA && n_close && warp == SETTLER) settle_places(lane, 32);
     if (warp >= D / 32 && warp != WARPS - 1) return;
     float Z = 0.0f;
 #pragma unroll
@@ -1166,7 +1437,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         d.fallback = (delta < p.gap_threshold && ns < T) ? 1 : 0;
         d.status = 0;
         p.diag[unit] = d;
-        if (FUSED == 2)
+        if (CLUSTER)
             p.flags[unit] = d.fallback;
         else if (d.fallback)
             p.fallback_list[atomicAdd(p.fallback_count, 1)] = (int32_t)unit;
@@ -1180,12 +1451,12 @@ cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
     size_t smem = (size_t)p.lay.total * 4;
     // a scanning block has an SM of its own (two units of a solve on one SM, which a cluster's blocks otherwise share: one
     // sequence of 4k, four entropic iterations 27.2 against 20.7 us per layer)
-    if (FUSED == 2 && smem < 120 * 1024) smem = 120 * 1024;
+    if ((FUSED == 2 || FUSED == 4) && p.scan_per_sm == 1 && smem < 120 * 1024) smem = 120 * 1024;
     if (smem > 48 * 1024) {
         const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>, attr_done);
         if (e != cudaSuccess) return e;
     }
-    if constexpr (FUSED == 2)
+    if constexpr (FUSED == 2 || FUSED == 4)
         return launch_pdl_cluster(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>,
                                   dim3((unsigned)(p.geo.n_q_heads >> p.heads_shift << p.cluster_shift), (unsigned)p.geo.batch),
                                   dim3(THREADS), 1u << p.cluster_shift, smem, stream, p);
@@ -1198,7 +1469,11 @@ template <int D, bool FP8>
 cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t stream)
 {
     const bool fused = p.page_scores != nullptr;
-    if (p.summaries) return threads == 512 ? launch_step_variant<512, 2, D, FP8>(p, stream) : cudaErrorInvalidValue;
+    if (p.summaries && !fused) {
+        if (threads == 256 && p.scan_mma) return launch_step_variant<256, 4, D, FP8>(p, stream);
+        if (threads != 512) return cudaErrorInvalidValue;
+        return p.scan_mma ? launch_step_variant<512, 4, D, FP8>(p, stream) : launch_step_variant<512, 2, D, FP8>(p, stream);
+    }
     // Five blocks per SM at 96 registers against four at 128, which make a unit 5 - 10 % faster: five
     // where they save a wave of blocks, and from three waves of four on, where units in flight count for more.  Microseconds
     // per layer, four / five, T = 8k.  A wave saved: 32 pages a unit, 640 units 41.6 / 31.9, 704 43.5 / 32.5, 1280 65.4 / 56.0,
@@ -1210,9 +1485,12 @@ cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t st
     // pages a unit: four 1 % faster).
     const long long units = (long long)p.geo.batch * p.geo.n_q_heads, four = 4LL * device_sm_count(), five = 5LL * device_sm_count();
     const bool fits = (size_t)p.lay.total * 4 + 1024 <= (size_t)228 * 1024 / 5;   // (1 KB of each block is the system's)
-    if (threads == 128 && fused && fits &&
-        ((units + five - 1) / five < (units + four - 1) / four || units >= 3 * four))
-        return launch_step_variant<128, 1, D, FP8, 0, 5>(p, stream);
+    const bool five_blocks = fits && ((units + five - 1) / five < (units + four - 1) / four || units >= 3 * four);
+    if (p.bounds) {
+        if (threads != 128) return cudaErrorInvalidValue;
+        return five_blocks ? launch_step_variant<128, 3, D, FP8, 0, 5>(p, stream) : launch_step_variant<128, 3, D, FP8>(p, stream);
+    }
+    if (threads == 128 && fused && five_blocks) return launch_step_variant<128, 1, D, FP8, 0, 5>(p, stream);
 #define VSA_STEP_CASE(T)                                                                    \
     if (threads == T)                                                                       \
         return fused ? launch_step_variant<T, 1, D, FP8>(p, stream)                      \

@@ -164,6 +164,15 @@ cudaError_t launch_route_scan(const Geometry& g, const void* q, const void* summ
                               const int32_t* seq_lens, void* ws, int32_t* zero_word, int32_t* zero_words,
                               int zero_count, cudaStream_t stream, const float* radii = nullptr,
                               float* rad_logical = nullptr);
+// The scan ahead of a step on the tensor cores (route_mma.cu), for the shapes that it is faster for: scores within page_score_slack(A) / 2 of the fixed-order ones, where bounds[batch][virtual KV
+// heads][blocks of kBoundPages pages] receives the bits of the largest A = sum |q_i k_i| of a block's pages and the group's heads.
+constexpr int kBoundPages = 32;
+__host__ __device__ inline int bound_blocks(int max_pages) { return (max_pages + kBoundPages - 1) / kBoundPages; }
+size_t route_bound_bytes(const Geometry& g);
+bool route_mma_wins(const Geometry& g);
+cudaError_t launch_route_mma(const Geometry& g, const void* q, const void* summaries, const int32_t* block_table, const int32_t* seq_lens,
+                             float* scores, uint32_t* bounds, int32_t* zero_word, int32_t* zero_words, int zero_count,
+                             cudaStream_t stream);
 // page_budget (device, per unit, or nullptr): at most that many pages of a unit are routed (two-level
 // routing: the pages that were scored; the rest of the unit's score row is marked)
 cudaError_t launch_route_select(const Geometry& g, const void* ws, const int32_t* seq_lens, int P,
@@ -200,8 +209,11 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
                           const int32_t* unit_count = nullptr, int routed_stride = 0,
                           const void* tl_summaries = nullptr, int P_super = 0, const float* k_scale = nullptr,
                           const float* v_scale = nullptr, const void* scan_summaries = nullptr, int32_t* flags = nullptr,
-                          int32_t* tickets = nullptr);
-// scan_summaries != nullptr (step_scans() of the shape, page_scores nullptr): the kernel scores the pages itself, writes
+                          int32_t* tickets = nullptr, const uint32_t* bounds = nullptr);
+// bounds != nullptr (with page_scores and scan_summaries): the page scores and their bounds are launch_route_mma's
+// (closed form, step_takes_bounds() of the shape).
+bool step_takes_bounds(const Geometry& g, int P);
+// scan_summaries != nullptr and page_scores nullptr (step_scans() of the shape): the kernel scores the pages itself, writes
 // every unit's fallback flag instead of the list and clears the dense pass's tickets.
 bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve);
 // k_scale / v_scale != nullptr: k_cache / v_cache hold e4m3 bytes, value = byte * scale[pool page][KV head]
@@ -239,6 +251,9 @@ int sparse_register_select_max_pages(long long units);
 
 // ---- dense split-K pass -------------------------------------------------------------------------
 size_t dense_workspace_bytes(const Geometry& g);
+// the partial results in a dense workspace: written by the dense pass only, free before it
+void* dense_partials(const Geometry& g, void* ws_dense);
+size_t dense_partials_bytes(const Geometry& g);
 cudaError_t launch_dense(const Geometry& g, const void* q, const void* k_cache, const void* v_cache,
                          const int32_t* block_table, const int32_t* seq_lens, const int32_t* fallback_list,
                          const int32_t* fallback_count, float epsilon, float* out, vsa_diag_t* diag, void* ws,
