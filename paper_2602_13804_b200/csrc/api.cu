@@ -555,8 +555,7 @@ static int decode_step_impl(const vsa_shape_t* shape, const void* q, const void*
     // The scan kernel clears fallback_count and the dense pass's tickets: the step enqueues no memset.  The bounds of scores by
     // MMAs lie in the place of the dense pass's partial results.
     uint32_t* bounds = nullptr;
-    if (!cert && !solve && vsa::step_takes_bounds(g, P) && vsa::route_mma_wins(g) && vsa::route_bound_bytes(g) <= vsa::dense_partials_bytes(g))
-        bounds = (uint32_t*)vsa::dense_partials(g, ws_dense);
+    if (!cert && !solve && vsa::step_takes_bounds(g, P)) bounds = (uint32_t*)vsa::dense_partials(g, ws_dense);
     cudaError_t e = bounds ? vsa::launch_route_mma(g, q, summaries, block_table, seq_lens, (float*)ws, bounds, fallback_count,
                                                    vsa::dense_tickets(ws_dense), vsa::dense_ticket_count(g), st)
                            : vsa::launch_route_scan(g, q, summaries, block_table, seq_lens, ws, fallback_count,

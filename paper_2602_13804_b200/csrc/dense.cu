@@ -284,6 +284,7 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
     // sparse pass, the only kernel it can then overlap, writes.
     pdl_launch_dependents();
     pdl_wait();
+    if (!flags && fallback_count && ld_cg_s32(fallback_count) <= 0) return;   // the usual case: the shortest way
 
     // ---- which heads of which groups are listed? ----
     if (flags) {
@@ -310,7 +311,6 @@ dense_split_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t*
         __syncthreads();
     } else if (fallback_count) {
         const int count = *fallback_count;
-        if (count <= 0) return;
         for (int i = tid; i < n_groups; i += kDenseThreads) sm.group_mask[i] = 0;
         __syncthreads();
         for (int i = tid; i < count; i += kDenseThreads) {

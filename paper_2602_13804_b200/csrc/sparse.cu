@@ -110,7 +110,10 @@ bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve)
            (size_t)(c.per_sm == 2 ? 113 : 227) * 1024;
 }
 
-bool step_takes_bounds(const Geometry& g, int P) { return step_threads(g, P) == 128; }
+bool step_takes_bounds(const Geometry& g, int P)
+{
+    return step_threads(g, P) == 128 && route_mma_wins(g) && route_bound_bytes(g) <= dense_partials_bytes(g);
+}
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)
 {
@@ -160,6 +163,8 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         p.flags = flags;
         p.tickets = tickets;
         p.n_tickets = tickets ? dense_ticket_count(g) : 0;
+        p.by_position = step_by_position(threads, g.head_dim, k_scale != nullptr) || step_takes_bounds(g, P) ||
+                        (step_scans(g, P, K_c, k_scale != nullptr, solve != nullptr) && scan_cluster(g, threads).mma);
         p.group_shift = 0;
         while ((1 << p.group_shift) < g.group) ++p.group_shift;
         p.epsilon = epsilon;

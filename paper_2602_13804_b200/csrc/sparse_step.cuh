@@ -11,8 +11,7 @@
 //   * Page scores are staged in shared memory (16-byte copies, any table width).  In every warp the r-th largest
 //     of the lanes' maxima, r = ceil(P / warps), has r scores at or above it; the smallest of these over the warps
 //     bounds the P-th best score from below and leaves about 1.6 P scores, which are listed and ranked exactly.
-//   * Routed pages are listed by position, so that the heads of a group walk the pages that they share at about
-//     the same time (L1 and L2 hits).  Ties are decided by (key << 32) | ~position.
+//   * Ties are decided by (key << 32) | ~position.
 //   * A warp that scored a tile keeps its keys in shared memory and selects among them; the candidates of all warps
 //     are then compacted into one list, whose value rows are dealt out evenly to the groups of lanes.
 //   * Every score is a chain of mixed-precision FMAs on the packed bf16 words (no unpacking).
@@ -63,6 +62,7 @@ struct StepParams {
     int heads_shift;            // log2(heads of a cluster)
     int scan_per_sm;            // blocks of such a launch that share an SM
     bool scan_mma;              // scores by MMAs (page_mma.cuh)
+    bool by_position;           // pages as an input: the step of this shape has the tiles in the order of positions
     int32_t* flags;             // with summaries: fallback flag of every unit, from which the dense pass makes the list
     int32_t* tickets;           // with summaries: the dense pass's tickets, cleared here
     int n_tickets;
@@ -104,8 +104,7 @@ enum : int {
     kCtlNext,           // key of the best page that is not routed
     kCtlCut,            // (tokens above the cut bucket << 20) | (tokens inside << 8) | bucket
     kCtlNear = 16,      // 4 words: bit t, the scores of the pages of rank t and t + 1 are too close to tell (P is 128 at most)
-    kCtlClose = 20,     // pages that have such a neighbour
-    kCtlBound,          // bits of the largest sum |q_i k_i| of the pages (scan by the cluster)
+    kCtlBound = 20,     // bits of the largest sum |q_i k_i| of the pages (scan by the cluster)
     kCtlWords = 24
 };
 
@@ -119,6 +118,9 @@ __host__ __device__ constexpr int step_value_stages(int threads, bool solve)
 
 // Tiles of 16 summary rows in flight per warp of a scanning block: 8 KB.
 __host__ __device__ constexpr int step_scan_stages(int D) { return D == 64 ? 4 : D == 128 ? 2 : 1; }
+
+// Order of the tiles of a block that selects its pages by fixed-order scores, see BY_POSITION
+__host__ __device__ constexpr bool step_by_position(int threads, int D, bool fp8) { return threads == 256 || (threads == 128 && D >= 128 && !fp8); }
 
 inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
                               int cluster = 0, int heads = 0, bool mma = false)
@@ -139,7 +141,7 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.warp_stat = o, o += 2 * 16;
     s.misc = o, o += 16;
     s.win = o, o += (P + 15) & ~15;
-    s.win_key = o, o += (P + 3) & ~3;
+    s.win_key = o, o += 2 * ((P + 3) & ~3);   // and those of the fixed order, where they are needed
     s.loc = o, o += kStepList;
     s.tile_off = o, o += 2 * ((PT + 1) & ~1);
     s.tile_pos = o, o += (PT + 3) & ~3;
@@ -250,7 +252,7 @@ __device__ __noinline__ void step_rescore_row(const StepParams& p, const int32_t
 // the scores do).
 template <int THREADS, int D>
 __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_t* bt, uint4 qraw, unsigned long long* list, int m,
-                                               float lowest, int g)
+                                               float lowest, int g, uint32_t* ctl)
 {
     constexpr int LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     const int c = (threadIdx.x & 31) % LPR, grp = threadIdx.x / LPR, warp = threadIdx.x >> 5;
@@ -270,6 +272,7 @@ __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_
         if (c == 0 && s != -INFINITY)   // (key 1: below the rest, -inf included)
             list[t] = ((unsigned long long)(near ? float_to_key(exact) : 1u) << 32) | (uint32_t)e;
     }
+    if (threadIdx.x == 0) ctl[kCtlBad] = ctl[kCtlMissing] = 0u;   // the pages are put into their slots anew
     __syncthreads();
 }
 
@@ -278,13 +281,19 @@ __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_
 // which is unselected as well.
 __device__ __noinline__ uint32_t step_tokens_exact(const BlockTeam& tm, uint32_t* own_keys, int n_own, const int32_t* tile_pos,
                                                    int nt, int lanes, int R, uint32_t* hist, uint32_t* scratch, uint32_t* wred,
-                                                   uint32_t* work)
+                                                   uint32_t* work, uint32_t* place)
 {
     const int N = nt * 16;
     const int tpl = lanes == 8 ? 2 : 1, group = tm.tid / lanes, c = tm.tid % lanes, groups = tm.size / lanes;
-    auto index_of = [&](int o) {   // array index of own key o, or -1 (tiles are in position order)
+    for (int t = tm.tid; t < nt; t += tm.size) {   // tiles by position (a page may be listed twice)
+        int at = 0;
+        for (int x = 0; x < nt; ++x) at += (int)((tile_pos[x] < tile_pos[t]) | ((tile_pos[x] == tile_pos[t]) & (x < t)));
+        place[t] = (uint32_t)at;
+    }
+    tm.sync();
+    auto index_of = [&](int o) {   // array index of own key o, or -1
         const int slot = (o / tpl) * groups + group;
-        return slot >= nt || (lanes == 32 && (c & 1)) ? -1 : slot * 16 + (lanes == 8 ? 2 * c + o % 2 : lanes == 32 ? c >> 1 : c);
+        return slot >= nt || (lanes == 32 && (c & 1)) ? -1 : (int)place[slot] * 16 + (lanes == 8 ? 2 * c + o % 2 : lanes == 32 ? c >> 1 : c);
     };
     tm.sync();
     for (int o = 0; o < n_own; ++o) {
@@ -607,8 +616,9 @@ __device__ __forceinline__ int rank_below(const int32_t* win, int n, int l, int 
 
 // THREADS: 512 (one block per SM) when there are no more units than SMs, 256 (two) up to two units per SM, 128
 //   (four, or BLOCKS = five) beyond: a unit is a latency chain, so units in flight count for more than threads per unit.
-// FUSED: the unit's pages are selected here from page_scores (1) or from scores computed here (2: the blocks of a cluster are
-//   the query heads of a KV head, eight at most); otherwise (0) routed_pages is an input.
+// FUSED: the unit's pages are selected here from page_scores (1, by MMAs 3) or from scores computed here (2, by MMAs 4: the blocks of a
+//   cluster are the query heads of a KV head, eight at most); otherwise routed_pages is an input, and its tiles are taken in
+//   the order that it has (0) or by position (5), whichever the step of the shape does, so that both sum in one order.
 // D: head dimension.  A row is spread over D / 8 lanes, 8 elements (16 bytes; fp8: 8 bytes) each, so a warp works
 //   on 4, 2 or 1 tiles of 16 rows at a time.
 // FP8: k / v hold e4m3 bytes with one scale per (pool page, KV head); strides count bytes.  Scores and weights are
@@ -619,7 +629,15 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     constexpr bool BULK = THREADS == 128;   // key tiles by bulk copies
-    constexpr bool CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED >= 3;
+    // The routed pages fill the slots of tiles in the order of their scores or, where a group of lanes has several rounds of tiles as a
+    // rule, of their positions: the heads of a KV head then walk the pages that they share at about the same time.  The latter
+    // takes a phase more.  Microseconds per layer by score / position: 512 threads, batch 1 of 4k 10.8 / 11.2, 4 of 4k 11.8 / 12.1,
+    // 64 pages 4 of 16k 19.5 / 19.2; 256, 8 of 16k 19.2 / 19.0, 64 pages 26.4 / 25.7; 128
+    // threads 64 of 8k 79.4 / 77.2, 32 of 8k with 64 pages 72.7 / 71.1, D = 256 78.8 / 75.9, but rows of 128 bytes D = 64 38.3 / 40.0,
+    // e4m3 29.6 / 30.3.
+    // (Scores by MMAs: by position, since near ties would leave their order open.)
+    constexpr bool SELECT = FUSED != 0 && FUSED != 5, CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED == 3 || FUSED == 4;
+    constexpr bool BY_POSITION = SELECT ? MMA || step_by_position(THREADS, D, FP8) : FUSED == 5;
     constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
     static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
     static_assert(SOLVE == 0 || (THREADS == 256 && D == 128 && !FP8), "the solve maps one candidate to each of 256 lanes");
@@ -636,6 +654,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     unsigned long long* tokens = reinterpret_cast<unsigned long long*>(smem + lay.tokens);
     int32_t* win = (int32_t*)(smem + lay.win);
     uint32_t* win_key = smem + lay.win_key;   // key of the page with that rank
+    int32_t* win_phys = (int32_t*)(smem + lay.loc);   // (until the token selection)
+    uint32_t* settled = win_key + ((p.P + 3) & ~3);
     long long* tile_off = reinterpret_cast<long long*>(smem + lay.tile_off);   // element offset of a tile's first row, -1 = none
     int32_t* tile_pos = (int32_t*)(smem + lay.tile_pos);                       // its first token's position
     int32_t* tile_phys = (int32_t*)(smem + lay.tile_phys);                     // its pool page
@@ -659,13 +679,14 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     const int T = ld_ca_s32(p.seq_lens + b);
     uint4 qraw;
     if constexpr (!CLUSTER) qraw = ld_nc_16B(p.q + unit * D + c * 8);
-    if (FUSED && lay.stage_bt) {
+    if (SELECT && lay.stage_bt) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(bt_s);
         for (int i = tid; i < geo.max_pages; i += THREADS) cp_async_4(dst + 4u * (uint32_t)i, bt + i);
     }
     cp_async_commit_group();
     for (int i = tid; i < lay.zeroed / 4; i += THREADS) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = tid; i < ((P + 15) & ~15); i += THREADS) win[i] = INT_MAX;
+    if (SELECT && BY_POSITION)
+        for (int i = tid; i < ((P + 15) & ~15); i += THREADS) win[i] = INT_MAX;
     const bool length_ok = geo.length_ok(T);
     const int nb = length_ok ? geo.pages_of(T) : 0;
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(smem + lay.bar) + 8u * (uint32_t)grp;   // BULK: of this group of lanes
@@ -686,7 +707,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         if constexpr (CLUSTER) cluster_wait();
         if (helper) return;
         cp_async_wait_all();
-        step_failed_unit(tm, p, unit, VSA_UNIT_BAD_LENGTH, D, FUSED);
+        step_failed_unit(tm, p, unit, VSA_UNIT_BAD_LENGTH, D, SELECT);
         return;
     }
 
@@ -705,7 +726,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
 
     int np;
     float slack = 0.0f;   // page scores further apart than this are in the order of the fixed-order ones (0: they are those)
-    if constexpr (FUSED) {
+    if constexpr (SELECT) {
         // ---- stage the scores of the sequence's pages, four to a chunk; a thread only reads back what it copied.
         //      Short rows spread over the warps (all of them have to vouch for r_warp scores) ----
         const float* row = !CLUSTER ? p.page_scores + unit * geo.max_pages : nullptr;
@@ -864,7 +885,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, warp_stat, pages, &ctl[kCtlPages]);
             m = np;
         }
-        // ---- exact ranks, four lanes per listed page ----
+        // ---- exact ranks, four lanes per listed page; the page of rank t fills slot t ----
+        for (int t = np + tid; t < P; t += THREADS) p.routed_pages[unit * P + t] = -1;
 #pragma unroll 1
         while (true) {
 #pragma unroll 1
@@ -872,10 +894,20 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 const int t = t0 + (tid >> 2);
                 const unsigned long long e = t < m ? pages[t] : ~0ull;
                 if (t0 + (warp << 3) >= m) break;   // nothing left for this warp
+                const int l = (int)~(uint32_t)e;
+                int phys = 0;
+                if constexpr (!BY_POSITION) {
+                    const int at = t < m && l >= 0 ? l : 0;   // (a word beside the row is ranked last)
+                    phys = lay.stage_bt ? bt_s[at] : ld_ca_s32(bt + at);
+                }
                 const int rank = rank_in_list(pages, m, e, tid & 3);
                 if (t < m && rank < np + (MMA ? 1 : 0) && (tid & 3) == 0) {
                     if (rank < np) {
-                        win[rank] = (int)~(uint32_t)e;
+                        if constexpr (!BY_POSITION) {
+                            put_page(rank, l, phys);
+                            p.routed_pages[unit * P + rank] = l;
+                        }
+                        if constexpr (BY_POSITION || MMA) win[rank] = l;
                         if constexpr (MMA) win_key[rank] = (uint32_t)(e >> 32);
                     } else if constexpr (MMA) {
                         ctl[kCtlNext] = (uint32_t)(e >> 32);
@@ -887,38 +919,25 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             const uint32_t next = ctl[kCtlNext];   // (0: no page, but a word beside the row)
             const float kth = key_to_float(win_key[np - 1]);
             if (next == 0u || kth - key_to_float(next) > slack) break;
-            step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, g);
+            step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, g, ctl);
             slack = 0.0f;   // the scores are the fixed-order ones
         }
-        // ---- routed pages by position ----
-        for (int t = np + tid; t < P; t += THREADS) p.routed_pages[unit * P + t] = -1;
+        if constexpr (BY_POSITION) {
 #pragma unroll 1
-        for (int t0 = 0; t0 < np; t0 += THREADS / 4) {
-            if (t0 + (warp << 3) >= np) break;
-            const int t = t0 + (tid >> 2);
-            const int l = t < np ? win[t] : 0;
-            const int phys = lay.stage_bt ? bt_s[l] : ld_ca_s32(bt + l);
-            // too close to tell from the neighbours in the order by score?  (-inf, a page outside the pool, is exact)
-            bool near = false, close = false;
-            if (MMA && slack != 0.0f && t < np) {
-                const float s = key_to_float(win_key[t]), next = t + 1 < np ? key_to_float(win_key[t + 1]) : -INFINITY,
-                            last = t > 0 ? key_to_float(win_key[t - 1]) : INFINITY;
-                near = next != -INFINITY && !(s - next > slack);
-                close = near || (s != -INFINITY && !(last - s > slack));
-            }
-            const int rank = rank_below(win, np, l, tid & 3);
-            if (t < np && (tid & 3) == 0) {
-                put_page(rank, l, phys);
-                p.routed_pages[unit * P + t] = l;
-                if (MMA && close) {
-                    if (near) atomicOr(&ctl[kCtlNear + (t >> 5)], 1u << (t & 31));
-                    const uint32_t i = atomicAdd(&ctl[kCtlClose], 1u);
-                    smem[lay.loc + i] = (uint32_t)t;
-                    smem[lay.loc + kMaxRouted + i] = (uint32_t)phys;
+            for (int t0 = 0; t0 < np; t0 += THREADS / 4) {
+                if (t0 + (warp << 3) >= np) break;
+                const int t = t0 + (tid >> 2);
+                const int l = t < np ? win[t] : 0;
+                const int phys = lay.stage_bt ? bt_s[l] : ld_ca_s32(bt + l);
+                const int slot = rank_below(win, np, l, tid & 3);
+                if (t < np && (tid & 3) == 0) {
+                    put_page(slot, l, phys);
+                    p.routed_pages[unit * P + t] = l;
+                    if constexpr (MMA) win_phys[t] = phys;
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
     } else {
         for (int t = tid; t < P; t += THREADS) {
             const int l = p.routed_pages[unit * P + t];
@@ -929,35 +948,59 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             const int l = win[t];
             if (l == INT_MAX) continue;
             const int phys = ld_ca_s32(bt + l);
-            int rank = 0;
+            int slot = 0;
 #pragma unroll 4
-            for (int j = 0; j < P; ++j) rank += (int)((win[j] < l) | ((win[j] == l) & (j < t)));
-            put_page(rank, l, phys);
+            for (int j = 0; j < P; ++j) slot += BY_POSITION ? (int)((win[j] < l) | ((win[j] == l) & (j < t))) : (int)((j < t) & (win[j] != INT_MAX));
+            put_page(slot, l, phys);
             atomicAdd(&ctl[kCtlNp], 1u);
         }
         __syncthreads();
         np = (int)ctl[kCtlNp];
     }
-    // The list of routed pages is ordered by score (nothing else depends on that order): pages whose scores are too close to tell
-    // get their fixed-order scores, each by a group of lanes, ...
-    const int n_close = MMA ? (int)ctl[kCtlClose] : 0;
-    auto close_row = [&](int i) {
-        const uint8_t* from = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
-        return ld_nc_16B(from + (unsigned long long)smem[lay.loc + kMaxRouted + min(i, n_close - 1)] * (unsigned)(geo.n_kv_heads * 2 * D));
+    // The list of routed pages is ordered by score: pages whose scores are too close to tell from a neighbour's get their
+    // fixed-order scores (a warp settles 32 ranks, a group of lanes a page at a time), ...
+    unsigned close = 0u;   // of ranks 32 * warp ...
+    if (MMA && slack != 0.0f && warp * 32 < np) {
+        const int t = warp * 32 + lane;
+        bool near = false, either = false;   // (-inf, a page outside the pool, is exact)
+        if (t < np) {
+            const float s = key_to_float(win_key[t]), next = t + 1 < np ? key_to_float(win_key[t + 1]) : -INFINITY,
+                        last = t > 0 ? key_to_float(win_key[t - 1]) : INFINITY;
+            near = next != -INFINITY && !(s - next > slack);
+            either = near || (s != -INFINITY && !(last - s > slack));
+        }
+        const unsigned word = __ballot_sync(kFullMask, near);
+        close = __ballot_sync(kFullMask, either);
+        if (lane == 0) ctl[kCtlNear + warp] = word;
+    }
+    auto next_close = [&] {   // this group of lanes' next one, or -1
+        int t = -1;
+#pragma unroll
+        for (int k = 0; k < GPW; ++k) {
+            if (close && k == lane / LPR) t = warp * 32 + __ffs(close) - 1;
+            close &= close - 1u;
+        }
+        return t;
     };
-    auto settle_score = [&](int i, const uint4& row) {   // (by all lanes of a warp)
+    auto close_row = [&](int t) {
+        const uint8_t* from = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
+        return ld_nc_16B(from + (unsigned long long)(unsigned)(t >= 0 ? (BY_POSITION ? win_phys[t] : tile_phys[t << tsh]) : 0) * (unsigned)(geo.n_kv_heads * 2 * D));
+    };
+    auto settle_score = [&](int t, const uint4& row) {   // (by all lanes of a warp)
         const float s = page_score<LPR>(qraw, row);
-        if (c == 0 && i < n_close) win_key[smem[lay.loc + i]] = float_to_key(s);
+        if (c == 0 && t >= 0) settled[t] = float_to_key(s);
     };
     // ... and, later, their places among the neighbours that are close to one another
     auto settle_places = [&](int first, int step) {
+        const uint4 words = *reinterpret_cast<const uint4*>(ctl + kCtlNear);
+        if (!(words.x | words.y | words.z | words.w)) return;
         auto near = [&](int x) { return x >= 0 && ((ctl[kCtlNear + (x >> 5)] >> (x & 31)) & 1u); };
 #pragma unroll 1
         for (int t = first; t < np; t += step) {
             if (!near(t) && !near(t - 1)) continue;
-            const uint32_t key = win_key[t];
+            const uint32_t key = settled[t];
             const int l = win[t];
-            auto before = [&](int x) { return win_key[x] > key || (win_key[x] == key && win[x] < l); };
+            auto before = [&](int x) { return settled[x] > key || (settled[x] == key && win[x] < l); };
             int at = t;
             for (int x = t - 1; near(x); --x) at -= !before(x);
             for (int x = t + 1; near(x - 1); ++x) at += before(x);
@@ -965,9 +1008,14 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         }
     };
     if (ctl[kCtlBad]) {
-        for (int i0 = 0; i0 + warp * GPW < n_close; i0 += GROUPS) settle_score(i0 + grp, close_row(i0 + grp));
-        __syncthreads();
-        if (n_close) settle_places(tid, THREADS);
+        if constexpr (MMA) {
+            while (close) {
+                const int t = next_close();
+                settle_score(t, close_row(t));
+            }
+            __syncthreads();
+            settle_places(tid, THREADS);
+        }
         step_failed_unit(tm, p, unit, VSA_UNIT_BAD_PAGE, D, false);
         return;
     }
@@ -976,7 +1024,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     const int rounds = (nt + GROUPS - 1) / GROUPS;
 
     uint4 first_close;   // asked for ahead of the keys
-    if (warp * GPW < n_close) first_close = close_row(grp);
+    int first_t = -1;
+    if (MMA && close) {
+        first_t = next_close();
+        first_close = close_row(first_t);
+    }
 
     // ---- token routing: one tile of 16 rows per group of lanes and round ----
     uint32_t a1 = 0u, a2 = 0u, amin = 0xffffffffu;   // best, second best and smallest key of this thread
@@ -1080,10 +1132,13 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             }
         }
     }
-    if (warp * GPW < n_close) {
-        settle_score(grp, first_close);
+    if (MMA && __any_sync(kFullMask, first_t >= 0)) {
+        settle_score(first_t, first_close);
 #pragma unroll 1
-        for (int i0 = GROUPS; i0 + warp * GPW < n_close; i0 += GROUPS) settle_score(i0 + grp, close_row(i0 + grp));
+        while (close) {
+            const int t = next_close();
+            settle_score(t, close_row(t));
+        }
     }
     // Largest and smallest key, and a bracket of the bulk of the scores: the smallest of the warps' largest keys and
     // the largest of the warps' smallest (the histogram's range; a few outliers do not stretch it).  All four as
@@ -1096,7 +1151,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     __syncthreads();
     const uint4 stat = *reinterpret_cast<const uint4*>(ctl + kCtlStat);
     if (BULK && ctl[kCtlLate]) {
-        if (n_close) settle_places(tid, THREADS);
+        if (MMA) settle_places(tid, THREADS);
         step_failed_unit(tm, p, unit, VSA_UNIT_COPY_TIMEOUT, D, false);
         return;
     }
@@ -1166,8 +1221,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 const uint32_t key = own[o * THREADS];
                 if (key != 0u && bucket_of(key) == cut) {
                     const int slot = (o / TPL) * GROUPS + grp;
-                    // (tiles are in position order; a page that the caller lists twice has tiles of its own)
-                    const int order = slot * 16 + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
+                    // by position; a page that the caller lists twice has tiles of its own
+                    const int order = (tile_pos[slot] >> 4 << 11) + slot * 16 + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
                     const uint32_t i = atomicAdd(&ctl[kCtlTokens], 1u);
                     tokens[i] = ((unsigned long long)key << 32) | (uint32_t)~order;
                     loc[i] = (uint32_t)(o * THREADS + tid);
@@ -1190,7 +1245,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             __syncthreads();
         } else {
             cut = -1;
-            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, warp_stat, work);
+            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, warp_stat, work, smem + lay.loc);
             if (tid == 0) ctl[kCtlOut] = k;
         }
     }
@@ -1406,7 +1461,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     }
     __syncthreads();
     constexpr int SETTLER = D / 32 < WARPS - 1 ? D / 32 : 0;   // a warp that has nothing else to do, if there is one
-    if (MMA && n_close && warp == SETTLER) settle_places(lane, 32);
+    if (MMA && warp == SETTLER) settle_places(lane, 32);
     if (warp >= D / 32 && warp != WARPS - 1) return;
     float Z = 0.0f;
 #pragma unroll
@@ -1492,9 +1547,12 @@ cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t st
     }
     if (threads == 128 && fused && five_blocks) return launch_step_variant<128, 1, D, FP8, 0, 5>(p, stream);
 #define VSA_STEP_CASE(T)                                                                    \
-    if (threads == T)                                                                       \
-        return fused ? launch_step_variant<T, 1, D, FP8>(p, stream)                      \
-                     : launch_step_variant<T, 0, D, FP8>(p, stream);
+    if (threads == T) {                                                                     \
+        if (fused) return launch_step_variant<T, 1, D, FP8>(p, stream);                     \
+        if constexpr (!step_by_position(T, D, FP8))                                         \
+            if (!p.by_position) return launch_step_variant<T, 0, D, FP8>(p, stream);        \
+        return launch_step_variant<T, 5, D, FP8>(p, stream);                                \
+    }
     VSA_STEP_CASE(512)
     VSA_STEP_CASE(256)
     VSA_STEP_CASE(128)
