@@ -120,7 +120,7 @@ __host__ __device__ constexpr int step_value_stages(int threads, bool solve)
 __host__ __device__ constexpr int step_scan_stages(int D) { return D == 64 ? 4 : D == 128 ? 2 : 1; }
 
 // Order of the tiles of a block that selects its pages by fixed-order scores, see BY_POSITION
-__host__ __device__ constexpr bool step_by_position(int threads, int D, bool fp8) { return fp8 ? threads >= 256 : threads == 256 || (threads == 128 && D >= 128); }
+__host__ __device__ constexpr bool step_by_position(int threads, int D, bool fp8) { return fp8 || threads == 256 || (threads == 128 && D >= 128); }
 
 inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
                               int cluster = 0, int heads = 0, bool mma = false)
@@ -633,8 +633,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     // rule, of their positions: the heads of a KV head then walk the pages that they share at about the same time.  The latter
     // takes a phase more.  Microseconds per layer by score / position: 512 threads, batch 1 of 4k 10.8 / 11.2, 4 of 4k 11.8 / 12.1,
     // 64 pages 4 of 16k 19.5 / 19.2; 256, 8 of 16k 19.2 / 19.0, 64 pages 26.4 / 25.7; 128
-    // threads 64 of 8k 79.4 / 77.2, 32 of 8k with 64 pages 72.7 / 71.1, D = 256 78.8 / 75.9, but rows of 128 bytes D = 64 38.3 / 40.0,
-    // e4m3 29.6 / 30.3 (512 threads 4 of 16k 14.3 / 14.1).
+    // threads 64 of 8k 79.4 / 77.2, 32 of 8k with 64 pages 72.7 / 71.1, D = 256 78.8 / 75.9, but rows of 128 bytes D = 64 38.3 / 40.0.
+    // e4m3 16 of 16k 29.6 / 30.3, but 4 of 16k 14.3 / 14.1 and sixteen heads of one KV head, 19 of 3k, 41.8 / 40.9.
     // (Scores by MMAs: by position, since near ties would leave their order open.)
     constexpr bool SELECT = FUSED != 0 && FUSED != 5, CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED == 3 || FUSED == 4;
     constexpr bool BY_POSITION = SELECT ? MMA || step_by_position(THREADS, D, FP8) : FUSED == 5;
