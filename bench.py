@@ -242,8 +242,9 @@ def oracle_layer_time(w, reps_budget_s: float = 12.0, dense: bool = False, input
     return t_total / reps, reps, oracle.num_threads()
 
 
-def algorithmic_bytes(spec, seq_lens, routed_pages=None, cand_pos=None, fallback=None):
+def algorithmic_bytes(spec, seq_lens, routed_pages=None, cand_pos=None, fallback=None, scan_inside=False):
     """Bytes one launch of each kernel has to move for this layer ("algorithmic bytes").
+    With scan_inside the sparse kernel scores the pages itself: its bytes include the scan's, q once.
 
     scan:   every owned page's summary row of every KV head + its block-table entry + q.
     sparse: per (sequence, KV head) the UNION over the group's query heads of the routed pages x 4 KB
@@ -275,6 +276,11 @@ def algorithmic_bytes(spec, seq_lens, routed_pages=None, cand_pos=None, fallback
                 rows += np.unique(c[c >= 0]).size
         out["sparse_decode"] = pages * spec.page_size * row + rows * row + units * (row + 2 * row)
         out["sparse_union_pages"], out["sparse_union_rows"] = int(pages), int(rows)
+    if scan_inside:
+        scan = out.pop("route_scan") - units * row
+        for k in ("sparse_decode_per_head_model", "sparse_decode"):
+            if k in out:
+                out[k] += scan
     if fallback is not None:
         fb = np.asarray(fallback).reshape(B, Hkv, G).any(axis=2)
         out["dense_fallback"] = int((fb * sl[:, None]).sum()) * 2 * row
@@ -482,7 +488,8 @@ class Harness:
         """us per launch of each kernel: event intervals around the kernels of the same launch sequence
         (vsa_decode_step_timed).  The interval between two event records holds the kernel plus the cost of
         the records themselves; the second slot of the timed step brackets no kernel (the page selection
-        is fused into the sparse kernel) and reads that cost, which is reported, not subtracted."""
+        is fused into the sparse kernel) and reads that cost, which is reported, not subtracted.  Where the sparse
+        kernel also scans the pages the first slot brackets none either and is left out."""
         import numpy as np
         torch, B, shape = self.torch, self.B, self.shape
         L = self.L
@@ -512,8 +519,16 @@ class Harness:
                 self.stream.synchronize()
                 for row in evs:
                     acc += np.array([row[j].elapsed_time(row[j + 1]) for j in range(4)])
-        return dict(zip(["route_scan", "event_pair_overhead", "sparse_decode", "dense_fallback"],
-                        (acc / (n_rep * L) * 1e3).tolist()))    # us per launch
+        us = dict(zip(["route_scan", "event_pair_overhead", "sparse_decode", "dense_fallback"],
+                      (acc / (n_rep * L) * 1e3).tolist()))    # us per launch
+        if self.scan_inside():
+            del us["route_scan"]
+        return us
+
+    def scan_inside(self, step=None):
+        """Whether the sparse kernel of the step scans the pages itself (two launches a layer instead of three)."""
+        B = self.B
+        return B.vsa_step_scan(self.shape, self.P, self.K_c, B.VSA_STEP_CLOSED if step is None else step) >= B.VSA_STEP_SCAN_INSIDE
 
     def fallback_units(self):
         n = int(self.fcount.item())
@@ -572,7 +587,7 @@ def measure_point(spec, dev, steps, want_kernels=True, use_graph=True, oracle_se
         st = oracle.decode_step(geo, q, K, V, bt, sl, spec.P, spec.K_c, w0.epsilon, w0.gap_threshold)
         rp, cp = st.route.pages, st.sparse.cand_pos
     sl = h.layers[0].seq_lens.cpu().numpy()
-    alg = algorithmic_bytes(spec, sl, rp, cp, fallback)
+    alg = algorithmic_bytes(spec, sl, rp, cp, fallback, h.scan_inside())
     peak, _ = measured_peak()
     point = {"workload": spec.name, "batch": spec.batch, "context": int(sl.max()), "layers": h.L,
              "distinct_layer_caches": h.distinct, "us_per_layer": us_layer,
@@ -823,11 +838,19 @@ def run_ours(args):
     solve, cert = h.solve, h.cert
     summary_ms = h.summary_ms_per_layer
 
-    kernels_per_layer = 1 if args.dense_baseline else 3   # scan, sparse (top-P selection fused in), dense
-    if cert is not None and args.expand:
-        kernels_per_layer = 3 + vsa_expand_rounds(P, args.expand)
-    if args.two_level:
-        kernels_per_layer = 6     # prep, representative scan, super-page selection, inner scan, sparse, dense
+    # scan, sparse (top-P selection fused in), dense; two where the sparse pass scans the pages itself.  The steps with a
+    # certificate, two-level or group-shared routing always have a scan ahead
+    scan_inside = not args.dense_baseline and h.scan_inside()        # of the closed-form step, whose kernels are timed
+    kernels_per_layer = 3
+    if args.dense_baseline:
+        kernels_per_layer = 1
+    elif cert is not None:
+        kernels_per_layer += vsa_expand_rounds(P, args.expand) if args.expand else 0
+    elif args.two_level:
+        if B.n_super_pages(shape) <= args.two_level and scan_inside:     # every super-page is kept: the plain step
+            kernels_per_layer = 2
+    elif not args.group_shared and h.scan_inside(B.VSA_STEP_SOLVE if solve is not None else None):
+        kernels_per_layer = 2
     use_graph = not args.no_graph
     step = h.capture(use_graph)
 
@@ -974,7 +997,7 @@ def run_ours(args):
     # ---- algorithmic bytes per launch and the roofline fractions ----
     fallback = np.zeros(units, np.int32)
     fallback[fb_units] = 1
-    alg = algorithmic_bytes(spec, sl, rp, cp, fallback)
+    alg = algorithmic_bytes(spec, sl, rp, cp, fallback, scan_inside)
     peak, peak_kind = measured_peak()
     step_us = ms_per_step * 1e3 / L
     if args.dense_baseline:
@@ -984,7 +1007,7 @@ def run_ours(args):
         dom = "dense_fallback"
     else:
         kern = kernel_fracs(alg, per_kernel, step_us, peak)
-        dom = max(("route_scan", "sparse_decode", "dense_fallback"), key=lambda k: per_kernel[k])
+        dom = max((k for k in per_kernel if k != "event_pair_overhead"), key=lambda k: per_kernel[k])
         if solve is not None or cert is not None or args.two_level or args.group_shared:
             # the events bracket the plain step's kernels; the cost of the iterations (of the certificate)
             # is the difference of the two graph-replayed steps and is booked on the sparse kernel
@@ -1001,8 +1024,9 @@ def run_ours(args):
                 "traffic": traffic, "kernel": dom, "bytes_per_launch": d["bytes_per_launch"],
                 "us_per_launch": d["us_per_launch"], "peak_kind": f"of {peak_kind}",
                 "frac_of_8TBps": d["frac_of_8TBps"],
-                "bytes_model": "union over each GQA group of routed K pages and candidate V rows (oracle sets of "
-                               "one layer)" if "sparse_union_pages" in alg else "per kernel, see `kernels`",
+                "bytes_model": ("union over each GQA group of routed K pages and candidate V rows (oracle sets of "
+                                "one layer)" if "sparse_union_pages" in alg else "per kernel, see `kernels`") +
+                               (", and every page summary: the kernel scans the pages itself" if scan_inside else ""),
                 "us_is": "CUDA-event interval around the kernel inside vsa_decode_step_timed; nothing subtracted",
                 "us_event_pair_overhead": per_kernel["event_pair_overhead"] if per_kernel else None,
                 "frac_traffic_based": (traffic / (d["us_per_launch"] * 1e-6) / 1e9 / peak) if traffic else None}
@@ -1041,7 +1065,7 @@ def run_ours(args):
                    "context": int(sl.max()), "P": P, "K_c": K_c, "epsilon": eps, "gap_threshold": tau,
                    "layers_per_step": L, "distinct_layer_caches": distinct,
                    "l2": f"inputs larger than L2: {distinct} distinct layer caches, "
-                         f"{(alg['route_scan'] + alg.get('sparse_decode', alg['sparse_decode_per_head_model'])) * distinct / 1e6:.0f}"
+                         f"{(alg.get('route_scan', 0) + alg.get('sparse_decode', alg['sparse_decode_per_head_model'])) * distinct / 1e6:.0f}"
                          f" MB touched per pass over them",
                    "launch": "cuda graph replay of the whole step" if use_graph else "plain stream launches",
                    "path": "dense split-K baseline" if args.dense_baseline else

@@ -414,7 +414,8 @@ int vsa_decode_step_two_level(const vsa_shape_t* shape, const void* q, const voi
  *   [3] after the fused sparse pass, [4] after the dense fallback pass.
  * The top-P selection runs inside the fused sparse kernel, so the interval [1] -> [2] brackets no
  * kernel: it reads what a pair of event records costs on the stream, which every other interval
- * also contains.
+ * also contains.  Where the fused kernel also scans the pages (vsa_step_scan below) [0] -> [1]
+ * brackets none either, and the scan is part of [2] -> [3].
  */
 int vsa_decode_step_timed(const vsa_shape_t* shape, const void* q, const void* summaries, const void* k_cache,
                           const void* v_cache, const int32_t* block_table, const int32_t* seq_lens, int32_t P,
@@ -535,6 +536,22 @@ int vsa_cp_token_candidates(const vsa_shape_t* shape, const void* q, const void*
 int vsa_cp_partial_readout(const vsa_shape_t* shape, const void* v_cache, const int32_t* block_table,
                            const int32_t* seq_lens, const int32_t* cand_pos, const float* cand_score,
                            int32_t K_c, float epsilon, float* out_partial, float* lse_partial, void* stream);
+
+/*
+ * Where a step scores the pages of a shape on the current device: by a kernel ahead of the fused sparse pass (three
+ * launches a step) or inside it (two), in the fixed order or on the tensor cores with the near ties settled
+ * in the fixed order.  The results do not depend on it.
+ *   step: VSA_STEP_CLOSED for vsa_decode_step, _timed and _host, VSA_STEP_FP8 for vsa_decode_step_fp8,
+ *   VSA_STEP_SOLVE for vsa_decode_step_entropic and _frank_wolfe.  Returns VSA_STEP_SCAN_* or a VSA_ERR_* code.
+ */
+#define VSA_STEP_CLOSED 0
+#define VSA_STEP_FP8 1
+#define VSA_STEP_SOLVE 2
+#define VSA_STEP_SCAN_AHEAD 0
+#define VSA_STEP_SCAN_AHEAD_MMA 1
+#define VSA_STEP_SCAN_INSIDE 2
+#define VSA_STEP_SCAN_INSIDE_MMA 3
+int vsa_step_scan(const vsa_shape_t* shape, int32_t P, int32_t K_c, int step);
 
 /* Scratch bytes needed by one call kind for this shape (0 if the shape is invalid). */
 size_t vsa_workspace_bytes(const vsa_shape_t* shape, int32_t P, int32_t K_c, int which_call);

@@ -18,6 +18,8 @@ LIB_PATH = os.path.join(_HERE, "libvsa.so")
 
 VSA_WS_ROUTE, VSA_WS_SPARSE, VSA_WS_DENSE, VSA_WS_STEP, VSA_WS_STEP_CERTIFIED, VSA_WS_STEP_EXPAND = 1, 2, 3, 4, 5, 6
 VSA_WS_ROUTE_TWO_LEVEL, VSA_WS_STEP_TWO_LEVEL = 7, 8
+VSA_STEP_CLOSED, VSA_STEP_FP8, VSA_STEP_SOLVE = 0, 1, 2
+VSA_STEP_SCAN_AHEAD, VSA_STEP_SCAN_AHEAD_MMA, VSA_STEP_SCAN_INSIDE, VSA_STEP_SCAN_INSIDE_MMA = 0, 1, 2, 3
 VSA_SUPER_PAGES = 16
 DIAG_BYTES = 32
 DIAG_FIELDS = ("delta", "delta12", "s_max", "lse", "leak_bound", "n_candidates", "fallback", "status")
@@ -64,6 +66,8 @@ def lib() -> C.CDLL:
         _lib.vsa_strerror.argtypes = [C.c_int]
         _lib.vsa_workspace_bytes.restype = sz
         _lib.vsa_workspace_bytes.argtypes = [shp, i32, i32, C.c_int]
+        _lib.vsa_step_scan.argtypes = [shp, i32, i32, C.c_int]
+        _lib.vsa_step_scan.restype = C.c_int
         _lib.vsa_build_page_summaries.argtypes = [shp, vp, vp, vp, vp, vp, vp]
         _lib.vsa_route_pages.argtypes = [shp, vp, vp, vp, vp, i32, vp, vp, vp, sz, vp]
         _lib.vsa_decode_step_group_shared.argtypes = [shp, vp, vp, vp, vp, vp, vp, i32, i32, f32, f32, vp, vp, vp, vp,
@@ -154,6 +158,14 @@ def vsa_strerror(code: int) -> str:
 
 def vsa_workspace_bytes(shape: vsa_shape_t, P: int, K_c: int, which_call: int) -> int:
     return int(lib().vsa_workspace_bytes(C.byref(shape), P, K_c, which_call))
+
+
+def vsa_step_scan(shape: vsa_shape_t, P: int, K_c: int, step: int = VSA_STEP_CLOSED) -> int:
+    """Where the step scores the pages: VSA_STEP_SCAN_* (from VSA_STEP_SCAN_INSIDE on a step is two launches, else three)."""
+    rc = int(lib().vsa_step_scan(C.byref(shape), P, K_c, step))
+    if rc < 0:
+        _check(rc, "vsa_step_scan")
+    return rc
 
 
 def vsa_build_page_summaries(shape, k_cache, block_table, seq_lens, first_page, summaries, stream=None) -> None:

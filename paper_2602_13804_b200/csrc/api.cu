@@ -208,6 +208,22 @@ size_t vsa_workspace_bytes(const vsa_shape_t* shape, int32_t P, int32_t K_c, int
     }
 }
 
+int vsa_step_scan(const vsa_shape_t* shape, int32_t P, int32_t K_c, int step)
+{
+    Geometry g;
+    int rc = make_geometry(shape, &g);
+    if (rc) return rc;
+    if ((rc = check_routing_sizes(g, P, K_c, true))) return rc;
+    const bool fp8 = step == VSA_STEP_FP8, solve = step == VSA_STEP_SOLVE;
+    if (!fp8 && !solve && step != VSA_STEP_CLOSED) return VSA_ERR_INVALID_ARGUMENT;
+    if (g.head_dim != vsa::kHeadDim && (fp8 || solve)) return VSA_ERR_UNSUPPORTED_SHAPE;
+    if (solve && (rc = check_solver_sizes(K_c, 0))) return rc;
+    if (!vsa::sparse_shared_memory_fits(g, P, K_c, true, solve, false)) return VSA_ERR_UNSUPPORTED_SHAPE;
+    static_assert((int)vsa::StepScan::Ahead == VSA_STEP_SCAN_AHEAD && (int)vsa::StepScan::AheadMma == VSA_STEP_SCAN_AHEAD_MMA &&
+                  (int)vsa::StepScan::Inside == VSA_STEP_SCAN_INSIDE && (int)vsa::StepScan::InsideMma == VSA_STEP_SCAN_INSIDE_MMA, "one order");
+    return (int)vsa::step_scan(g, P, K_c, fp8, solve);
+}
+
 int vsa_build_page_summaries(const vsa_shape_t* shape, const void* k_cache, const int32_t* block_table,
                              const int32_t* seq_lens, const int32_t* first_page, void* summaries, void* stream)
 {
@@ -539,23 +555,30 @@ static int decode_step_impl(const vsa_shape_t* shape, const void* q, const void*
             ev[i] = (cudaEvent_t)events[i];
         }
     void* ws_dense = (char*)ws + step_route_part(g);
-    if (!events && !cert && vsa::step_scans(g, P, K_c, fp8, solve != nullptr)) {
+    const vsa::StepScan scan = cert ? vsa::StepScan::Ahead : vsa::step_scan(g, P, K_c, fp8, solve != nullptr);
+    if (ev[0] && cudaEventRecord(ev[0], st) != cudaSuccess) return VSA_ERR_CUDA;
+    if (scan == vsa::StepScan::Inside || scan == vsa::StepScan::InsideMma) {
         // two launches: the sparse pass scores the pages itself, and the dense pass makes the list from its flags
         // (in the place of the page scores)
+        for (int i = 1; i < 3; ++i)
+            if (ev[i] && cudaEventRecord(ev[i], st) != cudaSuccess) return VSA_ERR_CUDA;
         int32_t* flags = (int32_t*)ws;
         cudaError_t e = vsa::launch_sparse(g, q, k_cache, v_cache, block_table, seq_lens, routed_pages, nullptr, P, K_c, epsilon,
                                            gap_threshold, out, diag, fallback_list, fallback_count, st, solver_iters, solve, nullptr,
                                            nullptr, solver_kind, nullptr, nullptr, 0, nullptr, 0, k_scale, v_scale, summaries, flags,
                                            vsa::dense_tickets(ws_dense));
         if (e != cudaSuccess) return VSA_ERR_CUDA;
-        return cuda_rc(vsa::launch_dense(g, q, k_cache, v_cache, block_table, seq_lens, fallback_list, fallback_count, epsilon, out,
-                                         diag, ws_dense, st, /*tickets_cleared=*/true, k_scale, v_scale, flags));
+        if (ev[3] && cudaEventRecord(ev[3], st) != cudaSuccess) return VSA_ERR_CUDA;
+        e = vsa::launch_dense(g, q, k_cache, v_cache, block_table, seq_lens, fallback_list, fallback_count, epsilon, out, diag,
+                              ws_dense, st, /*tickets_cleared=*/true, k_scale, v_scale, flags);
+        if (e != cudaSuccess) return VSA_ERR_CUDA;
+        if (ev[4] && cudaEventRecord(ev[4], st) != cudaSuccess) return VSA_ERR_CUDA;
+        return VSA_OK;
     }
-    if (ev[0] && cudaEventRecord(ev[0], st) != cudaSuccess) return VSA_ERR_CUDA;
     // The scan kernel clears fallback_count and the dense pass's tickets: the step enqueues no memset.  The bounds of scores by
     // MMAs lie in the place of the dense pass's partial results.
     uint32_t* bounds = nullptr;
-    if (!cert && !solve && vsa::step_takes_bounds(g, P)) bounds = (uint32_t*)vsa::dense_partials(g, ws_dense);
+    if (scan == vsa::StepScan::AheadMma) bounds = (uint32_t*)vsa::dense_partials(g, ws_dense);
     cudaError_t e = bounds ? vsa::launch_route_mma(g, q, summaries, block_table, seq_lens, (float*)ws, bounds, fallback_count,
                                                    vsa::dense_tickets(ws_dense), vsa::dense_ticket_count(g), st)
                            : vsa::launch_route_scan(g, q, summaries, block_table, seq_lens, ws, fallback_count,

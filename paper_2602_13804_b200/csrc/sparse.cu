@@ -101,18 +101,14 @@ int sparse_block_threads(const Geometry& g, int P, bool listed, bool two_level, 
 
 }  // namespace
 
-bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve)
+StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, bool solve)
 {
     const int threads = solve ? 256 : step_threads(g, P);
     const ScanCluster c = scan_cluster(g, threads);
-    if (!c.blocks || threads < 256) return false;
-    return (size_t)step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, true, fp8, solve, c.blocks, scan_heads(g), c.mma).total * 4 <=
-           (size_t)(c.per_sm == 2 ? 113 : 227) * 1024;
-}
-
-bool step_takes_bounds(const Geometry& g, int P)
-{
-    return step_threads(g, P) == 128 && route_mma_wins(g) && route_bound_bytes(g) <= dense_partials_bytes(g);
+    if (c.blocks && (size_t)step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, true, fp8, solve, c.blocks, scan_heads(g), c.mma).total * 4 <=
+                        (size_t)(c.per_sm == 2 ? 113 : 227) * 1024)
+        return c.mma ? StepScan::InsideMma : StepScan::Inside;
+    return threads == 128 && route_mma_wins(g) && route_bound_bytes(g) <= dense_partials_bytes(g) ? StepScan::AheadMma : StepScan::Ahead;
 }
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)
@@ -163,8 +159,8 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         p.flags = flags;
         p.tickets = tickets;
         p.n_tickets = tickets ? dense_ticket_count(g) : 0;
-        p.by_position = step_by_position(threads, g.head_dim, k_scale != nullptr) || step_takes_bounds(g, P) ||
-                        (step_scans(g, P, K_c, k_scale != nullptr, solve != nullptr) && scan_cluster(g, threads).mma);
+        const StepScan of_step = step_scan(g, P, K_c, k_scale != nullptr, solve != nullptr);
+        p.by_position = step_by_position(threads, g.head_dim, k_scale != nullptr) || of_step == StepScan::AheadMma || of_step == StepScan::InsideMma;
         p.group_shift = 0;
         while ((1 << p.group_shift) < g.group) ++p.group_shift;
         p.epsilon = epsilon;

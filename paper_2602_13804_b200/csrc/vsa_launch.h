@@ -211,11 +211,13 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
                           const float* v_scale = nullptr, const void* scan_summaries = nullptr, int32_t* flags = nullptr,
                           int32_t* tickets = nullptr, const uint32_t* bounds = nullptr);
 // bounds != nullptr (with page_scores and scan_summaries): the page scores and their bounds are launch_route_mma's
-// (closed form, step_takes_bounds() of the shape).
-bool step_takes_bounds(const Geometry& g, int P);
-// scan_summaries != nullptr and page_scores nullptr (step_scans() of the shape): the kernel scores the pages itself, writes
+// (step_scan() AheadMma).
+// scan_summaries != nullptr and page_scores nullptr (step_scan() Inside or InsideMma): the kernel scores the pages itself, writes
 // every unit's fallback flag instead of the list and clears the dense pass's tickets.
-bool step_scans(const Geometry& g, int P, int K_c, bool fp8, bool solve);
+// Where the step of a shape scores its pages: by a kernel ahead of the sparse pass, in the fixed order or by MMAs, or inside it
+// (the values are those of vsa.h's VSA_STEP_SCAN_*)
+enum class StepScan : int { Ahead = 0, AheadMma = 1, Inside = 2, InsideMma = 3 };
+StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, bool solve);
 // k_scale / v_scale != nullptr: k_cache / v_cache hold e4m3 bytes, value = byte * scale[pool page][KV head]
 // (closed-form family, head dimension 128).
 // tl_summaries != nullptr: the two-level front end - page_scores then holds the scores of the super-pages'

@@ -59,6 +59,16 @@ def test_workspace_sizes(lib):
     assert B.vsa_workspace_bytes(s, 32, 256, 77) == 0
 
 
+def test_step_scan_refuses_what_the_steps_refuse(lib):
+    ok = B.make_shape(2, 8, 2, 64, 256)
+    assert lib.vsa_step_scan(C.byref(ok), 16, 64, B.VSA_STEP_CLOSED) >= 0
+    assert lib.vsa_step_scan(None, 16, 64, 0) == -1 and lib.vsa_step_scan(C.byref(ok), 16, 64, 3) == -1
+    assert lib.vsa_step_scan(C.byref(ok), 0, 64, 0) == -1 and lib.vsa_step_scan(C.byref(ok), 4, 65, 0) == -2
+    assert lib.vsa_step_scan(C.byref(ok), 32, 257, B.VSA_STEP_SOLVE) == -2
+    d64 = B.make_shape(2, 8, 2, 64, 256, head_dim=64)
+    assert lib.vsa_step_scan(C.byref(d64), 16, 64, 0) >= 0 and lib.vsa_step_scan(C.byref(d64), 16, 64, B.VSA_STEP_FP8) == -2
+
+
 FAKE = 0x10000   # an aligned non-NULL address that is never dereferenced: validation fails first
 ODD = 0x10008    # not 16-byte aligned
 

@@ -34,6 +34,11 @@ def test_union_bytes_count_each_page_and_row_once_per_group():
     assert a["sparse_decode"] == union_pages * 16 * 256 + union_rows * 256 + units * (256 + 512)
     # scan: one 256-byte summary row per (page, KV head) + a block-table entry per page + q
     assert a["route_scan"] == (7 + 3) * (2 * 256 + 4) + units * 256
+    # a sparse kernel that scans the pages itself: the scan's bytes are its own, q counted once
+    b = bench.algorithmic_bytes(spec, sl, rp, cp, fb, scan_inside=True)
+    scan = a["route_scan"] - units * 256
+    assert "route_scan" not in b and b["sparse_decode"] == a["sparse_decode"] + scan
+    assert b["sparse_decode_per_head_model"] == a["sparse_decode_per_head_model"] + scan
     # dense: K and V rows of every (sequence, KV head) with a flagged head
     assert a["dense_fallback"] == 100 * 2 * 256
     # the paper's per-query-head model books every head's pages and rows
