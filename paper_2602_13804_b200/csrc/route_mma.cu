@@ -117,7 +117,9 @@ mma_list_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* __
                     const int l = t * 16 + h * 8 + r;
                     const bool ok = __shfl_sync(kFullMask, entry, l) >= 0;
                     // (magnitudes are not negative: their order is that of their bits, an infinity or NaN above all)
-                    if (ok) most = max(most, max(__float_as_uint(a[2 * h]), __float_as_uint(a[2 * h + 1])));
+                    uint32_t a0 = __float_as_uint(a[2 * h]), a1 = __float_as_uint(a[2 * h + 1]);
+                    if (max(a0, a1) >= kNoBound) mark_without_bound(s[2 * h], a0), mark_without_bound(s[2 * h + 1], a1);
+                    if (ok) most = max(most, max(a0, a1));
                     if (page + l < end) {
                         if (has0) out[page + l] = ok ? s[2 * h] : -INFINITY;
                         if (has1) out[geo.max_pages + page + l] = ok ? s[2 * h + 1] : -INFINITY;

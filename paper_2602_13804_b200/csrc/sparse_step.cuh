@@ -247,12 +247,12 @@ __device__ __noinline__ void step_rescore_row(const StepParams& p, const int32_t
     __syncthreads();
 }
 
-// The P-th and the next of the listed pages' scores are too close to tell: the pages from `lowest` on get their fixed-order
-// scores, which then decide.  Pages below it are not among the P best, whatever the rounding (the P-th best score moves by no more than
-// the scores do).
+// Fixed-order scores for listed pages.  marks: for those whose score is a mark (page_mma.cuh).  Otherwise the P-th and the next of the
+// scores are too close to tell: the pages from `lowest` on get theirs, which then decide.  Pages below it are not among the P best,
+// whatever the rounding (the P-th best score moves by no more than the scores do).
 template <int THREADS, int D>
 __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_t* bt, uint4 qraw, unsigned long long* list, int m,
-                                               float lowest, int g, uint32_t* ctl)
+                                               float lowest, bool marks, int g, uint32_t* ctl)
 {
     constexpr int LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     const int c = (threadIdx.x & 31) % LPR, grp = threadIdx.x / LPR, warp = threadIdx.x >> 5;
@@ -264,12 +264,12 @@ __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_
         const unsigned long long e = t < m ? list[t] : 0ull;
         // (0: a word beside the row; -inf, a page outside the pool, is exact)
         const float s = e != 0ull ? key_to_float((uint32_t)(e >> 32)) : -INFINITY;
-        const bool near = s != -INFINITY && !(s < lowest);
+        const bool near = marks ? s != s : s != -INFINITY && !(s < lowest);
         const int phys = near ? ld_ca_s32(bt + (int)~(uint32_t)e) : 0;
         const uint4 row = ld_nc_16B(base + (unsigned long long)(unsigned)phys * page_bytes);
         __syncwarp();
         const float exact = page_score<LPR>(qraw, row);
-        if (c == 0 && s != -INFINITY)   // (key 1: below the rest, -inf included)
+        if (c == 0 && (near || (!marks && s != -INFINITY)))   // (key 1: below the rest, -inf included)
             list[t] = ((unsigned long long)(near ? float_to_key(exact) : 1u) << 32) | (uint32_t)e;
     }
     if (threadIdx.x == 0) ctl[kCtlBad] = ctl[kCtlMissing] = 0u;   // the pages are put into their slots anew
@@ -543,7 +543,9 @@ __device__ __forceinline__ void step_scan_pages_mma(const StepParams& p, const i
             const int l = tile * 16 + h * 8 + r;
             if (l >= nb) continue;
             const bool ok = page_ok(bt_s[l]);
-            if (ok) most = max(most, max(__float_as_uint(a[2 * h]), __float_as_uint(a[2 * h + 1])));
+            uint32_t a0 = __float_as_uint(a[2 * h]), a1 = __float_as_uint(a[2 * h + 1]);
+            if (max(a0, a1) >= kNoBound) mark_without_bound(s[2 * h], a0), mark_without_bound(s[2 * h + 1], a1);
+            if (ok) most = max(most, max(a0, a1));
             if (has0) cluster_store(dst0 + 4u * (uint32_t)l, ok ? s[2 * h] : -INFINITY);
             if (has1) cluster_store(dst1 + 4u * (uint32_t)l, ok ? s[2 * h + 1] : -INFINITY);
         }
@@ -874,13 +876,13 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
         }
         __syncthreads();
         int m = (int)ctl[kCtlPages];
-        // (a bound that is no ordinary number, or so large that a sum may overflow: the fixed-order scores of all pages)
-        const bool unbounded = MMA && bound >= 0x7e800000u;
-        if (m > kStepPages || unbounded) {
+        bool marks = MMA;   // pages whose score is a mark may be listed (they always are: NaN is not below theta)
+        if (m > kStepPages) {
             if (single && chunk0 < n_chunks) sc4[chunk0] = own_chunk;
             if constexpr (MMA) {
                 step_rescore_row<THREADS, D>(p, bt, qraw, sc + mis, nb, g);
                 slack = 0.0f;
+                marks = false;
             }
             step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, warp_stat, pages, &ctl[kCtlPages]);
             m = np;
@@ -915,11 +917,20 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 }
             }
             __syncthreads();
-            if (!MMA || slack == 0.0f || m <= np) break;
+            if (!MMA) break;
+            if (marks) {   // they rank first
+                marks = false;
+                const float best = key_to_float(win_key[0]);
+                if (best != best) {
+                    step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, 0.0f, true, g, ctl);
+                    continue;
+                }
+            }
+            if (slack == 0.0f || m <= np) break;
             const uint32_t next = ctl[kCtlNext];   // (0: no page, but a word beside the row)
             const float kth = key_to_float(win_key[np - 1]);
             if (next == 0u || kth - key_to_float(next) > slack) break;
-            step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, g, ctl);
+            step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, false, g, ctl);
             slack = 0.0f;   // the scores are the fixed-order ones
         }
         if constexpr (BY_POSITION) {

@@ -14,11 +14,19 @@ pytestmark = pytest.mark.gpu
 NAN, INF = float("nan"), float("inf")
 
 
-def clean_workload(batch, hq, hkv, P=32, K_c=100, d=128):
+def clean_workload(batch, hq, hkv, P=32, K_c=100, d=128, table=0):
     # sequences 0 - 3 are the ones `poison` spoils; 2 has fewer pages than are routed, 1 and 3 have more
     lens = (2003, 1500, 100, 9001) + tuple(40 + 61 * (i % 19) for i in range(batch - 4))
-    return make_workload(WorkloadSpec(name="nonfinite", config=9, batch=batch, n_q_heads=hq, n_kv_heads=hkv, P=P, K_c=K_c,
-                                      seq_lens=lens, needles=1, head_dim=d), seed=4100 + batch)
+    w = make_workload(WorkloadSpec(name="nonfinite", config=9, batch=batch, n_q_heads=hq, n_kv_heads=hkv, P=P, K_c=K_c,
+                                   seq_lens=lens, needles=1, head_dim=d), seed=4100 + batch)
+    if table:                              # a wider block table, whose width decides where the pages are scored
+        w.block_table = torch.nn.functional.pad(w.block_table, (0, table - w.block_table.shape[1]), value=-1)
+    return w
+
+
+def shape_of(w):
+    from paper_2602_13804_b200 import binding as B
+    return B.shape_of(w.q, w.k_cache, w.block_table)
 
 
 def poison(w):
@@ -73,6 +81,78 @@ def test_step(batch, hq, hkv, P, K_c, d):
         assert np.array_equal(got.step_diag[name][4 * hq:], ref.step_diag[name][4 * hq:]), name
     # the page that holds the NaN key has a NaN score, which ranks first for every head that reads it
     assert (got.step_routed[1, : hq // hkv, 0] == 40).all()
+
+
+@pytest.mark.parametrize("batch,hq,hkv,P,K_c,d,table,scan", [
+    (6, 16, 2, 32, 100, 128, 563, "INSIDE"),           # 512 threads, more rounds than one
+    (5, 4, 1, 32, 100, 64, 563, "INSIDE"),             # with helpers
+    (13, 8, 2, 32, 100, 128, 4096, "INSIDE_MMA"),      # 512 threads
+    (10, 16, 2, 32, 100, 128, 600, "INSIDE_MMA"),      # 256, eight heads
+    (20, 8, 2, 64, 300, 128, 2048, "INSIDE_MMA"),
+    (10, 16, 4, 32, 100, 64, 2040, "INSIDE_MMA"),
+    (38, 4, 1, 32, 300, 256, 2040, "INSIDE_MMA"),
+    (40, 8, 1, 64, 100, 128, 1024, "AHEAD_MMA"),       # 128 threads
+    (150, 8, 1, 32, 100, 64, 1024, "AHEAD_MMA"),       # five blocks of 128 threads per SM
+])
+def test_scans(batch, hq, hkv, P, K_c, d, table, scan):
+    """Every place where a step scores the pages.  Beside the values of `poison`: products that overflow where a sum in another order need
+    not, and sums of such size that cancel, whose pages rank among ordinary ones."""
+    from paper_2602_13804_b200 import binding as B
+    w = clean_workload(batch, hq, hkv, P, K_c, d, table)
+    assert B.vsa_step_scan(shape_of(w), P, K_c) == getattr(B, "VSA_STEP_SCAN_" + scan)
+    ref = run_gpu(w, gap_threshold=-INF)
+    bad = poison(w)
+    bt = bad.block_table
+    bad.q[1, 0, 20:24] = torch.tensor([3e19, 3e19, 2.0, 0.0], dtype=torch.bfloat16)
+    for page, tail in ((3, 1.0), (7, 30.0), (11, -5.0), (60, 1e4)):      # 9e38 - 9e38 (an overflow: NaN or an infinity) + ...
+        bad.k_cache[bt[1, page], 0, :, 20:23] = torch.tensor([3e19, -3e19, tail], dtype=torch.bfloat16)
+    for page, tail in ((4, 1.0), (9, 30.0), (44, 300.0)):                # 9e37 - 9e37 + ...
+        bad.k_cache[bt[1, page], 0, :, 20:23] = torch.tensor([3e18, -3e18, tail], dtype=torch.bfloat16)
+    got = run_gpu(bad, gap_threshold=-INF)
+    check_pages(got.step_routed, w, P)
+    check_pages(got.routed_pages, w, P)
+    assert np.array_equal(got.step_routed, got.routed_pages)
+    for name in ("out", "step_out", "step_routed"):
+        assert np.array_equal(getattr(got, name)[4:], getattr(ref, name)[4:]), name
+    for name in ref.step_diag:
+        assert np.array_equal(got.step_diag[name][4 * hq:], ref.step_diag[name][4 * hq:]), name
+        assert np.array_equal(got.step_diag[name], got.diag[name], equal_nan=True), name
+    assert (got.step_routed[1, 1 : hq // hkv, 0] == 40).all()
+
+
+@pytest.mark.parametrize("batch,hq,hkv,P,table,scan", [
+    (20, 8, 2, 32, 2048, "INSIDE_MMA"), (13, 8, 2, 32, 4096, "INSIDE_MMA"), (40, 8, 1, 64, 1024, "AHEAD_MMA"), (6, 16, 2, 32, 563, "INSIDE"),
+])
+def test_one_nan_key_costs_little(batch, hq, hkv, P, table, scan):
+    """One NaN in every sequence: only the pages that it spoils are scored anew.  (Scoring every page anew took more than twice the
+    time of the step; 1.6 leaves room for the clock of a shared machine.)"""
+    from paper_2602_13804_b200 import SparsePagedDecoder
+    from paper_2602_13804_b200 import binding as B
+    T, dev = table * 16, "cuda:0"
+    gen = torch.Generator(device=dev).manual_seed(3)
+    shape = B.make_shape(batch, hq, hkv, table, table)                   # (all sequences share their pages)
+    assert B.vsa_step_scan(shape, P, 100) == getattr(B, "VSA_STEP_SCAN_" + scan)
+    k = torch.randn((table, hkv, 16, 128), generator=gen, device=dev).bfloat16()
+    bt = torch.arange(table, dtype=torch.int32, device=dev).expand(batch, -1).contiguous()
+    lens = torch.full((batch,), T, dtype=torch.int32, device=dev)
+    q = torch.randn((batch, hq, 128), generator=gen, device=dev).bfloat16()
+    dec = SparsePagedDecoder(shape, P, 100, 11.0, -INF, device=dev)
+    us = []
+    for spoil in (False, True):
+        if spoil:
+            k[5, :, 0, 0] = NAN
+        summ = dec.build_summaries(k, bt, lens)
+        best = INF
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                dec.step(q, summ, k, k, bt, lens)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 50.0)
+        us.append(best)
+    assert us[1] < 1.6 * us[0], us
 
 
 @pytest.mark.parametrize("batch,hq,hkv,P", [(6, 8, 2, 32), (40, 8, 2, 64)])
