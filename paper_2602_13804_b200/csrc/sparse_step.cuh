@@ -235,7 +235,7 @@ __device__ __noinline__ void step_rescore_row(const StepParams& p, const int32_t
             if (e[u] >= p.geo.pool_pages) e[u] = -1;
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) row[u] = ld_nc_16B(base + (unsigned long long)(unsigned)max(e[u], 0) * page_bytes);
+        for (int u = 0; u < U; ++u) row[u] = ld_cg_16B(base + (unsigned long long)(unsigned)max(e[u], 0) * page_bytes);
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -266,7 +266,7 @@ __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_
         const float s = e != 0ull ? key_to_float((uint32_t)(e >> 32)) : -INFINITY;
         const bool near = marks ? s != s : s != -INFINITY && !(s < lowest);
         const int phys = near ? ld_ca_s32(bt + (int)~(uint32_t)e) : 0;
-        const uint4 row = ld_nc_16B(base + (unsigned long long)(unsigned)phys * page_bytes);
+        const uint4 row = ld_cg_16B(base + (unsigned long long)(unsigned)phys * page_bytes);
         __syncwarp();
         const float exact = page_score<LPR>(qraw, row);
         if (c == 0 && (near || (!marks && s != -INFINITY)))   // (key 1: below the rest, -inf included)
@@ -640,6 +640,9 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     // (Scores by MMAs: by position, since near ties would leave their order open.)
     constexpr bool SELECT = FUSED != 0 && FUSED != 5, CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED == 3 || FUSED == 4;
     constexpr bool BY_POSITION = SELECT ? MMA || step_by_position(THREADS, D, FP8) : FUSED == 5;
+    // A scan ahead of this kernel has waited for whatever wrote the cache before this kernel starts.  Without one its blocks may already run
+    // beside the append, and what that writes is not read-only: no ld.global.nc.  (Nothing here writes an e4m3 cache's rows.)
+    constexpr bool BEHIND_SCAN = FUSED == 1 || FUSED == 3;
     constexpr int TPL = LPR == 8 ? 2 : 1;   // tokens of a tile per lane (D = 256: the even lanes own one each)
     static_assert(!FP8 || D == 128, "fp8 cache: head dimension 128");
     static_assert(SOLVE == 0 || (THREADS == 256 && D == 128 && !FP8), "the solve maps one candidate to each of 256 lanes");
@@ -995,7 +998,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     };
     auto close_row = [&](int t) {
         const uint8_t* from = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
-        return ld_nc_16B(from + (unsigned long long)(unsigned)(t >= 0 ? (BY_POSITION ? win_phys[t] : tile_phys[t << tsh]) : 0) * (unsigned)(geo.n_kv_heads * 2 * D));
+        return ld_cg_16B(from + (unsigned long long)(unsigned)(t >= 0 ? (BY_POSITION ? win_phys[t] : tile_phys[t << tsh]) : 0) * (unsigned)(geo.n_kv_heads * 2 * D));
     };
     auto settle_score = [&](int t, const uint4& row) {   // (by all lanes of a warp)
         const float s = page_score<LPR>(qraw, row);
@@ -1099,7 +1102,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                     if constexpr (FP8)
                         rows[t] = ld_nc_8B(src + t * stride);
                     else
-                        rows[t] = CLUSTER ? ld_cg_16B(src + t * stride) : ld_nc_16B(src + t * stride);
+                        rows[t] = BEHIND_SCAN ? ld_nc_16B(src + t * stride) : ld_cg_16B(src + t * stride);
                 }
             } else if constexpr (BULK) {
                 if (active && !mbar_wait(bar, (uint32_t)(r - 1) & 1u)) ctl[kCtlLate] = 1u;
@@ -1413,7 +1416,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                     if constexpr (FP8)
                         rows[t][u] = ld_nc_8B(vbase + row.off * kElem);
                     else
-                        rows[t][u] = ld_nc_16B(vbase + row.off * kElem);
+                        rows[t][u] = BEHIND_SCAN ? ld_nc_16B(vbase + row.off * kElem) : ld_cg_16B(vbase + row.off * kElem);
                 }
             };
 #pragma unroll
