@@ -37,20 +37,28 @@ mma_list_kernel(Geometry geo, const uint16_t* __restrict__ q, const uint16_t* __
         const int T = ld_ca_s32(seq_lens + b);
         return geo.length_ok(T) ? geo.pages_of(T) : 0;
     };
-    if (warp == 0) {
+    // Every warp sums up its own part of the batch (one warp alone takes 0.3 us for 32 sequences), then adds what lies before it.
+    {
+        __shared__ int warp_units[kWarps];
+        const int part = (geo.batch + kThreads - 1) / kThreads * 32, end = min((warp + 1) * part, geo.batch);
         int base = 0;
-        for (int b0 = 0; b0 < geo.batch; b0 += 32) {
-            const int u = b0 + lane < geo.batch ? (pages_in(b0 + lane) + kBlock - 1) / kBlock : 0;
+        for (int b0 = warp * part; b0 < end; b0 += 32) {
+            const int u = b0 + lane < end ? (pages_in(b0 + lane) + kBlock - 1) / kBlock : 0;
             int incl = u;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
                 const int o = __shfl_up_sync(kFullMask, incl, off);
                 if (lane >= off) incl += o;
             }
-            if (b0 + lane < geo.batch) first_unit[b0 + lane] = base + incl - u;
+            if (b0 + lane < end) first_unit[b0 + lane] = base + incl - u;
             base += __shfl_sync(kFullMask, incl, 31);
         }
-        if (lane == 0) first_unit[geo.batch] = base;
+        if (lane == 0) warp_units[warp] = base;
+        __syncthreads();
+        int before = 0;
+        for (int i = 0; i < warp; ++i) before += warp_units[i];
+        for (int i = warp * part + lane; i < end; i += 32) first_unit[i] += before;
+        if (warp == kWarps - 1 && lane == 0) first_unit[geo.batch] = before + base;
     }
     __syncthreads();
     const int n_units = first_unit[geo.batch];
