@@ -30,6 +30,7 @@
 #include <limits.h>
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "page_mma.cuh"
@@ -40,7 +41,7 @@
 
 namespace vsa {
 
-// Shared-memory layout in 4-byte words; every part starts on a 16-byte boundary.
+// Shared-memory layout in 4-byte words, see step_layout.
 struct StepLayout {
     int hist, warp_stat, misc, win_key, list, tokens, zeroed /* words from 0 cleared at the start */, win, loc, tile_off, tile_pos, tile_phys, keys, red, zred, bar, cand, solve, work, vring, bt, scan_q, scan_ring;
     int total;
@@ -122,16 +123,18 @@ __host__ __device__ constexpr int step_scan_stages(int D) { return D == 64 ? 4 :
 // Order of the tiles of a block that selects its pages by fixed-order scores, see BY_POSITION
 __host__ __device__ constexpr bool step_by_position(int threads, int D, bool fp8) { return fp8 || threads == 256 || (threads == 128 && D >= 128); }
 
-inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
-                              int cluster = 0, int heads = 0, bool mma = false)
+// line: words that the parts which rows pass through start on a multiple of
+inline StepLayout step_layout_on(int line, int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
+                              int cluster, int heads, bool mma)
 {
     StepLayout s;
+    auto up = [&](int words) { return (words + line - 1) / line * line; };
     const int groups = threads / step_lanes_per_row(D), warps = threads / 32;
     const int tt = (PT + groups - 1) / groups;   // tiles of a group of lanes
     const int cands = (K_c + 4 * groups - 1) / (4 * groups) * (4 * groups);   // (the value gather takes four rows per group at a time)
     const int lane_words = fp8 ? 2 : 4;          // a lane's piece of a row
     const int keys = tt * groups * 16 * (D == 256 ? 2 : 1);   // [round][sub][thread]
-    int o = kCtlWords;
+    int o = up(kCtlWords);
     s.hist = o, o += kStepBins;
     s.tokens = o, o += 2 * kStepList;
     s.list = o;
@@ -148,11 +151,12 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.tile_phys = o, o += (PT + 3) & ~3;
     s.zred = o, o += (warps + 3) & ~3;
     s.bar = o, o += 2 * groups;
+    o = up(o);
     s.solve = s.cand = s.red = o;
     if (solve) {
-        s.cand = s.solve + kSolveWords;
+        s.cand = up(s.solve + kSolveWords);
         s.red = s.cand + 4 * cands;
-        o = s.red + warps * D;
+        o = up(s.red + warps * D);
     }
     s.work = o;
     // work area: page scores, then the key tiles of the next round (or, in the exact token fallback, the keys in position
@@ -161,16 +165,16 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     s.vring = s.work;
     if (!solve) {
         s.cand = s.work;
-        s.red = s.work + 4 * cands;
-        s.vring = s.red + warps * D;
+        s.red = up(s.work + 4 * cands);
+        s.vring = up(s.red + warps * D);
     }
     const int stages = solve ? cands / (4 * groups) : step_value_stages(threads, false);   // (of a solve: those that K_c needs)
     const int vring_end = s.vring + 4 * stages * threads * lane_words - s.work;
     w = vring_end > w ? vring_end : w;
     if (fused && ((max_pages + 11) & ~3) > w) w = (max_pages + 11) & ~3;
     // page scan: the queries of the cluster's heads and the summary rows of the next round, beside the scores
-    s.scan_q = s.work + ((max_pages + 11) & ~3);
-    s.scan_ring = s.scan_q + heads * (D / 2);
+    s.scan_q = up(s.work + ((max_pages + 11) & ~3));
+    s.scan_ring = up(s.scan_q + heads * (D / 2));
     if (cluster) {
         const bool ahead = (max_pages + 15) / 16 > cluster * groups;   // more than one round
         const int scan_end = s.scan_ring + (mma ? threads * step_scan_stages(D) * (D / 32) * 8 : ahead ? threads * 16 * 4 : 0) - s.work;
@@ -178,13 +182,27 @@ inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, 
     }
     if (tt > 1 && threads * 16 * lane_words > w) w = threads * 16 * lane_words;
     if (solve && ((K_c + 31) & ~31) * 64 > w) w = ((K_c + 31) & ~31) * 64;
-    o += w;
+    o = up(o + w);
     s.bt = o;
     // (not where it would cost the second block of an SM)
     s.stage_bt = fused && (cluster || (threads >= 256 && max_pages <= 8192 && (threads == 512 || o + max_pages <= 113 * 256)));
     if (s.stage_bt) o += (max_pages + 15) & ~15;
     s.total = (o + 3) & ~3;
     return s;
+}
+
+// Rows that pass through shared memory in pieces of 16 bytes (bulk and asynchronous copies, vector loads) start on 128-byte lines.  On
+// 16-byte boundaries, wherever the parts before them ended, microseconds per layer: 160 units of D = 256 with 46 pages 29.6 -> 24.0, 64 sequences of
+// 4k - 128k with eight heads a group 300 -> 293, 1184 units of 3k - 18k with 48 pages 67.5 -> 64.6, 352 of at most 1.3k 56.6 -> 54.7, 32
+// of 8k at D = 64 41.0 -> 40.5, one sequence of 4k with 100 pages 18.7 -> 17.9; with one round of tiles no difference.
+// Where the lines would cost a block on an SM the parts start on 16-byte boundaries.
+inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
+                              int cluster = 0, int heads = 0, bool mma = false)
+{
+    auto on = [&](int line) { return step_layout_on(line, threads, D, max_pages, P, PT, K_c, fused, fp8, solve, cluster, heads, mma); };
+    auto blocks = [&](const StepLayout& s) { return std::min(threads == 128 ? 5 : 512 / threads, 228 * 1024 / (s.total * 4 + 1024)); };
+    const StepLayout lines = on(32), tight = on(4);
+    return blocks(lines) < blocks(tight) ? tight : lines;
 }
 
 // Exact page selection when the list overflows (many equal scores).  Leaves exactly K entries in list[] and
