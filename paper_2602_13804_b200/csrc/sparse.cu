@@ -88,6 +88,14 @@ ScanCluster scan_cluster(const Geometry& g, int threads)
     return threads == 256 && fits(heads, 2) ? ScanCluster{heads, 2, true} : ScanCluster{0, 0, false};
 }
 
+// Order of a unit's tiles, see BY_POSITION (sparse_step.cuh); not a matter of the stream, so that the sums are not.
+bool step_by_position(const Geometry& g, int P, int threads, bool fp8, StepScan rule)
+{
+    if (!step_order_open(threads, g.head_dim, fp8) || rule == StepScan::AheadMma || rule == StepScan::InsideMma) return true;
+    const bool rounds = (P << g.tile_shift) > threads / step_lanes_per_row(g.head_dim);
+    return threads == 512 && rule == StepScan::Ahead && rounds && g.group > 1 && 2LL * g.batch * g.n_q_heads > sm_count();
+}
+
 // thread-block size of the routing variants for a launch
 int sparse_block_threads(const Geometry& g, int P, bool listed, bool two_level, int P_super)
 {
@@ -101,14 +109,52 @@ int sparse_block_threads(const Geometry& g, int P, bool listed, bool two_level, 
 
 }  // namespace
 
+// What a launch of the closed-form family depends on beside its arrays.  selects: the pages are selected from scores, by MMAs with near
+static StepParams step_params(const Geometry& g, int P, int K_c, int threads, bool selects, bool near, bool fp8, bool solve, const ScanCluster& scan)
+{
+    StepParams p = {};
+    p.geo = g;
+    p.P = P;
+    p.K_c = K_c;
+    p.lay = step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, selects, fp8, solve, scan.blocks, scan_heads(g), near);
+    p.scan_per_sm = scan.per_sm;
+    p.scan_mma = scan.mma;
+    while ((1 << p.cluster_shift) < scan.blocks) ++p.cluster_shift;
+    while ((1 << p.heads_shift) < scan_heads(g)) ++p.heads_shift;
+    while ((1 << p.group_shift) < g.group) ++p.group_shift;
+    return p;
+}
+
+static cudaError_t launch_step_of(const StepParams& p, int threads, bool fp8, int solver, cudaStream_t stream)
+{
+    if (solver) return launch_step_solve(p, solver, stream);
+    if (fp8) return launch_step_fp8(p, threads, stream);
+    if (p.geo.head_dim == 64) return launch_step_d64(p, threads, stream);
+    if (p.geo.head_dim == 256) return launch_step_d256(p, threads, stream);
+    return launch_step(p, threads, stream);
+}
+
+// Where the step of a shape scores its pages, and its parameters if that is inside
+struct ScanRule {
+    StepScan scan;
+    StepParams inside;
+};
+
+static ScanRule scan_rule(const Geometry& g, int P, int K_c, int threads, bool fp8, int solver)
+{
+    const ScanCluster c = scan_cluster(g, threads);
+    if (c.blocks) {
+        const StepParams p = step_params(g, P, K_c, threads, true, c.mma, fp8, solver != 0, c);
+        if ((size_t)p.lay.total * 4 <= (size_t)(c.per_sm == 2 ? 113 : 227) * 1024) return {c.mma ? StepScan::InsideMma : StepScan::Inside, p};
+    }
+    const bool mma = threads == 128 && route_mma_wins(g) && route_bound_bytes(g) <= dense_partials_bytes(g) &&
+                     (size_t)step_params(g, P, K_c, threads, true, true, fp8, false, {0, 0, false}).lay.total * 4 <= (size_t)227 * 1024;
+    return {mma ? StepScan::AheadMma : StepScan::Ahead, {}};
+}
+
 StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, bool solve)
 {
-    const int threads = solve ? 256 : step_threads(g, P);
-    const ScanCluster c = scan_cluster(g, threads);
-    if (c.blocks && (size_t)step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, true, fp8, solve, c.blocks, scan_heads(g), c.mma).total * 4 <=
-                        (size_t)(c.per_sm == 2 ? 113 : 227) * 1024)
-        return c.mma ? StepScan::InsideMma : StepScan::Inside;
-    return threads == 128 && route_mma_wins(g) && route_bound_bytes(g) <= dense_partials_bytes(g) ? StepScan::AheadMma : StepScan::Ahead;
+    return scan_rule(g, P, K_c, solve ? 256 : step_threads(g, P), fp8, solve).scan;
 }
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)
@@ -132,8 +178,12 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         return cudaErrorInvalidValue;
     if (g.head_dim != kHeadDim && (solve || cert || tl_summaries)) return cudaErrorInvalidValue;   // (refused by the entry points)
     if (!cert && !tl_summaries) {
-        StepParams p;
-        p.geo = g;
+        const int threads = solve ? 256 : step_threads(g, P), solver = solve ? solver_kind : 0;
+        const bool fp8 = k_scale != nullptr;
+        const ScanRule rule = scan_rule(g, P, K_c, threads, fp8, solver);
+        const bool inside = !page_scores && scan_summaries;
+        StepParams p = inside ? rule.inside
+                              : step_params(g, P, K_c, threads, page_scores != nullptr, bounds != nullptr, fp8, solve != nullptr, {0, 0, false});
         p.q = (const uint16_t*)q;
         p.k = (const uint16_t*)k_cache;
         p.v = (const uint16_t*)v_cache;
@@ -141,28 +191,12 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         p.seq_lens = seq_lens;
         p.routed_pages = routed_pages;
         p.page_scores = page_scores;
-        p.P = P;
-        p.K_c = K_c;
-        const int threads = solve ? 256 : step_threads(g, P);
-        const ScanCluster scan = page_scores || !scan_summaries ? ScanCluster{0, 0, false} : scan_cluster(g, threads);
-        const int cluster = scan.blocks;
-        p.lay = step_layout(threads, g.head_dim, g.max_pages, P, P << g.tile_shift, K_c, page_scores || scan_summaries,
-                            k_scale != nullptr, solve != nullptr, cluster, scan_heads(g), scan.mma);
         p.summaries = (const uint16_t*)scan_summaries;
         p.bounds = bounds;
-        p.scan_per_sm = scan.per_sm;
-        p.scan_mma = scan.mma;
-        p.cluster_shift = 0;
-        while ((1 << p.cluster_shift) < cluster) ++p.cluster_shift;
-        p.heads_shift = 0;
-        while ((1 << p.heads_shift) < scan_heads(g)) ++p.heads_shift;
         p.flags = flags;
         p.tickets = tickets;
         p.n_tickets = tickets ? dense_ticket_count(g) : 0;
-        const StepScan of_step = step_scan(g, P, K_c, k_scale != nullptr, solve != nullptr);
-        p.by_position = step_by_position(threads, g.head_dim, k_scale != nullptr) || of_step == StepScan::AheadMma || of_step == StepScan::InsideMma;
-        p.group_shift = 0;
-        while ((1 << p.group_shift) < g.group) ++p.group_shift;
+        p.by_position = step_by_position(g, P, threads, fp8, rule.scan);
         p.epsilon = epsilon;
         p.gap_threshold = gap_threshold;
         p.out = out;
@@ -173,11 +207,7 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
         p.solve = solve;
         p.k_scale = k_scale;
         p.v_scale = v_scale;
-        if (solve) return launch_step_solve(p, solver_kind, stream);
-        if (k_scale) return launch_step_fp8(p, threads, stream);
-        if (g.head_dim == 64) return launch_step_d64(p, threads, stream);
-        if (g.head_dim == 256) return launch_step_d256(p, threads, stream);
-        return launch_step(p, threads, stream);
+        return launch_step_of(p, threads, fp8, solver, stream);
     }
     SparseArgs a;
     a.g = g;

@@ -15,9 +15,9 @@ cudaError_t launch_step_solve(const StepParams& p, int kind, cudaStream_t stream
     }
     if (kind == 2)
         return fused ? launch_step_variant<256, 1, kHeadDim, false, 2>(p, stream)
-                     : launch_step_variant<256, 5, kHeadDim, false, 2>(p, stream);
+                     : launch_step_variant<256, 0, kHeadDim, false, 2>(p, stream);
     return fused ? launch_step_variant<256, 1, kHeadDim, false, 1>(p, stream)
-                 : launch_step_variant<256, 5, kHeadDim, false, 1>(p, stream);
+                 : launch_step_variant<256, 0, kHeadDim, false, 1>(p, stream);
 }
 
 }  // namespace vsa

@@ -63,7 +63,7 @@ struct StepParams {
     int heads_shift;            // log2(heads of a cluster)
     int scan_per_sm;            // blocks of such a launch that share an SM
     bool scan_mma;              // scores by MMAs (page_mma.cuh)
-    bool by_position;           // pages as an input: the step of this shape has the tiles in the order of positions
+    bool by_position;           // tiles in the order of positions instead of scores (see BY_POSITION)
     int32_t* flags;             // with summaries: fallback flag of every unit, from which the dense pass makes the list
     int32_t* tickets;           // with summaries: the dense pass's tickets, cleared here
     int n_tickets;
@@ -120,12 +120,12 @@ __host__ __device__ constexpr int step_value_stages(int threads, bool solve)
 // Tiles of 16 summary rows in flight per warp of a scanning block: 8 KB.
 __host__ __device__ constexpr int step_scan_stages(int D) { return D == 64 ? 4 : D == 128 ? 2 : 1; }
 
-// Order of the tiles of a block that selects its pages by fixed-order scores, see BY_POSITION
-__host__ __device__ constexpr bool step_by_position(int threads, int D, bool fp8) { return fp8 || threads == 256 || (threads == 128 && D >= 128); }
+// Blocks whose tiles may come in either order, see BY_POSITION
+__host__ __device__ constexpr bool step_order_open(int threads, int D, bool fp8) { return !fp8 && (threads == 512 || (threads == 128 && D == 64)); }
 
-// line: words that the parts which rows pass through start on a multiple of
+// near: page scores by MMAs, whose near ties are settled.  line: words that the parts which rows pass through start on a multiple of
 inline StepLayout step_layout_on(int line, int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
-                              int cluster, int heads, bool mma)
+                              int cluster, int heads, bool near)
 {
     StepLayout s;
     auto up = [&](int words) { return (words + line - 1) / line * line; };
@@ -144,7 +144,7 @@ inline StepLayout step_layout_on(int line, int threads, int D, int max_pages, in
     s.warp_stat = o, o += 2 * 16;
     s.misc = o, o += 16;
     s.win = o, o += (P + 15) & ~15;
-    s.win_key = o, o += 2 * ((P + 3) & ~3);   // and those of the fixed order, where they are needed
+    s.win_key = o, o += near ? 2 * ((P + 3) & ~3) : 0;   // and those of the fixed order, where they are needed
     s.loc = o, o += kStepList;
     s.tile_off = o, o += 2 * ((PT + 1) & ~1);
     s.tile_pos = o, o += (PT + 3) & ~3;
@@ -177,7 +177,7 @@ inline StepLayout step_layout_on(int line, int threads, int D, int max_pages, in
     s.scan_ring = up(s.scan_q + heads * (D / 2));
     if (cluster) {
         const bool ahead = (max_pages + 15) / 16 > cluster * groups;   // more than one round
-        const int scan_end = s.scan_ring + (mma ? threads * step_scan_stages(D) * (D / 32) * 8 : ahead ? threads * 16 * 4 : 0) - s.work;
+        const int scan_end = s.scan_ring + (near ? threads * step_scan_stages(D) * (D / 32) * 8 : ahead ? threads * 16 * 4 : 0) - s.work;
         w = scan_end > w ? scan_end : w;
     }
     if (tt > 1 && threads * 16 * lane_words > w) w = threads * 16 * lane_words;
@@ -197,9 +197,9 @@ inline StepLayout step_layout_on(int line, int threads, int D, int max_pages, in
 // of 8k at D = 64 41.0 -> 40.5, one sequence of 4k with 100 pages 18.7 -> 17.9; with one round of tiles no difference.
 // Where the lines would cost a block on an SM the parts start on 16-byte boundaries.
 inline StepLayout step_layout(int threads, int D, int max_pages, int P, int PT, int K_c, bool fused, bool fp8, bool solve,
-                              int cluster = 0, int heads = 0, bool mma = false)
+                              int cluster = 0, int heads = 0, bool near = false)
 {
-    auto on = [&](int line) { return step_layout_on(line, threads, D, max_pages, P, PT, K_c, fused, fp8, solve, cluster, heads, mma); };
+    auto on = [&](int line) { return step_layout_on(line, threads, D, max_pages, P, PT, K_c, fused, fp8, solve, cluster, heads, near); };
     auto blocks = [&](const StepLayout& s) { return std::min(threads == 128 ? 5 : 512 / threads, 228 * 1024 / (s.total * 4 + 1024)); };
     const StepLayout lines = on(32), tight = on(4);
     return blocks(lines) < blocks(tight) ? tight : lines;
@@ -270,7 +270,7 @@ __device__ __noinline__ void step_rescore_row(const StepParams& p, const int32_t
 // whatever the rounding (the P-th best score moves by no more than the scores do).
 template <int THREADS, int D>
 __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_t* bt, uint4 qraw, unsigned long long* list, int m,
-                                               float lowest, bool marks, int g, uint32_t* ctl)
+                                               float lowest, bool marks, int g)
 {
     constexpr int LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     const int c = (threadIdx.x & 31) % LPR, grp = threadIdx.x / LPR, warp = threadIdx.x >> 5;
@@ -290,7 +290,6 @@ __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_
         if (c == 0 && (near || (!marks && s != -INFINITY)))   // (key 1: below the rest, -inf included)
             list[t] = ((unsigned long long)(near ? float_to_key(exact) : 1u) << 32) | (uint32_t)e;
     }
-    if (threadIdx.x == 0) ctl[kCtlBad] = ctl[kCtlMissing] = 0u;   // the pages are put into their slots anew
     __syncthreads();
 }
 
@@ -299,19 +298,21 @@ __device__ __noinline__ void step_settle_pages(const StepParams& p, const int32_
 // which is unselected as well.
 __device__ __noinline__ uint32_t step_tokens_exact(const BlockTeam& tm, uint32_t* own_keys, int n_own, const int32_t* tile_pos,
                                                    int nt, int lanes, int R, uint32_t* hist, uint32_t* scratch, uint32_t* wred,
-                                                   uint32_t* work, uint32_t* place)
+                                                   uint32_t* work, uint32_t* place)   // place: nullptr where tiles are in position order
 {
     const int N = nt * 16;
     const int tpl = lanes == 8 ? 2 : 1, group = tm.tid / lanes, c = tm.tid % lanes, groups = tm.size / lanes;
-    for (int t = tm.tid; t < nt; t += tm.size) {   // tiles by position (a page may be listed twice)
-        int at = 0;
-        for (int x = 0; x < nt; ++x) at += (int)((tile_pos[x] < tile_pos[t]) | ((tile_pos[x] == tile_pos[t]) & (x < t)));
-        place[t] = (uint32_t)at;
+    if (place) {   // tiles by position (a page may be listed twice)
+        for (int t = tm.tid; t < nt; t += tm.size) {
+            int at = 0;
+            for (int x = 0; x < nt; ++x) at += (int)((tile_pos[x] < tile_pos[t]) | ((tile_pos[x] == tile_pos[t]) & (x < t)));
+            place[t] = (uint32_t)at;
+        }
+        tm.sync();
     }
-    tm.sync();
     auto index_of = [&](int o) {   // array index of own key o, or -1
         const int slot = (o / tpl) * groups + group;
-        return slot >= nt || (lanes == 32 && (c & 1)) ? -1 : (int)place[slot] * 16 + (lanes == 8 ? 2 * c + o % 2 : lanes == 32 ? c >> 1 : c);
+        return slot >= nt || (lanes == 32 && (c & 1)) ? -1 : (place ? (int)place[slot] : slot) * 16 + (lanes == 8 ? 2 * c + o % 2 : lanes == 32 ? c >> 1 : c);
     };
     tm.sync();
     for (int o = 0; o < n_own; ++o) {
@@ -637,27 +638,29 @@ __device__ __forceinline__ int rank_below(const int32_t* win, int n, int l, int 
 // THREADS: 512 (one block per SM) when there are no more units than SMs, 256 (two) up to two units per SM, 128
 //   (four, or BLOCKS = five) beyond: a unit is a latency chain, so units in flight count for more than threads per unit.
 // FUSED: the unit's pages are selected here from page_scores (1, by MMAs 3) or from scores computed here (2, by MMAs 4: the blocks of a
-//   cluster are the query heads of a KV head, eight at most); otherwise routed_pages is an input, and its tiles are taken in
-//   the order that it has (0) or by position (5), whichever the step of the shape does, so that both sum in one order.
+//   cluster are the query heads of a KV head, eight at most); otherwise (0) routed_pages is an input.
+// BY_POSITION: order of the tiles, the same for pages as an input as in the step of the shape, so that both sum in one order.
 // D: head dimension.  A row is spread over D / 8 lanes, 8 elements (16 bytes; fp8: 8 bytes) each, so a warp works
 //   on 4, 2 or 1 tiles of 16 rows at a time.
 // FP8: k / v hold e4m3 bytes with one scale per (pool page, KV head); strides count bytes.  Scores and weights are
 //   multiplied by the scale afterwards (exact for powers of two).
 // SOLVE: the weights come from solver_iters entropic (1) or Frank-Wolfe (2) iterations (step_solve.cuh).
-template <int THREADS, int FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0, int BLOCKS = 512 / THREADS>
+template <int THREADS, int FUSED, int D = kHeadDim, bool FP8 = false, int SOLVE = 0, int BLOCKS = 512 / THREADS, bool BY_POSITION = true>
 __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __grid_constant__ StepParams p)
 {
     constexpr int WARPS = THREADS / 32, LPR = step_lanes_per_row(D), GPW = 32 / LPR, GROUPS = THREADS / LPR;
     constexpr bool BULK = THREADS == 128;   // key tiles by bulk copies
-    // The routed pages fill the slots of tiles in the order of their scores or, where a group of lanes has several rounds of tiles as a
-    // rule, of their positions: the heads of a KV head then walk the pages that they share at about the same time.  The latter
-    // takes a phase more.  Microseconds per layer by score / position: 512 threads, batch 1 of 4k 10.8 / 11.2, 4 of 4k 11.8 / 12.1,
-    // 64 pages 4 of 16k 19.5 / 19.2; 256, 8 of 16k 19.2 / 19.0, 64 pages 26.4 / 25.7; 128
-    // threads 64 of 8k 79.4 / 77.2, 32 of 8k with 64 pages 72.7 / 71.1, D = 256 78.8 / 75.9, but rows of 128 bytes D = 64 38.3 / 40.0.
-    // e4m3 16 of 16k 29.6 / 30.3, but 4 of 16k 14.3 / 14.1 and sixteen heads of one KV head, 19 of 3k, 41.8 / 40.9.
-    // (Scores by MMAs: by position, since near ties would leave their order open.)
-    constexpr bool SELECT = FUSED != 0 && FUSED != 5, CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED == 3 || FUSED == 4;
-    constexpr bool BY_POSITION = SELECT ? MMA || step_by_position(THREADS, D, FP8) : FUSED == 5;
+    // The routed pages fill the slots of tiles in the order of their scores or, in a phase more, of their positions: the heads of a KV head then
+    // walk the pages that they share at about the same time.  Microseconds per layer by score / position.  512 threads behind a scan (the
+    // rule is step_by_position in sparse.cu): one round of tiles 4 of 16k with 32 pages 14.1 / 14.3; more, 4 of 16k 48 pages 16.2 / 15.9, 64
+    // 17.7 / 17.4, D = 256 8 of 8k with two heads a group 26.3 / 25.3, but one head a group, 16 of 16k 23.1 / 23.3, D = 256 16 of 8k 25.9 / 26.3, and few
+    // units, D = 256 one of 8k 15.9 / 16.5.  In a cluster, whose blocks leave the scan together, 4 of 4k 48 pages 14.0 / 14.4, 64 14.7 / 15.1,
+    // one of 4k 100 pages 17.9 / 18.2.  Always by position (on 16-byte boundaries of shared memory): 256 threads 8 of 16k 19.2 / 19.0, 64 pages 26.4 /
+    // 25.7; 128 threads 64 of 8k 79.4 / 77.2, 32 of 8k with 64 pages 72.7 / 71.1, D = 256 78.8 / 75.9; e4m3 16 of 16k 29.6 / 30.3, but 4 of
+    // 16k 14.3 / 14.1 and sixteen heads of one KV head, 19 of 3k, 41.8 / 40.9.  Always by score: 128 threads of D = 64, 32 of 8k 41.5 / 41.9, in 32-token
+    // pages 36.5 / 37.0, but 64 of 8k with 32 pages 68.6 / 67.7.  (Scores by MMAs: by position, since near ties would leave their order open.)
+    constexpr bool SELECT = FUSED != 0, CLUSTER = FUSED == 2 || FUSED == 4, MMA = FUSED == 3 || FUSED == 4;
+    static_assert(BY_POSITION || (!MMA && step_order_open(THREADS, D, FP8)), "by position");
     // A scan ahead of this kernel has waited for whatever wrote the cache before this kernel starts.  Without one its blocks may already run
     // beside the append, and what that writes is not read-only: no ld.global.nc.  (Nothing here writes an e4m3 cache's rows.)
     constexpr bool BEHIND_SCAN = FUSED == 1 || FUSED == 3;
@@ -908,8 +911,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             step_pages_exact(tm, sc + mis, nb, np, hist, smem + lay.misc, warp_stat, pages, &ctl[kCtlPages]);
             m = np;
         }
-        // ---- exact ranks, four lanes per listed page; the page of rank t fills slot t ----
-        for (int t = np + tid; t < P; t += THREADS) p.routed_pages[unit * P + t] = -1;
+        // ---- exact ranks, four lanes per listed page.  By position the pages are put into slots in a phase of their own ----
 #pragma unroll 1
         while (true) {
 #pragma unroll 1
@@ -917,33 +919,33 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 const int t = t0 + (tid >> 2);
                 const unsigned long long e = t < m ? pages[t] : ~0ull;
                 if (t0 + (warp << 3) >= m) break;   // nothing left for this warp
-                const int l = (int)~(uint32_t)e;
-                int phys = 0;
-                if constexpr (!BY_POSITION) {
-                    const int at = t < m && l >= 0 ? l : 0;   // (a word beside the row is ranked last)
-                    phys = lay.stage_bt ? bt_s[at] : ld_ca_s32(bt + at);
-                }
-                const int rank = rank_in_list(pages, m, e, tid & 3);
-                if (t < m && rank < np + (MMA ? 1 : 0) && (tid & 3) == 0) {
-                    if (rank < np) {
-                        if constexpr (!BY_POSITION) {
-                            put_page(rank, l, phys);
-                            p.routed_pages[unit * P + rank] = l;
+                if constexpr (BY_POSITION) {
+                    const int rank = rank_in_list(pages, m, e, tid & 3);
+                    if (t < m && rank < np + (MMA ? 1 : 0) && (tid & 3) == 0) {
+                        if (rank < np) {
+                            win[rank] = (int)~(uint32_t)e;
+                            if constexpr (MMA) win_key[rank] = (uint32_t)(e >> 32);
+                        } else if constexpr (MMA) {
+                            ctl[kCtlNext] = (uint32_t)(e >> 32);
                         }
-                        if constexpr (BY_POSITION || MMA) win[rank] = l;
-                        if constexpr (MMA) win_key[rank] = (uint32_t)(e >> 32);
-                    } else if constexpr (MMA) {
-                        ctl[kCtlNext] = (uint32_t)(e >> 32);
+                    }
+                } else {   // the page of rank t fills slot t
+                    const int l = (int)~(uint32_t)e, at = t < m && l >= 0 ? l : 0;   // (a word beside the row is ranked last)
+                    const int phys = lay.stage_bt ? bt_s[at] : ld_ca_s32(bt + at);
+                    const int rank = rank_in_list(pages, m, e, tid & 3);
+                    if (t < m && rank < np && (tid & 3) == 0) {
+                        put_page(rank, l, phys);
+                        p.routed_pages[unit * P + rank] = l;
                     }
                 }
             }
             __syncthreads();
-            if (!MMA) break;
+            if constexpr (!MMA) break;
             if (marks) {   // they rank first
                 marks = false;
                 const float best = key_to_float(win_key[0]);
                 if (best != best) {
-                    step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, 0.0f, true, g, ctl);
+                    if constexpr (MMA) step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, 0.0f, true, g);
                     continue;
                 }
             }
@@ -951,9 +953,10 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             const uint32_t next = ctl[kCtlNext];   // (0: no page, but a word beside the row)
             const float kth = key_to_float(win_key[np - 1]);
             if (next == 0u || kth - key_to_float(next) > slack) break;
-            step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, false, g, ctl);
+            if constexpr (MMA) step_settle_pages<THREADS, D>(p, bt, qraw, pages, m, kth - slack, false, g);
             slack = 0.0f;   // the scores are the fixed-order ones
         }
+        for (int t = np + tid; t < P; t += THREADS) p.routed_pages[unit * P + t] = -1;
         if constexpr (BY_POSITION) {
 #pragma unroll 1
             for (int t0 = 0; t0 < np; t0 += THREADS / 4) {
@@ -1016,7 +1019,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     };
     auto close_row = [&](int t) {
         const uint8_t* from = reinterpret_cast<const uint8_t*>(p.summaries) + ((long long)g * D + c * 8) * 2;
-        return ld_cg_16B(from + (unsigned long long)(unsigned)(t >= 0 ? (BY_POSITION ? win_phys[t] : tile_phys[t << tsh]) : 0) * (unsigned)(geo.n_kv_heads * 2 * D));
+        return ld_cg_16B(from + (unsigned long long)(unsigned)(t >= 0 ? win_phys[t] : 0) * (unsigned)(geo.n_kv_heads * 2 * D));
     };
     auto settle_score = [&](int t, const uint4& row) {   // (by all lanes of a warp)
         const float s = page_score<LPR>(qraw, row);
@@ -1254,7 +1257,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
                 if (key != 0u && bucket_of(key) == cut) {
                     const int slot = (o / TPL) * GROUPS + grp;
                     // by position; a page that the caller lists twice has tiles of its own
-                    const int order = (tile_pos[slot] >> 4 << 11) + slot * 16 + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
+                    const int order = (BY_POSITION ? 0 : tile_pos[slot] >> 4 << 11) + slot * 16 + (LPR == 8 ? 2 * c + o % TPL : LPR == 32 ? c >> 1 : c);
                     const uint32_t i = atomicAdd(&ctl[kCtlTokens], 1u);
                     tokens[i] = ((unsigned long long)key << 32) | (uint32_t)~order;
                     loc[i] = (uint32_t)(o * THREADS + tid);
@@ -1277,7 +1280,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
             __syncthreads();
         } else {
             cut = -1;
-            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, warp_stat, work, smem + lay.loc);
+            const uint32_t k = step_tokens_exact(tm, smem + lay.keys, n_own, tile_pos, nt, LPR, R, hist, smem + lay.misc, warp_stat, work,
+                                                 BY_POSITION ? nullptr : smem + lay.loc);
             if (tid == 0) ctl[kCtlOut] = k;
         }
     }
@@ -1531,7 +1535,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS) sparse_step_kernel(const __gr
     }
 }
 
-template <int THREADS, int FUSED, int D, bool FP8, int SOLVE = 0, int BLOCKS = 512 / THREADS>
+template <int THREADS, int FUSED, int D, bool FP8, int SOLVE = 0, int BLOCKS = 512 / THREADS, bool BY_POSITION = true>
 cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
 {
     static bool attr_done[kMaxDevices] = {};   // per template instance
@@ -1544,16 +1548,25 @@ cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
     // Frank-Wolfe 25.9 -> 21.5.
     if (SOLVE != 0 && (long long)p.geo.batch * p.geo.n_q_heads <= device_sm_count() && smem < 120 * 1024) smem = 120 * 1024;
     if (smem > 48 * 1024) {
-        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>, attr_done);
+        const cudaError_t e = allow_large_dynamic_smem(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS, BY_POSITION>, attr_done);
         if (e != cudaSuccess) return e;
     }
-    if constexpr (FUSED == 2 || FUSED == 4)
-        return launch_pdl_cluster(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>,
+    if constexpr (FUSED == 2 || FUSED == 4) {
+        return launch_pdl_cluster(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS, BY_POSITION>,
                                   dim3((unsigned)(p.geo.n_q_heads >> p.heads_shift << p.cluster_shift), (unsigned)p.geo.batch),
                                   dim3(THREADS), 1u << p.cluster_shift, smem, stream, p);
-    else
-        return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS>,
+    } else
+        return launch_pdl(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS, BY_POSITION>,
                           dim3((unsigned)p.geo.n_q_heads, (unsigned)p.geo.batch), dim3(THREADS), smem, stream, p);
+}
+
+// in the order of the tiles that the launch has
+template <int THREADS, int FUSED, int D, bool FP8, int BLOCKS = 512 / THREADS>
+cudaError_t launch_step_order(const StepParams& p, cudaStream_t stream)
+{
+    if constexpr (step_order_open(THREADS, D, FP8))
+        if (!p.by_position) return launch_step_variant<THREADS, FUSED, D, FP8, 0, BLOCKS, false>(p, stream);
+    return launch_step_variant<THREADS, FUSED, D, FP8, 0, BLOCKS>(p, stream);
 }
 
 template <int D, bool FP8>
@@ -1563,7 +1576,7 @@ cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t st
     if (p.summaries && !fused) {
         if (threads == 256 && p.scan_mma) return launch_step_variant<256, 4, D, FP8>(p, stream);
         if (threads != 512) return cudaErrorInvalidValue;
-        return p.scan_mma ? launch_step_variant<512, 4, D, FP8>(p, stream) : launch_step_variant<512, 2, D, FP8>(p, stream);
+        return p.scan_mma ? launch_step_variant<512, 4, D, FP8>(p, stream) : launch_step_order<512, 2, D, FP8>(p, stream);
     }
     // Five blocks per SM at 96 registers against four at 128, which make a unit 5 - 10 % faster: five
     // where they save a wave of blocks, and from three waves of four on, where units in flight count for more.  Microseconds
@@ -1581,14 +1594,11 @@ cudaError_t launch_step_family(const StepParams& p, int threads, cudaStream_t st
         if (threads != 128) return cudaErrorInvalidValue;
         return five_blocks ? launch_step_variant<128, 3, D, FP8, 0, 5>(p, stream) : launch_step_variant<128, 3, D, FP8>(p, stream);
     }
-    if (threads == 128 && fused && five_blocks) return launch_step_variant<128, 1, D, FP8, 0, 5>(p, stream);
+    if (threads == 128 && fused && five_blocks) return launch_step_order<128, 1, D, FP8, 5>(p, stream);
 #define VSA_STEP_CASE(T)                                                                    \
-    if (threads == T) {                                                                     \
-        if (fused) return launch_step_variant<T, 1, D, FP8>(p, stream);                     \
-        if constexpr (!step_by_position(T, D, FP8))                                         \
-            if (!p.by_position) return launch_step_variant<T, 0, D, FP8>(p, stream);        \
-        return launch_step_variant<T, 5, D, FP8>(p, stream);                                \
-    }
+    if (threads == T)                                                                       \
+        return fused ? launch_step_order<T, 1, D, FP8>(p, stream)                           \
+                     : launch_step_order<T, 0, D, FP8>(p, stream);
     VSA_STEP_CASE(512)
     VSA_STEP_CASE(256)
     VSA_STEP_CASE(128)
