@@ -540,7 +540,8 @@ int vsa_cp_partial_readout(const vsa_shape_t* shape, const void* v_cache, const 
 /*
  * Where a step scores the pages of a shape on the current device: by a kernel ahead of the fused sparse pass (three
  * launches a step) or inside it (two), in the fixed order or on the tensor cores with the near ties settled
- * in the fixed order.  The results do not depend on it.
+ * in the fixed order.  The results do not depend on it.  (A stream that has a part of the device's SMs, too few in one
+ * place for the clusters of a pass that scores the pages itself, has them scored ahead.)
  *   step: VSA_STEP_CLOSED for vsa_decode_step, _timed and _host, VSA_STEP_FP8 for vsa_decode_step_fp8,
  *   VSA_STEP_SOLVE for vsa_decode_step_entropic and _frank_wolfe.  Returns VSA_STEP_SCAN_* or a VSA_ERR_* code.
  */

@@ -221,7 +221,7 @@ int vsa_step_scan(const vsa_shape_t* shape, int32_t P, int32_t K_c, int step)
     if (!vsa::sparse_shared_memory_fits(g, P, K_c, true, solve, false)) return VSA_ERR_UNSUPPORTED_SHAPE;
     static_assert((int)vsa::StepScan::Ahead == VSA_STEP_SCAN_AHEAD && (int)vsa::StepScan::AheadMma == VSA_STEP_SCAN_AHEAD_MMA &&
                   (int)vsa::StepScan::Inside == VSA_STEP_SCAN_INSIDE && (int)vsa::StepScan::InsideMma == VSA_STEP_SCAN_INSIDE_MMA, "one order");
-    return (int)vsa::step_scan(g, P, K_c, fp8, solve);
+    return (int)vsa::step_scan(g, P, K_c, fp8, solve ? 1 : 0, nullptr);
 }
 
 int vsa_build_page_summaries(const vsa_shape_t* shape, const void* k_cache, const int32_t* block_table,
@@ -555,7 +555,7 @@ static int decode_step_impl(const vsa_shape_t* shape, const void* q, const void*
             ev[i] = (cudaEvent_t)events[i];
         }
     void* ws_dense = (char*)ws + step_route_part(g);
-    const vsa::StepScan scan = cert ? vsa::StepScan::Ahead : vsa::step_scan(g, P, K_c, fp8, solve != nullptr);
+    const vsa::StepScan scan = cert ? vsa::StepScan::Ahead : vsa::step_scan(g, P, K_c, fp8, solve ? solver_kind : 0, st);
     if (ev[0] && cudaEventRecord(ev[0], st) != cudaSuccess) return VSA_ERR_CUDA;
     if (scan == vsa::StepScan::Inside || scan == vsa::StepScan::InsideMma) {
         // two launches: the sparse pass scores the pages itself, and the dense pass makes the list from its flags

@@ -134,7 +134,7 @@ static cudaError_t launch_step_of(const StepParams& p, int threads, bool fp8, in
     return launch_step(p, threads, stream);
 }
 
-// Where the step of a shape scores its pages, and its parameters if that is inside
+// Where the step of a shape scores its pages when it has the whole device, and its parameters if that is inside
 struct ScanRule {
     StepScan scan;
     StepParams inside;
@@ -152,9 +152,22 @@ static ScanRule scan_rule(const Geometry& g, int P, int K_c, int threads, bool f
     return {mma ? StepScan::AheadMma : StepScan::Ahead, {}};
 }
 
-StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, bool solve)
+StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, int solver, cudaStream_t stream)
 {
-    return scan_rule(g, P, K_c, solve ? 256 : step_threads(g, P), fp8, solve).scan;
+    const int threads = solver ? 256 : step_threads(g, P);
+    ScanRule rule = scan_rule(g, P, K_c, threads, fp8, solver);
+    if (rule.scan == StepScan::Ahead || rule.scan == StepScan::AheadMma) return rule.scan;
+    // The rule counts the SMs of one chip.  What a stream really has (another chip's GPCs, a green context, a share of the SMs
+    // under MPS) may hold fewer clusters at once, or none, and then there would be no launch: the scan ahead.
+    int n = 0;
+    const uint16_t any = 0;
+    rule.inside.summaries = &any;   // (of the kernels that scan)
+    rule.inside.active_clusters = &n;
+    if (launch_step_of(rule.inside, threads, fp8, solver, stream) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return StepScan::Ahead;
+    }
+    return (long long)n * scan_heads(g) >= (long long)g.batch * g.n_q_heads ? rule.scan : StepScan::Ahead;
 }
 
 bool sparse_shared_memory_fits(const Geometry& g, int P, int K_c, bool fused, bool solve, bool cert, int P_super)

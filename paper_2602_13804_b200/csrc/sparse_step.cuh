@@ -63,6 +63,7 @@ struct StepParams {
     int heads_shift;            // log2(heads of a cluster)
     int scan_per_sm;            // blocks of such a launch that share an SM
     bool scan_mma;              // scores by MMAs (page_mma.cuh)
+    int* active_clusters;       // not nullptr: no launch, but active_clusters() of it
     bool by_position;           // tiles in the order of positions instead of scores (see BY_POSITION)
     int32_t* flags;             // with summaries: fallback flag of every unit, from which the dense pass makes the list
     int32_t* tickets;           // with summaries: the dense pass's tickets, cleared here
@@ -1552,6 +1553,9 @@ cudaError_t launch_step_variant(const StepParams& p, cudaStream_t stream)
         if (e != cudaSuccess) return e;
     }
     if constexpr (FUSED == 2 || FUSED == 4) {
+        if (p.active_clusters)
+            return active_clusters(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS, BY_POSITION>, dim3(THREADS), 1u << p.cluster_shift, smem,
+                                   stream, p.active_clusters);
         return launch_pdl_cluster(sparse_step_kernel<THREADS, FUSED, D, FP8, SOLVE, BLOCKS, BY_POSITION>,
                                   dim3((unsigned)(p.geo.n_q_heads >> p.heads_shift << p.cluster_shift), (unsigned)p.geo.batch),
                                   dim3(THREADS), 1u << p.cluster_shift, smem, stream, p);

@@ -49,6 +49,25 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// How many clusters of `cluster` blocks of the kernel the SMs behind `stream` hold at once (0.2 us): a cluster needs its SMs in one
+// GPC, and a stream may have a part of the device only.
+template <typename... KArgs>
+inline cudaError_t active_clusters(void (*kernel)(KArgs...), dim3 block, unsigned cluster, size_t smem, cudaStream_t stream, int* n)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
+}
+
 // Ordinary kernel launch: starts when everything before it in the stream has finished.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_in_order(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
@@ -215,9 +234,9 @@ cudaError_t launch_sparse(const Geometry& g, const void* q, const void* k_cache,
 // scan_summaries != nullptr and page_scores nullptr (step_scan() Inside or InsideMma): the kernel scores the pages itself, writes
 // every unit's fallback flag instead of the list and clears the dense pass's tickets.
 // Where the step of a shape scores its pages: by a kernel ahead of the sparse pass, in the fixed order or by MMAs, or inside it
-// (the values are those of vsa.h's VSA_STEP_SCAN_*)
+// (the values are those of vsa.h's VSA_STEP_SCAN_*), for a launch in `stream`.  solver: 0 closed form, 1 entropic, 2 Frank-Wolfe
 enum class StepScan : int { Ahead = 0, AheadMma = 1, Inside = 2, InsideMma = 3 };
-StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, bool solve);
+StepScan step_scan(const Geometry& g, int P, int K_c, bool fp8, int solver, cudaStream_t stream);
 // k_scale / v_scale != nullptr: k_cache / v_cache hold e4m3 bytes, value = byte * scale[pool page][KV head]
 // (closed-form family, head dimension 128).
 // tl_summaries != nullptr: the two-level front end - page_scores then holds the scores of the super-pages'
