@@ -123,6 +123,15 @@ __device__ __forceinline__ uint4 ld_cg_16B(const void* p)
     return v;
 }
 
+// What an earlier kernel may have been writing when this one started: an ordinary load, whose value the wait for that kernel
+// orders, of what is read once.
+__device__ __forceinline__ uint4 ld_once_16B(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 __device__ __forceinline__ void prefetch_L2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ int ld_ca_s32(const int32_t* p)
