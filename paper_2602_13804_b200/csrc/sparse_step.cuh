@@ -7,7 +7,7 @@
 // barriers on its longest thread and, since every instruction is executed once or twice per launch, the size
 // of the code (instruction fetch: an SM caches about 2000 instructions, straight code that is not there takes three or more
 // cycles each).  Hence: loops that run from memory instead of unrolled register arrays, one template instance for every
-// table width, P and K_c, the rare exact fallbacks out of line, twelve barriers.
+// table width, P and K_c, the rare exact fallbacks out of line, one barrier between phases.
 //   * Page scores are staged in shared memory (16-byte copies, any table width).  In every warp the r-th largest
 //     of the lanes' maxima, r = ceil(P / warps), has r scores at or above it; the smallest of these over the warps
 //     bounds the P-th best score from below and leaves about 1.6 P scores, which are listed and ranked exactly.
@@ -22,9 +22,10 @@
 // 83.0 -> 81.5 at batch 16, T = 128k; with scores in registers where a thread has one chunk (and the append's reads side by
 // side), 14.4 -> 14.2 at batch 1, T = 4k, the append included.
 // What bounds it:
-// no unit of the SM, but the chain of phases.  Counters at P = 32, K_c = 256: 20k warp instructions per unit of 256
-// threads, 0.41 of the issue slots at two units per SM (256 units), 0.38 at four of 128 threads (512 units); at P = 64,
-// K_c = 512 34k per unit, 0.52 at five per SM (2048 units).  The waits are for loads from L2, then for shared memory.
+// no unit of the SM, but the chain of phases, until there are units enough to fill one another's waits.  Counters at P = 32, K_c = 256: 20k
+// warp instructions per unit of 256 threads and 10k for the scan of its cluster, 0.40 of the issue slots at two units per SM (256
+// units, 32k); 16k at four units of 128 threads, 0.45 (512 units of 8k); at P = 64, K_c = 512 35k, 0.62 at five (2048 units).  The waits are for
+// the results of instructions, for shared memory and for loads from L2, in this order.
 #pragma once
 
 #include <limits.h>
